@@ -197,13 +197,14 @@ __global__ void __launch_bounds__(256) axis_kernel(const AxisArgs a) {
         __syncthreads();
         if (threadIdx.x == 0) s_last = (atomicAdd(a.ticket, 1u) == gridDim.x - 1) ? 1u : 0u;
         __syncthreads();
-        if (s_last && threadIdx.x == 0) {
+        if (s_last && threadIdx.x < 32) {
             __threadfence();
-            double f = 0.0;
-            for (unsigned q = 0; q < gridDim.x; ++q) f = __dadd_rn(f, __ldcg(a.flux_part + q));
-            *a.flux_cum = __dadd_rn(__ldcg(a.flux_cum), __dmul_rn(f, a.vol));
-            __threadfence();
-            *a.ticket = 0u;
+            const double f = fold_parts(a.flux_part, gridDim.x, threadIdx.x);
+            if (threadIdx.x == 0) {
+                *a.flux_cum = __dadd_rn(__ldcg(a.flux_cum), __dmul_rn(f, a.vol));
+                __threadfence();
+                *a.ticket = 0u;
+            }
         }
     }
 }
