@@ -847,13 +847,17 @@ void default_plan(dirac_grid *g) {
         // storage (bandwidth-bound), one in FP64 (bound by the FP64 pipe: the second step's halo would cost)
         int K3 = 1;
         if (!strang(g) && (pp == 0 || field_on(g))) K3 = k == 2 ? 2 : (k == 1 ? 1 : (g->fp32 ? 2 : 1));
-        make_plan(g, K3, pp > 0 ? pp : 2, 4, 16);
+        // FP64 two-pass plan: 32 warps an SM of segments (8.75 against 8.2 G at 256^3 with 16)
+        make_plan(g, K3, pp > 0 ? pp : 2, 4, g->fp32 ? 16 : 32);
         return;
     }
     if (sweep_mode(g) == 4) {
-        // FP64 with the field's phase matrix spills at two points per lane
-        const int P = pp == 1 || pp == 2 ? pp : ((field_on(g) && !g->fp32) ? 1 : 2);
-        make_plan(g, 1, P, 4, 8);
+        // FP64, K = 2, no field: one point a lane and 24 warps an SM of segments, whose sweeps fill the FP64 and the
+        // integer pipe (9.4 against 8.7 G point-steps/s at 2048^2); elsewhere two (with the field's phase matrix
+        // 4.5 against 4.2 G)
+        const bool one = !g->fp32 && char_shift(g) == 2 && !field_on(g);
+        const int P = pp == 1 || pp == 2 ? pp : (one ? 1 : 2);
+        make_plan(g, 1, P, 4, one && P == 1 ? 24 : 8);
         return;
     }
     const int mode = sweep_mode(g);
@@ -867,10 +871,12 @@ void default_plan(dirac_grid *g) {
         make_plan(g, K, P, 4, 16);
         return;
     }
-    int K = g->fp32 ? 2 : 1, P = (g->fp32 || mode >= 2) ? 2 : 4;
+    // FP64: one point a lane, 16 warps an SM (four blocks of 128 registers): the sweeps' pairs split over the FP64 and
+    // the integer pipe need warps to overlap (2048^2: 13.1 against 10.0 G with two points and 8 warps; second order
+    // 6.35 against 5.1; in a laser field 7.6 against 6.4)
+    int K = g->fp32 ? 2 : 1, P = g->fp32 ? 2 : 1;
     if (mode == 3 || mode == 5) K = 1;  // measured: the field's phase matrix makes k = 2 register-bound
     if (mode == 2) K = g->fp32 ? 2 : 1;  // FP32 second order: two steps per pass with the history in shared memory
-    if (mode == 5 && !g->fp32) P = 1;  // the FP64 two-level matrix step spills at P = 2
     if (k > 0) K = k;
     if (pp > 0) P = pp;
     if (!sweep_supported(g->fp32, mode, K, P)) P = sweep_supported(g->fp32, mode, K, 4) ? 4 : 2;
@@ -881,7 +887,7 @@ void default_plan(dirac_grid *g) {
     // FP32 P = 2 with the sweep history in shared memory: four blocks per SM fit (first order two steps per
     // pass, second order one)
     const bool four = g->fp32 && P == 2 && ((mode == 0 && K == 2) || (mode == 2 && K == 1));
-    make_plan(g, K, P, 4, g->fp32 ? (four ? 16 : 12) : 8);
+    make_plan(g, K, P, 4, g->fp32 ? (four ? 16 : 12) : (P == 1 ? 16 : 8));
 }
 
 }  // namespace
@@ -1505,25 +1511,25 @@ dirac_status dirac_autotune(dirac_grid *g) {
         cands.push_back({2, 2, 4, 16, 16});  // two steps per fused pass
     } else if (sweep_mode(g) == 4) {
         for (int P : {1, 2})
-            for (int wsm : {4, 8, 12, 16}) cands.push_back({1, P, 4, wsm});
+            for (int wsm : {4, 8, 12, 16, 24}) cands.push_back({1, P, 4, wsm});
     } else if (sweep_mode(g) == 3 || sweep_mode(g) == 5) {
         const int KP[][2] = {{1, 1}, {1, 2}, {2, 2}};
         for (auto &kp : KP)
             if (sweep_supported(g->fp32, sweep_mode(g), kp[0], kp[1]))
-                for (int wsm : {4, 8, 12}) cands.push_back({kp[0], kp[1], 4, wsm});
+                for (int wsm : {4, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else if (strang(g)) {
         const int KP[][2] = {{1, 1}, {1, 2}, {1, 4}, {2, 2}};
         for (auto &kp : KP)
             if (sweep_supported(g->fp32, 2, kp[0], kp[1]))
-                for (int wsm : {4, 8, 12}) cands.push_back({kp[0], kp[1], 4, wsm});
+                for (int wsm : {4, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else if (g->fp32) {
         const int KP[][2] = {{1, 2}, {1, 4}, {2, 2}, {2, 4}, {4, 2}};
         for (auto &kp : KP)
             for (int wsm : {8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else {
-        const int KP[][2] = {{1, 2}, {1, 4}, {2, 2}};
+        const int KP[][2] = {{1, 1}, {1, 2}, {2, 2}};
         for (auto &kp : KP)
-            for (int wsm : {4, 8, 12}) cands.push_back({kp[0], kp[1], 4, wsm});
+            for (int wsm : {8, 12, 16, 24}) cands.push_back({kp[0], kp[1], 4, wsm});
     }
     // save state and counters
     const size_t bytes = (size_t)g->ncells * 8 * g->elem;

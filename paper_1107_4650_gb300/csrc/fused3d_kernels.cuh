@@ -131,8 +131,8 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
             for (int c = 0; c < 4; ++c) ring[j][c] = ring[j + 1][c];
         if (k + LA <= z_end) load_row(k + LA, ring[LA - 1]);
         // x characteristics and the x sweep (neighbours by shuffle; lanes 0 and 31 are halo cells)
-        const Cx<T> u14 = cadd(st[0], st[3]), w14 = csub(st[0], st[3]);
-        const Cx<T> u23 = cadd(st[1], st[2]), w23 = csub(st[1], st[2]);
+        Cx<T> u14, w14, u23, w23;
+        x_chars<false>(st, u14, w14, u23, w23);
         if (face_lane && k >= z_begin && k < z_end) {
             using F = typename FaceAcc<T>::type;
             const F v = (x == face - 1) ? face_sq(u14, u23) : -face_sq(w14, w23);
@@ -144,34 +144,27 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
         }
         const Cx<T> lu14 = shfl_c(u14, (lane + 31) & 31), lu23 = shfl_c(u23, (lane + 31) & 31);
         const Cx<T> rw14 = shfl_c(w14, (lane + 1) & 31), rw23 = shfl_c(w23, (lane + 1) & 31);
-        const Cx<T> b0 = cadd(lu14, rw14), b3 = csub(lu14, rw14);
-        const Cx<T> b1 = cadd(lu23, rw23), b2 = csub(lu23, rw23);
-        // y characteristics (Eq. sol_dis_2): "+y" movers (b1 - i b4, b2 + i b3), "-y" movers (b1 + i b4, b2 - i b3)
+        Cx<T> b4[4], U14, W14, U23, W23;
+        x_join<false>(lu14, rw14, lu23, rw23, b4);
+        y_chars<false>(b4, U14, W14, U23, W23);
         Cx<T> *buf = ych + (size_t)((k - z_begin + 1) & 1) * (W * 4 * 32);
-        buf[(w * 4 + 0) * 32 + lane] = csub_ib(b0, b3);
-        buf[(w * 4 + 1) * 32 + lane] = cadd_ib(b1, b2);
-        buf[(w * 4 + 2) * 32 + lane] = cadd_ib(b0, b3);
-        buf[(w * 4 + 3) * 32 + lane] = csub_ib(b1, b2);
+        buf[(w * 4 + 0) * 32 + lane] = U14;
+        buf[(w * 4 + 1) * 32 + lane] = U23;
+        buf[(w * 4 + 2) * 32 + lane] = W14;
+        buf[(w * 4 + 3) * 32 + lane] = W23;
         __syncthreads();
         if (owned_row) {
             // y sweep of row y: "+y" movers of row y-1, "-y" movers of row y+1 (x2 again: 4x the state)
             const Cx<T> U14 = buf[((w - 1) * 4 + 0) * 32 + lane], U23 = buf[((w - 1) * 4 + 1) * 32 + lane];
             const Cx<T> W14 = buf[((w + 1) * 4 + 2) * 32 + lane], W23 = buf[((w + 1) * 4 + 3) * 32 + lane];
-            Cx<T> s[4];
-            s[0] = cadd(U14, W14);
-            s[3] = cmul_i(csub(U14, W14));
-            s[1] = cadd(U23, W23);
-            s[2] = cmul_mi(csub(U23, W23));
-            // z sweep (Eq. sol_dis_3): +z movers (s1+s3, s2-s4) of plane k-2, -z movers (s1-s3, s2+s4) of plane k
-            const Cx<T> U13 = cadd(s[0], s[2]), U24 = csub(s[1], s[3]);
-            const Cx<T> W13 = csub(s[0], s[2]), W24 = cadd(s[1], s[3]);
+            Cx<T> s[4], U13, W13, U24, W24;
+            y_join<false>(U14, W14, U23, W23, s);
+            // z sweep (Eq. sol_dis_3): +z movers of plane k-2, -z movers of plane k
+            z_chars<false>(s, U13, W13, U24, W24);
             const ZI zo = k - 1;
             if (zo >= z_begin && zo < z_end) {
                 Cx<T> o[4];
-                o[0] = cadd(UA[0], W13);
-                o[2] = csub(UA[0], W13);
-                o[1] = cadd(UA[1], W24);
-                o[3] = csub(W24, UA[1]);
+                z_join<false>(UA[0], W13, UA[1], W24, o);
                 const Cx<T> qu = a.full_table ? tu : pu, qd = a.full_table ? td : pd;
                 if (FIELD) {
                     Cx<T> m6[FIELD ? 6 : 1];
@@ -291,39 +284,31 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A
     };
     // x sweep of a row held one cell per lane (valid where both neighbours are); face terms of its input
     auto xsweep = [&](const Cx<T> s[4], Cx<T> o[4], T &acc, bool count) {
-        const Cx<T> u14 = cadd(s[0], s[3]), w14 = csub(s[0], s[3]);
-        const Cx<T> u23 = cadd(s[1], s[2]), w23 = csub(s[1], s[2]);
+        Cx<T> u14, w14, u23, w23;
+        x_chars<false>(s, u14, w14, u23, w23);
         if (count && fl_u) acc = Ar<T>::add(acc, face_term(u14, u23));
         if (count && fl_w) acc = Ar<T>::sub(acc, face_term(w14, w23));
         const Cx<T> lu14 = shfl_c(u14, (lane + 31) & 31), lu23 = shfl_c(u23, (lane + 31) & 31);
         const Cx<T> rw14 = shfl_c(w14, (lane + 1) & 31), rw23 = shfl_c(w23, (lane + 1) & 31);
-        o[0] = cadd(lu14, rw14);
-        o[3] = csub(lu14, rw14);
-        o[1] = cadd(lu23, rw23);
-        o[2] = csub(lu23, rw23);
+        x_join<false>(lu14, rw14, lu23, rw23, o);
     };
     // y characteristics (Eq. sol_dis_2): "+y" movers (b1 - i b4, b2 + i b3), "-y" movers (b1 + i b4, b2 - i b3)
     auto ywrite = [&](Cx<T> *buf, const Cx<T> b4[4]) {
-        buf[(w * 4 + 0) * 32 + lane] = csub_ib(b4[0], b4[3]);
-        buf[(w * 4 + 1) * 32 + lane] = cadd_ib(b4[1], b4[2]);
-        buf[(w * 4 + 2) * 32 + lane] = cadd_ib(b4[0], b4[3]);
-        buf[(w * 4 + 3) * 32 + lane] = csub_ib(b4[1], b4[2]);
+        Cx<T> U14, W14, U23, W23;
+        y_chars<false>(b4, U14, W14, U23, W23);
+        buf[(w * 4 + 0) * 32 + lane] = U14;
+        buf[(w * 4 + 1) * 32 + lane] = U23;
+        buf[(w * 4 + 2) * 32 + lane] = W14;
+        buf[(w * 4 + 3) * 32 + lane] = W23;
     };
     // y sweep from rows w - 1 and w + 1, z sweep against the history (output plane = input plane - 1), phase
     auto yz_phase = [&](const Cx<T> *buf, Cx<T> (&HA)[2], Cx<T> (&HB)[2], Cx<T> qu, Cx<T> qd, int st, Cx<T> o[4]) {
         const Cx<T> U14 = buf[((w - 1) * 4 + 0) * 32 + lane], U23 = buf[((w - 1) * 4 + 1) * 32 + lane];
         const Cx<T> W14 = buf[((w + 1) * 4 + 2) * 32 + lane], W23 = buf[((w + 1) * 4 + 3) * 32 + lane];
-        Cx<T> s[4];
-        s[0] = cadd(U14, W14);
-        s[3] = cmul_i(csub(U14, W14));
-        s[1] = cadd(U23, W23);
-        s[2] = cmul_mi(csub(U23, W23));
-        const Cx<T> U13 = cadd(s[0], s[2]), U24 = csub(s[1], s[3]);
-        const Cx<T> W13 = csub(s[0], s[2]), W24 = cadd(s[1], s[3]);
-        o[0] = cadd(HA[0], W13);
-        o[2] = csub(HA[0], W13);
-        o[1] = cadd(HA[1], W24);
-        o[3] = csub(W24, HA[1]);
+        Cx<T> s[4], U13, W13, U24, W24;
+        y_join<false>(U14, W14, U23, W23, s);
+        z_chars<false>(s, U13, W13, U24, W24);
+        z_join<false>(HA[0], W13, HA[1], W24, o);
         HA[0] = HB[0];
         HA[1] = HB[1];
         HB[0] = U13;

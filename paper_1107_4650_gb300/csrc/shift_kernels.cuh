@@ -22,6 +22,9 @@ namespace dirac {
 // FIELD: a uniform vector potential; the phase is U(step) exp(-i V dt) applied as in the one-cell field mode.
 template <typename T, int S, int P, bool FIELD>
 __device__ __forceinline__ void shift_warp(const SweepArgs &a, const int64_t wid, const int lane) {
+    // FP64 pairs over two pipes: with one point a lane at S = 2 (9.4 against 8.7 G at 2048^2, 24 warps an SM); the
+    // longer histories of S = 3 and 4 leave no registers for it (8.3 and 5.0 against 8.4 and 8.1 G)
+    constexpr bool HY = P == 1 && S == 2;
     const int64_t seg = wid / a.nstrips;
     const int64_t strip = wid - seg * a.nstrips;
     const int64_t nx = a.nx, nr = a.nr;
@@ -115,12 +118,7 @@ __device__ __forceinline__ void shift_warp(const SweepArgs &a, const int64_t wid
             // point group, lanes >= 32 - S the next one)
             Cx<T> u14[P], u23[P], w14[P], w23[P];
 #pragma unroll
-            for (int j = 0; j < P; ++j) {
-                u14[j] = cadd(st[j][0], st[j][3]);
-                w14[j] = csub(st[j][0], st[j][3]);
-                u23[j] = cadd(st[j][1], st[j][2]);
-                w23[j] = csub(st[j][1], st[j][2]);
-            }
+            for (int j = 0; j < P; ++j) x_chars<HY>(st[j], u14[j], w14[j], u23[j], w23[j]);
             Cx<T> pu14[P], pu23[P], nw14[P], nw23[P];
 #pragma unroll
             for (int j = 0; j < P; ++j) {
@@ -163,19 +161,13 @@ __device__ __forceinline__ void shift_warp(const SweepArgs &a, const int64_t wid
                 const Cx<T> rw14 = (lane >= 32 - S) ? nw14[jn] : nw14[j];
                 const Cx<T> rw23 = (lane >= 32 - S) ? nw23[jn] : nw23[j];
                 // x sweep (Eq. sol_dis_1 with neighbours at -+S), x2
-                const Cx<T> b0 = cadd(lu14, rw14);
-                const Cx<T> b3 = csub(lu14, rw14);
-                const Cx<T> b1 = cadd(lu23, rw23);
-                const Cx<T> b2 = csub(lu23, rw23);
-                // z sweep (Eq. sol_dis_3 with rows -+S): +z movers (b1+b3, b2-b4), -z movers (b1-b3, b2+b4)
-                const Cx<T> U13 = cadd(b0, b2), U24 = csub(b1, b3);
+                Cx<T> b[4], U13, W13, U24, W24;
+                x_join<HY>(lu14, rw14, lu23, rw23, b);
+                // z sweep (Eq. sol_dis_3 with rows -+S)
+                z_chars<HY>(b, U13, W13, U24, W24);
                 if (out_row) {
-                    const Cx<T> W13 = csub(b0, b2), W24 = cadd(b1, b3);
                     Cx<T> o[4];
-                    o[0] = cadd(UH[t][j][0], W13);
-                    o[2] = csub(UH[t][j][0], W13);
-                    o[1] = cadd(UH[t][j][1], W24);
-                    o[3] = csub(W24, UH[t][j][1]);
+                    z_join<HY>(UH[t][j][0], W13, UH[t][j][1], W24, o);
                     Cx<T> qu, qd;
                     if (a.full_table) {
                         load_tab(tab + (q * nx + xl[j]) * 4, qu, qd);

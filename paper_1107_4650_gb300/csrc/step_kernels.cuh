@@ -25,25 +25,8 @@
 #include <atomic>
 #include <type_traits>
 
+#include "butterfly.cuh"
 #include "dirac_internal.cuh"
-
-// Compile-time tunables of the 2-D step kernels: resident 4-warp blocks per SM the register budget is fitted to
-// (fixed point k = 1, P = 1; FP32 k = 2, P = 2; FP64 k = 1, P = 2 and 4), and rows per loop iteration of the
-// fixed-point kernel.  Fixed point: 4 blocks with two rows per iteration fit 128 registers without spilling (33.1
-// against 26.7 G point-steps/s at 150 registers and 3 blocks, 2048^2).  FP32 k = 2, P = 2 (and the second-order
-// step at k = 1, P = 2): 4 blocks fit once the z sweep's history lives in shared memory (HistSmem below).
-#ifndef FX_MIN_BLOCKS
-#define FX_MIN_BLOCKS 4
-#endif
-#ifndef F32_MIN_BLOCKS
-#define F32_MIN_BLOCKS 4
-#endif
-#ifndef F64_MIN_BLOCKS
-#define F64_MIN_BLOCKS 1
-#endif
-#ifndef FX_ROW_UNROLL
-#define FX_ROW_UNROLL 2
-#endif
 
 namespace dirac {
 
@@ -97,6 +80,57 @@ template <typename T> __device__ __forceinline__ Cx<T> cadd_ib(Cx<T> a, Cx<T> b)
 }
 template <typename T> __device__ __forceinline__ Cx<T> csub_ib(Cx<T> a, Cx<T> b) {
     return {Ar<T>::add(a.re, b.im), Ar<T>::sub(a.im, b.re)};
+}
+// Two pairs: s = a + b, d = a - b for (a0, b0) and (a1, b1).  HY: FP64 pairs over the FP64 and the integer pipe
+// (butterfly.cuh), the same bits.
+template <bool HY, typename T>
+__device__ __forceinline__ void butterfly2(Cx<T> a0, Cx<T> b0, Cx<T> a1, Cx<T> b1, Cx<T> &s0, Cx<T> &d0, Cx<T> &s1, Cx<T> &d1) {
+    if constexpr (HY && std::is_same<T, double>::value) {
+        butterfly(a0.re, b0.re, s0.re, d0.re);
+        butterfly(a0.im, b0.im, s0.im, d0.im);
+        butterfly(a1.re, b1.re, s1.re, d1.re);
+        butterfly(a1.im, b1.im, s1.im, d1.im);
+    } else {
+        s0 = cadd(a0, b0);
+        d0 = csub(a0, b0);
+        s1 = cadd(a1, b1);
+        d1 = csub(a1, b1);
+    }
+}
+// x characteristics of a point: u14 = 1 + 4, w14 = 1 - 4, u23 = 2 + 3, w23 = 2 - 3
+template <bool HY, typename T>
+__device__ __forceinline__ void x_chars(const Cx<T> s[4], Cx<T> &u14, Cx<T> &w14, Cx<T> &u23, Cx<T> &w23) {
+    butterfly2<HY>(s[0], s[3], s[1], s[2], u14, w14, u23, w23);
+}
+// x sweep from the left cell's u and the right cell's w (twice the swept point)
+template <bool HY, typename T> __device__ __forceinline__ void x_join(Cx<T> u14, Cx<T> w14, Cx<T> u23, Cx<T> w23, Cx<T> o[4]) {
+    butterfly2<HY>(u14, w14, u23, w23, o[0], o[3], o[1], o[2]);
+}
+// y characteristics (Eq. sol_dis_2): "+y" movers U14 = 1 - i 4, U23 = 2 + i 3, "-y" movers W14 = 1 + i 4, W23 = 2 - i 3
+template <bool HY, typename T>
+__device__ __forceinline__ void y_chars(const Cx<T> b[4], Cx<T> &U14, Cx<T> &W14, Cx<T> &U23, Cx<T> &W23) {
+    Cx<T> s0, d0, s1, d1;
+    butterfly2<HY>(b[0], Cx<T>{b[3].im, b[3].re}, b[1], Cx<T>{b[2].im, b[2].re}, s0, d0, s1, d1);
+    U14 = {s0.re, d0.im};
+    W14 = {d0.re, s0.im};
+    U23 = {d1.re, s1.im};
+    W23 = {s1.re, d1.im};
+}
+// y sweep from the "+y" movers of the row below and the "-y" movers of the row above (twice the swept point)
+template <bool HY, typename T> __device__ __forceinline__ void y_join(Cx<T> U14, Cx<T> W14, Cx<T> U23, Cx<T> W23, Cx<T> o[4]) {
+    Cx<T> d0, d1;
+    butterfly2<HY>(U14, W14, U23, W23, o[0], d0, o[1], d1);
+    o[3] = {-d0.im, d0.re};
+    o[2] = {d1.im, -d1.re};
+}
+// z characteristics (Eq. sol_dis_3): "+z" movers U13 = 1 + 3, U24 = 2 - 4, "-z" movers W13 = 1 - 3, W24 = 2 + 4
+template <bool HY, typename T>
+__device__ __forceinline__ void z_chars(const Cx<T> b[4], Cx<T> &U13, Cx<T> &W13, Cx<T> &U24, Cx<T> &W24) {
+    butterfly2<HY>(b[0], b[2], b[1], b[3], U13, W13, W24, U24);
+}
+// z sweep from the "+z" movers of the row below and the "-z" movers of the row above (twice the swept point)
+template <bool HY, typename T> __device__ __forceinline__ void z_join(Cx<T> U13, Cx<T> W13, Cx<T> U24, Cx<T> W24, Cx<T> o[4]) {
+    butterfly2<HY>(U13, W13, W24, U24, o[0], o[2], o[1], o[3]);
 }
 // i z and -i z (exact)
 template <typename T> __device__ __forceinline__ Cx<T> cmul_i(Cx<T> a) { return {-a.im, a.re}; }
@@ -215,18 +249,22 @@ __device__ __forceinline__ int64_t pmod(int64_t a, int64_t n) {
 // alternate instead of moving, which pays where the loop body is short).
 template <typename T, int K, int MODE> struct RowUnroll {
     static constexpr bool FX = sizeof(T) == 8 && (T)0.5 == (T)0;  // the int64 fixed-point state
-    static constexpr int value = (sizeof(T) == 4 && K == 1 && MODE == 0) ? 2 : ((FX && K == 1 && MODE == 0) ? FX_ROW_UNROLL : 1);
+    static constexpr int value = (sizeof(T) == 4 && K == 1 && MODE == 0) ? 2 : ((FX && K == 1 && MODE == 0) ? 2 : 1);
 };
+template <typename T> struct IsFx { static constexpr bool value = std::is_same<T, long long>::value; };  // int64 fixed point
+template <typename T> struct IsF64 { static constexpr bool value = std::is_same<T, double>::value; };
 // Whether the z sweep's history (the "+" sums of the two previous rows per level) lives in the warp's shared
-// memory instead of registers, one slot per row parity so that nothing moves.  Measured for the single-grid
-// FP32 kernels with P = 2: at k = 2 the registers it frees let four blocks (16 warps) per SM run without
-// spilling, 114.5 against 105.0 G point-steps/s at 2048^2; at k = 4 it takes the kernel from 208 to 128
-// registers, 105.3 against 67.1 G; in the second-order step (mode 2) 150 -> 114 registers at k = 1 and
-// 197 -> 126 at k = 2, the best plan 60.8 against 56.8 G; the same bits every time.  The batched kernel, which
-// runs the same warp routine, keeps the history in registers (107.5 against 116.0 G with it in shared memory).
+// memory instead of registers, one slot per row parity so that nothing moves.  Measured at 2048^2 (G point-steps/s,
+// the same bits every time):
+//   FP32, P = 2: at k = 2 the registers it frees let four blocks (16 warps) per SM run without spilling, 114.5
+//     against 105.0; at k = 4 208 -> 128 registers, 105.3 against 67.1; second order (mode 2) 60.8 against 56.8.
+//   FP64, P = 1: four blocks without spilling, 13.1 against 12.3 first order.
+// The batched kernel, which runs the same warp routine, keeps the history in registers (107.5 against 116.0 G with
+// it in shared memory).
 template <typename T, int K, int P, int MODE> struct HistSmem {
     static constexpr bool value =
-        sizeof(T) == 4 && P == 2 && ((MODE == 0 && (K == 2 || K == 4)) || (MODE == 2 && (K == 1 || K == 2)));
+        (IsF64<T>::value && P == 1 && K == 1 && MODE != 1) ||
+        (sizeof(T) == 4 && P == 2 && ((MODE == 0 && (K == 2 || K == 4)) || (MODE == 2 && (K == 1 || K == 2))));
 };
 template <typename T, int K, int P, int MODE, int UNR = RowUnroll<T, K, MODE>::value, bool HS = false>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem);
@@ -245,15 +283,14 @@ template <int K, int MODE> struct Levels { static constexpr int value = (MODE ==
 //         Eq. sol_dis_4, U(step) exp(-i V dt), with the table holding g = exp(-i V dt) / 4 per column or cell.
 // MODE 5: MODE 2 with a uniform vector potential (the phase of each step's first level is the matrix, the
 //         table holding g = exp(-i V dt) / 16).
-// Resident 4-warp blocks per SM the register budget is fitted to (1: the compiler's choice).
+// Resident 4-warp blocks per SM the register budget is fitted to (1: the compiler's choice).  Four (128 registers)
+// where the history in shared memory, or two rows per iteration (fixed point first order: 33.1 against 26.7 G at
+// 150 registers and 3 blocks), lets them fit; FP64's shared magnitude sums need the warps to fill both pipes.
 template <typename T, int K, int P, int MODE> struct SweepMinBlocks {
-    static constexpr bool FX = sizeof(T) == 8 && (T)0.5 == (T)0;
-    static constexpr bool F64 = sizeof(T) == 8 && !FX;
-    static constexpr int value = (FX && K == 1 && P == 1 && MODE == 0)                  ? FX_MIN_BLOCKS
-                                 : (sizeof(T) == 4 && K == 2 && P == 2 && MODE == 0)   ? F32_MIN_BLOCKS
-                                 : (sizeof(T) == 4 && K == 1 && P == 2 && MODE == 2)   ? F32_MIN_BLOCKS
-                                 : (F64 && K == 1 && (P == 2 || P == 4) && MODE == 0) ? F64_MIN_BLOCKS
-                                                                                       : 1;
+    static constexpr int value = (IsFx<T>::value && K == 1 && P == 1 && MODE == 0)                            ? 4
+                                 : (sizeof(T) == 4 && P == 2 && ((K == 2 && MODE == 0) || (K == 1 && MODE == 2))) ? 4
+                                 : (IsF64<T>::value && K == 1 && P == 1)                                       ? 4
+                                                                                                               : 1;
 };
 
 template <typename T, int K, int P, int MODE>
@@ -358,10 +395,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 
 // Per-warp shared memory: 128 B of mbarriers, the row ring, the flux hand-off area (K levels x 8 values x 32
 // lanes), then with HS the sweep history ([row parity 2][level K][lane 32][point P][2] complex values; the ring
-// keeps three rows so that four blocks fit).
+// keeps three rows so that four blocks fit, two of the 8-byte types, whose rows last long enough).
 template <typename T, int K, int P, bool HS> struct Ring {
     static constexpr int ROW_BYTES = 32 * P * 8 * (int)sizeof(T);  // one warp row: 32P cells
-    static constexpr int SLOTS = (HS || ROW_BYTES >= 8192) ? 3 : 4;
+    static constexpr int SLOTS = (HS && sizeof(T) == 8) ? 2 : (HS || ROW_BYTES >= 8192) ? 3 : 4;
     static constexpr int FLUX_BYTES = K * 8 * 32 * (int)sizeof(T);
     static constexpr int HIST_BYTES = HS ? 2 * K * 32 * P * 2 * 2 * (int)sizeof(T) : 0;
     static constexpr int WARP_BYTES = 128 + SLOTS * ROW_BYTES + FLUX_BYTES + HIST_BYTES;
@@ -390,17 +427,12 @@ __device__ __forceinline__ void push_row(Cx<T> (&s0)[2], Cx<T> (&s1)[2], Cx<T> (
 // x characteristics of a row (u = a + b travels +x, w = a - b travels -x) and the neighbours the x sweep
 // takes: u of the left cell and w of the right cell (warp shuffles; lane 0 and lane 31 take them from the
 // adjacent point of lanes 31 and 0).
-template <typename T, int P>
+template <bool HY, typename T, int P>
 __device__ __forceinline__ void x_characteristics(const Cx<T> (*s)[4], int lane, int src_prev, int src_next, Cx<T> *u14,
                                                   Cx<T> *u23, Cx<T> *w14, Cx<T> *w23, Cx<T> *lu14, Cx<T> *lu23,
                                                   Cx<T> *rw14, Cx<T> *rw23) {
 #pragma unroll
-    for (int j = 0; j < P; ++j) {
-        u14[j] = cadd(s[j][0], s[j][3]);
-        w14[j] = csub(s[j][0], s[j][3]);
-        u23[j] = cadd(s[j][1], s[j][2]);
-        w23[j] = csub(s[j][1], s[j][2]);
-    }
+    for (int j = 0; j < P; ++j) x_chars<HY>(s[j], u14[j], w14[j], u23[j], w23[j]);
     Cx<T> pu14[P], pu23[P], nw14[P], nw23[P];
 #pragma unroll
     for (int j = 0; j < P; ++j) {
@@ -456,6 +488,9 @@ __device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, c
 template <typename T, int K, int P, int MODE, int UNR, bool HS>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem) {
     constexpr int L = Levels<K, MODE>::value;  // pipelined levels (one row and one x cell of halo each)
+    // FP64 pairs over two pipes, except where the registers run out: four points a lane (8.5 against 9.6 G at 2048^2)
+    // and the batched kernel's two steps a launch (6.2 against 8.6 G on 12 runs; one step: 9.8 against 8.9 G)
+    constexpr bool HY = P <= 2 && !(K == 2 && UNR == 2);
     const int64_t per_plane = a.nstrips * a.nsegs;
     const int64_t plane = wid / per_plane;
     const int64_t rem = wid - plane * per_plane;
@@ -638,15 +673,12 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                 Cx<T> zs[P][4];
 #pragma unroll
                 for (int j = 0; j < P; ++j) {
-                    const Cx<T> U13 = cadd(st[j][0], st[j][2]), U24 = csub(st[j][1], st[j][3]);
-                    const Cx<T> W13 = csub(st[j][0], st[j][2]), W24 = cadd(st[j][1], st[j][3]);
+                    Cx<T> U13, W13, U24, W24;
+                    z_chars<HY>(st[j], U13, W13, U24, W24);
                     Cx<T>(&UO)[2] = UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j];  // row q - 2
                     Cx<T> *hq = hist + ((((int)(q & 1) * L + lev) * 32 + lane) * P + j) * 2;  // HS: its slot
                     const Cx<T> o0 = HS ? hq[0] : UO[0], o1 = HS ? hq[1] : UO[1];
-                    zs[j][0] = cadd(o0, W13);
-                    zs[j][2] = csub(o0, W13);
-                    zs[j][1] = cadd(o1, W24);
-                    zs[j][3] = csub(W24, o1);
+                    z_join<HY>(o0, W13, o1, W24, zs[j]);
                     if (HS) {
                         hq[0] = U13;
                         hq[1] = U24;
@@ -665,30 +697,23 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                     continue;
                 }
                 Cx<T> u14[P], u23[P], w14[P], w23[P], lu14[P], lu23[P], rw14[P], rw23[P];
-                x_characteristics<T, P>(zs, lane, src_prev, src_next, u14, u23, w14, w23, lu14, lu23, rw14, rw23);
+                x_characteristics<HY, T, P>(zs, lane, src_prev, src_next, u14, u23, w14, w23, lu14, lu23, rw14, rw23);
                 if (has_face && q - 1 >= r_begin && q - 1 < r_end)
                     flux_row<T, P>(lu14, lu23, w14, w23, face_j, face_lane, lane, q - 1 - r_begin, q - 1 == r_end - 1,
                                    gsm + lev * 8 * 32, 2.0 * a.flux_unit, facc[lev]);
 #pragma unroll
                 for (int j = 0; j < P; ++j) {
                     const bool keep = per || (zrow_ok && xin[j]);
-                    const Cx<T> b0 = cadd(lu14[j], rw14[j]), b3 = csub(lu14[j], rw14[j]);
-                    const Cx<T> b1 = cadd(lu23[j], rw23[j]), b2 = csub(lu23[j], rw23[j]);
-                    st[j][0] = keep ? b0 : Cx<T>{T(0), T(0)};
-                    st[j][1] = keep ? b1 : Cx<T>{T(0), T(0)};
-                    st[j][2] = keep ? b2 : Cx<T>{T(0), T(0)};
-                    st[j][3] = keep ? b3 : Cx<T>{T(0), T(0)};
+                    Cx<T> b[4];
+                    x_join<HY>(lu14[j], rw14[j], lu23[j], rw23[j], b);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) st[j][c] = keep ? b[c] : Cx<T>{T(0), T(0)};
                 }
                 continue;
             }
             Cx<T> u14[P], u23[P], w14[P], w23[P];
 #pragma unroll
-            for (int j = 0; j < P; ++j) {
-                u14[j] = cadd(st[j][0], st[j][3]);
-                w14[j] = csub(st[j][0], st[j][3]);
-                u23[j] = cadd(st[j][1], st[j][2]);
-                w23[j] = csub(st[j][1], st[j][2]);
-            }
+            for (int j = 0; j < P; ++j) x_chars<HY>(st[j], u14[j], w14[j], u23[j], w23[j]);
             Cx<T> pu14[P], pu23[P], nw14[P], nw23[P];
 #pragma unroll
             for (int j = 0; j < P; ++j) {
@@ -714,14 +739,12 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
 #pragma unroll
             for (int j = 0; j < P; ++j) {
                 // x sweep (Eq. sol_dis_1), x2
-                const Cx<T> b0 = cadd(lu14[j], rw14[j]);
-                const Cx<T> b3 = csub(lu14[j], rw14[j]);
-                const Cx<T> b1 = cadd(lu23[j], rw23[j]);
-                const Cx<T> b2 = csub(lu23[j], rw23[j]);
-                Cx<T> o[4];
+                Cx<T> b[4], o[4];
+                x_join<HY>(lu14[j], rw14[j], lu23[j], rw23[j], b);
                 if (MODE != 1) {
-                    // z sweep (Eq. sol_dis_3): +z movers (b1+b3, b2-b4), -z movers (b1-b3, b2+b4)
-                    const Cx<T> U13 = cadd(b0, b2), U24 = csub(b1, b3);
+                    // z sweep (Eq. sol_dis_3)
+                    Cx<T> U13, W13, U24, W24;
+                    z_chars<HY>(b, U13, W13, U24, W24);
                     // row q - 2's sums: the slot of q's parity (HS) or the register slot
                     Cx<T> *hp = hist + ((((int)(q & 1) * L + lev) * 32 + lane) * P + j) * 2;
                     Cx<T> h0, h1;
@@ -733,11 +756,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                         h1 = UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][1];
                     }
                     if (need_out) {
-                        const Cx<T> W13 = csub(b0, b2), W24 = cadd(b1, b3);
-                        o[0] = cadd(h0, W13);
-                        o[2] = csub(h0, W13);
-                        o[1] = cadd(h1, W24);
-                        o[3] = csub(W24, h1);
+                        z_join<HY>(h0, W13, h1, W24, o);
                         // phase (Eq. sol_dis_4) with the deferred 1/4
                         Cx<T> qu, qd;
                         if (a.full_table) {
@@ -778,14 +797,12 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                         push_row<T, UNR>(UH[0][lev][j], UH[1][lev][j], UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j], U13, U24);
                     }
                 } else {
-                    // y sweep (Eq. sol_dis_2): +y movers (b1 - i b4, b2 + i b3), -y movers (b1 + i b4, b2 - i b3)
-                    const Cx<T> U14 = csub_ib(b0, b3), U23 = cadd_ib(b1, b2);
+                    // y sweep (Eq. sol_dis_2)
+                    Cx<T> U14, W14, U23, W23;
+                    y_chars<HY>(b, U14, W14, U23, W23);
                     if (need_out) {
-                        const Cx<T> W14 = cadd_ib(b0, b3), W23 = csub_ib(b1, b2);
-                        o[0] = cadd(UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][0], W14);
-                        o[3] = cmul_i(csub(UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][0], W14));
-                        o[1] = cadd(UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][1], W23);
-                        o[2] = cmul_mi(csub(UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][1], W23));
+                        Cx<T>(&UO)[2] = UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j];
+                        y_join<HY>(UO[0], W14, UO[1], W23, o);
                     }
                     push_row<T, UNR>(UH[0][lev][j], UH[1][lev][j], UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j], U14, U23);
                 }
@@ -901,15 +918,12 @@ __global__ void __launch_bounds__(128) zphase_kernel(const ZArgs a) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) s[c] = {T(0), T(0)};
         }
-        const Cx<T> U13 = cadd(s[0], s[2]), U24 = csub(s[1], s[3]);
-        const Cx<T> W13 = csub(s[0], s[2]), W24 = cadd(s[1], s[3]);
+        Cx<T> U13, W13, U24, W24;
+        z_chars<true>(s, U13, W13, U24, W24);
         const int64_t zo = z - 1;
         if (zo >= z_begin && zo < z_end) {
             Cx<T> o[4];
-            o[0] = cadd(UA[0], W13);
-            o[2] = csub(UA[0], W13);
-            o[1] = cadd(UA[1], W24);
-            o[3] = csub(W24, UA[1]);
+            z_join<true>(UA[0], W13, UA[1], W24, o);
             Cx<T> qu = pu, qd = pd;
             if (a.full_table) load_tab(tab + (zo * ncol + col) * 4, qu, qd);
             o[0] = cmulp(o[0], qu);

@@ -87,25 +87,24 @@ template <typename T>
 __device__ __forceinline__ void xsweep_row(const Cx<T> s[4], Cx<T> o[4], int lane, bool fl_u, bool fl_w,
                                            typename FaceAcc<T>::type &fp) {
     using F = typename FaceAcc<T>::type;
-    const Cx<T> u14 = cadd(s[0], s[3]), w14 = csub(s[0], s[3]);
-    const Cx<T> u23 = cadd(s[1], s[2]), w23 = csub(s[1], s[2]);
+    Cx<T> u14, w14, u23, w23;
+    x_chars<false>(s, u14, w14, u23, w23);
     if (fl_u) fp = Ar<F>::add(fp, face_term(u14, u23));
     if (fl_w) fp = Ar<F>::sub(fp, face_term(w14, w23));
     const Cx<T> lu14 = shfl_c(u14, (lane + 31) & 31), lu23 = shfl_c(u23, (lane + 31) & 31);
     const Cx<T> rw14 = shfl_c(w14, (lane + 1) & 31), rw23 = shfl_c(w23, (lane + 1) & 31);
-    o[0] = cadd(lu14, rw14);
-    o[3] = csub(lu14, rw14);
-    o[1] = cadd(lu23, rw23);
-    o[2] = csub(lu23, rw23);
+    x_join<false>(lu14, rw14, lu23, rw23, o);
 }
 
 // y characteristics of row w (Eq. sol_dis_2): "+y" movers (a1 - i a4, a2 + i a3), "-y" movers (a1 + i a4, a2 - i a3)
 template <typename T>
 __device__ __forceinline__ void ywrite_row(Cx<T> *buf, int w, int lane, const Cx<T> a[4]) {
-    buf[(w * 4 + 0) * 32 + lane] = csub_ib(a[0], a[3]);
-    buf[(w * 4 + 1) * 32 + lane] = cadd_ib(a[1], a[2]);
-    buf[(w * 4 + 2) * 32 + lane] = cadd_ib(a[0], a[3]);
-    buf[(w * 4 + 3) * 32 + lane] = csub_ib(a[1], a[2]);
+    Cx<T> U14, W14, U23, W23;
+    y_chars<false>(a, U14, W14, U23, W23);
+    buf[(w * 4 + 0) * 32 + lane] = U14;
+    buf[(w * 4 + 1) * 32 + lane] = U23;
+    buf[(w * 4 + 2) * 32 + lane] = W14;
+    buf[(w * 4 + 3) * 32 + lane] = W23;
 }
 
 // B: y sweep, two cells, of row w: "+y" movers of row w - 2, "-y" movers of row w + 2
@@ -113,10 +112,7 @@ template <typename T>
 __device__ __forceinline__ void ysweep_row(const Cx<T> *buf, int w, int lane, Cx<T> q[4]) {
     const Cx<T> U14 = buf[((w - 2) * 4 + 0) * 32 + lane], U23 = buf[((w - 2) * 4 + 1) * 32 + lane];
     const Cx<T> W14 = buf[((w + 2) * 4 + 2) * 32 + lane], W23 = buf[((w + 2) * 4 + 3) * 32 + lane];
-    q[0] = cadd(U14, W14);
-    q[3] = cmul_i(csub(U14, W14));
-    q[1] = cadd(U23, W23);
-    q[2] = cmul_mi(csub(U23, W23));
+    y_join<false>(U14, W14, U23, W23, q);
 }
 
 template <typename T>
@@ -362,13 +358,9 @@ __global__ void __launch_bounds__(128, ZMinBlocks<T, FIELD>::value) strang_z_ker
                 load_phase(k + 2 * LA, tpu[LA - 1], tpd[LA - 1]);
             }
             // C: z sweep, two cells (Eq. sol_dis_3): output plane j = k - 2 from U(k - 4) and W(k)
-            const Cx<T> U13 = cadd(s[0], s[2]), U24 = csub(s[1], s[3]);
-            const Cx<T> W13 = csub(s[0], s[2]), W24 = cadd(s[1], s[3]);
-            Cx<T> o[4];
-            o[0] = cadd(R1[t][0], W13);
-            o[2] = csub(R1[t][0], W13);
-            o[1] = cadd(R1[t][1], W24);
-            o[3] = csub(W24, R1[t][1]);
+            Cx<T> U13, W13, U24, W24, o[4];
+            z_chars<false>(s, U13, W13, U24, W24);
+            z_join<false>(R1[t][0], W13, R1[t][1], W24, o);
             R1[t][0] = U13;
             R1[t][1] = U24;
             // D: phase of Eq. sol_dis_4 at plane j (zero outside the grid under the zero boundary)
@@ -399,13 +391,9 @@ __global__ void __launch_bounds__(128, ZMinBlocks<T, FIELD>::value) strang_z_ker
                 for (int c = 0; c < 4; ++c) o[c] = {T(0), T(0)};
             }
             // C: z sweep, two cells: output plane m = j - 2 from the phased U(j - 4) and W(j)
-            const Cx<T> V13 = cadd(o[0], o[2]), V24 = csub(o[1], o[3]);
-            const Cx<T> X13 = csub(o[0], o[2]), X24 = cadd(o[1], o[3]);
-            Cx<T> r[4];
-            r[0] = cadd(R2[t][0], X13);
-            r[2] = csub(R2[t][0], X13);
-            r[1] = cadd(R2[t][1], X24);
-            r[3] = csub(X24, R2[t][1]);
+            Cx<T> V13, X13, V24, X24, r[4];
+            z_chars<false>(o, V13, X13, V24, X24);
+            z_join<false>(R2[t][0], X13, R2[t][1], X24, r);
             R2[t][0] = V13;
             R2[t][1] = V24;
             const ZI m = k - 4;
