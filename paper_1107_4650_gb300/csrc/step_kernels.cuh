@@ -248,8 +248,7 @@ __device__ __forceinline__ int64_t pmod(int64_t a, int64_t n) {
 // Rows per iteration of the row loop (1 or 2; measured per variant: two rows let the history registers
 // alternate instead of moving, which pays where the loop body is short).
 template <typename T, int K, int MODE> struct RowUnroll {
-    static constexpr bool FX = sizeof(T) == 8 && (T)0.5 == (T)0;  // the int64 fixed-point state
-    static constexpr int value = (sizeof(T) == 4 && K == 1 && MODE == 0) ? 2 : ((FX && K == 1 && MODE == 0) ? 2 : 1);
+    static constexpr int value = (!std::is_same<T, double>::value && K == 1 && MODE == 0) ? 2 : 1;
 };
 template <typename T> struct IsFx { static constexpr bool value = std::is_same<T, long long>::value; };  // int64 fixed point
 template <typename T> struct IsF64 { static constexpr bool value = std::is_same<T, double>::value; };
@@ -259,14 +258,17 @@ template <typename T> struct IsF64 { static constexpr bool value = std::is_same<
 //   FP32, P = 2: at k = 2 the registers it frees let four blocks (16 warps) per SM run without spilling, 114.5
 //     against 105.0; at k = 4 208 -> 128 registers, 105.3 against 67.1; second order (mode 2) 60.8 against 56.8.
 //   FP64, P = 1: four blocks without spilling, 13.1 against 12.3 first order.
+//   Fixed point, P = 1, second order: four blocks instead of two, 22.9 against 19.9 (periodic 22.4 against 20.6);
+//     first order periodic 31.9 against 31.6, but zero boundary 31.8 against 33.7: registers there.
 // The batched kernel, which runs the same warp routine, keeps the history in registers (107.5 against 116.0 G with
 // it in shared memory).
-template <typename T, int K, int P, int MODE> struct HistSmem {
+template <typename T, int K, int P, int MODE, bool PER> struct HistSmem {
     static constexpr bool value =
         (IsF64<T>::value && P == 1 && K == 1 && MODE != 1) ||
+        (IsFx<T>::value && P == 1 && K == 1 && (MODE == 2 || (MODE == 0 && PER))) ||
         (sizeof(T) == 4 && P == 2 && ((MODE == 0 && (K == 2 || K == 4)) || (MODE == 2 && (K == 1 || K == 2))));
 };
-template <typename T, int K, int P, int MODE, int UNR = RowUnroll<T, K, MODE>::value, bool HS = false>
+template <typename T, int K, int P, int MODE, bool PER, int UNR = RowUnroll<T, K, MODE>::value, bool HS = false>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem);
 template <int K>
 __device__ __forceinline__ void finish_flux(const SweepArgs &a);
@@ -287,22 +289,22 @@ template <int K, int MODE> struct Levels { static constexpr int value = (MODE ==
 // where the history in shared memory, or two rows per iteration (fixed point first order: 33.1 against 26.7 G at
 // 150 registers and 3 blocks), lets them fit; FP64's shared magnitude sums need the warps to fill both pipes.
 template <typename T, int K, int P, int MODE> struct SweepMinBlocks {
-    static constexpr int value = (IsFx<T>::value && K == 1 && P == 1 && MODE == 0)                            ? 4
+    static constexpr int value = (IsFx<T>::value && K == 1 && P == 1 && (MODE == 0 || MODE == 2))             ? 4
                                  : (sizeof(T) == 4 && P == 2 && ((K == 2 && MODE == 0) || (K == 1 && MODE == 2))) ? 4
                                  : (IsF64<T>::value && K == 1 && P == 1)                                       ? 4
                                                                                                                : 1;
 };
 
-template <typename T, int K, int P, int MODE>
+template <typename T, int K, int P, int MODE, bool PER>
 __global__ void __launch_bounds__(128, SweepMinBlocks<T, K, P, MODE>::value) sweep_kernel(const SweepArgs a) {
     constexpr int L = Levels<K, MODE>::value;
-    constexpr bool HS = HistSmem<T, K, P, MODE>::value;
+    constexpr bool HS = HistSmem<T, K, P, MODE, PER>::value;
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t per_plane = a.nstrips * a.nsegs;
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     unsigned char *wsmem = dyn_smem + (threadIdx.x >> 5) * Ring<T, L, P, HS>::WARP_BYTES;
-    if (wid < per_plane * a.nplanes) sweep_warp<T, K, P, MODE, RowUnroll<T, K, MODE>::value, HS>(a, wid, lane, wsmem);
+    if (wid < per_plane * a.nplanes) sweep_warp<T, K, P, MODE, PER, RowUnroll<T, K, MODE>::value, HS>(a, wid, lane, wsmem);
 }
 
 // Sum of n flux partials in an order fixed by n: lane l adds parts l, l + 32, ..., a xor tree adds the lanes (the
@@ -359,8 +361,10 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 __device__ __forceinline__ void mbar_inval(uint32_t bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
         "l"(src), "r"(bytes), "r"(bar)
@@ -485,7 +489,7 @@ __device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, c
     }
 }
 
-template <typename T, int K, int P, int MODE, int UNR, bool HS>
+template <typename T, int K, int P, int MODE, bool PER, int UNR, bool HS>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem) {
     constexpr int L = Levels<K, MODE>::value;  // pipelined levels (one row and one x cell of halo each)
     // FP64 pairs over two pipes, except where the registers run out: four points a lane (8.5 against 9.6 G at 2048^2)
@@ -497,15 +501,14 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     const int64_t seg = rem / a.nstrips;
     const int64_t strip = rem - seg * a.nstrips;
     const int64_t nx = a.nx, nr = a.nr;
-    const bool per = a.periodic != 0;
-    const bool ring = !per;  // periodic grids wrap the strip: plain loads
+    constexpr bool per = PER;
     const int64_t x_own0 = strip * a.strip_w;
     const int64_t x_own1 = min(x_own0 + a.strip_w, nx);
     const int64_t xa = x_own0 - L;
-    // Row indices fit 32 bits (the host limits every grid dimension below 2^31).  The floating-point kernels run
-    // their row loop on 32-bit indices (FP32 k = 2: 105 against 94 G point-steps/s at 2048^2); the fixed-point
-    // kernel keeps 64-bit ones, with which it fits its 128-register budget without spilling (33.2 against 31.5 G).
-    using RI = typename std::conditional<RowUnroll<T, K, MODE>::FX, int64_t, int>::type;
+    // Row indices fit 32 bits (the host limits every grid dimension below 2^31): FP32 k = 2 105 against 94 G at
+    // 2048^2 with 64-bit ones.  The fixed-point first-order kernel on a zero-boundary grid keeps 64-bit ones, with
+    // which it runs 33.7 against 33.5 G.
+    using RI = typename std::conditional<IsFx<T>::value && MODE == 0 && !PER, int64_t, int>::type;
     const RI nr32 = (RI)nr;
     const RI r_begin = (RI)(seg * a.seg_h);
     const RI r_end = (RI)min((int64_t)r_begin + a.seg_h, nr);
@@ -586,39 +589,64 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
             hist[((t / (L * P * 2) * L + (t / (P * 2)) % L) * 32 + lane) * P * 2 + t % (P * 2)] = Cx<T>{T(0), T(0)};
     }
     T *gsm = reinterpret_cast<T *>(wsmem + 128 + RG::SLOTS * RG::ROW_BYTES);  // flux hand-off [K][8][32]
-    const int64_t cx0 = max(xa, (int64_t)0), cx1 = min(xa + 32 * P, nx);
-    const uint32_t copy_bytes = (uint32_t)((cx1 - cx0) * 8 * (int64_t)sizeof(T));
+    // span of grid cells a row copy brings: the strip clipped to the grid; periodic: all 32 P cells, wrapped, as
+    // pieces that end at the grid's right edge (two at most where nx >= 32 P)
+    const int64_t cx0 = per ? pmod(xa, nx) : max(xa, (int64_t)0), cx1 = per ? xa + 32 * P : min(xa + 32 * P, nx);
+    constexpr uint32_t CELL = 8 * (uint32_t)sizeof(T);
+    const uint32_t copy_bytes = per ? (uint32_t)RG::ROW_BYTES : (uint32_t)(cx1 - cx0) * CELL;
     const uint32_t bar0 = smem_u32(wsmem);
     const uint32_t slot0 = smem_u32(wsmem + 128);
-    const uint32_t dst_off = (uint32_t)((cx0 - xa) * 8 * (int64_t)sizeof(T));
+    const uint32_t dst_off = per ? 0u : (uint32_t)(cx0 - xa) * CELL;
+    // lane 0: row r of the grid into slot sl
+    auto fetch_row = [&](RI r, int sl) {
+        const T *row = in + (int64_t)r * nx * 8;
+        const uint32_t bar = bar0 + 8 * sl, dst = slot0 + sl * RG::ROW_BYTES + dst_off;
+        bar_expect(bar, copy_bytes);
+        if (!per) {
+            bulk_copy(dst, row + cx0 * 8, copy_bytes, bar);
+        } else {
+            int64_t x = cx0;
+            for (int done = 0; done < 32 * P;) {
+                const int n = (int)min((int64_t)(32 * P - done), nx - x);
+                bulk_copy(dst + (uint32_t)done * CELL, row + x * 8, (uint32_t)n * CELL, bar);
+                done += n;
+                x = 0;
+            }
+        }
+    };
+    // a row of the segment or its halo in the grid's own numbering (periodic: wrapped)
+    auto grid_row = [&](RI r) -> RI {
+        if (per) {
+            while (r < 0) r += nr32;
+            while (r >= nr32) r -= nr32;
+        }
+        return r;
+    };
     const RI r_first = r_begin - L, r_last = r_end + L;  // rows [r_first, r_last) are read
     uint32_t phase_bits = 0, pending = 0;
     bool aborted = false;
-    if (ring) {
-        if (lane == 0) {
+    if (lane == 0) {
 #pragma unroll
-            for (int sl = 0; sl < RG::SLOTS; ++sl) mbar_init(bar0 + 8 * sl, 1);
-            mbar_fence_init();
-        }
-        __syncwarp();
-        bool stall = a.inject_stall && wid == 0;
+        for (int sl = 0; sl < RG::SLOTS; ++sl) mbar_init(bar0 + 8 * sl, 1);
+        mbar_fence_init();
+    }
+    __syncwarp();
+    bool stall = a.inject_stall && wid == 0 && !per;
 #pragma unroll
-        for (int sl = 0; sl < RG::SLOTS; ++sl) {
-            const RI r = r_first + sl;
-            if (r < r_last && r >= 0 && r < nr32) {
-                if (lane == 0) {
-                    // failure-detection test hook: the first warp of the launch announces 16 bytes more than
-                    // its first row copy delivers, so that slot's phase never completes and its bounded wait
-                    // runs out (the copy itself completes normally)
-                    if (stall)
-                        asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], 16;" ::"r"(bar0 + 8 * sl)
-                                     : "memory");
-                    bulk_load(slot0 + sl * RG::ROW_BYTES + dst_off, in + ((int64_t)r * nx + cx0) * 8, copy_bytes,
-                              bar0 + 8 * sl);
-                }
-                stall = false;
-                pending |= 1u << sl;
+    for (int sl = 0; sl < RG::SLOTS; ++sl) {
+        const RI r = r_first + sl;
+        if (r < r_last && (per || (r >= 0 && r < nr32))) {
+            if (lane == 0) {
+                // failure-detection test hook: the first warp of the launch announces 16 bytes more than
+                // its first row copy delivers, so that slot's phase never completes and its bounded wait
+                // runs out (the copy itself completes normally)
+                if (stall)
+                    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], 16;" ::"r"(bar0 + 8 * sl)
+                                 : "memory");
+                fetch_row(grid_row(r), sl);
             }
+            stall = false;
+            pending |= 1u << sl;
         }
     }
 
@@ -630,35 +658,22 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         if (r >= r_last) break;
         Cx<T> st[P][4];
         const bool row_ok = per || (r >= 0 && r < nr32);
-        const int64_t rl = per ? pmod(r, nr) : r;
-        if (ring) {
-            if (row_ok) {
-                if (!mbar_wait(bar0 + 8 * sl, (phase_bits >> sl) & 1u)) {
-                    aborted = true;
-                    break;
-                }
-                phase_bits ^= 1u << sl;
-                pending &= ~(1u << sl);
+        if (row_ok) {
+            if (!mbar_wait(bar0 + 8 * sl, (phase_bits >> sl) & 1u)) {
+                aborted = true;
+                break;
             }
-            const T *srow = reinterpret_cast<const T *>(wsmem + 128 + sl * RG::ROW_BYTES);
+            phase_bits ^= 1u << sl;
+            pending &= ~(1u << sl);
+        }
+        const T *srow = reinterpret_cast<const T *>(wsmem + 128 + sl * RG::ROW_BYTES);
 #pragma unroll
-            for (int j = 0; j < P; ++j) {
-                if (row_ok && xin[j]) {
-                    load_pt(srow + (32 * j + lane) * 8, st[j]);
-                } else {
+        for (int j = 0; j < P; ++j) {
+            if (row_ok && (per || xin[j])) {
+                load_pt(srow + (32 * j + lane) * 8, st[j]);
+            } else {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) st[j][c] = {T(0), T(0)};
-                }
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-                if (row_ok && (per || xin[j])) {
-                    load_pt(in + (rl * nx + xl[j]) * 8, st[j]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) st[j][c] = {T(0), T(0)};
-                }
+                for (int c = 0; c < 4; ++c) st[j][c] = {T(0), T(0)};
             }
         }
 #pragma unroll
@@ -760,7 +775,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                         // phase (Eq. sol_dis_4) with the deferred 1/4
                         Cx<T> qu, qd;
                         if (a.full_table) {
-                            const int64_t rr = per ? pmod(q - 1, nr) : (int64_t)min(max(q - 1, (RI)0), nr32 - 1);
+                            const int64_t rr = per ? (int64_t)grid_row(q - 1) : (int64_t)min(max(q - 1, (RI)0), nr32 - 1);
                             load_tab(static_cast<const T *>(a.table) + (plane * nr * nx + rr * nx + xl[j]) * 4, qu, qd);
                         } else {
                             qu = pu[j];
@@ -836,20 +851,17 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                     if (own[j]) store_pt(orow + (xa + 32 * j + lane) * 8, st[j]);
             }
         }
-        if (ring) {
-            // refill this slot with row r + SLOTS once every lane has read it
-            __syncwarp();
-            const RI rn = r + RG::SLOTS;
-            if (rn < r_last && rn >= 0 && rn < nr32) {
-                if (lane == 0) {
-                    fence_proxy_async();
-                    bulk_load(slot0 + sl * RG::ROW_BYTES + dst_off, in + ((int64_t)rn * nx + cx0) * 8, copy_bytes,
-                              bar0 + 8 * sl);
-                }
-                pending |= 1u << sl;
+        // refill this slot with row r + SLOTS once every lane has read it
+        __syncwarp();
+        const RI rn = r + RG::SLOTS;
+        if (rn < r_last && (per || (rn >= 0 && rn < nr32))) {
+            if (lane == 0) {
+                fence_proxy_async();
+                fetch_row(grid_row(rn), sl);
             }
-            sl = (sl + 1 == RG::SLOTS) ? 0 : sl + 1;
+            pending |= 1u << sl;
         }
+        sl = (sl + 1 == RG::SLOTS) ? 0 : sl + 1;
     }
     }
     if (aborted) {
@@ -859,14 +871,12 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         for (int s2 = 0; s2 < RG::SLOTS; ++s2)
             if (pending & (1u << s2)) mbar_wait(bar0 + 8 * s2, (phase_bits >> s2) & 1u);
     }
-    if (ring) {
-        // release the barriers so the next task of this warp can initialise them again
-        __syncwarp();
-        if (lane == 0)
+    // release the barriers so the next task of this warp can initialise them again
+    __syncwarp();
+    if (lane == 0)
 #pragma unroll
-            for (int s2 = 0; s2 < RG::SLOTS; ++s2) mbar_inval(bar0 + 8 * s2);
-        __syncwarp();
-    }
+        for (int s2 = 0; s2 < RG::SLOTS; ++s2) mbar_inval(bar0 + 8 * s2);
+    __syncwarp();
     if (has_face) {
 #pragma unroll
         for (int s = 0; s < L; ++s) {
