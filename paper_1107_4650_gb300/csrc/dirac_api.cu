@@ -277,8 +277,61 @@ dirac_status upload_field_aux(dirac_grid *g) {
     return put_doubles(g, g->fabs_dev, g->fabs_bytes, g->absorb.data(), g->absorb.size());
 }
 
-// Launch geometry for (K, P, warps per block): strips of 32P - 2K owned cells, segments sized so the
-// launch holds about `target` warps per SM.
+// Rows (or planes) per segment: the split of n rows that minimises a launch's time,
+//   (rows + halo) x (full waves x row_time(resident) + row_time(the rest)),
+// where each segment streams `halo` extra rows, `units` units of work per segment run `per_block` to a block, an SM
+// holds `resident` blocks and row_time(b) is the time of one row with b blocks on an SM.  uneven: the part of a block
+// that a launch loses at its end where its blocks differ (tiles cut by the grid's edge, the face's strip).
+template <typename F>
+int64_t pick_rows(int64_t n, int64_t units, int per_block, int64_t sms, int64_t resident, double halo, double uneven,
+                  F row_time) {
+    int64_t best_h = n;
+    double best = 1e300;
+    for (int64_t h = n; h >= 1;) {
+        const int64_t segs = (n + h - 1) / h;
+        const int64_t blocks = (units * segs + per_block - 1) / per_block;
+        const int64_t per_sm = (blocks + sms - 1) / sms;  // on the fullest SM
+        const int64_t waves = per_sm / resident, rest = per_sm % resident;
+        const double t = ((double)h + halo) * (waves * row_time(resident) + (rest ? row_time(rest) : 0.0)) + uneven * h * row_time(1);
+        if (t < best * 0.999) {  // near ties: the longer segments
+            best = t;
+            best_h = h;
+        }
+        const int64_t next = (n + segs) / (segs + 1);  // the longest segment of one split more
+        h = next < h ? next : h - 1;
+    }
+    return best_h;
+}
+
+// Time of one row of the 2-D step's row loop (microseconds) with w warps on an SM: a warp alone is bound by its chain
+// of dependent instructions (lat), a full SM by the pipes (w x thr); in between the two add like independent delays.
+// Fitted to measured launches (128^2 to 2048^2, segments of 1 to 64 rows); a fit within a quarter of the truth picks the
+// segments, since the optimum is flat.  The launches of small grids were sized for few halo rows before (16 rows or
+// more a segment): 256^2 FP64 42.5 us a step with 144 warps on the chip, 14.7 with 1152; FP32 13.6 -> 6.5.
+struct RowTime {
+    double lat, thr;
+    double operator()(int64_t w) const { return std::sqrt(lat * lat + (w * thr) * (w * thr)); }
+};
+RowTime row_time_of(const dirac_grid *g, int K, int P) {
+    const int mode = sweep_mode(g);
+    const bool matrix = mode == 3 || mode == 5;
+    // the second level of a second-order step has no phase (FP64: the phase is a third of the first's FP64 work)
+    const double lv = strang(g) ? (g->fp32 || g->fx ? 1.5 : 2.0) * K : K;
+    RowTime t = g->fx ? RowTime{1.03, 0.129} : (g->fp32 ? RowTime{0.5, 0.033} : RowTime{2.1, 0.31});
+    t.lat *= lv * (matrix ? 1.4 : 1.0);
+    t.thr *= lv * P * (matrix ? 1.7 : 1.0) * (!g->fp32 && !g->fx && P > 1 ? 1.4 : 1.0);
+    return t;
+}
+// 4-warp blocks of the 2-D step resident on an SM (SweepMinBlocks; FP32 with one point a lane and one step fits five).
+int resident_blocks(const dirac_grid *g, int K, int P) {
+    if (sweep_mode(g) == 4) return g->fp32 ? 4 : (P == 1 ? 3 : 2);
+    if (P == 1) return g->fp32 && K == 1 ? 5 : 4;
+    if (P == 4) return 2;
+    return g->fp32 ? (levels(g, K) == 4 ? 3 : 4) : 2;  // FP32, four levels: 18.5 KB of shared memory a warp
+}
+
+// Launch geometry for (K, P, warps per block): strips of 32P - 2K owned cells; segments for about `target` warps per
+// SM, or, with target 0, by the row-time model above.
 void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
     Plan &p = g->plan;
     p.K = K;
@@ -290,28 +343,35 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
     const int Lv = halo_of(g, K);
     p.strip_w = 32 * P - 2 * Lv;
     p.nstrips = (nx + p.strip_w - 1) / p.strip_w;
-    const int64_t want = (int64_t)g->sm_count * target_warps_per_sm;
-    int64_t nsegs = std::max<int64_t>(1, want / std::max<int64_t>(1, p.nstrips * planes));
-    // keep segments at least 8 levels' worth of rows so halo rows stay a small fraction
-    const int64_t min_rows = std::max<int64_t>(8 * Lv, 16);
-    nsegs = std::min<int64_t>(nsegs, std::max<int64_t>(1, nr / min_rows));
-    p.seg_h = (nr + nsegs - 1) / nsegs;
+    const bool model = target_warps_per_sm == 0;
+    const int64_t want = (int64_t)g->sm_count * (model ? 16 : target_warps_per_sm);
+    if (model) {
+        const RowTime rt = row_time_of(g, K, P);
+        p.seg_h = pick_rows(nr, p.nstrips * planes, wpb, g->sm_count, resident_blocks(g, K, P), 2.0 * Lv, 0.0,
+                            [&](int64_t blocks) { return rt(blocks * wpb); });
+    } else {
+        int64_t nsegs = std::max<int64_t>(1, want / std::max<int64_t>(1, p.nstrips * planes));
+        // keep segments at least 8 levels' worth of rows so halo rows stay a small fraction
+        const int64_t min_rows = std::max<int64_t>(8 * Lv, 16);
+        nsegs = std::min<int64_t>(nsegs, std::max<int64_t>(1, nr / min_rows));
+        p.seg_h = (nr + nsegs - 1) / nsegs;
+    }
     p.nsegs = (nr + p.seg_h - 1) / p.seg_h;
     // 3-D z pass: one thread per column, segments until ~target warps per SM
     if (ndim_of(g) == 3) {
         const int64_t ncol = g->cfg.n[0] * g->cfg.n[1];
         const int64_t nz = g->cfg.n[2];
         int64_t zs = std::max<int64_t>(1, want * 32 / std::max<int64_t>(1, ncol));
-        zs = std::min<int64_t>(zs, std::max<int64_t>(1, nz / 32));
+        zs = std::min<int64_t>(zs, std::max<int64_t>(1, nz / (ncol * nz < 32 * want * 32 ? 4 : 32)));  // small grids: short ones
         p.z_seg_h = (nz + zs - 1) / zs;
         p.z_nsegs = (nz + p.z_seg_h - 1) / p.z_seg_h;
-        // fused pass: 30-cell strips x (warps - 2)-row tiles, z segments until ~8 blocks per SM have work
+        // fused pass: 30-cell strips x (warps - 2)-row tiles, z segments that fill whole waves (each carries two halo
+        // planes and one plane's worth of start-up)
         p.f_nstrips = (g->cfg.n[0] + 29) / 30;
         p.f_nytiles = (g->cfg.n[1] + (p.f_warps - 2) - 1) / (p.f_warps - 2);
         const int64_t tiles = p.f_nstrips * p.f_nytiles;
-        int64_t fz = std::max<int64_t>(1, (8 * (int64_t)g->sm_count + tiles - 1) / tiles);
-        fz = std::min<int64_t>(fz, std::max<int64_t>(1, nz / 16));
-        p.f_zseg_h = (nz + fz - 1) / fz;
+        const auto whole = [](int64_t blocks) { return (double)blocks; };  // the passes: time as the blocks on an SM
+        p.f_zseg_h = pick_rows(nz, tiles, 1, g->sm_count, 1, 3.0, 0.5, whole);
         p.f_nzsegs = (nz + p.f_zseg_h - 1) / p.f_zseg_h;
         // two steps per fused pass: 28-cell strips x (warps - 4)-row tiles (16 warps in FP32, 8 in FP64), z
         // segments as above (each carries two halo planes a side)
@@ -319,12 +379,10 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         p.f2_nstrips = (g->cfg.n[0] + 27) / 28;
         p.f2_nytiles = (g->cfg.n[1] + (p.f2_warps - 4) - 1) / (p.f2_warps - 4);
         const int64_t tiles2 = p.f2_nstrips * p.f2_nytiles;
-        int64_t fz2 = std::max<int64_t>(1, (8 * (int64_t)g->sm_count + tiles2 - 1) / tiles2);
-        fz2 = std::min<int64_t>(fz2, std::max<int64_t>(1, nz / 16));
-        p.f2_zseg_h = (nz + fz2 - 1) / fz2;
+        p.f2_zseg_h = pick_rows(nz, tiles2, 1, g->sm_count, 1, 5.0, 0.0, whole);
         p.f2_nzsegs = (nz + p.f2_zseg_h - 1) / p.f2_zseg_h;
         // second-order passes: x-y-x(-x-y-x) blocks over (32 - 4 nh)-cell strips x (warps - 4 nh)-row tiles x
-        // z segments (planes are independent: ~8 blocks per SM of work); z-phase-z columns x 2 plane parities
+        // z segments (planes are independent; whole waves); z-phase-z columns x 2 plane parities
         // x z segments (~s3_zfactor x 1024 threads per SM, segments of at least 16 planes: four halo planes
         // each side)
         for (int nh = 1; nh <= 2; ++nh) {
@@ -333,13 +391,11 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
             q.nstrips = (g->cfg.n[0] + own - 1) / own;
             q.nytiles = (g->cfg.n[1] + rows - 1) / rows;
             const int64_t tiles = q.nstrips * q.nytiles;
-            int64_t sz = std::max<int64_t>(1, (8 * (int64_t)g->sm_count + tiles - 1) / tiles);
-            sz = std::min<int64_t>(sz, nz);
-            q.zseg_h = (nz + sz - 1) / sz;
+            q.zseg_h = pick_rows(nz, tiles, 1, g->sm_count, 1, 1.0, 0.5, whole);
             q.nzsegs = (nz + q.zseg_h - 1) / q.zseg_h;
         }
         int64_t zz = std::max<int64_t>(1, ((int64_t)p.s3_zfactor * 1024 * g->sm_count + ncol) / std::max<int64_t>(1, 2 * ncol));
-        zz = std::min<int64_t>(zz, std::max<int64_t>(1, nz / 16));
+        zz = std::min<int64_t>(zz, std::max<int64_t>(1, nz / (ncol * nz < 32 * 1024 * (int64_t)g->sm_count ? 8 : 16)));
         p.s3_z_seg_h = (nz + zz - 1) / zz;
         p.s3_z_nsegs = (nz + p.s3_z_seg_h - 1) / p.s3_z_seg_h;
     }
@@ -857,7 +913,7 @@ void default_plan(dirac_grid *g) {
         // 4.5 against 4.2 G)
         const bool one = !g->fp32 && char_shift(g) == 2 && !field_on(g);
         const int P = pp == 1 || pp == 2 ? pp : (one ? 1 : 2);
-        make_plan(g, 1, P, 4, one && P == 1 ? 24 : 8);
+        make_plan(g, 1, P, 4, 0);
         return;
     }
     const int mode = sweep_mode(g);
@@ -868,7 +924,7 @@ void default_plan(dirac_grid *g) {
             K = 1;
             P = 1;
         }
-        make_plan(g, K, P, 4, 16);
+        make_plan(g, K, P, 4, 0);
         return;
     }
     // FP64: one point a lane, 16 warps an SM (four blocks of 128 registers): the sweeps' pairs split over the FP64 and
@@ -877,6 +933,9 @@ void default_plan(dirac_grid *g) {
     int K = g->fp32 ? 2 : 1, P = g->fp32 ? 2 : 1;
     if (mode == 3 || mode == 5) K = 1;  // measured: the field's phase matrix makes k = 2 register-bound
     if (mode == 2) K = g->fp32 ? 2 : 1;  // FP32 second order: two steps per pass with the history in shared memory
+    // small FP32 grids, second order: one step a launch with one cell a lane, whose short rows spread over the chip
+    // (300 x 257: 11.5 us a step against 13; 900 x 700: 25.4 against 26.2; 1400^2: 45.1 against 44.0)
+    if (mode == 2 && g->fp32 && k == 0 && pp == 0 && g->ncells < (1 << 20)) K = P = 1;
     if (k > 0) K = k;
     if (pp > 0) P = pp;
     if (!sweep_supported(g->fp32, mode, K, P)) P = sweep_supported(g->fp32, mode, K, 4) ? 4 : 2;
@@ -884,10 +943,7 @@ void default_plan(dirac_grid *g) {
         K = 1;
         P = 2;
     }
-    // FP32 P = 2 with the sweep history in shared memory: four blocks per SM fit (first order two steps per
-    // pass, second order one)
-    const bool four = g->fp32 && P == 2 && ((mode == 0 && K == 2) || (mode == 2 && K == 1));
-    make_plan(g, K, P, 4, g->fp32 ? (four ? 16 : 12) : (P == 1 ? 16 : 8));
+    make_plan(g, K, P, 4, 0);
 }
 
 }  // namespace
@@ -1502,7 +1558,7 @@ dirac_status dirac_autotune(dirac_grid *g) {
         const int KP[][2] = {{1, 1}, {1, 2}, {1, 4}, {2, 2}};
         for (auto &kp : KP)
             if (sweep_supported_fx(sweep_mode(g), kp[0], kp[1]))
-                for (int wsm : {8, 12, 16, 24}) cands.push_back({kp[0], kp[1], 4, wsm});
+                for (int wsm : {0, 8, 12, 16, 24}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else if (g->cfg.ndim == 3) {
         if (!field_on(g))  // with a vector potential only the fused pass applies the phase matrix
             for (int P : {1, 2, 4})
@@ -1511,25 +1567,25 @@ dirac_status dirac_autotune(dirac_grid *g) {
         cands.push_back({2, 2, 4, 16, 16});  // two steps per fused pass
     } else if (sweep_mode(g) == 4) {
         for (int P : {1, 2})
-            for (int wsm : {4, 8, 12, 16, 24}) cands.push_back({1, P, 4, wsm});
+            for (int wsm : {0, 4, 8, 12, 16, 24}) cands.push_back({1, P, 4, wsm});
     } else if (sweep_mode(g) == 3 || sweep_mode(g) == 5) {
         const int KP[][2] = {{1, 1}, {1, 2}, {2, 2}};
         for (auto &kp : KP)
             if (sweep_supported(g->fp32, sweep_mode(g), kp[0], kp[1]))
-                for (int wsm : {4, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
+                for (int wsm : {0, 4, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else if (strang(g)) {
         const int KP[][2] = {{1, 1}, {1, 2}, {1, 4}, {2, 2}};
         for (auto &kp : KP)
             if (sweep_supported(g->fp32, 2, kp[0], kp[1]))
-                for (int wsm : {4, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
+                for (int wsm : {0, 4, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else if (g->fp32) {
         const int KP[][2] = {{1, 2}, {1, 4}, {2, 2}, {2, 4}, {4, 2}};
         for (auto &kp : KP)
-            for (int wsm : {8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
+            for (int wsm : {0, 8, 12, 16}) cands.push_back({kp[0], kp[1], 4, wsm});
     } else {
         const int KP[][2] = {{1, 1}, {1, 2}, {2, 2}};
         for (auto &kp : KP)
-            for (int wsm : {8, 12, 16, 24}) cands.push_back({kp[0], kp[1], 4, wsm});
+            for (int wsm : {0, 8, 12, 16, 24}) cands.push_back({kp[0], kp[1], 4, wsm});
     }
     // save state and counters
     const size_t bytes = (size_t)g->ncells * 8 * g->elem;
@@ -1589,7 +1645,7 @@ dirac_status dirac_autotune(dirac_grid *g) {
         if (best.s3) g->plan.s3_warps = best.s3;
         g->plan.s3_zfactor = best.s3z;
         g->plan.s3_zpass = best.s3zp;
-        make_plan(g, best.K, best.P, best.wpb, best.wsm ? best.wsm : 8);
+        make_plan(g, best.K, best.P, best.wpb, best.wsm);
         st = ensure_flux_part(g);
     }
     g->cur = cur_saved;
