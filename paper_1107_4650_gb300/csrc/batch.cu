@@ -7,7 +7,7 @@ namespace dirac {
 namespace {
 template <typename T, int K, int P>
 cudaError_t launch_batch_t(const BatchArgs &b, int blocks, cudaStream_t s) {
-    const int smem = ring_smem_bytes<T, K, P>(4);
+    const int smem = ring_smem_bytes<T, K, P, BatchHist<T, K, P>::value>(4);
     cudaError_t e = cudaFuncSetAttribute(batch_kernel<T, K, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     batch_kernel<T, K, P><<<blocks, 128, smem, s>>>(b);
@@ -15,7 +15,7 @@ cudaError_t launch_batch_t(const BatchArgs &b, int blocks, cudaStream_t s) {
 }
 template <typename T, int K, int P>
 cudaError_t occupancy_t(int *blocks_per_sm) {
-    const int smem = ring_smem_bytes<T, K, P>(4);
+    const int smem = ring_smem_bytes<T, K, P, BatchHist<T, K, P>::value>(4);
     cudaError_t e = cudaFuncSetAttribute(batch_kernel<T, K, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<T, K, P>, 128, smem);

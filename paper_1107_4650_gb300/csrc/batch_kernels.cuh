@@ -40,11 +40,19 @@ struct BatchArgs {
     double vol;
 };
 
+// FP32 with two points a lane and two or four steps a launch: the sweep history in shared memory and one row per
+// iteration (24 runs of sides 768 and 1024, four steps: 196 against 157 G point-steps/s with it in registers and two
+// rows per iteration; two steps: 168 against 167; sides 256 to 1024: 158 against 133 and 131 against 135).
+template <typename T, int K, int P> struct BatchHist {
+    static constexpr bool value = sizeof(T) == 4 && P == 2 && K >= 2;
+    static constexpr int unroll = value ? 1 : 2;
+};
+
 template <typename T, int K, int P>
 __global__ void __launch_bounds__(128) batch_kernel(const BatchArgs b) {
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     const int lane = threadIdx.x & 31;
-    unsigned char *wsmem = dyn_smem + (threadIdx.x >> 5) * Ring<T, K, P>::WARP_BYTES;
+    unsigned char *wsmem = dyn_smem + (threadIdx.x >> 5) * Ring<T, K, P, BatchHist<T, K, P>::value>::WARP_BYTES;
     const int64_t total = b.task_off[b.n_active];
     for (;;) {
         unsigned task = 0;
@@ -78,7 +86,8 @@ __global__ void __launch_bounds__(128) batch_kernel(const BatchArgs b) {
         a.periodic = 0;
         a.full_table = 0;
         a.flux_unit = 1.0;  // floating-point states
-        sweep_warp<T, K, P, 0, false, 2>(a, (int64_t)task - b.task_off[lo], lane, wsmem);  // two rows per iteration: measured faster here
+        a.wide = 1;         // the pool is the library's own, a cell 32 or 64 bytes
+        sweep_warp<T, K, P, 0, false, BatchHist<T, K, P>::unroll, BatchHist<T, K, P>::value>(a, (int64_t)task - b.task_off[lo], lane, wsmem);
     }
     // last block folds the flux partials of every active run and resets the counters
     __shared__ unsigned s_last;

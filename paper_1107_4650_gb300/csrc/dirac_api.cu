@@ -292,7 +292,8 @@ int64_t pick_rows(int64_t n, int64_t units, int per_block, int64_t sms, int64_t 
         const int64_t blocks = (units * segs + per_block - 1) / per_block;
         const int64_t per_sm = (blocks + sms - 1) / sms;  // on the fullest SM
         const int64_t waves = per_sm / resident, rest = per_sm % resident;
-        const double t = ((double)h + halo) * (waves * row_time(resident) + (rest ? row_time(rest) : 0.0)) + uneven * h * row_time(1);
+        const double t = ((double)h + halo) * (waves * row_time(resident) + (rest ? row_time(rest) : 0.0)) +
+                         uneven * h * row_time(std::min(resident, per_sm));
         if (t < best * 0.999) {  // near ties: the longer segments
             best = t;
             best_h = h;
@@ -347,7 +348,9 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
     const int64_t want = (int64_t)g->sm_count * (model ? 16 : target_warps_per_sm);
     if (model) {
         const RowTime rt = row_time_of(g, K, P);
-        p.seg_h = pick_rows(nr, p.nstrips * planes, wpb, g->sm_count, resident_blocks(g, K, P), 2.0 * Lv, 0.0,
+        // a wave's blocks end apart: FP32 at 4096^2, k = 2, 165 G point-steps/s in one wave, 170-175 in two to four; at
+        // 2048^2 145 in one, 130 in two; fixed point at 2048^2 33.7 in one, 32.8 in two
+        p.seg_h = pick_rows(nr, p.nstrips * planes, wpb, g->sm_count, resident_blocks(g, K, P), 2.0 * Lv, g->fp32 ? 0.2 : 0.1,
                             [&](int64_t blocks) { return rt(blocks * wpb); });
     } else {
         int64_t nsegs = std::max<int64_t>(1, want / std::max<int64_t>(1, p.nstrips * planes));
@@ -438,6 +441,11 @@ dirac_status ensure_flux_part(dirac_grid *g) {
     return DIRAC_OK;
 }
 
+// Both state buffers lie on 32-byte boundaries (always, but for caller-owned ones).
+int wide_state(const dirac_grid *g) {
+    return ((reinterpret_cast<uintptr_t>(g->psi[0]) | reinterpret_cast<uintptr_t>(g->psi[1])) & 31u) == 0;
+}
+
 // One block of work: K steps (2-D) or one step (3-D), from psi[parity] to psi[parity ^ 1] (2-D) or back
 // to psi[parity] (3-D).  Enqueued on s.  K_override > 0 runs that many steps with P from the plan.
 dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int64_t step0) {
@@ -447,6 +455,7 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
     SweepArgs a{};
     a.in = g->psi[parity];
     a.out = g->psi[parity ^ 1];
+    a.wide = wide_state(g);
     a.table = g->table;
     a.nx = g->cfg.n[0];
     a.nr = (ndim_of(g) == 3) ? g->cfg.n[1] : g->cfg.n[2];
@@ -675,6 +684,7 @@ dirac_status enqueue_strang3d_run(dirac_grid *g, int parity, int64_t m, cudaStre
         const Plan::XY &q = p.s3_xy[nh - 1];
         a.in = g->psi[par];
         a.out = g->psi[par ^ 1];
+        a.wide = wide_state(g);
         a.nsegs = q.nzsegs * q.nytiles * p.s3_warps;  // flux parts per x sweep
         double fsu[4];
         for (int i = 0; i < 4; ++i) fsu[i] = fs[i] * funit;
@@ -937,6 +947,7 @@ void default_plan(dirac_grid *g) {
     // (300 x 257: 11.5 us a step against 13; 900 x 700: 25.4 against 26.2; 1400^2: 45.1 against 44.0)
     if (mode == 2 && g->fp32 && k == 0 && pp == 0 && g->ncells < (1 << 20)) K = P = 1;
     if (k > 0) K = k;
+    if (mode == 0 && g->fp32 && K == 1) P = 1;  // one step a launch: 84.9 against 76.8 G at 2048^2
     if (pp > 0) P = pp;
     if (!sweep_supported(g->fp32, mode, K, P)) P = sweep_supported(g->fp32, mode, K, 4) ? 4 : 2;
     if (!sweep_supported(g->fp32, mode, K, P)) {

@@ -41,6 +41,7 @@ struct SweepArgs {
     // failure-detection test hook (DIRAC_INJECT_STALL): the launch's first warp makes its first row-copy
     // wait run out, so the kernel reports DIRAC_ERR_TIMEOUT through *err
     int inject_stall;
+    int wide = 0;  // `out` is 32-byte aligned: points are stored in 32-byte pieces
     // multiplies the face-flux sums: 1 for floating-point states, 2^-2S for a fixed-point state q = psi 2^S
     double flux_unit = 1.0;
 };

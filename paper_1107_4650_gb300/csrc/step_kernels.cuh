@@ -74,6 +74,22 @@ template <typename T> __device__ __forceinline__ Cx<T> cadd(Cx<T> a, Cx<T> b) {
 template <typename T> __device__ __forceinline__ Cx<T> csub(Cx<T> a, Cx<T> b) {
     return {Ar<T>::sub(a.re, b.re), Ar<T>::sub(a.im, b.im)};
 }
+// FP32: real and imaginary part in one packed instruction (two independent round-to-nearest adds: the same bits as two
+// scalar ones in half the issue slots)
+template <> __device__ __forceinline__ Cx<float> cadd<float>(Cx<float> a, Cx<float> b) {
+    Cx<float> r;
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 c, a, b;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "=f"(r.re), "=f"(r.im)
+        : "f"(a.re), "f"(a.im), "f"(b.re), "f"(b.im));
+    return r;
+}
+template <> __device__ __forceinline__ Cx<float> csub<float>(Cx<float> a, Cx<float> b) {
+    Cx<float> r;
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tsub.rn.f32x2 c, a, b;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "=f"(r.re), "=f"(r.im)
+        : "f"(a.re), "f"(a.im), "f"(b.re), "f"(b.im));
+    return r;
+}
 // a + i b and a - i b
 template <typename T> __device__ __forceinline__ Cx<T> cadd_ib(Cx<T> a, Cx<T> b) {
     return {Ar<T>::sub(a.re, b.im), Ar<T>::add(a.im, b.re)};
@@ -222,6 +238,72 @@ __device__ __forceinline__ void store_pt(long long *p, const Cx<long long> s[4])
 #pragma unroll
     for (int c = 0; c < 4; ++c) q[c] = make_longlong2(s[c].re, s[c].im);
 }
+// A point stored to global memory in 32-byte pieces (whole sectors, half the store instructions), where the buffer is
+// 32-byte aligned (`wide`; caller-owned buffers need only 16 bytes).
+template <typename T> __device__ __forceinline__ void store_cell(T *p, const Cx<T> s[4], bool wide) {
+    if (wide) {
+        if constexpr (sizeof(T) == 4) {
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(s[0].re), "f"(s[0].im),
+                         "f"(s[1].re), "f"(s[1].im), "f"(s[2].re), "f"(s[2].im), "f"(s[3].re), "f"(s[3].im)
+                         : "memory");
+        } else if constexpr (std::is_same<T, double>::value) {
+            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(s[0].re), "d"(s[0].im), "d"(s[1].re),
+                         "d"(s[1].im)
+                         : "memory");
+            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p + 4), "d"(s[2].re), "d"(s[2].im), "d"(s[3].re),
+                         "d"(s[3].im)
+                         : "memory");
+        } else {
+            asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(s[0].re), "l"(s[0].im), "l"(s[1].re),
+                         "l"(s[1].im)
+                         : "memory");
+            asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p + 4), "l"(s[2].re), "l"(s[2].im), "l"(s[3].re),
+                         "l"(s[3].im)
+                         : "memory");
+        }
+    } else {
+        store_pt(p, s);
+    }
+}
+// A point of a row in shared memory, lane l holding point l (consecutive points).  FP32: lanes 4-7 of every eight take
+// their two 16-byte halves in the other order, so that eight lanes' reads cover all banks once (in one order the halves
+// of points four apart meet in one bank).
+template <typename T> __device__ __forceinline__ void load_row_pt(const T *p, int lane, Cx<T> s[4]) {
+    if constexpr (sizeof(T) == 4) {
+        const int swap = (lane >> 2) & 1;
+        const float4 *q = reinterpret_cast<const float4 *>(p);
+        const float4 f = q[swap], g = q[swap ^ 1];
+        s[0] = {swap ? g.x : f.x, swap ? g.y : f.y};
+        s[1] = {swap ? g.z : f.z, swap ? g.w : f.w};
+        s[2] = {swap ? f.x : g.x, swap ? f.y : g.y};
+        s[3] = {swap ? f.z : g.z, swap ? f.w : g.w};
+    } else {
+        load_pt(p, s);
+    }
+}
+// The two sums a level keeps of a row's point, in the warp's shared memory: consecutive lanes 16 bytes apart (no bank
+// conflict).  `p` is the pair's place for this lane: 4-byte types keep both sums there, 8-byte types 32 lanes apart.
+template <typename T> __device__ __forceinline__ Cx<T> *hist_at(Cx<T> *hist, int slot, int lane) {
+    return sizeof(T) == 4 ? hist + (slot * 32 + lane) * 2 : hist + slot * 64 + lane;
+}
+template <typename T> __device__ __forceinline__ void hist_load(const Cx<T> *p, Cx<T> &a, Cx<T> &b) {
+    if constexpr (sizeof(T) == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(p);
+        a = {v.x, v.y};
+        b = {v.z, v.w};
+    } else {
+        a = p[0];
+        b = p[32];
+    }
+}
+template <typename T> __device__ __forceinline__ void hist_store(Cx<T> *p, Cx<T> a, Cx<T> b) {
+    if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4 *>(p) = make_float4(a.re, a.im, b.re, b.im);
+    } else {
+        p[0] = a;
+        p[32] = b;
+    }
+}
 __device__ __forceinline__ void load_tab(const long long *p, Cx<long long> &pu, Cx<long long> &pd) {
     const longlong2 *q = reinterpret_cast<const longlong2 *>(p);
     longlong2 a = q[0], b = q[1];
@@ -256,12 +338,12 @@ template <typename T> struct IsF64 { static constexpr bool value = std::is_same<
 // memory instead of registers, one slot per row parity so that nothing moves.  Measured at 2048^2 (G point-steps/s,
 // the same bits every time):
 //   FP32, P = 2: at k = 2 the registers it frees let four blocks (16 warps) per SM run without spilling, 114.5
-//     against 105.0; at k = 4 208 -> 128 registers, 105.3 against 67.1; second order (mode 2) 60.8 against 56.8.
+//     against 105.0 (145 since its accesses are free of bank conflicts); at k = 4 208 -> 128 registers, 105.3 against
+//     67.1 (146); second order (mode 2) 60.8 against 56.8 (81).
 //   FP64, P = 1: four blocks without spilling, 13.1 against 12.3 first order.
 //   Fixed point, P = 1, second order: four blocks instead of two, 22.9 against 19.9 (periodic 22.4 against 20.6);
 //     first order periodic 31.9 against 31.6, but zero boundary 31.8 against 33.7: registers there.
-// The batched kernel, which runs the same warp routine, keeps the history in registers (107.5 against 116.0 G with
-// it in shared memory).
+// (batch_kernels.cuh has its own choice.)
 template <typename T, int K, int P, int MODE, bool PER> struct HistSmem {
     static constexpr bool value =
         (IsF64<T>::value && P == 1 && K == 1 && MODE != 1) ||
@@ -370,6 +452,15 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_
         "l"(src), "r"(bytes), "r"(bar)
         : "memory");
 }
+// The lane with `issue` set: orders the warp's reads of a slot before its refill, announces the bytes and starts the copy.
+__device__ __forceinline__ void refill_row(bool issue, uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p fence.proxy.async.shared::cta;\n\t"
+        "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%4], %3;\n\t"
+        "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%1], [%2], %3, [%4];\n\t}" ::"r"((uint32_t)issue),
+        "r"(dst), "l"(src), "r"(bytes), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -398,7 +489,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 }
 
 // Per-warp shared memory: 128 B of mbarriers, the row ring, the flux hand-off area (K levels x 8 values x 32
-// lanes), then with HS the sweep history ([row parity 2][level K][lane 32][point P][2] complex values; the ring
+// lanes), then with HS the sweep history ([row parity 2][level K][point P][lane 32], two complex values each; the ring
 // keeps three rows so that four blocks fit, two of the 8-byte types, whose rows last long enough).
 template <typename T, int K, int P, bool HS> struct Ring {
     static constexpr int ROW_BYTES = 32 * P * 8 * (int)sizeof(T);  // one warp row: 32P cells
@@ -585,8 +676,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     Cx<T> *hist = reinterpret_cast<Cx<T> *>(wsmem + 128 + RG::SLOTS * RG::ROW_BYTES + RG::FLUX_BYTES);
     if (HS) {
 #pragma unroll
-        for (int t = 0; t < 2 * L * P * 2; ++t)
-            hist[((t / (L * P * 2) * L + (t / (P * 2)) % L) * 32 + lane) * P * 2 + t % (P * 2)] = Cx<T>{T(0), T(0)};
+        for (int t = 0; t < 2 * L * P; ++t) hist_store(hist_at(hist, t, lane), Cx<T>{T(0), T(0)}, Cx<T>{T(0), T(0)});
     }
     T *gsm = reinterpret_cast<T *>(wsmem + 128 + RG::SLOTS * RG::ROW_BYTES);  // flux hand-off [K][8][32]
     // span of grid cells a row copy brings: the strip clipped to the grid; periodic: all 32 P cells, wrapped, as
@@ -630,6 +720,14 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         for (int sl = 0; sl < RG::SLOTS; ++sl) mbar_init(bar0 + 8 * sl, 1);
         mbar_fence_init();
     }
+    if (!strip_in) {  // cells outside the grid: zero in every slot, and no copy reaches them
+        const Cx<T> none[4] = {{T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}};
+#pragma unroll
+        for (int sl = 0; sl < RG::SLOTS; ++sl)
+#pragma unroll
+            for (int j = 0; j < P; ++j)
+                if (!xin[j]) store_pt(reinterpret_cast<T *>(wsmem + 128 + sl * RG::ROW_BYTES) + (32 * j + lane) * 8, none);
+    }
     __syncwarp();
     bool stall = a.inject_stall && wid == 0 && !per;
 #pragma unroll
@@ -650,27 +748,31 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         }
     }
 
+    // One input row through the levels.  STEADY: every level's output row is wanted and lies inside the grid (all rows
+    // but a segment's first 2 L and the last ones beyond the grid), so nothing is tested per level: FP32 k = 2 at 2048^2
+    // 42.0 -> 31.4 M warp instructions a launch with the packed adds, k = 4 125 -> 139 G point-steps/s, the batched
+    // kernel 154 -> 164.  What then bounds the FP32 kernel is the shared-memory pipe (82 % busy at k = 2, half of it bank
+    // conflicts of the history and the row reads): without the conflicts and with 32-byte stores 124 -> 145 G.
+    T *orow = out + ((int64_t)(r_first - L) * nx + xa + lane) * 8;       // this lane's cell of output row r - L
+    const T *frow = in + ((int64_t)(r_first + RG::SLOTS) * nx + cx0) * 8;  // zero boundary: span of row r + SLOTS
+    const RI f_end = per ? r_last : min(r_last, nr32);                   // rows [.., f_end) are fetched
+    const int64_t row_step = nx * 8;
     int sl = 0;
-    for (RI r0 = r_first; r0 < r_last && !aborted; r0 += UNR) {
-#pragma unroll
-    for (int par = 0; par < UNR; ++par) {
-        const RI r = r0 + par;
-        if (r >= r_last) break;
+    auto do_row = [&](auto steady_c, auto par_c, const RI r) -> bool {
+        constexpr bool STEADY = decltype(steady_c)::value;
+        constexpr int par = decltype(par_c)::value;
         Cx<T> st[P][4];
-        const bool row_ok = per || (r >= 0 && r < nr32);
+        const bool row_ok = STEADY || per || (r >= 0 && r < nr32);
         if (row_ok) {
-            if (!mbar_wait(bar0 + 8 * sl, (phase_bits >> sl) & 1u)) {
-                aborted = true;
-                break;
-            }
+            if (!mbar_wait(bar0 + 8 * sl, (phase_bits >> sl) & 1u)) return false;
             phase_bits ^= 1u << sl;
             pending &= ~(1u << sl);
         }
-        const T *srow = reinterpret_cast<const T *>(wsmem + 128 + sl * RG::ROW_BYTES);
+        const T *srow = reinterpret_cast<const T *>(wsmem + 128 + sl * RG::ROW_BYTES) + lane * 8;
 #pragma unroll
         for (int j = 0; j < P; ++j) {
-            if (row_ok && (per || xin[j])) {
-                load_pt(srow + (32 * j + lane) * 8, st[j]);
+            if (row_ok) {
+                load_row_pt(srow + 32 * 8 * j, lane, st[j]);
             } else {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) st[j][c] = {T(0), T(0)};
@@ -679,24 +781,24 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
 #pragma unroll
         for (int lev = 0; lev < L; ++lev) {
             const RI q = r - lev;  // row of the level-lev state in st
-            // rows of level lev+1 that later levels (or the store) use: [r_first + lev + 1, r_last - lev - 1)
-            const bool need_out = (q - 1 >= r_first + lev + 1) && (q - 1 < r_last - lev - 1);
+            // rows of level lev+1 that later levels (or the store) use begin at r_first + lev + 1
+            const bool need_out = STEADY || r >= r_first + 2 * lev + 2;
             if ((MODE == 2 || MODE == 5) && (lev & 1)) {
                 // second half of a Strang step: z sweep of rows q-2 and q into row q-1, then the x sweep of
                 // row q-1.  The input is 1/4 of the state (the phase carried 1/16), the z-swept row 1/2 of it.
-                const bool zrow_ok = per || (q - 1 >= 0 && q - 1 < nr32);
+                const bool zrow_ok = STEADY || per || (q - 1 >= 0 && q - 1 < nr32);
                 Cx<T> zs[P][4];
 #pragma unroll
                 for (int j = 0; j < P; ++j) {
                     Cx<T> U13, W13, U24, W24;
                     z_chars<HY>(st[j], U13, W13, U24, W24);
                     Cx<T>(&UO)[2] = UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j];  // row q - 2
-                    Cx<T> *hq = hist + ((((int)(q & 1) * L + lev) * 32 + lane) * P + j) * 2;  // HS: its slot
-                    const Cx<T> o0 = HS ? hq[0] : UO[0], o1 = HS ? hq[1] : UO[1];
+                    Cx<T> *hq = hist_at(hist, ((int)(q & 1) * L + lev) * P + j, lane);  // HS: its slot
+                    Cx<T> o0 = UO[0], o1 = UO[1];
+                    if (HS) hist_load(hq, o0, o1);
                     z_join<HY>(o0, W13, o1, W24, zs[j]);
                     if (HS) {
-                        hq[0] = U13;
-                        hq[1] = U24;
+                        hist_store(hq, U13, U24);
                     } else {
                         push_row<T, UNR>(UH[0][lev][j], UH[1][lev][j], UO, U13, U24);
                     }
@@ -750,7 +852,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
             if (has_face && q >= r_begin && q < r_end)
                 flux_row<T, P>(lu14, lu23, w14, w23, face_j, face_lane, lane, q - r_begin, q == r_end - 1,
                                gsm + lev * 8 * 32, 0.5 * a.flux_unit, facc[lev]);
-            const bool out_row_ok = per || (q - 1 >= 0 && q - 1 < nr32);
+            const bool out_row_ok = STEADY || per || (q - 1 >= 0 && q - 1 < nr32);
 #pragma unroll
             for (int j = 0; j < P; ++j) {
                 // x sweep (Eq. sol_dis_1), x2
@@ -761,11 +863,10 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                     Cx<T> U13, W13, U24, W24;
                     z_chars<HY>(b, U13, W13, U24, W24);
                     // row q - 2's sums: the slot of q's parity (HS) or the register slot
-                    Cx<T> *hp = hist + ((((int)(q & 1) * L + lev) * 32 + lane) * P + j) * 2;
+                    Cx<T> *hp = hist_at(hist, ((int)(q & 1) * L + lev) * P + j, lane);
                     Cx<T> h0, h1;
                     if (HS) {
-                        h0 = hp[0];
-                        h1 = hp[1];
+                        hist_load(hp, h0, h1);
                     } else {
                         h0 = UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][0];
                         h1 = UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j][1];
@@ -806,8 +907,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                         }
                     }
                     if (HS) {  // row q's sums replace row q - 2's
-                        hp[0] = U13;
-                        hp[1] = U24;
+                        hist_store(hp, U13, U24);
                     } else {
                         push_row<T, UNR>(UH[0][lev][j], UH[1][lev][j], UH[UNR == 2 ? (par + lev) & 1 : 0][lev][j], U13, U24);
                     }
@@ -836,33 +936,44 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                 }
             }
         }
-        const RI ro = r - L;
-        if (ro >= r_begin && ro < r_end) {
-            if constexpr (sizeof(RI) == 8) {
+        if (STEADY || r >= r_first + 2 * L) {
 #pragma unroll
-                for (int j = 0; j < P; ++j) {
-                    const int64_t x = xa + 32 * j + lane;
-                    if (x >= x_own0 && x < x_own1) store_pt(out + (ro * nx + x) * 8, st[j]);
-                }
-            } else {
-                T *orow = out + (int64_t)ro * nx * 8;
-#pragma unroll
-                for (int j = 0; j < P; ++j)
-                    if (own[j]) store_pt(orow + (xa + 32 * j + lane) * 8, st[j]);
-            }
+            for (int j = 0; j < P; ++j)
+                if (own[j]) store_cell(orow + 32 * 8 * j, st[j], a.wide != 0);
         }
         // refill this slot with row r + SLOTS once every lane has read it
         __syncwarp();
         const RI rn = r + RG::SLOTS;
-        if (rn < r_last && (per || (rn >= 0 && rn < nr32))) {
-            if (lane == 0) {
-                fence_proxy_async();
-                fetch_row(grid_row(rn), sl);
+        if (rn < f_end && (STEADY || per || rn >= 0)) {
+            if (per) {
+                if (lane == 0) {
+                    fence_proxy_async();
+                    fetch_row(grid_row(rn), sl);
+                }
+            } else {
+                refill_row(lane == 0, slot0 + sl * RG::ROW_BYTES + dst_off, frow, copy_bytes, bar0 + 8 * sl);
             }
             pending |= 1u << sl;
         }
         sl = (sl + 1 == RG::SLOTS) ? 0 : sl + 1;
-    }
+        orow += row_step;
+        frow += row_step;
+        return true;
+    };
+    using Even = std::integral_constant<int, 0>;
+    using Odd = std::integral_constant<int, 1>;
+    // (FP64 rows are long beside the tests, and a second copy of them costs more than it saves: 13.0 against 13.4 G)
+    constexpr bool SPLIT = !IsF64<T>::value;
+    const RI steady0 = r_first + 2 * L, steady1 = f_end;
+    for (RI r = r_first; r < r_last && !aborted; r += UNR) {
+        if (UNR == 1) {
+            aborted = !(SPLIT && r >= steady0 && r < steady1 ? do_row(std::true_type{}, Even{}, r) : do_row(std::false_type{}, Even{}, r));
+        } else if (SPLIT && r >= steady0 && r + 1 < steady1) {
+            aborted = !(do_row(std::true_type{}, Even{}, r) && do_row(std::true_type{}, Odd{}, r + 1));
+        } else {
+            aborted = !do_row(std::false_type{}, Even{}, r);
+            if (!aborted && r + 1 < r_last) aborted = !do_row(std::false_type{}, Odd{}, r + 1);
+        }
     }
     if (aborted) {
         // a copy never completed: report, then wait (bounded) for this warp's copies still in flight
