@@ -374,7 +374,8 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         p.f_nytiles = (g->cfg.n[1] + (p.f_warps - 2) - 1) / (p.f_warps - 2);
         const int64_t tiles = p.f_nstrips * p.f_nytiles;
         const auto whole = [](int64_t blocks) { return (double)blocks; };  // the passes: time as the blocks on an SM
-        p.f_zseg_h = pick_rows(nz, tiles, 1, g->sm_count, 1, 3.0, 0.5, whole);
+        const int f_resident = !g->fp32 && p.f_warps == 8 ? 2 : 1;
+        p.f_zseg_h = pick_rows(nz, tiles, 1, g->sm_count, f_resident, 3.0, 0.5, whole);
         p.f_nzsegs = (nz + p.f_zseg_h - 1) / p.f_zseg_h;
         // two steps per fused pass: 28-cell strips x (warps - 4)-row tiles (16 warps in FP32, 8 in FP64), z
         // segments as above (each carries two halo planes a side)
@@ -890,7 +891,7 @@ void default_plan(dirac_grid *g) {
         // the fused passes (bandwidth-bound integer sweeps: the passes move a seventh of the single sweeps' bytes),
         // 4 = single x and y sweeps with one z-phase-z pass
         g->plan.fused3d = pp > 0 ? 0 : 1;
-        g->plan.f_warps = g->cfg.n[1] <= 12 ? 8 : 16;
+        g->plan.f_warps = 8;  // two blocks an SM (fused3d_kernels.cuh)
         g->plan.s3_fused = (strang(g) && pp != 1 && pp != 4) ? 1 : 0;
         g->plan.s3_zpass = (strang(g) && pp == 4) ? 1 : 0;
         g->plan.s3_warps = 32;  // measured at 384^3: 12.5 G point-steps/s against 10.5 with 16-warp blocks (fewer
@@ -901,7 +902,9 @@ void default_plan(dirac_grid *g) {
     if (ndim_of(g) == 3) {
         // points_per_lane 0: the fused single-pass step; 1, 2 or 4: the x-y pass + z/phase pass with that P
         g->plan.fused3d = pp > 0 ? 0 : 1;
-        g->plan.f_warps = g->cfg.n[1] <= 12 ? 8 : 16;  // short y extents: 6-row tiles waste fewer halo rows
+        // FP64: 8-warp blocks, two on an SM (fused3d_kernels.cuh); FP32: 16, short y extents 8 (6-row tiles waste fewer
+        // halo rows)
+        g->plan.f_warps = !g->fp32 || g->cfg.n[1] <= 12 ? 8 : 16;
         // second-order step: points_per_lane 1 = eight single-sweep launches, 2 = the three fused passes, 4 = x and
         // y single sweeps with one z-phase-z pass, 0 = library choice (fused passes for FP32 storage, which is
         // bandwidth-bound; for FP64, which is bound by the FP64 pipe and would recompute the x-y-x pass's halo

@@ -7,8 +7,8 @@
 //   * each warp loads its row of the plane, x-sweeps it with warp shuffles and writes the row's y
 //     characteristics (U = "+y" movers, W = "-y" movers) to shared memory (double-buffered by plane);
 //   * after one block barrier the owned warps y-sweep their row from the rows above and below;
-//   * the z sweep keeps the "+z" sums of the two previous planes per cell in registers (output plane
-//     k - 1 = U(k - 2) + W(k)), then the phase with the table pre-scaled by 1/8, and the store.
+//   * the z sweep keeps the "+z" sums of the two previous planes per cell, in registers or in shared memory
+//     (output plane k - 1 = U(k - 2) + W(k)), then the phase with the table pre-scaled by 1/8, and the store.
 // Arithmetic order is that of the two-kernel 3-D path (x-y pass at 4x scale, then z sweep and phase), so
 // the FP64 result is the same bit for bit.  Face flux: the lanes holding cells face-1 and face of owned
 // rows and planes add 1/2 (|u14|^2+|u23|^2) and subtract 1/2 (|w14|^2+|w23|^2) of the state entering the x
@@ -47,9 +47,18 @@ __device__ __forceinline__ typename FaceAcc<T>::type face_sq(Cx<T> p14, Cx<T> p2
                       Ar<F>::fma((F)p14.im, (F)p14.im, Ar<F>::fma((F)p23.re, (F)p23.re, Ar<F>::mul((F)p23.im, (F)p23.im))));
 }
 
+// FP64 and fixed-point states keep the z sweep's history (the "+z" sums of the two previous planes) in shared memory,
+// one slot per plane parity: the registers it frees let two 8-warp blocks run on an SM, whose barriers then fall at
+// different times (256^3: FP64 with its pairs over two pipes 7.2 G point-steps/s against 6.9 in one 16-warp block and 6.05
+// on the FP64 pipe alone; in a laser field 4.3 against 3.8 and 3.6; fixed point 23.4 against 19.9), although 6 of 8 rows are
+// owned instead of 14 of 16.
+template <typename T> struct Fused3DHist { static constexpr bool value = sizeof(T) == 8; };
+template <typename T, int W> struct Fused3DMinBlocks { static constexpr int value = sizeof(T) == 8 && W == 8 ? 2 : 1; };
 template <typename T, int W, bool FIELD>
-__global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A) {
+__global__ void __launch_bounds__(32 * W, Fused3DMinBlocks<T, W>::value) fused3d_kernel(const Fused3DArgs A) {
     constexpr int H = W - 2;
+    constexpr bool HY = true;  // FP64 pairs over two pipes
+    constexpr bool HS = Fused3DHist<T>::value;
     const SweepArgs &a = A.s;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t b = blockIdx.x;
@@ -88,7 +97,12 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
     double facc = 0.0;
     typename FaceAcc<T>::type fpart = 0;
 
+    // "+z" sums of the two previous planes: registers, or (HS) the warp's shared memory, slot = plane parity
     Cx<T> UA[2] = {{T(0), T(0)}, {T(0), T(0)}}, UB[2] = {{T(0), T(0)}, {T(0), T(0)}};
+    Cx<T> *zh = ych + 2 * W * 4 * 32 + w * 4 * 32 + lane;  // [slot][2][32]
+    if (HS)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) zh[q * 32] = Cx<T>{T(0), T(0)};
 
     // cell (xl, yl) of a plane: plane k at (k nx ny + cell) (periodic: halo planes wrap)
     const int64_t plane_cells = nx * ny, cell = yl * nx + xl;
@@ -132,7 +146,7 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
         if (k + LA <= z_end) load_row(k + LA, ring[LA - 1]);
         // x characteristics and the x sweep (neighbours by shuffle; lanes 0 and 31 are halo cells)
         Cx<T> u14, w14, u23, w23;
-        x_chars<false>(st, u14, w14, u23, w23);
+        x_chars<HY>(st, u14, w14, u23, w23);
         if (face_lane && k >= z_begin && k < z_end) {
             using F = typename FaceAcc<T>::type;
             const F v = (x == face - 1) ? face_sq(u14, u23) : -face_sq(w14, w23);
@@ -145,8 +159,8 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
         const Cx<T> lu14 = shfl_c(u14, (lane + 31) & 31), lu23 = shfl_c(u23, (lane + 31) & 31);
         const Cx<T> rw14 = shfl_c(w14, (lane + 1) & 31), rw23 = shfl_c(w23, (lane + 1) & 31);
         Cx<T> b4[4], U14, W14, U23, W23;
-        x_join<false>(lu14, rw14, lu23, rw23, b4);
-        y_chars<false>(b4, U14, W14, U23, W23);
+        x_join<HY>(lu14, rw14, lu23, rw23, b4);
+        y_chars<HY>(b4, U14, W14, U23, W23);
         Cx<T> *buf = ych + (size_t)((k - z_begin + 1) & 1) * (W * 4 * 32);
         buf[(w * 4 + 0) * 32 + lane] = U14;
         buf[(w * 4 + 1) * 32 + lane] = U23;
@@ -158,13 +172,20 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
             const Cx<T> U14 = buf[((w - 1) * 4 + 0) * 32 + lane], U23 = buf[((w - 1) * 4 + 1) * 32 + lane];
             const Cx<T> W14 = buf[((w + 1) * 4 + 2) * 32 + lane], W23 = buf[((w + 1) * 4 + 3) * 32 + lane];
             Cx<T> s[4], U13, W13, U24, W24;
-            y_join<false>(U14, W14, U23, W23, s);
+            y_join<HY>(U14, W14, U23, W23, s);
             // z sweep (Eq. sol_dis_3): +z movers of plane k-2, -z movers of plane k
-            z_chars<false>(s, U13, W13, U24, W24);
+            z_chars<HY>(s, U13, W13, U24, W24);
             const ZI zo = k - 1;
+            Cx<T> *zk = zh + (int)((k - z_begin) & 1) * 64;
+            if (HS) {
+                UA[0] = zk[0];
+                UA[1] = zk[32];
+                zk[0] = U13;
+                zk[32] = U24;
+            }
             if (zo >= z_begin && zo < z_end) {
                 Cx<T> o[4];
-                z_join<false>(UA[0], W13, UA[1], W24, o);
+                z_join<HY>(UA[0], W13, UA[1], W24, o);
                 const Cx<T> qu = a.full_table ? tu : pu, qd = a.full_table ? td : pd;
                 if (FIELD) {
                     Cx<T> m6[FIELD ? 6 : 1];
@@ -187,10 +208,12 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d_kernel(const Fused3DArgs A)
                 }
                 if (x >= x_own0 && x < x_own1) store_pt(out + ((int64_t)zo * plane_cells + cell) * 8, o);
             }
-            UA[0] = UB[0];
-            UA[1] = UB[1];
-            UB[0] = U13;
-            UB[1] = U24;
+            if (!HS) {
+                UA[0] = UB[0];
+                UA[1] = UB[1];
+                UB[0] = U13;
+                UB[1] = U24;
+            }
         }
     }
     if (face >= 0 && face >= x_own0 && face < x_own1) {
@@ -429,7 +452,7 @@ template <typename T, int W, bool FIELD>
 static cudaError_t launch_fused3d_one(const Fused3DArgs &A, cudaStream_t s) {
     const int64_t blocks = A.nstrips * A.nytiles * A.nzsegs;
     if (blocks <= 0) return cudaSuccess;
-    const int smem = 2 * W * 4 * 32 * (int)sizeof(Cx<T>);
+    const int smem = (2 + (Fused3DHist<T>::value ? 1 : 0)) * W * 4 * 32 * (int)sizeof(Cx<T>);
     static std::atomic<unsigned long long> done{0};
     cudaError_t e = optin_smem(fused3d_kernel<T, W, FIELD>, smem, done);
     if (e != cudaSuccess) return e;
