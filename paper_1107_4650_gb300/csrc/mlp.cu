@@ -20,24 +20,24 @@ namespace mlp {
 
 namespace {
 
-// ---- tcgen05 (5th-generation tensor core) GEMM for the hidden layers.
+// ---- tcgen05 (5th-generation tensor core) GEMM of the training step.
 //
-// C[M x N] (FP32, row-major, ldc) = sum_k A(m,k) B(k,n) (+ C when accumulate), A(m,k) = A[m*sam + k*sak],
-// B(k,n) = B[k*sbk + n*sbn], BF16 operands with arbitrary strides (the backward pass reads transposes).
-// One CTA of 4 warps computes a 128 x 64 tile of C in tensor memory: K is consumed in chunks of 64,
-// staged by all threads into shared memory in the canonical no-swizzle K-major layout (8-row x 16-byte
-// core matrices; K-direction core-matrix stride 128 B, 8-row-group stride 256 B; one 16-deep K slab per
-// MMA), double-buffered so the next chunk is staged while the tensor core consumes the current one.
-// One thread issues tcgen05.mma (M = 128, N = 64, K = 16, BF16 x BF16 -> FP32) and commits each chunk
-// to an mbarrier; every wait is bounded (about one second of the global timer) and a timeout sets
-// *err instead of hanging.  The accumulator (64 TMEM columns) is read back with tcgen05.ld, each warp
-// its 32 lanes = 32 rows of the tile.  The 64-wide N tile gives a 256 x 256 product 8 CTAs: these GEMMs
-// are small, so the time goes to staging operands, which more CTAs run in parallel.
-constexpr int GM = 128, GN = 64, GK = 64;
+// One CTA of 8 warps computes a 128 x 32 tile of C[m][n] = sum_k A[m][k] B[n][k] (BF16 operands, both with k
+// contiguous; FP32 accumulator in 32 columns of tensor memory) and finishes the layer in its epilogue.  The products
+// are small (256 x 256 x 256 for a batch of 256), so the time is the operands' latency: every 16-byte piece of a
+// K = 64 stage goes to shared memory by cp.async, four stages in flight, so a whole K = 256 is under way at once, and
+// 32-column tiles give such a product 16 CTAs.  Operands that a product needs the other way round (the weight
+// gradients' dz and h, the data gradients' W) are kept transposed by the kernels that produce them: an accumulator
+// row is a lane, so a column's 32 values leave as 64 consecutive bytes.  Measured for 256 x 256 x 256: see `step`.
+// Shared memory holds the canonical no-swizzle K-major layout (8-row x 16-byte core matrices; K-direction core-matrix
+// stride 128 B, 8-row-group stride 256 B; one 16-deep K slab per MMA).  One thread issues tcgen05.mma (M = 128, N = 32,
+// K = 16) in ascending k and commits each stage to an mbarrier; every wait is bounded (about one second of the global
+// timer) and a timeout sets *err instead of hanging.
+constexpr int GM = 128, GN = 32, GK = 64, GSTAGES = 4;
 constexpr int A_SLAB = GM * 16 * 2;  // bytes of one 16-deep K slab of the A tile (4 KB)
-constexpr int B_SLAB = GN * 16 * 2;  // (2 KB)
-constexpr int STAGE_BYTES = 4 * A_SLAB + 4 * B_SLAB;  // 24 KB per K chunk
-constexpr int GEMM_SMEM = 2 * STAGE_BYTES + 1024;     // two stages + alignment slack
+constexpr int B_SLAB = GN * 16 * 2;  // (1 KB)
+constexpr int STAGE_BYTES = 4 * A_SLAB + 4 * B_SLAB;         // 20 KB per K chunk
+constexpr int GEMM_SMEM = GSTAGES * STAGE_BYTES + 1024;      // + alignment slack
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -74,82 +74,89 @@ __device__ __forceinline__ int tile_off(int row, int k, int slab) {
     return (k >> 4) * slab + (row >> 3) * 256 + ((k >> 3) & 1) * 128 + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// Stages rows [r0, r0 + rows) x k [k0, k0 + 64) of X(r,k) = X[r*sr + k*sk] (zero outside [0,R) x [0,K)).
-__device__ __forceinline__ void stage(unsigned char *dst, int slab, const __nv_bfloat16 *X, int64_t sr, int64_t sk,
-                                      int r0, int rows, int R, int k0, int K) {
-    const __nv_bfloat16 zero = __float2bfloat16(0.f);
-    if (sk == 1 && (sr & 7) == 0 && ((uintptr_t)X & 15) == 0 && k0 + GK <= K) {
-        // K-contiguous source: 8 elements (16 bytes) per load, one core-matrix row per store
-        for (int e = threadIdx.x; e < rows * (GK / 8); e += blockDim.x) {
-            const int r = e / (GK / 8), c = e % (GK / 8);
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (r0 + r < R) v = *reinterpret_cast<const uint4 *>(X + (int64_t)(r0 + r) * sr + k0 + 8 * c);
-            *reinterpret_cast<uint4 *>(dst + tile_off(r, 8 * c, slab)) = v;
-        }
-    } else if (sr == 1 && (sk & 7) == 0 && ((uintptr_t)X & 15) == 0 && r0 + rows <= R && k0 + GK <= K) {
-        // row-contiguous source (a transpose), whole tile inside: 8 rows of one k per 16-byte load
-        for (int e = threadIdx.x; e < (rows / 8) * GK; e += blockDim.x) {
-            const int k = e / (rows / 8), r8 = 8 * (e % (rows / 8));
-            const uint4 v = *reinterpret_cast<const uint4 *>(X + (int64_t)(r0 + r8) + (int64_t)(k0 + k) * sk);
-            const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&v);
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
+    const __nv_bfloat16 lo = __float2bfloat16(a), hi = __float2bfloat16(b);
+    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+}
+
+// Starts the copies of rows [r0, r0 + ROWS) x k [k0, k0 + 64) of X[r][k] (row pitch ld) into a stage; rows past R are
+// zero.  The caller's buffers are readable up to the 64-multiple of k that it asks for.
+template <int ROWS>
+__device__ __forceinline__ void stage_async(unsigned char *dst, int slab, const __nv_bfloat16 *X, int64_t ld, int r0, int R,
+                                            int k0) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) *reinterpret_cast<__nv_bfloat16 *>(dst + tile_off(r8 + i, k, slab)) = h[i];
-        }
-    } else if (sr == 1) {
-        // row-contiguous source at the edges: consecutive threads take consecutive rows
-        for (int e = threadIdx.x; e < rows * GK; e += blockDim.x) {
-            const int k = e / rows, r = e % rows;
-            const int rr = r0 + r, kk = k0 + k;
-            *reinterpret_cast<__nv_bfloat16 *>(dst + tile_off(r, k, slab)) =
-                (rr < R && kk < K) ? X[(int64_t)rr + (int64_t)kk * sk] : zero;
-        }
-    } else {
-        for (int e = threadIdx.x; e < rows * GK; e += blockDim.x) {
-            const int r = e / GK, k = e % GK;
-            const int rr = r0 + r, kk = k0 + k;
-            *reinterpret_cast<__nv_bfloat16 *>(dst + tile_off(r, k, slab)) =
-                (rr < R && kk < K) ? X[(int64_t)rr * sr + (int64_t)kk * sk] : zero;
-        }
+    for (int e = threadIdx.x; e < ROWS * (GK / 8); e += 256) {
+        const int r = e / (GK / 8), c = e % (GK / 8);
+        const uint32_t bytes = r0 + r < R ? 16u : 0u;  // 0: zero fill, nothing read
+        const __nv_bfloat16 *src = X + (int64_t)(r0 + r < R ? r0 + r : 0) * ld + k0 + 8 * c;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst + tile_off(r, 8 * c, slab))), "l"(src),
+                     "r"(bytes)
+                     : "memory");
     }
 }
 
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *A, int64_t sam, int64_t sak,
-                                                           const __nv_bfloat16 *B, int64_t sbk, int64_t sbn, float *C,
-                                                           int64_t ldc, int M, int N, int K, int accumulate, unsigned *err) {
+// What a GEMM launch computes.
+//   FWD    h = tanh(A . B^T + bias): FP32 h, its BF16 copy and the copy's transpose
+//   DGRAD  dz = (A . B^T) (1 - h^2) (h: this layer's activations): FP32 dz, its BF16 copy and the copy's transpose
+//   WGRAD  C = A . B^T, FP32
+enum { FWD = 0, DGRAD = 1, WGRAD = 2 };
+struct GemmArgs {
+    const __nv_bfloat16 *A, *B;
+    int64_t lda, ldb;
+    int M, K;
+    float *C;                 // h, dz or the gradient: [M][256]
+    __nv_bfloat16 *Cb, *Ct;   // BF16 copy [M][256] and transpose [256][ldt] (FWD, DGRAD); rows past M leave zeros in Ct
+    int64_t ldt;
+    const float *bias, *h;
+    unsigned *err;
+};
+
+template <int KIND> __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
     extern __shared__ unsigned char gsm_raw[];
     unsigned char *gsm = reinterpret_cast<unsigned char *>(((uintptr_t)gsm_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ float tr[4][32][33];  // epilogue: each warp's 32 x 32 block, rows padded (no bank conflicts)
-    __shared__ __align__(8) uint64_t mbar[2];
+    __shared__ __align__(8) uint64_t mbar[GSTAGES];
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
-    const int nchunks = (K + GK - 1) / GK;
+    const int nchunks = (g.K + GK - 1) / GK;
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(smem_addr(&tmem_slot))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_addr(&tmem_slot))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar[0])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar[1])) : "memory");
+#pragma unroll
+        for (int i = 0; i < GSTAGES; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar[i])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (nchunks > 0) {
-        stage(gsm, A_SLAB, A, sam, sak, m0, GM, M, 0, K);
-        stage(gsm + 4 * A_SLAB, B_SLAB, B, sbn, sbk, n0, GN, N, 0, K);
-    }
+    auto load_chunk = [&](int c) {
+        unsigned char *buf = gsm + (c % GSTAGES) * STAGE_BYTES;
+        if (c < nchunks) {
+            stage_async<GM>(buf, A_SLAB, g.A, g.lda, m0, g.M, c * GK);
+            stage_async<GN>(buf + 4 * A_SLAB, B_SLAB, g.B, g.ldb, n0, HID, c * GK);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
+    };
+#pragma unroll
+    for (int c = 0; c < GSTAGES - 1; ++c) load_chunk(c);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    // instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, N = 64, M = 128
+    // instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, N = 32, M = 128
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GN >> 3) << 17) | ((uint32_t)(GM >> 4) << 24);
     bool ok = true;
     for (int c = 0; c < nchunks && ok; ++c) {
-        unsigned char *buf = gsm + (c & 1) * STAGE_BYTES;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // staged stores -> tensor core's view
+        // chunk c + GSTAGES - 1 goes where chunk c - 1 was: its MMAs have to be done with it
+        if (c >= 1 && c + GSTAGES - 1 < nchunks)
+            ok = __syncthreads_and(bar_wait(smem_addr(&mbar[(c - 1) % GSTAGES]), (uint32_t)(((c - 1) / GSTAGES) & 1)));
+        if (!ok) break;
+        load_chunk(c + GSTAGES - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(GSTAGES - 1) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // landed pieces -> the tensor core's view
         __syncthreads();
         if (tid == 0) {
+            unsigned char *buf = gsm + (c % GSTAGES) * STAGE_BYTES;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int j = 0; j < GK / 16; ++j) {
@@ -162,196 +169,260 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *A, 
                              : "memory");
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_addr(&mbar[c & 1]))
+                             smem_addr(&mbar[c % GSTAGES]))
                          : "memory");
         }
-        if (c + 1 < nchunks) {
-            // the other buffer was read by chunk c - 1: wait for its commit before overwriting it
-            if (c >= 1) ok = __syncthreads_and(bar_wait(smem_addr(&mbar[(c - 1) & 1]), (uint32_t)(((c - 1) >> 1) & 1)));
-            if (ok) {
-                unsigned char *nb = gsm + ((c + 1) & 1) * STAGE_BYTES;
-                stage(nb, A_SLAB, A, sam, sak, m0, GM, M, (c + 1) * GK, K);
-                stage(nb + 4 * A_SLAB, B_SLAB, B, sbn, sbk, n0, GN, N, (c + 1) * GK, K);
-            }
-        }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // commits complete in order: the last one covers every MMA
-    if (ok && nchunks > 0)
-        ok = __syncthreads_and(bar_wait(smem_addr(&mbar[(nchunks - 1) & 1]), (uint32_t)(((nchunks - 1) >> 1) & 1)));
+    if (ok) ok = __syncthreads_and(bar_wait(smem_addr(&mbar[(nchunks - 1) % GSTAGES]), (uint32_t)(((nchunks - 1) / GSTAGES) & 1)));
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
-#pragma unroll 1
-        for (int c0 = 0; c0 < GN; c0 += 32) {
-            uint32_t r[32];
-            if (nchunks > 0) {
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                    "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                      "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                      "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-                      "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-                      "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                    : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0)
-                    : "memory");
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            } else {
+        // warps w and w + 4 read the same 32 accumulator rows, 16 columns each
+        const int m = m0 + (warp & 3) * 32 + lane, nc = n0 + (warp >> 2) * 16;
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 16))
+            : "memory");
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        const bool in = m < g.M;
+        float v[16];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) r[j] = 0u;
-            }
-            // lane = row in the accumulator's layout: through shared memory, so that each store instruction writes
-            // 32 consecutive columns of one row (128 bytes) instead of one column of 32 rows
+        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+        if (KIND == FWD) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) tr[warp][lane][j] = __uint_as_float(r[j]);
-            __syncwarp();
-            const int n = n0 + c0 + lane;
-            for (int rr = 0; rr < 32; ++rr) {
-                const int mr = m0 + warp * 32 + rr;
-                if (mr < M && n < N) {
-                    float *p = C + (int64_t)mr * ldc + n;
-                    const float v = tr[warp][rr][lane];
-                    *p = accumulate ? (*p + v) : v;
-                }
+            for (int j = 0; j < 16; ++j) v[j] = tanhf(v[j] + g.bias[nc + j]);
+        } else if (KIND == DGRAD && in) {
+            const float4 *hp = reinterpret_cast<const float4 *>(g.h + (int64_t)m * HID + nc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 y = hp[j];
+                v[4 * j + 0] = v[4 * j + 0] * (1.f - y.x * y.x);
+                v[4 * j + 1] = v[4 * j + 1] * (1.f - y.y * y.y);
+                v[4 * j + 2] = v[4 * j + 2] * (1.f - y.z * y.z);
+                v[4 * j + 3] = v[4 * j + 3] * (1.f - y.w * y.w);
             }
-            __syncwarp();
+        }
+        if (KIND == WGRAD) {
+            // the gradient's place in the parameter vector is a multiple of 16 bytes for W2-W4
+            float4 *cp = reinterpret_cast<float4 *>(g.C + (int64_t)m * HID + nc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) cp[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        } else {
+            uint32_t pk[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) pk[j] = in ? pack_bf16x2(v[2 * j], v[2 * j + 1]) : 0u;
+            if (in) {
+                float4 *cp = reinterpret_cast<float4 *>(g.C + (int64_t)m * HID + nc);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) cp[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                uint4 *bp = reinterpret_cast<uint4 *>(g.Cb + (int64_t)m * HID + nc);
+                bp[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                bp[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                g.Ct[(int64_t)(nc + j) * g.ldt + m] = __ushort_as_bfloat16((unsigned short)(pk[j / 2] >> (16 * (j & 1))));
         }
     } else if (lane == 0) {
-        atomicOr(err, 1u);
+        atomicOr(g.err, 1u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
 }
 
-// z1 = x . bf16(W1)^T + b1, h1 = tanh(z1); x is [B][3] FP32, W1 [256][3] BF16.
-__global__ void layer1_fwd_kernel(const float *x, const __nv_bfloat16 *W1, const float *b1, float *h, __nv_bfloat16 *hb,
-                                  int Bn) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)Bn * HID) return;
-    const int b = (int)(e / HID), j = (int)(e % HID);
-    float z = b1[j];
-    z = fmaf(x[b * 3 + 0], __bfloat162float(W1[j * 3 + 0]), z);
-    z = fmaf(x[b * 3 + 1], __bfloat162float(W1[j * 3 + 1]), z);
-    z = fmaf(x[b * 3 + 2], __bfloat162float(W1[j * 3 + 2]), z);
-    const float y = tanhf(z);
-    h[e] = y;
-    hb[e] = __float2bfloat16(y);
+template <int KIND> __global__ void __launch_bounds__(256) layer_gemm_kernel(const GemmArgs g) {
+    gemm_tile<KIND>(g, blockIdx.y * GM, blockIdx.x * GN);
 }
 
-// h = tanh(z + b) in place on z (FP32), plus the BF16 copy.
-__global__ void bias_tanh_kernel(float *z, const float *bias, __nv_bfloat16 *hb, int Bn) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)Bn * HID) return;
-    const float y = tanhf(z[e] + bias[e % HID]);
-    z[e] = y;
-    hb[e] = __float2bfloat16(y);
-}
+// A training batch: sample b is row idx[b] of X and T (idx null: row b).
+struct BatchIn {
+    const float *X, *T;
+    const int *idx;
+    int B;
+    __device__ __forceinline__ int row(int b) const { return idx ? idx[b] : b; }
+};
 
-// y = sigmoid(bf16(h4) . bf16(w5) + b5): one warp per sample.
-__global__ void out_fwd_kernel(const __nv_bfloat16 *h4b, const __nv_bfloat16 *w5, const float *b5, float *y, int Bn) {
-    const int lane = threadIdx.x & 31;
-    const int b = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (b >= Bn) return;
-    float s = 0.f;
-    for (int j = lane; j < HID; j += 32) s = fmaf(__bfloat162float(h4b[(int64_t)b * HID + j]), __bfloat162float(w5[j]), s);
+// z1 = x . bf16(W1)^T + b1, h1 = tanh(z1) (x is 3 FP32, W1 [256][3] BF16): h1, its BF16 copy and the copy's transpose
+// (zeros for the samples that pad the batch to a multiple of 128).  A block of 256 threads takes 32 samples x 32 units.
+__global__ void __launch_bounds__(256) layer1_fwd_kernel(const BatchIn in, const __nv_bfloat16 *W1, const float *b1, float *h,
+                                                         __nv_bfloat16 *hb, __nv_bfloat16 *ht, int64_t ldt) {
+    __shared__ __nv_bfloat16 tr[32][34];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+    const int j = j0 + tx;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) y[b] = 1.f / (1.f + expf(-(s + b5[0])));
-}
-
-// dz5 = 2 (y - t) y (1 - y) / B, and the per-sample squared error.
-__global__ void out_bwd_kernel(const float *y, const float *t, float *dz5, float *sqerr, int Bn) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= Bn) return;
-    const float d = y[b] - t[b];
-    dz5[b] = 2.f * d * y[b] * (1.f - y[b]) / (float)Bn;
-    sqerr[b] = d * d;
-}
-
-// dW5[j] = sum_b dz5[b] bf16(h4)[b][j], db5 = sum_b dz5[b] (block j = HID handles db5); then dh4 = dz5 w5.
-__global__ void out_wgrad_kernel(const float *dz5, const __nv_bfloat16 *h4b, float *gW5, float *gb5, int Bn) {
-    __shared__ float sh[32];
-    const int j = blockIdx.x;
-    float s = 0.f;
-    for (int b = threadIdx.x; b < Bn; b += blockDim.x)
-        s += dz5[b] * (j < HID ? __bfloat162float(h4b[(int64_t)b * HID + j]) : 1.f);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float v = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w];
-        if (j < HID) gW5[j] = v; else gb5[0] = v;
+    for (int i = ty; i < 32; i += 8) {
+        const int b = b0 + i;
+        __nv_bfloat16 o = __float2bfloat16(0.f);
+        if (b < in.B) {
+            const float *x = in.X + (int64_t)in.row(b) * 3;
+            float z = b1[j];
+            z = fmaf(x[0], __bfloat162float(W1[j * 3 + 0]), z);
+            z = fmaf(x[1], __bfloat162float(W1[j * 3 + 1]), z);
+            z = fmaf(x[2], __bfloat162float(W1[j * 3 + 2]), z);
+            const float y = tanhf(z);
+            h[(int64_t)b * HID + j] = y;
+            o = __float2bfloat16(y);
+            hb[(int64_t)b * HID + j] = o;
+        }
+        tr[i][tx] = o;
     }
-}
-
-// dz = dh (1 - h^2) with dh = dz5 (x) w5 for the last hidden layer (from_out = 1) or dh given (from_out = 0);
-// writes FP32 dz and its BF16 copy.
-__global__ void tanh_bwd_kernel(const float *dh, const float *dz5, const __nv_bfloat16 *w5, const float *h, float *dz,
-                                __nv_bfloat16 *dzb, int Bn, int from_out) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)Bn * HID) return;
-    const float g = from_out ? dz5[e / HID] * __bfloat162float(w5[e % HID]) : dh[e];
-    const float y = h[e];
-    const float v = g * (1.f - y * y);
-    dz[e] = v;
-    dzb[e] = __float2bfloat16(v);
-}
-
-// db[j] = sum_b dz[b][j] (FP32), one block per column.
-__global__ void colsum_kernel(const float *dz, float *db, int Bn, int ncol) {
-    __shared__ float sh[32];
-    const int j = blockIdx.x;
-    float s = 0.f;
-    for (int b = threadIdx.x; b < Bn; b += blockDim.x) s += dz[(int64_t)b * ncol + j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float v = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w];
-        db[j] = v;
-    }
-}
-
-// dW1[j][i] = sum_b dz1[b][j] x[b][i] (FP32), one block per (j, i).
-__global__ void layer1_wgrad_kernel(const float *dz1, const float *x, float *gW1, int Bn) {
-    __shared__ float sh[32];
-    const int j = blockIdx.x / 3, i = blockIdx.x % 3;
-    float s = 0.f;
-    for (int b = threadIdx.x; b < Bn; b += blockDim.x) s += dz1[(int64_t)b * HID + j] * x[b * 3 + i];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float v = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w];
-        gW1[j * 3 + i] = v;
+    for (int i = ty; i < 32; i += 8) ht[(int64_t)(j0 + i) * ldt + b0 + tx] = tr[tx][i];
+}
+
+// The output layer both ways, one warp per sample: y = sigmoid(bf16(h4) . bf16(w5) + b5); dz5 = 2 (y - t) y (1 - y) / B and
+// the squared error; the last hidden layer's dz = dz5 w5 (1 - h4^2), its BF16 copy and the copy's transpose (32 samples of
+// a block through shared memory; zeros for the samples that pad the batch).
+__global__ void __launch_bounds__(1024) out_layer_kernel(const BatchIn in, const __nv_bfloat16 *h4b, const float *h4,
+                                                         const __nv_bfloat16 *w5, const float *b5, float *y, float *dz5,
+                                                         float *sqerr, float *dz, __nv_bfloat16 *dzb, __nv_bfloat16 *dzt,
+                                                         int64_t ldt) {
+    __shared__ __nv_bfloat16 tr[32][HID + 2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int b = blockIdx.x * 32 + w;
+    if (b < in.B) {
+        float s = 0.f;
+        for (int j = lane; j < HID; j += 32) s = fmaf(__bfloat162float(h4b[(int64_t)b * HID + j]), __bfloat162float(w5[j]), s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float yb = 1.f / (1.f + expf(-(s + b5[0])));
+        const float d = yb - in.T[in.row(b)];
+        const float g5 = 2.f * d * yb * (1.f - yb) / (float)in.B;
+        if (lane == 0) {
+            y[b] = yb;
+            dz5[b] = g5;
+            sqerr[b] = d * d;
+        }
+        for (int j = lane; j < HID; j += 32) {
+            const float g = g5 * __bfloat162float(w5[j]);
+            const float a = h4[(int64_t)b * HID + j];
+            const float v = g * (1.f - a * a);
+            dz[(int64_t)b * HID + j] = v;
+            const __nv_bfloat16 o = __float2bfloat16(v);
+            dzb[(int64_t)b * HID + j] = o;
+            tr[w][j] = o;
+        }
+    } else {
+        for (int j = lane; j < HID; j += 32) tr[w][j] = __float2bfloat16(0.f);
     }
+    __syncthreads();
+    for (int j = w; j < HID; j += 32) dzt[(int64_t)j * ldt + blockIdx.x * 32 + lane] = tr[lane][j];
 }
 
-// Adam on the FP32 master parameters; refreshes the BF16 copies of the weight entries.
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, int64_t n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float upd = lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    const float np = p[i] - upd;
-    p[i] = np;
-    pb[i] = __float2bfloat16(np);
+// Sum over the batch of term(b), one warp: 256 partial sums (b mod 256), each 32 of them by an xor tree, the eight
+// trees in order.
+template <typename F> __device__ __forceinline__ float batch_sum(int B, int lane, F term) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        float s = 0.f;
+        for (int b = 32 * w + lane; b < B; b += 256) s += term(b);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        v += s;
+    }
+    return v;
 }
 
-__global__ void to_bf16_kernel(const float *p, __nv_bfloat16 *pb, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) pb[i] = __float2bfloat16(p[i]);
+// The gradients, one launch: blocks [0, 48) the three hidden weight matrices (16 tiles each), then one warp each for the
+// sums over the batch: db of the four hidden layers, dW1 = dz1^T x, dW5 = sum_b dz5 bf16(h4), db5 = sum_b dz5.
+struct GradArgs {
+    GemmArgs w[3];             // dW2, dW3, dW4
+    const float *dz[4], *dz5;  // hidden layers' dz [B][256]
+    const __nv_bfloat16 *h4b;
+    float *gb[4], *gW1, *gW5, *gb5;
+    BatchIn in;
+};
+constexpr int kGradTiles = 3 * (HID / GM) * (HID / GN), kGradSums = 4 * HID + 3 * HID + HID + 1;
+__global__ void __launch_bounds__(256) grad_kernel(const __grid_constant__ GradArgs a) {
+    if (blockIdx.x < kGradTiles) {
+        const int per = kGradTiles / 3, t = blockIdx.x % per;
+        gemm_tile<WGRAD>(a.w[blockIdx.x / per], (t / (HID / GN)) * GM, (t % (HID / GN)) * GN);
+        return;
+    }
+    const int lane = threadIdx.x & 31, q = (blockIdx.x - kGradTiles) * 8 + (threadIdx.x >> 5), B = a.in.B;
+    if (q >= kGradSums) return;
+    float v;
+    float *to;
+    if (q < 4 * HID) {
+        const float *dz = a.dz[q / HID] + q % HID;
+        v = batch_sum(B, lane, [&](int b) { return dz[(int64_t)b * HID]; });
+        to = a.gb[q / HID] + q % HID;
+    } else if (q < 7 * HID) {
+        const int e = q - 4 * HID, j = e / 3, i = e % 3;
+        v = batch_sum(B, lane, [&](int b) { return a.dz[0][(int64_t)b * HID + j] * a.in.X[(int64_t)a.in.row(b) * 3 + i]; });
+        to = a.gW1 + j * 3 + i;
+    } else {
+        const int j = q - 7 * HID;
+        v = batch_sum(B, lane, [&](int b) { return a.dz5[b] * (j < HID ? __bfloat162float(a.h4b[(int64_t)b * HID + j]) : 1.f); });
+        to = j < HID ? a.gW5 + j : a.gb5;
+    }
+    if (lane == 0) *to = v;
+}
+
+// One Adam step's scalars: the learning rate and the moments' bias corrections.
+struct AdamStep {
+    float lr, c1, c2;
+};
+// Adam on the FP32 master parameter i (UPDATE), and its BF16 copy.
+template <bool UPDATE>
+__device__ __forceinline__ __nv_bfloat16 adam_one(float *p, const float *g, float *m, float *v, __nv_bfloat16 *pb, int64_t i,
+                                                  AdamStep st) {
+    float np = p[i];
+    if (UPDATE) {
+        const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+        const float gi = g[i];
+        const float mi = b1 * m[i] + (1.f - b1) * gi;
+        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+        m[i] = mi;
+        v[i] = vi;
+        const float upd = st.lr * (mi / st.c1) / (sqrtf(vi / st.c2) + eps);
+        np = np - upd;
+        p[i] = np;
+    }
+    const __nv_bfloat16 o = __float2bfloat16(np);
+    pb[i] = o;
+    return o;
+}
+// Blocks [0, 192): 32 x 32 tiles of W2-W4, whose BF16 copy is kept transposed too (the data gradients' operand); then the
+// other parameters, 256 to a block.
+constexpr int kAdamTiles = 3 * (HID / 32) * (HID / 32);
+struct ParamArgs {
+    float *p;
+    const float *g;
+    float *m, *v;
+    __nv_bfloat16 *pb, *wt;  // wt: [3][256][256], wt[l][k][j] = bf16(W_{l+2}[j][k])
+    int64_t off_w[5];
+    int64_t n;
+};
+template <bool UPDATE> __global__ void __launch_bounds__(256) param_kernel(const __grid_constant__ ParamArgs a, AdamStep st) {
+    if (blockIdx.x < kAdamTiles) {
+        __shared__ __nv_bfloat16 tr[32][34];
+        const int per = kAdamTiles / 3, l = blockIdx.x / per, t = blockIdx.x % per;
+        const int j0 = (t / (HID / 32)) * 32, k0 = (t % (HID / 32)) * 32;
+        const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+        for (int i = ty; i < 32; i += 8)
+            tr[i][tx] = adam_one<UPDATE>(a.p, a.g, a.m, a.v, a.pb, a.off_w[l + 1] + (int64_t)(j0 + i) * HID + k0 + tx, st);
+        __syncthreads();
+#pragma unroll
+        for (int i = ty; i < 32; i += 8) a.wt[(int64_t)l * HID * HID + (int64_t)(k0 + i) * HID + j0 + tx] = tr[tx][i];
+        return;
+    }
+    // W1 and b1, then b2, b3, b4 (each after its matrix), w5 and b5
+    int64_t e = (int64_t)(blockIdx.x - kAdamTiles) * 256 + threadIdx.x;
+    const int64_t first = a.off_w[1], mat = (int64_t)HID * HID;
+    if (e >= first) {
+        const int64_t r = e - first;
+        e = r < 3 * HID ? a.off_w[1 + r / HID] + mat + r % HID : a.off_w[4] + (r - 3 * HID);
+    }
+    if (e < a.n) adam_one<UPDATE>(a.p, a.g, a.m, a.v, a.pb, e, st);
 }
 
 inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
@@ -403,10 +474,6 @@ __device__ __forceinline__ void load_layer_weights(uint32_t ws, const unsigned c
     for (int c = 0; c < 4; ++c) bulk_copy(ws + c * (IW_BYTES / 4), src + c * (IW_BYTES / 4), IW_BYTES / 4, bar);
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-    const __nv_bfloat16 lo = __float2bfloat16(a), hi = __float2bfloat16(b);
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
 
 template <int NW>
 __global__ void __launch_bounds__(32 * NW, 1) mlp_infer_kernel(const float *x, const __nv_bfloat16 *W1, const float *b1,
@@ -561,24 +628,6 @@ __global__ void __launch_bounds__(32 * NW, 1) mlp_infer_kernel(const float *x, c
 
 }  // namespace
 
-cudaError_t gemm_bf16(const __nv_bfloat16 *A, int64_t sam, int64_t sak, const __nv_bfloat16 *B, int64_t sbk, int64_t sbn,
-                      float *C, int64_t ldc, int M, int N, int K, int accumulate, unsigned *err, cudaStream_t s) {
-    if (M <= 0 || N <= 0) return cudaSuccess;
-    // per device: > 48 KB of dynamic shared memory opted in once
-    static std::atomic<unsigned long long> attr_set{0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
-    if (!bit || !(attr_set.load(std::memory_order_relaxed) & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
-        if (e != cudaSuccess) return e;
-        if (bit) attr_set.fetch_or(bit, std::memory_order_relaxed);
-    }
-    dim3 grid((N + GN - 1) / GN, (M + GM - 1) / GM);
-    gemm_bf16_kernel<<<grid, 128, GEMM_SMEM, s>>>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, accumulate, err);
-    return cudaGetLastError();
-}
-
 cudaError_t pack_weights(const Net &n, cudaStream_t s) {
     if ((n.off_w[1] | n.off_w[2] | n.off_w[3]) & 7) return cudaErrorInvalidValue;  // 16-byte rows for the packing
     pack_weights_kernel<<<nblk(3 * HID * (HID / 8), 256), 256, 0, s>>>(n.wb, n.off_w[1], n.off_w[2], n.off_w[3], n.wpack);
@@ -608,58 +657,120 @@ cudaError_t infer(const Net &n, const float *x, float *y, int Bn, cudaStream_t s
     return cudaGetLastError();
 }
 
-// Forward pass for a batch: fills the activation buffers and y.
-cudaError_t forward(const Net &n, const Acts &a, const float *x, int Bn, cudaStream_t s) {
-    const int64_t E = (int64_t)Bn * HID;
-    layer1_fwd_kernel<<<nblk(E, 256), 256, 0, s>>>(x, n.wb + n.off_w[0], n.p + n.off_b[0], a.h[0], a.hb[0], Bn);
-    cudaError_t e = cudaGetLastError();
+namespace {
+// Per device: > 48 KB of dynamic shared memory opted in once.
+template <typename K> cudaError_t optin(K *kernel, int smem, std::atomic<unsigned long long> &done) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
+    if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
+template <int KIND> cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t s) {
+    static std::atomic<unsigned long long> done{0};
+    cudaError_t e = optin(layer_gemm_kernel<KIND>, GEMM_SMEM, done);
     if (e != cudaSuccess) return e;
-    for (int l = 1; l < 4; ++l) {
+    layer_gemm_kernel<KIND><<<dim3(HID / GN, nblk(g.M, GM)), 256, GEMM_SMEM, s>>>(g);
+    return cudaGetLastError();
+}
+}  // namespace
+
+// Forward and backward pass of a batch in nine launches: layer 1, three hidden layers, the output layer both ways, three
+// data gradients, all weight gradients.  Gradients of mean((y - t)^2) into g (same layout as the parameters).
+cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *T, const int *idx, float *g, int Bn,
+                      cudaStream_t s) {
+    const BatchIn in{X, T, idx, Bn};
+    const int pad = nblk(Bn, GM) * GM;
+    layer1_fwd_kernel<<<dim3(pad / 32, HID / 32), 256, 0, s>>>(in, n.wb + n.off_w[0], n.p + n.off_b[0], a.h[0], a.hb[0], a.ht[0],
+                                                              a.ldt);
+    cudaError_t e = cudaGetLastError();
+    GemmArgs q{};
+    q.err = n.err;
+    q.lda = q.ldb = HID;
+    q.M = Bn;
+    q.K = HID;
+    q.ldt = a.ldt;
+    for (int l = 1; l < 4 && e == cudaSuccess; ++l) {
         // z_l[b][j] = sum_k bf16(h_{l-1})[b][k] bf16(W_l)[j][k]
-        e = gemm_bf16(a.hb[l - 1], HID, 1, n.wb + n.off_w[l], 1, HID, a.h[l], HID, Bn, HID, HID, 0, n.err, s);
-        if (e != cudaSuccess) return e;
-        bias_tanh_kernel<<<nblk(E, 256), 256, 0, s>>>(a.h[l], n.p + n.off_b[l], a.hb[l], Bn);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        q.A = a.hb[l - 1];
+        q.B = n.wb + n.off_w[l];
+        q.bias = n.p + n.off_b[l];
+        q.C = a.h[l];
+        q.Cb = a.hb[l];
+        q.Ct = a.ht[l];
+        e = launch_gemm<FWD>(q, s);
     }
-    out_fwd_kernel<<<nblk((int64_t)Bn * 32, 256), 256, 0, s>>>(a.hb[3], n.wb + n.off_w[4], n.p + n.off_b[4], a.y, Bn);
+    if (e != cudaSuccess) return e;
+    out_layer_kernel<<<pad / 32, 1024, 0, s>>>(in, a.hb[3], a.h[3], n.wb + n.off_w[4], n.p + n.off_b[4], a.y, a.dz5, a.sqerr,
+                                               a.dz[3], a.dzb[3], a.dzt[3], a.ldt);
+    e = cudaGetLastError();
+    for (int l = 3; l >= 1 && e == cudaSuccess; --l) {
+        // dh_{l-1}[b][k] = sum_j bf16(dz_l)[b][j] bf16(W_l)[j][k]
+        q.A = a.dzb[l];
+        q.B = n.wt + (int64_t)(l - 1) * HID * HID;
+        q.h = a.h[l - 1];
+        q.C = a.dz[l - 1];
+        q.Cb = a.dzb[l - 1];
+        q.Ct = a.dzt[l - 1];
+        e = launch_gemm<DGRAD>(q, s);
+    }
+    if (e != cudaSuccess) return e;
+    GradArgs r{};
+    for (int l = 1; l < 4; ++l) {
+        // dW_l[j][k] = sum_b bf16(dz_l)[b][j] bf16(h_{l-1})[b][k]
+        GemmArgs &w = r.w[l - 1];
+        w.A = a.dzt[l];
+        w.B = a.ht[l - 1];
+        w.lda = w.ldb = a.ldt;
+        w.M = HID;
+        w.K = Bn;
+        w.C = g + n.off_w[l];
+        w.err = n.err;
+    }
+    for (int l = 0; l < 4; ++l) {
+        r.dz[l] = a.dz[l];
+        r.gb[l] = g + n.off_b[l];
+    }
+    r.dz5 = a.dz5;
+    r.h4b = a.hb[3];
+    r.gW1 = g + n.off_w[0];
+    r.gW5 = g + n.off_w[4];
+    r.gb5 = g + n.off_b[4];
+    r.in = in;
+    static std::atomic<unsigned long long> done{0};
+    e = optin(grad_kernel, GEMM_SMEM, done);
+    if (e != cudaSuccess) return e;
+    grad_kernel<<<kGradTiles + nblk(kGradSums, 8), 256, GEMM_SMEM, s>>>(r);
     return cudaGetLastError();
 }
 
-// Backward pass (after forward): gradients of mean((y - t)^2) into g (same layout as the parameters).
-cudaError_t backward(const Net &n, const Acts &a, const float *x, const float *t, float *g, int Bn, cudaStream_t s) {
-    const int64_t E = (int64_t)Bn * HID;
-    out_bwd_kernel<<<nblk(Bn, 256), 256, 0, s>>>(a.y, t, a.dz5, a.sqerr, Bn);
-    out_wgrad_kernel<<<HID + 1, 256, 0, s>>>(a.dz5, a.hb[3], g + n.off_w[4], g + n.off_b[4], Bn);
-    tanh_bwd_kernel<<<nblk(E, 256), 256, 0, s>>>(nullptr, a.dz5, n.wb + n.off_w[4], a.h[3], a.dz, a.dzb, Bn, 1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    for (int l = 3; l >= 1; --l) {
-        // dW_l[j][k] = sum_b bf16(dz)[b][j] bf16(h_{l-1})[b][k]:  A(m=j, k=b) = dzb[b*HID + j], B(k=b, n=k) = hb[b*HID + k]
-        e = gemm_bf16(a.dzb, 1, HID, a.hb[l - 1], HID, 1, g + n.off_w[l], HID, HID, HID, Bn, 0, n.err, s);
-        if (e != cudaSuccess) return e;
-        colsum_kernel<<<HID, 256, 0, s>>>(a.dz, g + n.off_b[l], Bn, HID);
-        // dh_{l-1}[b][k] = sum_j bf16(dz)[b][j] bf16(W_l)[j][k]:  A(m=b, k=j) = dzb[b*HID + j], B(k=j, n=k) = W[j*HID + k]
-        e = gemm_bf16(a.dzb, HID, 1, n.wb + n.off_w[l], HID, 1, a.dh, HID, Bn, HID, HID, 0, n.err, s);
-        if (e != cudaSuccess) return e;
-        tanh_bwd_kernel<<<nblk(E, 256), 256, 0, s>>>(a.dh, nullptr, nullptr, a.h[l - 1], a.dz, a.dzb, Bn, 0);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    layer1_wgrad_kernel<<<HID * 3, 256, 0, s>>>(a.dz, x, g + n.off_w[0], Bn);
-    colsum_kernel<<<HID, 256, 0, s>>>(a.dz, g + n.off_b[0], Bn, HID);
-    return cudaGetLastError();
+namespace {
+ParamArgs param_args(const Net &n, const float *g) {
+    ParamArgs a{};
+    a.p = n.p;
+    a.g = g;
+    a.m = n.m;
+    a.v = n.v;
+    a.pb = n.wb;
+    a.wt = n.wt;
+    for (int l = 0; l < 5; ++l) a.off_w[l] = n.off_w[l];
+    a.n = NPARAM;
+    return a;
 }
+constexpr int kParamBlocks = kAdamTiles + (int)((NPARAM - 3 * (int64_t)HID * HID + 255) / 256);
+}  // namespace
 
 cudaError_t adam(const Net &n, const float *g, float lr, int64_t step, cudaStream_t s) {
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-    adam_kernel<<<nblk(NPARAM, 256), 256, 0, s>>>(n.p, g, n.m, n.v, n.wb, NPARAM, lr, b1, b2, eps, c1, c2);
+    const float b1 = 0.9f, b2 = 0.999f;
+    const AdamStep st{lr, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step)};
+    param_kernel<true><<<kParamBlocks, 256, 0, s>>>(param_args(n, g), st);
     return cudaGetLastError();
 }
 
 cudaError_t refresh_bf16(const Net &n, cudaStream_t s) {
-    to_bf16_kernel<<<nblk(NPARAM, 256), 256, 0, s>>>(n.p, n.wb, NPARAM);
+    param_kernel<false><<<kParamBlocks, 256, 0, s>>>(param_args(n, nullptr), AdamStep{});
     return cudaGetLastError();
 }
 

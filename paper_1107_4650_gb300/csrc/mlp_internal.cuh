@@ -17,17 +17,22 @@ struct Net {
     float *p = nullptr;           // FP32 master parameters
     float *m = nullptr, *v = nullptr;  // Adam moments
     __nv_bfloat16 *wb = nullptr;  // BF16 copy of p
+    __nv_bfloat16 *wt = nullptr;  // BF16 W2, W3, W4 transposed, [3][256][256]
     unsigned *err = nullptr;      // set by a GEMM whose bounded tensor-core wait ran out
     unsigned char *wpack = nullptr;  // BF16 W2, W3, W4 in the tensor core's shared-memory layout (inference)
     int64_t off_w[5], off_b[5];
 };
 
+// A batch's activations and gradients, [B][256] but for the transposes [256][ldt] (ldt: B padded to a multiple of 128,
+// the padding zero).
 struct Acts {
-    float *h[4];              // tanh outputs per hidden layer [B][256] (FP32)
+    float *h[4];              // tanh outputs per hidden layer (FP32)
     __nv_bfloat16 *hb[4];     // their BF16 copies
+    __nv_bfloat16 *ht[4];     // and those transposed
     float *y, *dz5, *sqerr;   // [B]
-    float *dz, *dh;           // [B][256]
-    __nv_bfloat16 *dzb;       // [B][256]
+    float *dz[4];             // dL/dz per hidden layer
+    __nv_bfloat16 *dzb[4], *dzt[4];
+    int64_t ldt;
 };
 
 inline void layout(Net &n) {
@@ -42,18 +47,18 @@ inline void layout(Net &n) {
     n.off_b[4] = o; o += 1;
 }
 
-// C = A . B (+ C) on the tensor cores (tcgen05, accumulator in tensor memory); see mlp.cu.
-cudaError_t gemm_bf16(const __nv_bfloat16 *A, int64_t sam, int64_t sak, const __nv_bfloat16 *B, int64_t sbk, int64_t sbn,
-                      float *C, int64_t ldc, int M, int N, int K, int accumulate, unsigned *err, cudaStream_t s);
-cudaError_t forward(const Net &n, const Acts &a, const float *x, int Bn, cudaStream_t s);
+// Forward and backward pass of a batch of Bn samples, sample b being row idx[b] of X and T (idx null: row b): gradients
+// of mean((y - t)^2) into g, per-sample squared errors into a.sqerr; see mlp.cu.
+cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *T, const int *idx, float *g, int Bn,
+                      cudaStream_t s);
 // Inference only: y = network(x) for Bn queries in one fused launch, with the same rounding points as forward.
 // It reads W2-W4 from n.wpack, which pack_weights fills from n.wb (again after every change of the weights).
 constexpr int64_t WPACK_BYTES = 3 * (int64_t)HID * HID * 2;
 cudaError_t pack_weights(const Net &n, cudaStream_t s);
 // inject_stall (tests): the first CTA's first weight wait runs out, as a stuck copy would make it.
 cudaError_t infer(const Net &n, const float *x, float *y, int Bn, cudaStream_t s, int inject_stall);
-cudaError_t backward(const Net &n, const Acts &a, const float *x, const float *t, float *g, int Bn, cudaStream_t s);
 cudaError_t adam(const Net &n, const float *g, float lr, int64_t step, cudaStream_t s);
+// The BF16 copies (and transposes) of the parameters.
 cudaError_t refresh_bf16(const Net &n, cudaStream_t s);
 
 }  // namespace mlp

@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/dirac.h"
@@ -27,16 +28,6 @@ uint64_t splitmix64(uint64_t x) {
 }
 double unit(uint64_t seed, uint64_t i) { return (double)(splitmix64(seed * 0x100000001B3ull + i) >> 11) * 0x1.0p-53; }
 
-__global__ void gather_kernel(const float *X, const float *T, const int *idx, float *xb, float *tb, int Bn) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= Bn) return;
-    const int i = idx[b];
-    xb[b * 3 + 0] = X[i * 3 + 0];
-    xb[b * 3 + 1] = X[i * 3 + 1];
-    xb[b * 3 + 2] = X[i * 3 + 2];
-    if (T) tb[b] = T[i];
-}
-
 }  // namespace
 
 struct dirac_surrogate {
@@ -46,10 +37,14 @@ struct dirac_surrogate {
     cudaStream_t stream = nullptr;
     int device = 0;
     Net net;
-    Acts acts{};
+    Acts acts{};              // training buffers for batches up to acts_cap (allocated by the first that needs them)
+    int acts_cap = 0;
+    void *acts_mem = nullptr;
+    float *dX = nullptr, *dT = nullptr, *dsq = nullptr;  // training set, per-sample squared errors and order, up to data_cap
+    int *dIdx = nullptr;
+    int64_t data_cap = 0;
     float *grad = nullptr;
-    float *xb = nullptr, *tb = nullptr;
-    int *idx = nullptr;
+    float *xb = nullptr, *tb = nullptr, *yout = nullptr;
     float *host_pinned = nullptr;  // staging: max_batch * 4 floats
     unsigned *flag_pinned = nullptr;  // the tensor-wait flag, read back with a prediction's outputs
     bool packed = false;  // net.wpack holds the current W2-W4 (cleared whenever the weights change)
@@ -108,6 +103,54 @@ dirac_status stage(dirac_surrogate *s, const double *X, const double *T, int64_t
     return DIRAC_OK;
 }
 
+// Training buffers for batches of B samples, in one allocation (kept for the handle's life, grown when a larger batch
+// comes; freed by dirac_surrogate_destroy).
+dirac_status ensure_acts(dirac_surrogate *s, int B) {
+    if (B <= s->acts_cap) return DIRAC_OK;
+    SCK(s, cudaStreamSynchronize(s->stream));
+    if (s->acts_mem) SCK(s, cudaFree(s->acts_mem));
+    s->acts_mem = nullptr;
+    s->acts_cap = 0;
+    const size_t pad = ((size_t)B + 127) / 128 * 128, E = pad * HID;
+    // FP32 h and dz (4 each), BF16 copies and transposes of both (4 each), y, dz5 and sqerr
+    const size_t bytes = 8 * E * sizeof(float) + 16 * E * sizeof(__nv_bfloat16) + 3 * pad * sizeof(float);
+    SCK(s, cudaMalloc(&s->acts_mem, bytes));
+    char *at = static_cast<char *>(s->acts_mem);
+    auto take = [&](auto *&p, size_t n) {
+        p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(at);
+        at += n * sizeof(*p);
+    };
+    for (int l = 0; l < 4; ++l) {
+        take(s->acts.h[l], E);
+        take(s->acts.dz[l], E);
+        take(s->acts.hb[l], E);
+        take(s->acts.ht[l], E);
+        take(s->acts.dzb[l], E);
+        take(s->acts.dzt[l], E);
+    }
+    take(s->acts.y, pad);
+    take(s->acts.dz5, pad);
+    take(s->acts.sqerr, pad);
+    s->acts.ldt = (int64_t)pad;
+    s->acts_cap = B;
+    return DIRAC_OK;
+}
+
+// Device copies of a training set of n samples (inputs, targets, squared errors, order), kept and grown likewise.
+dirac_status ensure_data(dirac_surrogate *s, int64_t n) {
+    if (n <= s->data_cap) return DIRAC_OK;
+    SCK(s, cudaStreamSynchronize(s->stream));
+    if (s->dX) SCK(s, cudaFree(s->dX));
+    s->dX = nullptr;
+    s->data_cap = 0;
+    SCK(s, cudaMalloc(&s->dX, (size_t)n * 6 * sizeof(float)));
+    s->dT = s->dX + 3 * n;
+    s->dsq = s->dX + 4 * n;
+    s->dIdx = reinterpret_cast<int *>(s->dX + 5 * n);
+    s->data_cap = n;
+    return DIRAC_OK;
+}
+
 // Reads (and clears) the flag a GEMM sets when its bounded wait for the tensor cores ran out.
 dirac_status check_tensor_waits(dirac_surrogate *s) {
     unsigned flag = 0;
@@ -155,19 +198,10 @@ dirac_status dirac_surrogate_create(const double lo[3], const double hi[3], uint
     if (e == cudaSuccess) e = salloc(s, &s->net.wb, NPARAM * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = salloc(s, &s->net.wpack, WPACK_BYTES);
     if (e == cudaSuccess) e = salloc(s, &s->grad, NPARAM * sizeof(float));
-    for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
-        e = salloc(s, &s->acts.h[l], B * HID * sizeof(float));
-        if (e == cudaSuccess) e = salloc(s, &s->acts.hb[l], B * HID * sizeof(__nv_bfloat16));
-    }
-    if (e == cudaSuccess) e = salloc(s, &s->acts.y, B * sizeof(float));
-    if (e == cudaSuccess) e = salloc(s, &s->acts.dz5, B * sizeof(float));
-    if (e == cudaSuccess) e = salloc(s, &s->acts.sqerr, B * sizeof(float));
-    if (e == cudaSuccess) e = salloc(s, &s->acts.dz, B * HID * sizeof(float));
-    if (e == cudaSuccess) e = salloc(s, &s->acts.dh, B * HID * sizeof(float));
-    if (e == cudaSuccess) e = salloc(s, &s->acts.dzb, B * HID * sizeof(__nv_bfloat16));
+    if (e == cudaSuccess) e = salloc(s, &s->net.wt, 3 * (size_t)HID * HID * sizeof(__nv_bfloat16));
+    if (e == cudaSuccess) e = salloc(s, &s->yout, B * sizeof(float));
     if (e == cudaSuccess) e = salloc(s, &s->xb, B * 3 * sizeof(float));
     if (e == cudaSuccess) e = salloc(s, &s->tb, B * sizeof(float));
-    if (e == cudaSuccess) e = salloc(s, &s->idx, B * sizeof(int));
     if (e == cudaSuccess) e = salloc(s, &s->net.err, 16);
     if (e == cudaSuccess) e = cudaMemset(s->net.err, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMallocHost(&s->host_pinned, B * 4 * sizeof(float));
@@ -193,6 +227,8 @@ dirac_status dirac_surrogate_destroy(dirac_surrogate *s) {
     cudaSetDevice(s->device);
     cudaStreamSynchronize(s->stream);
     for (void *p : s->owned) cudaFree(p);
+    if (s->acts_mem) cudaFree(s->acts_mem);
+    if (s->dX) cudaFree(s->dX);
     if (s->host_pinned) cudaFreeHost(s->host_pinned);
     if (s->flag_pinned) cudaFreeHost(s->flag_pinned);
     delete s;
@@ -290,10 +326,10 @@ dirac_status dirac_surrogate_gradient(dirac_surrogate *s, const double *X, const
                                       double *loss_out) {
     if (!s || !X || !T || !grad_out || n < 1 || n > s->max_batch) return sfail(s, DIRAC_ERR_ARG, "bad arguments");
     SCK(s, cudaSetDevice(s->device));
-    dirac_status st = stage(s, X, T, 0, (int)n);
+    dirac_status st = ensure_acts(s, (int)n);
+    if (st == DIRAC_OK) st = stage(s, X, T, 0, (int)n);
     if (st != DIRAC_OK) return st;
-    SCK(s, forward(s->net, s->acts, s->xb, (int)n, s->stream));
-    SCK(s, backward(s->net, s->acts, s->xb, s->tb, s->grad, (int)n, s->stream));
+    SCK(s, gradients(s->net, s->acts, s->xb, s->tb, nullptr, s->grad, (int)n, s->stream));
     std::vector<float> sq(n);
     SCK(s, cudaMemcpyAsync(grad_out, s->grad, NPARAM * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
     SCK(s, cudaMemcpyAsync(sq.data(), s->acts.sqerr, n * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
@@ -314,27 +350,19 @@ dirac_status dirac_surrogate_train(dirac_surrogate *s, const double *X, const do
         return sfail(s, DIRAC_ERR_ARG, "dirac_surrogate_train: bad arguments");
     SCK(s, cudaSetDevice(s->device));
     s->packed = false;  // the Adam steps change the weights
-    float *dX = nullptr, *dT = nullptr;
-    int *dIdx = nullptr;
+    const int64_t nb = n / batch;  // full batches per epoch (at least one: a smaller n trains on all of it)
+    const int64_t per_epoch = std::max<int64_t>(1, nb);
+    const int bsz = nb > 0 ? batch : (int)n;
+    dirac_status st = ensure_acts(s, bsz);
+    if (st == DIRAC_OK) st = ensure_data(s, n);
+    if (st != DIRAC_OK) return st;
     std::vector<float> hx((size_t)n * 3), ht(n);
     for (int64_t i = 0; i < n; ++i) {
         normalise(s, X + i * 3, &hx[i * 3]);
         ht[i] = (float)T[i];
     }
-    cudaError_t e = cudaMalloc(&dX, hx.size() * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&dT, ht.size() * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&dIdx, (size_t)n * sizeof(int));
-    auto cleanup = [&]() {
-        cudaFree(dX);
-        cudaFree(dT);
-        cudaFree(dIdx);
-    };
-    if (e != cudaSuccess) {
-        cleanup();
-        return scuda(s, e, "training buffers");
-    }
-    e = cudaMemcpy(dX, hx.data(), hx.size() * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(dT, ht.data(), ht.size() * sizeof(float), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(s->dX, hx.data(), hx.size() * sizeof(float), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->dT, ht.data(), ht.size() * sizeof(float), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess && !s->bias_set) {
         // first training call: start the output at the mean target (bias = logit of the mean), so the
         // sigmoid does not begin in a saturated region where the squared-error gradient vanishes
@@ -346,42 +374,36 @@ dirac_status dirac_surrogate_train(dirac_surrogate *s, const double *X, const do
         s->bias_set = true;
     }
     std::vector<int> perm(n);
-    const int64_t nb = n / batch;  // full batches per epoch (at least one: a smaller n trains on all of it)
-    const int64_t per_epoch = std::max<int64_t>(1, nb);
-    const int bsz = nb > 0 ? batch : (int)n;
     const int64_t total = per_epoch * epochs;
-    std::vector<float> sq(bsz);
-    double last = 0.0;
+    std::vector<float> sq((size_t)(per_epoch * bsz));
+    Acts acts = s->acts;
     for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
         for (int64_t i = 0; i < n; ++i) perm[i] = (int)i;
         for (int64_t i = n - 1; i > 0; --i) {  // Fisher-Yates
             const int64_t j = (int64_t)(unit(s->seed ^ 0xA5A5A5A5ull, (uint64_t)ep * (uint64_t)n + i) * (i + 1));
             std::swap(perm[i], perm[std::min<int64_t>(j, i)]);
         }
-        e = cudaMemcpyAsync(dIdx, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, s->stream);
-        double ep_loss = 0.0;
+        e = cudaMemcpyAsync(s->dIdx, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, s->stream);
         for (int64_t bi = 0; bi < per_epoch && e == cudaSuccess; ++bi) {
-            gather_kernel<<<(bsz + 255) / 256, 256, 0, s->stream>>>(dX, dT, dIdx + bi * bsz, s->xb, s->tb, bsz);
-            e = cudaGetLastError();
-            if (e == cudaSuccess) e = forward(s->net, s->acts, s->xb, bsz, s->stream);
-            if (e == cudaSuccess) e = backward(s->net, s->acts, s->xb, s->tb, s->grad, bsz, s->stream);
+            if (ep == epochs - 1) acts.sqerr = s->dsq + bi * bsz;  // the last epoch's errors are read once, at its end
+            e = gradients(s->net, acts, s->dX, s->dT, s->dIdx + bi * bsz, s->grad, bsz, s->stream);
             const double t = (double)s->step / (double)std::max<int64_t>(1, total);
             const double lr_t = lr / 20.0 + 0.5 * (lr - lr / 20.0) * (1.0 + std::cos(M_PI * t));
             ++s->step;
             if (e == cudaSuccess) e = adam(s->net, s->grad, (float)lr_t, s->step, s->stream);
-            if (e == cudaSuccess && ep == epochs - 1) {
-                e = cudaMemcpyAsync(sq.data(), s->acts.sqerr, bsz * sizeof(float), cudaMemcpyDeviceToHost, s->stream);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-                for (float v : sq) ep_loss += v;
-            }
         }
-        if (ep == epochs - 1) last = ep_loss / (double)(per_epoch * bsz);
     }
+    if (e == cudaSuccess && epochs > 0)
+        e = cudaMemcpyAsync(sq.data(), s->dsq, sq.size() * sizeof(float), cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    cleanup();
     if (e != cudaSuccess) return scuda(s, e, "training step");
-    dirac_status st = check_tensor_waits(s);
+    st = check_tensor_waits(s);
     if (st != DIRAC_OK) return st;
+    double last = 0.0;
+    if (epochs > 0) {
+        for (float v : sq) last += v;
+        last /= (double)(per_epoch * bsz);
+    }
     if (loss_out) *loss_out = last;
     return DIRAC_OK;
 }
@@ -399,8 +421,8 @@ dirac_status dirac_surrogate_predict(dirac_surrogate *s, const double *X, int64_
         const int nb = (int)std::min<int64_t>(s->max_batch, n - i0);
         dirac_status st = stage(s, X, nullptr, i0, nb);
         if (st != DIRAC_OK) return st;
-        SCK(s, infer(s->net, s->xb, s->acts.y, nb, s->stream, s->inject_stall));
-        SCK(s, cudaMemcpyAsync(y.data(), s->acts.y, nb * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
+        SCK(s, infer(s->net, s->xb, s->yout, nb, s->stream, s->inject_stall));
+        SCK(s, cudaMemcpyAsync(y.data(), s->yout, nb * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
         if (i0 + nb >= n)  // the flag a timed-out tensor-core wait sets, read with the last outputs
             SCK(s, cudaMemcpyAsync(s->flag_pinned, s->net.err, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
         SCK(s, cudaStreamSynchronize(s->stream));
