@@ -28,7 +28,10 @@ namespace {
 // K = 64 stage goes to shared memory by cp.async, four stages in flight, so a whole K = 256 is under way at once, and
 // 32-column tiles give such a product 16 CTAs.  Operands that a product needs the other way round (the weight
 // gradients' dz and h, the data gradients' W) are kept transposed by the kernels that produce them: an accumulator
-// row is a lane, so a column's 32 values leave as 64 consecutive bytes.  Measured for 256 x 256 x 256: see `step`.
+// row is a lane, so a column's 32 values leave as 64 consecutive bytes.  A launch of a
+// 256 x 256 x 256 product takes 8.3 us alone under the profiler, layer epilogue included (before: 33 us and a launch for
+// the epilogue); a training step of 256 samples 55 us in its chain of overlapping launches (93 us without the overlap,
+// 271 before).
 // Shared memory holds the canonical no-swizzle K-major layout (8-row x 16-byte core matrices; K-direction core-matrix
 // stride 128 B, 8-row-group stride 256 B; one 16-deep K slab per MMA).  One thread issues tcgen05.mma (M = 128, N = 32,
 // K = 16) in ascending k and commits each stage to an mbarrier; every wait is bounded (about one second of the global
@@ -60,6 +63,16 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
         if ((it & 63) == 63 && timer_ns() - t0 > 1000000000ull) return false;
     }
     return false;
+}
+
+// Programmatic dependent launch (the training step's chain of short kernels): a launch may begin while the previous one
+// runs; everything the previous kernel writes is touched after chain_wait only, which returns when that kernel has
+// finished.  Each kernel lets the next one begin after its own chain_wait, so whatever the kernel before the previous one
+// wrote is complete when a kernel starts: the weights (the step's last kernel writes them) may be read before the wait by
+// every kernel but the step's first.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Shared-memory matrix descriptor: no swizzle, K-major; start address, LBO (K-direction core-matrix
@@ -129,16 +142,21 @@ template <int KIND> __device__ __forceinline__ void gemm_tile(const GemmArgs &g,
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar[i])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    auto load_chunk = [&](int c) {
-        unsigned char *buf = gsm + (c % GSTAGES) * STAGE_BYTES;
-        if (c < nchunks) {
-            stage_async<GM>(buf, A_SLAB, g.A, g.lda, m0, g.M, c * GK);
-            stage_async<GN>(buf + 4 * A_SLAB, B_SLAB, g.B, g.ldb, n0, HID, c * GK);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
+    auto load_a = [&](int c) {
+        if (c < nchunks) stage_async<GM>(gsm + (c % GSTAGES) * STAGE_BYTES, A_SLAB, g.A, g.lda, m0, g.M, c * GK);
+        asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk (with its B), empty past the end
     };
+    auto load_b = [&](int c) {
+        if (c < nchunks)
+            stage_async<GN>(gsm + (c % GSTAGES) * STAGE_BYTES + 4 * A_SLAB, B_SLAB, g.B, g.ldb, n0, HID, c * GK);
+    };
+    // FWD and DGRAD: the weights while the previous kernel still runs
+    if (KIND == WGRAD) chain_wait();
 #pragma unroll
-    for (int c = 0; c < GSTAGES - 1; ++c) load_chunk(c);
+    for (int c = 0; c < GSTAGES - 1; ++c) load_b(c);
+    if (KIND != WGRAD) chain_wait();
+#pragma unroll
+    for (int c = 0; c < GSTAGES - 1; ++c) load_a(c);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -151,7 +169,8 @@ template <int KIND> __device__ __forceinline__ void gemm_tile(const GemmArgs &g,
         if (c >= 1 && c + GSTAGES - 1 < nchunks)
             ok = __syncthreads_and(bar_wait(smem_addr(&mbar[(c - 1) % GSTAGES]), (uint32_t)(((c - 1) / GSTAGES) & 1)));
         if (!ok) break;
-        load_chunk(c + GSTAGES - 1);
+        load_b(c + GSTAGES - 1);
+        load_a(c + GSTAGES - 1);
         asm volatile("cp.async.wait_group %0;" ::"n"(GSTAGES - 1) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // landed pieces -> the tensor core's view
         __syncthreads();
@@ -252,6 +271,7 @@ struct BatchIn {
 __global__ void __launch_bounds__(256) layer1_fwd_kernel(const BatchIn in, const __nv_bfloat16 *W1, const float *b1, float *h,
                                                          __nv_bfloat16 *hb, __nv_bfloat16 *ht, int64_t ldt) {
     __shared__ __nv_bfloat16 tr[32][34];
+    chain_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
     const int j = j0 + tx;
 #pragma unroll
@@ -277,60 +297,89 @@ __global__ void __launch_bounds__(256) layer1_fwd_kernel(const BatchIn in, const
 }
 
 // The output layer both ways, one warp per sample: y = sigmoid(bf16(h4) . bf16(w5) + b5); dz5 = 2 (y - t) y (1 - y) / B and
-// the squared error; the last hidden layer's dz = dz5 w5 (1 - h4^2), its BF16 copy and the copy's transpose (32 samples of
-// a block through shared memory; zeros for the samples that pad the batch).
-__global__ void __launch_bounds__(1024) out_layer_kernel(const BatchIn in, const __nv_bfloat16 *h4b, const float *h4,
-                                                         const __nv_bfloat16 *w5, const float *b5, float *y, float *dz5,
-                                                         float *sqerr, float *dz, __nv_bfloat16 *dzb, __nv_bfloat16 *dzt,
-                                                         int64_t ldt) {
-    __shared__ __nv_bfloat16 tr[32][HID + 2];
+// the squared error; the last hidden layer's dz = dz5 w5 (1 - h4^2), its BF16 copy and the copy's transpose (the 16 samples
+// of a block through shared memory; zeros for the samples that pad the batch).  Everything a sample needs is loaded before
+// the first sum.
+constexpr int OUT_B = 16;
+__global__ void __launch_bounds__(32 * OUT_B) out_layer_kernel(const BatchIn in, const __nv_bfloat16 *h4b, const float *h4,
+                                                               const __nv_bfloat16 *w5, const float *b5, float *y, float *dz5,
+                                                               float *sqerr, float *dz, __nv_bfloat16 *dzb,
+                                                               __nv_bfloat16 *dzt, int64_t ldt) {
+    __shared__ __nv_bfloat16 tr[OUT_B][HID + 2];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int b = blockIdx.x * 32 + w;
+    const int b = blockIdx.x * OUT_B + w;
+    constexpr int NJ = HID / 32;
+    float wj[NJ], hj[NJ], aj[NJ];
+#pragma unroll
+    for (int i = 0; i < NJ; ++i) wj[i] = __bfloat162float(w5[lane + 32 * i]);
+    const float t = b < in.B ? in.T[in.row(b)] : 0.f, b5v = b5[0];
+    chain_wait();
     if (b < in.B) {
+#pragma unroll
+        for (int i = 0; i < NJ; ++i) {
+            hj[i] = __bfloat162float(h4b[(int64_t)b * HID + lane + 32 * i]);
+            aj[i] = h4[(int64_t)b * HID + lane + 32 * i];
+        }
         float s = 0.f;
-        for (int j = lane; j < HID; j += 32) s = fmaf(__bfloat162float(h4b[(int64_t)b * HID + j]), __bfloat162float(w5[j]), s);
+#pragma unroll
+        for (int i = 0; i < NJ; ++i) s = fmaf(hj[i], wj[i], s);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const float yb = 1.f / (1.f + expf(-(s + b5[0])));
-        const float d = yb - in.T[in.row(b)];
+        const float yb = 1.f / (1.f + expf(-(s + b5v)));
+        const float d = yb - t;
         const float g5 = 2.f * d * yb * (1.f - yb) / (float)in.B;
         if (lane == 0) {
             y[b] = yb;
             dz5[b] = g5;
             sqerr[b] = d * d;
         }
-        for (int j = lane; j < HID; j += 32) {
-            const float g = g5 * __bfloat162float(w5[j]);
-            const float a = h4[(int64_t)b * HID + j];
-            const float v = g * (1.f - a * a);
+#pragma unroll
+        for (int i = 0; i < NJ; ++i) {
+            const int j = lane + 32 * i;
+            const float g = g5 * wj[i];
+            const float v = g * (1.f - aj[i] * aj[i]);
             dz[(int64_t)b * HID + j] = v;
             const __nv_bfloat16 o = __float2bfloat16(v);
             dzb[(int64_t)b * HID + j] = o;
             tr[w][j] = o;
         }
     } else {
-        for (int j = lane; j < HID; j += 32) tr[w][j] = __float2bfloat16(0.f);
+#pragma unroll
+        for (int i = 0; i < NJ; ++i) tr[w][lane + 32 * i] = __float2bfloat16(0.f);
     }
     __syncthreads();
-    for (int j = w; j < HID; j += 32) dzt[(int64_t)j * ldt + blockIdx.x * 32 + lane] = tr[lane][j];
+    for (int e = threadIdx.x; e < HID * OUT_B; e += 32 * OUT_B)
+        dzt[(int64_t)(e / OUT_B) * ldt + blockIdx.x * OUT_B + e % OUT_B] = tr[e % OUT_B][e / OUT_B];
 }
 
-// Sum over the batch of term(b), one warp: 256 partial sums (b mod 256), each 32 of them by an xor tree, the eight
-// trees in order.
-template <typename F> __device__ __forceinline__ float batch_sum(int B, int lane, F term) {
-    float v = 0.f;
+// Sums over the batch for 32 columns, a block of 256 threads: thread (w, column) adds the samples b = 32 w + l (mod 256) into
+// one partial for each l = 0..31, those by a tree (l with l + 16, + 8, ...), and the eight w in order.  Consecutive lanes
+// read consecutive columns.
+template <typename F> __device__ __forceinline__ void batch_sums(int B, F term, float *to, int stride, int columns) {
+    __shared__ float part[8][33];
+    const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float s[32];
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
-        float s = 0.f;
-        for (int b = 32 * w + lane; b < B; b += 256) s += term(b);
+    for (int l = 0; l < 32; ++l) s[l] = 0.f;
+    for (int b0 = 32 * w; b0 < B; b0 += 256)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        v += s;
+        for (int l = 0; l < 32; ++l)
+            if (b0 + l < B && c < columns) s[l] += term(b0 + l, c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int l = 0; l < o; ++l) s[l] = s[l] + s[l + o];
+    part[w][c] = s[0];
+    __syncthreads();
+    if (w == 0 && c < columns) {
+        float v = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v += part[i][c];
+        to[c * stride] = v;
     }
-    return v;
 }
 
-// The gradients, one launch: blocks [0, 48) the three hidden weight matrices (16 tiles each), then one warp each for the
+// The gradients, one launch: blocks [0, 48) the three hidden weight matrices (16 tiles each), then 32 columns each of the
 // sums over the batch: db of the four hidden layers, dW1 = dz1^T x, dW5 = sum_b dz5 bf16(h4), db5 = sum_b dz5.
 struct GradArgs {
     GemmArgs w[3];             // dW2, dW3, dW4
@@ -339,31 +388,30 @@ struct GradArgs {
     float *gb[4], *gW1, *gW5, *gb5;
     BatchIn in;
 };
-constexpr int kGradTiles = 3 * (HID / GM) * (HID / GN), kGradSums = 4 * HID + 3 * HID + HID + 1;
+constexpr int kGradTiles = 3 * (HID / GM) * (HID / GN), kColumnGroups = HID / 32;
+constexpr int kGradSums = (4 + 3 + 1) * kColumnGroups + 1;
 __global__ void __launch_bounds__(256) grad_kernel(const __grid_constant__ GradArgs a) {
     if (blockIdx.x < kGradTiles) {
         const int per = kGradTiles / 3, t = blockIdx.x % per;
         gemm_tile<WGRAD>(a.w[blockIdx.x / per], (t / (HID / GN)) * GM, (t % (HID / GN)) * GN);
         return;
     }
-    const int lane = threadIdx.x & 31, q = (blockIdx.x - kGradTiles) * 8 + (threadIdx.x >> 5), B = a.in.B;
-    if (q >= kGradSums) return;
-    float v;
-    float *to;
-    if (q < 4 * HID) {
-        const float *dz = a.dz[q / HID] + q % HID;
-        v = batch_sum(B, lane, [&](int b) { return dz[(int64_t)b * HID]; });
-        to = a.gb[q / HID] + q % HID;
-    } else if (q < 7 * HID) {
-        const int e = q - 4 * HID, j = e / 3, i = e % 3;
-        v = batch_sum(B, lane, [&](int b) { return a.dz[0][(int64_t)b * HID + j] * a.in.X[(int64_t)a.in.row(b) * 3 + i]; });
-        to = a.gW1 + j * 3 + i;
+    chain_wait();
+    const int q = blockIdx.x - kGradTiles, what = q / kColumnGroups, j0 = (q % kColumnGroups) * 32, B = a.in.B;
+    if (what < 4) {
+        const float *dz = a.dz[what] + j0;
+        batch_sums(B, [&](int b, int c) { return dz[(int64_t)b * HID + c]; }, a.gb[what] + j0, 1, 32);
+    } else if (what < 7) {
+        const float *dz = a.dz[0] + j0;
+        const int i = what - 4;
+        batch_sums(B, [&](int b, int c) { return dz[(int64_t)b * HID + c] * a.in.X[(int64_t)a.in.row(b) * 3 + i]; },
+                   a.gW1 + j0 * 3 + i, 3, 32);
+    } else if (what == 7) {
+        const __nv_bfloat16 *h = a.h4b + j0;
+        batch_sums(B, [&](int b, int c) { return a.dz5[b] * __bfloat162float(h[(int64_t)b * HID + c]); }, a.gW5 + j0, 1, 32);
     } else {
-        const int j = q - 7 * HID;
-        v = batch_sum(B, lane, [&](int b) { return a.dz5[b] * (j < HID ? __bfloat162float(a.h4b[(int64_t)b * HID + j]) : 1.f); });
-        to = j < HID ? a.gW5 + j : a.gb5;
+        batch_sums(B, [&](int b, int) { return a.dz5[b] * 1.f; }, a.gb5, 1, 1);
     }
-    if (lane == 0) *to = v;
 }
 
 // One Adam step's scalars: the learning rate and the moments' bias corrections.
@@ -402,6 +450,7 @@ struct ParamArgs {
     int64_t n;
 };
 template <bool UPDATE> __global__ void __launch_bounds__(256) param_kernel(const __grid_constant__ ParamArgs a, AdamStep st) {
+    chain_wait();
     if (blockIdx.x < kAdamTiles) {
         __shared__ __nv_bfloat16 tr[32][34];
         const int per = kAdamTiles / 3, l = blockIdx.x / per, t = blockIdx.x % per;
@@ -668,12 +717,26 @@ template <typename K> cudaError_t optin(K *kernel, int smem, std::atomic<unsigne
     if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_relaxed);
     return e;
 }
+// Launches a kernel of the chain: it may begin while its predecessor in the stream runs (see chain_wait).
+template <typename... KA, typename... A>
+cudaError_t launch_chain(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, args...);
+}
 template <int KIND> cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t s) {
     static std::atomic<unsigned long long> done{0};
     cudaError_t e = optin(layer_gemm_kernel<KIND>, GEMM_SMEM, done);
     if (e != cudaSuccess) return e;
-    layer_gemm_kernel<KIND><<<dim3(HID / GN, nblk(g.M, GM)), 256, GEMM_SMEM, s>>>(g);
-    return cudaGetLastError();
+    return launch_chain(layer_gemm_kernel<KIND>, dim3(HID / GN, nblk(g.M, GM)), dim3(256), GEMM_SMEM, s, g);
 }
 }  // namespace
 
@@ -683,9 +746,8 @@ cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *
                       cudaStream_t s) {
     const BatchIn in{X, T, idx, Bn};
     const int pad = nblk(Bn, GM) * GM;
-    layer1_fwd_kernel<<<dim3(pad / 32, HID / 32), 256, 0, s>>>(in, n.wb + n.off_w[0], n.p + n.off_b[0], a.h[0], a.hb[0], a.ht[0],
-                                                              a.ldt);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chain(layer1_fwd_kernel, dim3(pad / 32, HID / 32), dim3(256), 0, s, in, n.wb + n.off_w[0],
+                                 n.p + n.off_b[0], a.h[0], a.hb[0], a.ht[0], a.ldt);
     GemmArgs q{};
     q.err = n.err;
     q.lda = q.ldb = HID;
@@ -703,9 +765,8 @@ cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *
         e = launch_gemm<FWD>(q, s);
     }
     if (e != cudaSuccess) return e;
-    out_layer_kernel<<<pad / 32, 1024, 0, s>>>(in, a.hb[3], a.h[3], n.wb + n.off_w[4], n.p + n.off_b[4], a.y, a.dz5, a.sqerr,
-                                               a.dz[3], a.dzb[3], a.dzt[3], a.ldt);
-    e = cudaGetLastError();
+    e = launch_chain(out_layer_kernel, dim3(pad / OUT_B), dim3(32 * OUT_B), 0, s, in, a.hb[3], a.h[3], n.wb + n.off_w[4],
+                     n.p + n.off_b[4], a.y, a.dz5, a.sqerr, a.dz[3], a.dzb[3], a.dzt[3], a.ldt);
     for (int l = 3; l >= 1 && e == cudaSuccess; --l) {
         // dh_{l-1}[b][k] = sum_j bf16(dz_l)[b][j] bf16(W_l)[j][k]
         q.A = a.dzb[l];
@@ -742,8 +803,7 @@ cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *
     static std::atomic<unsigned long long> done{0};
     e = optin(grad_kernel, GEMM_SMEM, done);
     if (e != cudaSuccess) return e;
-    grad_kernel<<<kGradTiles + nblk(kGradSums, 8), 256, GEMM_SMEM, s>>>(r);
-    return cudaGetLastError();
+    return launch_chain(grad_kernel, dim3(kGradTiles + kGradSums), dim3(256), GEMM_SMEM, s, r);
 }
 
 namespace {
@@ -765,13 +825,11 @@ constexpr int kParamBlocks = kAdamTiles + (int)((NPARAM - 3 * (int64_t)HID * HID
 cudaError_t adam(const Net &n, const float *g, float lr, int64_t step, cudaStream_t s) {
     const float b1 = 0.9f, b2 = 0.999f;
     const AdamStep st{lr, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step)};
-    param_kernel<true><<<kParamBlocks, 256, 0, s>>>(param_args(n, g), st);
-    return cudaGetLastError();
+    return launch_chain(param_kernel<true>, dim3(kParamBlocks), dim3(256), 0, s, param_args(n, g), st);
 }
 
 cudaError_t refresh_bf16(const Net &n, cudaStream_t s) {
-    param_kernel<false><<<kParamBlocks, 256, 0, s>>>(param_args(n, nullptr), AdamStep{});
-    return cudaGetLastError();
+    return launch_chain(param_kernel<false>, dim3(kParamBlocks), dim3(256), 0, s, param_args(n, nullptr), AdamStep{});
 }
 
 }  // namespace mlp
