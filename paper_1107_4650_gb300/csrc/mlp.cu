@@ -675,34 +675,167 @@ __global__ void __launch_bounds__(32 * NW, 1) mlp_infer_kernel(const float *x, c
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
 }
 
+// Inference of small calls: 32 queries per CTA, so that up to 32 x 152 of them spread over the chip (a CTA of 128 queries
+// spends its time in tanh: 4 x 64 per thread; here 4 x 16).  The MMA's M stays 128: the 32 queries stand four times in the
+// A operand, so each of the four 32-lane groups of the accumulator holds all of them and the 16 warps take 16 columns
+// each from the group they can read.  Rows are independent in the product and every query's arithmetic is that of
+// mlp_infer_kernel, so the predictions are the same bits.  x, y and the timeout flag may be pinned host memory (a call
+// of this size is shorter than its copies).  Measured end to end, with the copies it does without: 4096 queries a call
+// 67 -> 39 us, one query 54 -> 27.
+constexpr int SQ = 32;
+__global__ void __launch_bounds__(512, 1) mlp_infer_small_kernel(const float *x, const __nv_bfloat16 *W1, const float *b1,
+                                                                 const unsigned char *pack, const float *b2, const float *b3,
+                                                                 const float *b4, const __nv_bfloat16 *w5, const float *b5,
+                                                                 float *y, int Bn, unsigned *err, int inject_stall) {
+    extern __shared__ unsigned char ism_raw[];
+    unsigned char *hs = reinterpret_cast<unsigned char *>(((uintptr_t)ism_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *wsm = hs + IH_BYTES;
+    __shared__ __align__(8) uint64_t bars[2];  // [0]: a layer's weights have landed, [1]: its MMAs are done
+    __shared__ uint32_t tmem_slot;
+    __shared__ int issued;
+    __shared__ float part[32][SQ + 1];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int NCOL = HID / 16;  // columns per warp
+    const int c0 = warp * NCOL;
+    const int q = blockIdx.x * SQ + lane;
+    const uint32_t wbar = smem_addr(&bars[0]), mbar = smem_addr(&bars[1]), ws = smem_addr(wsm);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_addr(&tmem_slot))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(wbar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // failure-detection test hook: the first CTA's first weight wait runs out
+        load_layer_weights(ws, pack, wbar, (inject_stall && blockIdx.x == 0) ? 16u : 0u);
+    }
+    // bf16 values of this warp's columns [c, c + 8) of the lane's query into its four places in the A operand
+    auto put8 = [&](int c, const uint32_t pk[4]) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            *reinterpret_cast<uint4 *>(hs + tile_off(r * 32 + lane, c, IH_SLAB)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    };
+    float x0 = 0.f, x1 = 0.f, x2 = 0.f;
+    if (q < Bn) {
+        x0 = x[(int64_t)q * 3 + 0];
+        x1 = x[(int64_t)q * 3 + 1];
+        x2 = x[(int64_t)q * 3 + 2];
+    }
+#pragma unroll
+    for (int j0 = 0; j0 < NCOL; j0 += 8) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            float h[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int j = c0 + j0 + i + u;
+                float z = b1[j];
+                z = fmaf(x0, __bfloat162float(W1[j * 3 + 0]), z);
+                z = fmaf(x1, __bfloat162float(W1[j * 3 + 1]), z);
+                z = fmaf(x2, __bfloat162float(W1[j * 3 + 2]), z);
+                h[u] = tanhf(z);
+            }
+            pk[i / 2] = pack_bf16x2(h[0], h[1]);
+        }
+        put8(c0 + j0, pk);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // activations -> the tensor core's view
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(HID >> 3) << 17) | ((uint32_t)(IQ >> 4) << 24);
+    // Every weight copy is waited for (bounded) before the MMAs that read it, and the next one is issued only
+    // after those MMAs completed, so no copy is in flight wherever the loop stops early.
+    bool ok = true;
+    for (int L = 0; L < 3 && ok; ++L) {
+        if (tid == 0) {
+            issued = 0;
+            if (bar_wait(wbar, (uint32_t)(L & 1))) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int j = 0; j < HID / 16; ++j) {
+                    const uint64_t ad = umma_desc(smem_addr(hs + j * IH_SLAB));
+                    const uint64_t bd = umma_desc(ws + j * IW_SLAB);
+                    const uint32_t acc = j > 0 ? 1u : 0u;
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+                                 "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                                 : "memory");
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
+                             : "memory");
+                issued = 1;
+            }
+        }
+        __syncthreads();
+        ok = __syncthreads_and(issued && bar_wait(mbar, (uint32_t)(L & 1)));
+        if (!ok) break;
+        // the MMAs have read both operands: the next layer's weights can land while this epilogue runs
+        if (tid == 0 && L < 2) load_layer_weights(ws, pack + (int64_t)(L + 1) * IW_BYTES, wbar, 0u);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const float *bias = L == 0 ? b2 : (L == 1 ? b3 : b4);
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0)
+            : "memory");
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < NCOL; i += 8) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int u = 0; u < 8; u += 2)
+                pk[u / 2] = pack_bf16x2(tanhf(__uint_as_float(r[i + u]) + bias[c0 + i + u]),
+                                        tanhf(__uint_as_float(r[i + u + 1]) + bias[c0 + i + u + 1]));
+            put8(c0 + i, pk);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    }
+    if (ok) {
+        // output layer: partial sum l takes columns l, l + 32, ... (two partial sums per warp), then the xor tree
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int l = 2 * warp + u;
+            float s = 0.f;
+#pragma unroll
+            for (int t = 0; t < HID / 32; ++t) {
+                const __nv_bfloat16 h = *reinterpret_cast<const __nv_bfloat16 *>(hs + tile_off(lane, 32 * t + l, IH_SLAB));
+                s = fmaf(__bfloat162float(h), __bfloat162float(w5[32 * t + l]), s);
+            }
+            part[l][lane] = s;
+        }
+        __syncthreads();
+        if (warp == 0 && q < Bn) {
+            float s[32];
+#pragma unroll
+            for (int l = 0; l < 32; ++l) s[l] = part[l][lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int l = 0; l < o; ++l) s[l] = s[l] + s[l + o];
+            y[q] = 1.f / (1.f + expf(-(s[0] + b5[0])));
+        }
+    }
+    if (!ok && tid == 0) *reinterpret_cast<volatile unsigned *>(err) = 1u;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+}
+
 }  // namespace
 
 cudaError_t pack_weights(const Net &n, cudaStream_t s) {
     if ((n.off_w[1] | n.off_w[2] | n.off_w[3]) & 7) return cudaErrorInvalidValue;  // 16-byte rows for the packing
     pack_weights_kernel<<<nblk(3 * HID * (HID / 8), 256), 256, 0, s>>>(n.wb, n.off_w[1], n.off_w[2], n.off_w[3], n.wpack);
-    return cudaGetLastError();
-}
-
-#ifndef MLP_INFER_WARPS
-#define MLP_INFER_WARPS 16
-#endif
-
-cudaError_t infer(const Net &n, const float *x, float *y, int Bn, cudaStream_t s, int inject_stall) {
-    if (Bn <= 0) return cudaSuccess;
-    constexpr int NW = MLP_INFER_WARPS;
-    static std::atomic<unsigned long long> attr_set{0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
-    if (!bit || !(attr_set.load(std::memory_order_relaxed) & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(mlp_infer_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, INFER_SMEM);
-        if (e != cudaSuccess) return e;
-        if (bit) attr_set.fetch_or(bit, std::memory_order_relaxed);
-    }
-    mlp_infer_kernel<NW><<<nblk(Bn, IQ), 32 * NW, INFER_SMEM, s>>>(x, n.wb + n.off_w[0], n.p + n.off_b[0], n.wpack,
-                                                                   n.p + n.off_b[1], n.p + n.off_b[2], n.p + n.off_b[3],
-                                                                   n.wb + n.off_w[4], n.p + n.off_b[4], y, Bn, n.err,
-                                                                   inject_stall);
     return cudaGetLastError();
 }
 
@@ -717,6 +850,32 @@ template <typename K> cudaError_t optin(K *kernel, int smem, std::atomic<unsigne
     if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_relaxed);
     return e;
 }
+}  // namespace
+
+cudaError_t infer(const Net &n, const float *x, float *y, unsigned *err, int Bn, cudaStream_t s, int inject_stall) {
+    if (Bn <= 0) return cudaSuccess;
+    if (Bn <= SMALL_INFER) {
+        static std::atomic<unsigned long long> done{0};
+        cudaError_t e = optin(mlp_infer_small_kernel, INFER_SMEM, done);
+        if (e != cudaSuccess) return e;
+        mlp_infer_small_kernel<<<nblk(Bn, SQ), 512, INFER_SMEM, s>>>(x, n.wb + n.off_w[0], n.p + n.off_b[0], n.wpack,
+                                                                     n.p + n.off_b[1], n.p + n.off_b[2], n.p + n.off_b[3],
+                                                                     n.wb + n.off_w[4], n.p + n.off_b[4], y, Bn, err,
+                                                                     inject_stall);
+        return cudaGetLastError();
+    }
+    constexpr int NW = 16;
+    static std::atomic<unsigned long long> done{0};
+    cudaError_t e = optin(mlp_infer_kernel<NW>, INFER_SMEM, done);
+    if (e != cudaSuccess) return e;
+    mlp_infer_kernel<NW><<<nblk(Bn, IQ), 32 * NW, INFER_SMEM, s>>>(x, n.wb + n.off_w[0], n.p + n.off_b[0], n.wpack,
+                                                                   n.p + n.off_b[1], n.p + n.off_b[2], n.p + n.off_b[3],
+                                                                   n.wb + n.off_w[4], n.p + n.off_b[4], y, Bn, err,
+                                                                   inject_stall);
+    return cudaGetLastError();
+}
+
+namespace {
 // Launches a kernel of the chain: it may begin while its predecessor in the stream runs (see chain_wait).
 template <typename... KA, typename... A>
 cudaError_t launch_chain(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {

@@ -55,8 +55,10 @@ cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *
 // It reads W2-W4 from n.wpack, which pack_weights fills from n.wb (again after every change of the weights).
 constexpr int64_t WPACK_BYTES = 3 * (int64_t)HID * HID * 2;
 cudaError_t pack_weights(const Net &n, cudaStream_t s);
+// A wait that runs out sets *err.  Up to SMALL_INFER queries (32 for each of 152 SMs) x, y and err may be pinned host memory.
 // inject_stall (tests): the first CTA's first weight wait runs out, as a stuck copy would make it.
-cudaError_t infer(const Net &n, const float *x, float *y, int Bn, cudaStream_t s, int inject_stall);
+constexpr int SMALL_INFER = 32 * 152;
+cudaError_t infer(const Net &n, const float *x, float *y, unsigned *err, int Bn, cudaStream_t s, int inject_stall);
 cudaError_t adam(const Net &n, const float *g, float lr, int64_t step, cudaStream_t s);
 // The BF16 copies (and transposes) of the parameters.
 cudaError_t refresh_bf16(const Net &n, cudaStream_t s);

@@ -415,17 +415,24 @@ dirac_status dirac_surrogate_predict(dirac_surrogate *s, const double *X, int64_
         SCK(s, pack_weights(s->net, s->stream));
         s->packed = true;
     }
-    std::vector<float> y(s->max_batch);
+    float *y = s->host_pinned + (size_t)s->max_batch * 3;
     *s->flag_pinned = 0;
     for (int64_t i0 = 0; i0 < n; i0 += s->max_batch) {
         const int nb = (int)std::min<int64_t>(s->max_batch, n - i0);
-        dirac_status st = stage(s, X, nullptr, i0, nb);
-        if (st != DIRAC_OK) return st;
-        SCK(s, infer(s->net, s->xb, s->yout, nb, s->stream, s->inject_stall));
-        SCK(s, cudaMemcpyAsync(y.data(), s->yout, nb * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
-        if (i0 + nb >= n)  // the flag a timed-out tensor-core wait sets, read with the last outputs
+        if (nb <= SMALL_INFER) {
+            // the kernel reads and writes the pinned buffers itself: shorter than a copy each way
+            for (int b = 0; b < nb; ++b) normalise(s, X + (i0 + b) * 3, s->host_pinned + b * 3);
+            SCK(s, infer(s->net, s->host_pinned, y, s->flag_pinned, nb, s->stream, s->inject_stall));
+        } else {
+            dirac_status st = stage(s, X, nullptr, i0, nb);
+            if (st != DIRAC_OK) return st;
+            SCK(s, infer(s->net, s->xb, s->yout, s->net.err, nb, s->stream, s->inject_stall));
+            SCK(s, cudaMemcpyAsync(y, s->yout, nb * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
+            // the flag a timed-out tensor-core wait sets, read with the outputs
             SCK(s, cudaMemcpyAsync(s->flag_pinned, s->net.err, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+        }
         SCK(s, cudaStreamSynchronize(s->stream));
+        if (*s->flag_pinned) break;
 #pragma omp parallel for schedule(static) if (nb >= 32768)
         for (int b = 0; b < nb; ++b) T_out[i0 + b] = y[b];
     }

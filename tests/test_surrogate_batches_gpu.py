@@ -64,3 +64,18 @@ def test_growing_and_shrinking_batches_leave_nothing_behind():
             D.dirac_surrogate_set_params(h, p0)
     finally:
         D.dirac_surrogate_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 127, 129, 4863, 4864, 4865, 6000])
+def test_small_and_large_calls_predict_the_same_bits(n):
+    """Calls of up to 32 queries for each of 152 SMs run on 32-query tiles and pinned buffers, larger ones on 128-query
+    tiles and device buffers: a query's prediction does not depend on which, nor on its neighbours."""
+    import paper_1107_4650_gb300 as D
+    q, _ = _data(6000, 3)
+    h = D.dirac_surrogate_create(LO, HI, seed=11, max_batch=8192)
+    try:
+        whole = D.dirac_surrogate_predict(h, q)
+        assert np.array_equal(D.dirac_surrogate_predict(h, q[:n]), whole[:n])
+        assert np.array_equal(D.dirac_surrogate_predict(h, q[6000 - n:]), whole[6000 - n:])
+    finally:
+        D.dirac_surrogate_destroy(h)
