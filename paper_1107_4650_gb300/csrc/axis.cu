@@ -34,7 +34,7 @@ cudaError_t launch_axis_cellfield(const AxisArgs &a, int precision, int blocks, 
 
 cudaError_t launch_axis(const void *in, void *out, const void *table, int64_t nx, int64_t ny, int64_t nz, int axis,
                         int64_t shift, int periodic, int full_table, int phase, int64_t flux_face, double fscale,
-                        double vol, double *flux_part, double *flux_cum, unsigned *ticket, const double *ucoef,
+                        double *flux_part, const double *ucoef,
                         int64_t ucoef_n, int64_t step0, int precision, int rshift, int blocks, cudaStream_t s) {
     AxisArgs a{};
     a.rshift = rshift;
@@ -52,10 +52,7 @@ cudaError_t launch_axis(const void *in, void *out, const void *table, int64_t nx
     a.full_table = full_table;
     a.flux_face = axis == 0 ? flux_face : -1;
     a.fscale = fscale;
-    a.vol = vol;
     a.flux_part = flux_part;
-    a.flux_cum = flux_cum;
-    a.ticket = ticket;
     if (precision == 1) return launch_axis_t<float>(a, axis, phase, blocks, s);
     if (precision == 2) return launch_axis_t<long long>(a, axis, phase, blocks, s);
     return launch_axis_t<double>(a, axis, phase, blocks, s);

@@ -13,7 +13,7 @@
 // threads, neighbouring rows, planes a few MB apart), so HBM sees about one read and one write per cell.
 // Face flux (x sweeps): threads whose cell lies in [face - shift, face) add |u14|^2 + |u23|^2 of the state
 // entering the sweep, those in [face, face + shift) subtract |w14|^2 + |w23|^2; the block's sum times
-// `fscale` (1/2 over the square of the state's scale) is its part, and the last block folds the parts.
+// `fscale` (1/2 over the square of the state's scale) is its part.
 #pragma once
 
 #include "step_kernels.cuh"
@@ -181,30 +181,18 @@ __global__ void __launch_bounds__(256) axis_kernel(const AxisArgs a) {
         store_pt(out + c * 8, o);
     }
     if (AXIS == 0 && a.flux_face >= 0) {
-        // block part in a fixed order (warp xor tree, then warps in index order), then the last-block fold
+        // block part in a fixed order (warp xor tree, then warps in index order)
         __shared__ double wpart[8];
+        if (__any_sync(0xffffffffu, facc != 0.0)) {  // (a tree over zeros gives zero)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) facc = __dadd_rn(facc, __shfl_xor_sync(0xffffffffu, facc, o));
+            for (int o = 16; o > 0; o >>= 1) facc = __dadd_rn(facc, __shfl_xor_sync(0xffffffffu, facc, o));
+        }
         if ((threadIdx.x & 31) == 0) wpart[threadIdx.x >> 5] = facc;
         __syncthreads();
         if (threadIdx.x == 0) {
             double b = 0.0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b = __dadd_rn(b, wpart[w]);
             a.flux_part[blockIdx.x] = __dmul_rn(a.fscale, b);
-        }
-        __shared__ unsigned s_last;
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) s_last = (atomicAdd(a.ticket, 1u) == gridDim.x - 1) ? 1u : 0u;
-        __syncthreads();
-        if (s_last && threadIdx.x < 32) {
-            __threadfence();
-            const double f = fold_parts(a.flux_part, gridDim.x, threadIdx.x);
-            if (threadIdx.x == 0) {
-                *a.flux_cum = __dadd_rn(__ldcg(a.flux_cum), __dmul_rn(f, a.vol));
-                __threadfence();
-                *a.ticket = 0u;
-            }
         }
     }
 }

@@ -40,6 +40,12 @@ cudaError_t launch_batch(const BatchArgs &b, int fp32, int K, int P, int blocks,
     return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_batch_flux_fold(const BatchFluxFold &f, cudaStream_t s) {
+    if (f.count <= 0 || f.n_active[0] <= 0) return cudaSuccess;
+    batch_flux_fold_kernel<<<(f.n_active[0] + 3) / 4, 128, 0, s>>>(f);
+    return cudaGetLastError();
+}
+
 cudaError_t batch_occupancy(int fp32, int K, int P, int *blocks_per_sm) {
 #define X(T, k, p) if ((fp32 != 0) == (sizeof(T) == 4) && K == k && P == p) return occupancy_t<T, k, p>(blocks_per_sm);
     DIRAC_BATCH_CASES(X)

@@ -42,6 +42,7 @@ struct dirac_batch {
     void *table_pool = nullptr;
     double *flux_part_pool = nullptr;
     size_t flux_part_n = 0;
+    int64_t flux_stride = 0;   // doubles of one launch's partials, all runs
     double *flux_cum = nullptr;
     double *norm0 = nullptr;
     double *norm_partial = nullptr;
@@ -51,7 +52,7 @@ struct dirac_batch {
     double *d_init = nullptr;  // x0, k0, width, C per run
     int64_t *d_absorb = nullptr;
     std::vector<std::vector<double>> mask;  // absorbing-layer factors per run (side values)
-    unsigned *counters = nullptr;  // counter, ticket, err, pad
+    unsigned *counters = nullptr;  // two task counters, err, pad
     int *d_order_main = nullptr, *d_order_rem = nullptr;
     int64_t *d_off_main = nullptr, *d_off_rem = nullptr;
     std::vector<int> nact_main, nact_rem;
@@ -110,9 +111,11 @@ dirac_status plan(dirac_batch *b) {
         R.nsegs = (R.side + R.seg_h - 1) / R.seg_h;
         R.parity_base = b->runs[r].nsteps / b->K;
     }
-    // flux partials: K x nsegs per run
+    // flux partials: K x nsegs per run, for kBatchSlots launches between folds
     size_t need = 0;
     for (int r = 0; r < n; ++r) need += (size_t)b->K * b->hrun[r].nsegs;
+    b->flux_stride = (int64_t)need;
+    need *= kBatchSlots;
     if (need > b->flux_part_n) {
         if (b->flux_part_pool) {
             cudaFree(b->flux_part_pool);
@@ -205,30 +208,58 @@ dirac_status enqueue_schedule(dirac_batch *b, cudaStream_t s, int64_t max_main =
     BatchArgs a{};
     a.runs = b->drun;
     a.counter = b->counters;
-    a.ticket = b->counters + 1;
     a.err = b->counters + 2;
-    a.vol = b->cfg.dx * b->cfg.dx;
+    BCK(b, cudaMemsetAsync(b->counters, 0, 2 * sizeof(unsigned), s));
+    BatchFluxFold f{};
+    f.runs = b->drun;
+    f.stride = b->flux_stride;
+    f.vol = b->cfg.dx * b->cfg.dx;
+    auto fold = [&]() -> dirac_status {
+        if (f.count > 0) {
+            BCK(b, launch_batch_flux_fold(f, s));
+            b->launches++;
+        }
+        f.count = 0;
+        return DIRAC_OK;
+    };
+    auto launch = [&](int K) -> dirac_status {
+        a.flux_off = f.count * b->flux_stride;
+        f.n_active[f.count++] = a.n_active;
+        BCK(b, launch_batch(a, b->fp32, K, b->P, b->blocks, s));
+        b->launches++;
+        a.turn ^= 1;
+        return f.count == kBatchSlots ? fold() : DIRAC_OK;
+    };
     const int64_t Lm = (max_main >= 0) ? std::min<int64_t>(max_main, b->nact_main.size()) : (int64_t)b->nact_main.size();
-    for (int64_t l = 0; l < Lm; ++l) {
-        a.order = b->d_order_main;
-        a.task_off = b->d_off_main;
+    a.order = f.order = b->d_order_main;
+    a.task_off = b->d_off_main;
+    a.parity_mode = 0;
+    f.K = b->K;
+    dirac_status st = DIRAC_OK;
+    for (int64_t l = 0; l < Lm && st == DIRAC_OK; ++l) {
         a.n_active = b->nact_main[l];
-        a.parity_mode = 0;
         a.launch = l;
-        BCK(b, launch_batch(a, b->fp32, b->K, b->P, b->blocks, s));
-        b->launches++;
+        st = launch(b->K);
     }
-    if (max_main >= 0) return DIRAC_OK;
-    for (size_t j = 0; j < b->nact_rem.size(); ++j) {
-        a.order = b->d_order_rem;
-        a.task_off = b->d_off_rem;
+    if (st == DIRAC_OK) st = fold();
+    if (max_main >= 0 || st != DIRAC_OK) return st;
+    a.order = f.order = b->d_order_rem;
+    a.task_off = b->d_off_rem;
+    a.parity_mode = 1;
+    f.K = 1;
+    for (size_t j = 0; j < b->nact_rem.size() && st == DIRAC_OK; ++j) {
         a.n_active = b->nact_rem[j];
-        a.parity_mode = 1;
         a.launch = (int64_t)j;
-        BCK(b, launch_batch(a, b->fp32, 1, b->P, b->blocks, s));
-        b->launches++;
+        st = launch(1);
     }
-    return DIRAC_OK;
+    return st == DIRAC_OK ? fold() : st;
+}
+
+// Kernels of one whole schedule: the step launches and their flux folds.
+int64_t run_launches(const dirac_batch *b) {
+    int64_t n = 0;
+    for (int64_t m : {(int64_t)b->nact_main.size(), (int64_t)b->nact_rem.size()}) n += m + (m + kBatchSlots - 1) / kBatchSlots;
+    return n;
 }
 
 dirac_status enqueue_norm(dirac_batch *b, cudaStream_t s) {
@@ -496,7 +527,7 @@ dirac_status dirac_batch_run(dirac_batch *b) {
             if (e != cudaSuccess) return bcuda(b, e, "cudaGraphInstantiate");
         }
         BCK(b, cudaGraphLaunch(b->graph, b->stream));
-        b->launches += (int64_t)b->nact_main.size() + (int64_t)b->nact_rem.size();
+        b->launches += run_launches(b);
     } else {
         st = enqueue_schedule(b, b->stream);
         if (st != DIRAC_OK) return st;
@@ -595,7 +626,7 @@ dirac_status dirac_batch_get_info(const dirac_batch *b, dirac_batch_info *info) 
     info->steps_per_launch = b->K;
     info->points_per_lane = b->P;
     info->segment_rows = b->seg_rows;
-    info->launches = (int64_t)b->nact_main.size() + (int64_t)b->nact_rem.size();
+    info->launches = run_launches(b);
     info->max_tasks = b->max_tasks;
     int64_t ps = 0;
     for (const auto &r : b->runs) ps += r.side * r.side * r.nsteps;

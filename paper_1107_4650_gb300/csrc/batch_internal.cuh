@@ -7,8 +7,10 @@ namespace dirac {
 struct BatchArgs;
 struct InitArgs;
 struct NormArgs;
+struct BatchFluxFold;
 bool batch_supported(int fp32, int K, int P);
 cudaError_t launch_batch(const BatchArgs &b, int fp32, int K, int P, int blocks, cudaStream_t s);
+cudaError_t launch_batch_flux_fold(const BatchFluxFold &f, cudaStream_t s);
 cudaError_t batch_occupancy(int fp32, int K, int P, int *blocks_per_sm);
 cudaError_t launch_batch_init(const InitArgs &ia, int fp32, cudaStream_t s);
 cudaError_t launch_batch_norm(const NormArgs &na, int64_t nchunks, const int64_t *chunk_off, int nruns, double vol,

@@ -5,8 +5,8 @@
 // cuts its grid; the tasks of all active runs form one list.  Resident warps take tasks from an
 // atomic counter until the list is exhausted (dynamic balance across runs of different sizes) and
 // run each task with the single-grid warp routine (sweep_warp), so the arithmetic, boundary and
-// flux handling are identical to dirac_step's.  The last block to finish folds every active run's
-// per-step face-flux partials into that run's cumulative flux (fixed order) and resets the counter.
+// flux handling are identical to dirac_step's.  After up to 16 launches a launch of its own folds the per-step
+// face-flux partials into the runs' cumulative fluxes (fixed order).
 //
 // Runs are ordered so that the active set of every launch is a prefix of an order array; the task
 // list's prefix offsets are precomputed per order, and a warp finds its run by binary search.
@@ -22,7 +22,7 @@ struct BatchRunDev {
     int64_t side;           // nx = nz = side
     int64_t face;           // flux face index
     int64_t nsegs, seg_h;   // row segments
-    double *flux_part;      // [K][nsegs]
+    double *flux_part;      // [slot][K][nsegs], slots flux_stride apart
     double *flux_cum;       // cumulative flux of this run
     int64_t parity_base;    // parity offset of the remainder phase (number of K-step launches)
 };
@@ -34,11 +34,40 @@ struct BatchArgs {
     int n_active;
     int parity_mode;        // 0: parity = launch & 1 (K-step phase); 1: (parity_base + launch) & 1
     int64_t launch;
-    unsigned *counter;      // task counter, 0 between launches
-    unsigned *ticket;       // block-completion ticket, 0 between launches
+    unsigned *counter;      // two task counters: a launch takes from [turn] and clears the other for the next one
+    int turn;
+    int64_t flux_off;       // this launch's slot of the flux partials
     unsigned *err;
-    double vol;
 };
+
+// The flux partials of `count` launches (slots 0 .. count - 1, slot i of the first n_active[i] runs of the order) into the
+// runs' cumulative fluxes, one warp per run, launch by launch and step by step (lane l adds segments l, l + 32, ..., then
+// an xor tree).
+constexpr int kBatchSlots = 16;
+struct BatchFluxFold {
+    const BatchRunDev *runs;
+    const int *order;
+    int count, K;
+    int64_t stride;
+    double vol;
+    int n_active[kBatchSlots];
+};
+static __global__ void batch_flux_fold_kernel(const __grid_constant__ BatchFluxFold f) {
+    const int lane = threadIdx.x & 31, i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (i >= f.n_active[0]) return;  // the active set only shrinks
+    const BatchRunDev &R = f.runs[f.order[i]];
+    double F = *R.flux_cum;
+    for (int l = 0; l < f.count && i < f.n_active[l]; ++l)
+        for (int s = 0; s < f.K; ++s) {
+            const double *part = R.flux_part + l * f.stride + s * R.nsegs;
+            double v = 0.0;
+            for (int64_t q = lane; q < R.nsegs; q += 32) v = __dadd_rn(v, part[q]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+            F = __dadd_rn(F, __dmul_rn(v, f.vol));
+        }
+    if (lane == 0) *R.flux_cum = F;
+}
 
 // FP32 with two points a lane and two or four steps a launch: the sweep history in shared memory and one row per
 // iteration (24 runs of sides 768 and 1024, four steps: 196 against 157 G point-steps/s with it in registers and two
@@ -54,9 +83,10 @@ __global__ void __launch_bounds__(128) batch_kernel(const BatchArgs b) {
     const int lane = threadIdx.x & 31;
     unsigned char *wsmem = dyn_smem + (threadIdx.x >> 5) * Ring<T, K, P, BatchHist<T, K, P>::value>::WARP_BYTES;
     const int64_t total = b.task_off[b.n_active];
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.counter[b.turn ^ 1] = 0u;  // nobody takes from it during this launch
     for (;;) {
         unsigned task = 0;
-        if (lane == 0) task = atomicAdd(b.counter, 1u);
+        if (lane == 0) task = atomicAdd(b.counter + b.turn, 1u);
         task = __shfl_sync(0xffffffffu, task, 0);
         if ((int64_t)task >= total) break;
         int lo = 0, hi = b.n_active;  // task_off[lo] <= task < task_off[hi]
@@ -78,41 +108,13 @@ __global__ void __launch_bounds__(128) batch_kernel(const BatchArgs b) {
         a.nsegs = R.nsegs;
         a.seg_h = R.seg_h;
         a.flux_face = R.face;
-        a.flux_part = R.flux_part;
-        a.flux_cum = R.flux_cum;
-        a.ticket = nullptr;
+        a.flux_part = R.flux_part + b.flux_off;
         a.err = b.err;
-        a.vol = b.vol;
         a.periodic = 0;
         a.full_table = 0;
         a.flux_unit = 1.0;  // floating-point states
         a.wide = 1;         // the pool is the library's own, a cell 32 or 64 bytes
         sweep_warp<T, K, P, 0, false, BatchHist<T, K, P>::unroll, BatchHist<T, K, P>::value>(a, (int64_t)task - b.task_off[lo], lane, wsmem);
-    }
-    // last block folds the flux partials of every active run and resets the counters
-    __shared__ unsigned s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(b.ticket, 1u) == gridDim.x - 1) ? 1u : 0u;
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        for (int i = threadIdx.x; i < b.n_active; i += blockDim.x) {
-            const BatchRunDev &R = b.runs[b.order[i]];
-            double F = __ldcg(R.flux_cum);
-            for (int s = 0; s < K; ++s) {
-                double f = 0.0;
-                for (int64_t q = 0; q < R.nsegs; ++q) f = __dadd_rn(f, __ldcg(R.flux_part + s * R.nsegs + q));
-                F = __dadd_rn(F, __dmul_rn(f, b.vol));
-            }
-            *R.flux_cum = F;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            *b.counter = 0u;
-            *b.ticket = 0u;
-        }
     }
 }
 

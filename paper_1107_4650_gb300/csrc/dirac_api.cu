@@ -62,8 +62,10 @@ struct dirac_grid {
     int table_full = 0;
     double *flux_part = nullptr;
     size_t flux_part_cap = 0;  // doubles
+    size_t flux_used = 0;      // doubles of it that launches since the last fold write
+    FluxFold flux{};           // and their places; empty between calls of dirac_step
     double *flux_dev = nullptr;
-    unsigned *ticket = nullptr;
+    unsigned *ticket = nullptr;  // [1]: set by a step kernel whose bounded wait ran out
     std::vector<double> absorb;      // per-x-column damping factors (empty: none)
     std::vector<double> v_host;      // last potential set (for rebuilding the table)
     int v_layout = DIRAC_V_NONE;
@@ -87,6 +89,7 @@ struct dirac_grid {
     int sm_count = 0;
     Plan plan;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    int64_t graph_launches[2] = {0, 0};  // kernels in each
     int64_t launches = 0;
     size_t device_bytes = 0;
     std::string err;
@@ -430,6 +433,8 @@ dirac_status ensure_flux_part(dirac_grid *g) {
             const Plan::XY &q = g->plan.s3_xy[nh - 1];
             need = std::max(need, (size_t)(2 * nh * q.nzsegs * q.nytiles * g->plan.s3_warps));
         }
+    // room for 32 launches between folds, within 4 MB (a launch that leaves more is folded by itself)
+    need = std::max(need, std::min<size_t>(32 * need, (size_t)1 << 19));
     if (need <= g->flux_part_cap) return DIRAC_OK;
     if (g->flux_part) {
         cudaFree(g->flux_part);
@@ -439,6 +444,39 @@ dirac_status ensure_flux_part(dirac_grid *g) {
     CK(g, cudaMalloc(&g->flux_part, need * sizeof(double)));
     g->flux_part_cap = need;
     g->device_bytes += need * sizeof(double);
+    return DIRAC_OK;
+}
+
+// Folds what the launches since the last fold have left.
+dirac_status fold_flux(dirac_grid *g, cudaStream_t s) {
+    if (g->flux.count == 0) return DIRAC_OK;
+    g->flux.part = g->flux_part;
+    g->flux.flux_cum = g->flux_dev;
+    g->flux.vol = cell_volume(g);
+    cudaError_t e = launch_flux_fold(g->flux, s);
+    g->flux.count = 0;
+    g->flux_used = 0;
+    if (e != cudaSuccess) return cuda_fail(g, e, "flux fold launch");
+    g->launches++;
+    return DIRAC_OK;
+}
+
+// A place for the flux partials of the next launch: `sums` sums (steps or x sweeps, in order) of n partials each.
+dirac_status flux_place(dirac_grid *g, int sums, int64_t n, cudaStream_t s, double **part) {
+    *part = g->flux_part;
+    if (g->cfg.flux_face < 0) return DIRAC_OK;
+    const size_t need = (size_t)sums * (size_t)n;
+    if (g->flux.count + sums > kFluxEntries || g->flux_used + need > g->flux_part_cap) {
+        dirac_status st = fold_flux(g, s);
+        if (st != DIRAC_OK) return st;
+    }
+    if (need > g->flux_part_cap) return fail(g, DIRAC_ERR_STATE, "flux scratch too small");
+    *part = g->flux_part + g->flux_used;
+    for (int i = 0; i < sums; ++i) {
+        g->flux.off[g->flux.count] = (unsigned)(g->flux_used + (size_t)i * n);
+        g->flux.n[g->flux.count++] = (unsigned)n;
+    }
+    g->flux_used += need;
     return DIRAC_OK;
 }
 
@@ -466,11 +504,7 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
     a.nsegs = p.nsegs;
     a.seg_h = p.seg_h;
     a.flux_face = flux ? g->cfg.flux_face : -1;
-    a.flux_part = g->flux_part;
-    a.flux_cum = g->flux_dev;
-    a.ticket = g->ticket;
     a.err = g->ticket + 1;
-    a.vol = cell_volume(g);
     a.periodic = g->cfg.boundary == DIRAC_BC_PERIODIC;
     a.full_table = g->table_full;
     a.ucoef = g->ucoef;
@@ -506,10 +540,14 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
                 ++q;  // sweep 4 is done too
                 continue;
             }
+            if (ax == 0) {
+                dirac_status st = flux_place(g, 1, blocks, s, &a.flux_part);
+                if (st != DIRAC_OK) return st;
+            }
             cudaError_t e = launch_axis(g->psi[par], g->psi[par ^ 1], g->table, g->cfg.n[0], g->cfg.n[1], g->cfg.n[2], ax,
                                         ax == 0 ? K : 2 * K, a.periodic, g->table_full, q == 3 ? 1 : 0,
                                         ax == 0 ? a.flux_face : -1, (g->fx ? fscale_fx[q] : fscale[q]) * a.flux_unit,
-                                        a.vol, g->flux_part, g->flux_dev, g->ticket, q == 3 ? a.ucoef : nullptr,
+                                        a.flux_part, q == 3 ? a.ucoef : nullptr,
                                         q == 3 ? a.ucoef_n : 0, step0,
                                         g->fx ? DIRAC_FX64 : (g->fp32 ? DIRAC_FP32 : DIRAC_FP64),
                                         (g->fx && q == 7) ? 4 : 0, blocks, s);
@@ -568,9 +606,13 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
                 z.fscale_phase = scale_of(g);
                 e = launch_axis_cellfield(z, prec, blocks, s);
             } else {
+                if (w.axis == 0) {
+                    dirac_status st = flux_place(g, 1, blocks, s, &a.flux_part);
+                    if (st != DIRAC_OK) return st;
+                }
                 e = launch_axis(g->psi[par], g->psi[par ^ 1], g->table, g->cfg.n[0], g->cfg.n[1], g->cfg.n[2], w.axis,
-                                sh, a.periodic, g->table_full, 0, w.axis == 0 ? a.flux_face : -1, w.fscale, a.vol,
-                                g->flux_part, g->flux_dev, g->ticket, nullptr, 0, step0, prec, 0, blocks, s);
+                                sh, a.periodic, g->table_full, 0, w.axis == 0 ? a.flux_face : -1, w.fscale,
+                                a.flux_part, nullptr, 0, step0, prec, 0, blocks, s);
             }
             if (e != cudaSuccess) return cuda_fail(g, e, "cell-field sweep launch");
             g->launches++;
@@ -595,10 +637,14 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
         int par = parity;
         for (int q = 0; q < nseq; ++q) {
             const Sw &w = seq[q];
+            if (w.axis == 0) {
+                dirac_status st = flux_place(g, 1, blocks, s, &a.flux_part);
+                if (st != DIRAC_OK) return st;
+            }
             cudaError_t e = launch_axis(g->psi[par], g->psi[par ^ 1], g->table, g->cfg.n[0], g->cfg.n[1], g->cfg.n[2],
                                         w.axis, char_shift(g), a.periodic, g->table_full, w.phase,
-                                        w.axis == 0 ? a.flux_face : -1, w.fscale, a.vol, g->flux_part, g->flux_dev,
-                                        g->ticket, w.phase ? a.ucoef : nullptr, w.phase ? a.ucoef_n : 0, step0,
+                                        w.axis == 0 ? a.flux_face : -1, w.fscale, a.flux_part,
+                                        w.phase ? a.ucoef : nullptr, w.phase ? a.ucoef_n : 0, step0,
                                         g->fp32 ? DIRAC_FP32 : DIRAC_FP64, 0, blocks, s);
             if (e != cudaSuccess) return cuda_fail(g, e, "characteristic-shift sweep launch");
             g->launches++;
@@ -611,10 +657,14 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
         a.nplanes = 1;
         if (K == 2) {
             a.nsegs = p.f2_nzsegs * p.f2_nytiles * p.f2_warps;  // flux parts per step of the fused pass
+            dirac_status st = flux_place(g, 2, a.nsegs, s, &a.flux_part);
+            if (st != DIRAC_OK) return st;
             e = launch_fused3d(a, g->fx ? 2 : g->fp32, p.f2_warps, 2, g->cfg.n[1], g->cfg.n[2], p.f2_nstrips, p.f2_nytiles,
                                p.f2_nzsegs, p.f2_zseg_h, s);
         } else {
             a.nsegs = p.f_nzsegs * p.f_nytiles * p.f_warps;  // flux parts of the fused pass
+            dirac_status st = flux_place(g, 1, a.nsegs, s, &a.flux_part);
+            if (st != DIRAC_OK) return st;
             e = launch_fused3d(a, g->fx ? 2 : g->fp32, p.f_warps, 1, g->cfg.n[1], g->cfg.n[2], p.f_nstrips, p.f_nytiles,
                                p.f_nzsegs, p.f_zseg_h, s);
         }
@@ -622,6 +672,8 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
         g->launches++;
         return DIRAC_OK;
     }
+    dirac_status st = flux_place(g, mode == 4 ? 1 : levels(g, K), a.nsegs * planes, s, &a.flux_part);
+    if (st != DIRAC_OK) return st;
     cudaError_t e = mode == 4 ? launch_shift(a, g->fp32, char_shift(g), p.P, p.wpb, s)
                     : g->fx   ? launch_sweep_fx(a, mode, K, p.P, p.wpb, s)
                     : g->fp32 ? launch_sweep_f32(a, mode, K, p.P, p.wpb, s)
@@ -671,11 +723,7 @@ dirac_status enqueue_strang3d_run(dirac_grid *g, int parity, int64_t m, cudaStre
     a.nx = g->cfg.n[0];
     a.nplanes = 1;
     a.flux_face = flux ? g->cfg.flux_face : -1;
-    a.flux_part = g->flux_part;
-    a.flux_cum = g->flux_dev;
-    a.ticket = g->ticket;
     a.err = g->ticket + 1;
-    a.vol = cell_volume(g);
     a.periodic = g->cfg.boundary == DIRAC_BC_PERIODIC;
     const double *ucoef = field_on(g) ? g->ucoef : nullptr;
     const int64_t ucoef_n = (int64_t)(g->avec.size() / 3);
@@ -687,6 +735,8 @@ dirac_status enqueue_strang3d_run(dirac_grid *g, int parity, int64_t m, cudaStre
         a.out = g->psi[par ^ 1];
         a.wide = wide_state(g);
         a.nsegs = q.nzsegs * q.nytiles * p.s3_warps;  // flux parts per x sweep
+        dirac_status st = flux_place(g, 2 * nh, a.nsegs, s, &a.flux_part);
+        if (st != DIRAC_OK) return st;
         double fsu[4];
         for (int i = 0; i < 4; ++i) fsu[i] = fs[i] * funit;
         const int rmid = (g->fx && nh == 2) ? 4 : 0, rend = (g->fx && ends_step) ? 4 : 0;
@@ -735,8 +785,10 @@ dirac_status get_graph(dirac_grid *g, int parity, cudaGraphExec_t *out) {
             par ^= block_flips(g);
         }
     }
+    if (st == DIRAC_OK) st = fold_flux(g, g->cap_stream);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(g->cap_stream, &graph);
+    g->graph_launches[parity] = g->launches - l0;
     g->launches = l0;  // captured, not launched
     if (st != DIRAC_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -752,14 +804,9 @@ dirac_status get_graph(dirac_grid *g, int parity, cudaGraphExec_t *out) {
     return DIRAC_OK;
 }
 
-int64_t launches_per_block(const dirac_grid *g) {
-    if (sweep_mode(g) == 6) return strang3d_zpass(g) ? 7 : 8;
-    if (sweep_mode(g) == 7) return ndim_of(g) == 3 ? 3 : 4;
-    if (sweep_mode(g) == 8) return strang(g) ? (ndim_of(g) == 3 ? 8 : 4) : (ndim_of(g) == 3 ? 3 : 2);
-    return 1 + ((ndim_of(g) == 3 && !fused_pass(g)) ? 1 : 0);
-}
-
 dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
+    g->flux.count = 0;  // nothing is left over but by a call that failed
+    g->flux_used = 0;
     const int K = (ndim_of(g) == 3) ? (fused_pass(g) ? g->plan.K : 1) : g->plan.K;
     int64_t blocks = nsteps / K;
     int64_t rem = nsteps % K;
@@ -779,7 +826,7 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
                 dirac_status st = get_graph(g, g->cur, &ex);
                 if (st != DIRAC_OK) return st;
                 CK(g, cudaGraphLaunch(ex, g->stream));
-                g->launches += 2 * kGraphBlocks + 1;
+                g->launches += g->graph_launches[g->cur];
                 g->cur ^= 1;
                 left -= kGraphBlocks;
                 t += kGraphBlocks;
@@ -790,7 +837,7 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
             g->cur ^= 1;
         }
         g->step += nsteps;
-        return DIRAC_OK;
+        return fold_flux(g, g->stream);
     }
     // launches with a field take their step index as an argument: no graph replay
     if (g->cfg.use_graphs && !field && blocks >= kGraphBlocks) {
@@ -799,7 +846,7 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
             dirac_status st = get_graph(g, g->cur, &ex);
             if (st != DIRAC_OK) return st;
             CK(g, cudaGraphLaunch(ex, g->stream));
-            g->launches += kGraphBlocks * launches_per_block(g);
+            g->launches += g->graph_launches[g->cur];
             blocks -= kGraphBlocks;
             // kGraphBlocks is even: parity unchanged
         }
@@ -817,7 +864,7 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
         t += 1;
     }
     g->step += nsteps;
-    return DIRAC_OK;
+    return fold_flux(g, g->stream);
 }
 
 void release(dirac_grid *g) {

@@ -26,11 +26,8 @@ struct SweepArgs {
     int64_t nx, nr, nplanes;
     int64_t strip_w, nstrips, nsegs, seg_h;
     int64_t flux_face;     // x face index or -1
-    double *flux_part;     // [K][nplanes*nsegs] per-step face-flux partial sums (unscaled)
-    double *flux_cum;      // cumulative flux; the last block of a launch adds vol * (sum of each step)
-    unsigned *ticket;      // block-completion counter, 0 between launches (the last block resets it)
+    double *flux_part;     // [K][nplanes*nsegs] per-step face-flux partial sums (unscaled), folded by launch_flux_fold
     unsigned *err;         // set non-zero by a kernel whose bounded wait ran out
-    double vol;            // cell volume dx^d
     int periodic;
     int full_table;
     // mode 3 (uniform vector potential): per-step entries of U (Sec. 2.3) as 6 complex values
@@ -70,10 +67,7 @@ struct AxisArgs {
     int full_table;
     int64_t flux_face;   // x sweeps: face index, or -1
     double fscale;       // multiplies the summed |.|^2 of the face cells
-    double vol;          // cell volume
     double *flux_part;   // [gridDim.x]
-    double *flux_cum;
-    unsigned *ticket;
     // uniform vector potential (phase epilogue only): 12 doubles of U entries per step, this launch's step
     const double *ucoef;
     int64_t ucoef_n, step0;
@@ -119,6 +113,18 @@ struct ObsArgs {
 // precision: DIRAC_FP64, DIRAC_FP32 or DIRAC_FX64 (the state then is int64 q, psi = q * a.scale)
 cudaError_t launch_observables(const ObsArgs &a, int precision, int nblocks, cudaStream_t s);
 
+// Folds flux partials into the cumulative flux, in order: for each entry, *flux_cum += vol * (sum of its n partials from
+// part + off).  One launch of one block.
+constexpr int kFluxEntries = 128;
+struct FluxFold {
+    const double *part;
+    double *flux_cum;
+    double vol;
+    int count;
+    unsigned off[kFluxEntries], n[kFluxEntries];
+};
+cudaError_t launch_flux_fold(const FluxFold &f, cudaStream_t s);
+
 // Instantiated (K, P) pairs of the sweep kernels.
 bool sweep_supported(int fp32, int mode, int K, int P);
 
@@ -135,7 +141,7 @@ bool shift_supported(int S, int P);
 // output by 2^rshift with rounding to nearest, halves up).
 cudaError_t launch_axis(const void *in, void *out, const void *table, int64_t nx, int64_t ny, int64_t nz, int axis,
                         int64_t shift, int periodic, int full_table, int phase, int64_t flux_face, double fscale,
-                        double vol, double *flux_part, double *flux_cum, unsigned *ticket, const double *ucoef,
+                        double *flux_part, const double *ucoef,
                         int64_t ucoef_n, int64_t step0, int precision, int rshift, int blocks, cudaStream_t s);
 
 // Fused 3-D step (x, y, z sweeps and phase in one pass, `steps` = 1 or 2 steps per launch): blocks of

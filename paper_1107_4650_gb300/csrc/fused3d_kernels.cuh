@@ -218,11 +218,9 @@ __global__ void __launch_bounds__(32 * W, Fused3DMinBlocks<T, W>::value) fused3d
     }
     if (face >= 0 && face >= x_own0 && face < x_own1) {
         // one flux part per (y tile, z segment, warp) of the strip that owns the face; halo warps write 0
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) facc = __dadd_rn(facc, __shfl_xor_sync(0xffffffffu, facc, o));
+        facc = face_lanes_sum(facc, face, x_own0 - 1);
         if (lane == 0) a.flux_part[(zseg * A.nytiles + ytile) * W + w] = __dmul_rn(0.5 * a.flux_unit, facc);
     }
-    if (face >= 0) finish_flux<1>(a);
 }
 
 // Two first-order steps per pass (temporal block k = 2): HBM is read and written once per two steps.
@@ -427,13 +425,10 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A
         const int64_t q = (zseg * A.nytiles + ytile) * W + w;
 #pragma unroll
         for (int st = 0; st < 2; ++st) {
-            double f = facc[st];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) f = __dadd_rn(f, __shfl_xor_sync(0xffffffffu, f, o));
+            const double f = face_lanes_sum(facc[st], face, x_own0 - 2);
             if (lane == 0) a.flux_part[st * nparts + q] = __dmul_rn(0.5, f);
         }
     }
-    if (face >= 0) finish_flux<2>(a);
 }
 
 template <typename T, int W, bool FIELD>

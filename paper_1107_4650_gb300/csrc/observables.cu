@@ -87,6 +87,27 @@ __global__ void __launch_bounds__(OBS_THREADS) obs_final_kernel(const double *pa
         for (int k = 0; k < 5; ++k) out[k] = v[k];
 }
 
+// Flux partials of up to kFluxEntries launches' steps into the cumulative flux, in order (FluxFold): warp w sums entry
+// w, w + 32, ... (lane l adds partials l, l + 32, ..., then an xor tree), thread 0 adds vol times each to the total.
+__global__ void __launch_bounds__(1024) flux_fold_kernel(const __grid_constant__ FluxFold f) {
+    __shared__ double sum[kFluxEntries];
+    const int lane = threadIdx.x & 31;
+    for (int e = threadIdx.x >> 5; e < f.count; e += 32) {
+        const double *part = f.part + f.off[e];
+        double v = 0.0;
+        for (unsigned q = lane; q < f.n[e]; q += 32) v = __dadd_rn(v, part[q]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if (lane == 0) sum[e] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double F = *f.flux_cum;
+        for (int e = 0; e < f.count; ++e) F = __dadd_rn(F, __dmul_rn(sum[e], f.vol));
+        *f.flux_cum = F;
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_observables(const ObsArgs &a, int precision, int nblocks, cudaStream_t s) {
@@ -99,6 +120,11 @@ cudaError_t launch_observables(const ObsArgs &a, int precision, int nblocks, cud
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     obs_final_kernel<<<1, OBS_THREADS, 0, s>>>(a.partial, nblocks, a.out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_flux_fold(const FluxFold &f, cudaStream_t s) {
+    flux_fold_kernel<<<1, 1024, 0, s>>>(f);
     return cudaGetLastError();
 }
 

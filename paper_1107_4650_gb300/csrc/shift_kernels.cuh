@@ -214,7 +214,6 @@ __global__ void __launch_bounds__(128) shift_kernel(const SweepArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid < a.nstrips * a.nsegs) shift_warp<T, S, P, FIELD>(a, wid, lane);
-    if (a.flux_face >= 0) finish_flux<1>(a);
 }
 
 template <typename T, int S, int P>

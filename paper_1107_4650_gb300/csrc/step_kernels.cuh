@@ -352,8 +352,6 @@ template <typename T, int K, int P, int MODE, bool PER> struct HistSmem {
 };
 template <typename T, int K, int P, int MODE, bool PER, int UNR = RowUnroll<T, K, MODE>::value, bool HS = false>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem);
-template <int K>
-__device__ __forceinline__ void finish_flux(const SweepArgs &a);
 template <typename T, int K, int P, bool HS = false> struct Ring;
 
 // Pipelined levels of one launch: K steps, or 2K levels for the second-order splitting (mode 2).
@@ -389,44 +387,11 @@ __global__ void __launch_bounds__(128, SweepMinBlocks<T, K, P, MODE>::value) swe
     if (wid < per_plane * a.nplanes) sweep_warp<T, K, P, MODE, PER, RowUnroll<T, K, MODE>::value, HS>(a, wid, lane, wsmem);
 }
 
-// Sum of n flux partials in an order fixed by n: lane l adds parts l, l + 32, ..., a xor tree adds the lanes (the
-// result is the same in every lane).
-__device__ __forceinline__ double fold_parts(const double *part, int64_t n, int lane) {
-    double f = 0.0;
-    for (int64_t q = lane; q < n; q += 32) f = __dadd_rn(f, __ldcg(part + q));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) f = __dadd_rn(f, __shfl_xor_sync(0xffffffffu, f, o));
-    return f;
-}
-
-// One warp adds vol * (sum of each of the K steps' partials) to the cumulative flux and resets the ticket.
-__device__ __forceinline__ void fold_flux(const SweepArgs &a, int K, int lane) {
-    __threadfence();
-    const int64_t nparts = a.nsegs * a.nplanes;
-    double F = __ldcg(a.flux_cum);
-    for (int s = 0; s < K; ++s) F = __dadd_rn(F, __dmul_rn(fold_parts(a.flux_part + s * nparts, nparts, lane), a.vol));
-    if (lane == 0) {
-        *a.flux_cum = F;
-        __threadfence();
-        *a.ticket = 0u;
-    }
-}
-
-// Last-block fold of the flux partials: every block takes a ticket after its partials are visible; the first warp
-// of the block that takes the last one folds them.  No block waits.  The lanes load and add the partials side by
-// side: a launch leaves up to a few thousand of them, and one thread adding them one after the other (a load and a
-// dependent FP64 add each) kept the launch open at its end.  Measured at 256^3, one thread against one warp: FP32
-// second order 1522 -> 711 us a step, FP32 first order 423 -> 311, fixed-point second order 2644 -> 1851, FP64
-// first order 2898 -> 2771; FP32 2-D at 2048^2 36.9 -> 34.2.
-template <int K>
-__device__ __forceinline__ void finish_flux(const SweepArgs &a) {
-    __shared__ unsigned s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(a.ticket, 1u) == gridDim.x - 1) ? 1u : 0u;
-    __syncthreads();
-    if (s_last && threadIdx.x < 32) fold_flux(a, K, threadIdx.x);
-}
+// Face flux: a launch leaves one partial sum per step (or x sweep) and warp, block or segment that owns the face; they are
+// folded into the cumulative flux by a launch of its own after up to 32 of them (flux_fold_kernel, observables.cu), not
+// by each launch's last block.  That fold, with the fence and the ticket that find the last block, was half of a small
+// grid's launch: 128^2 FP32 5.8 us a step, 4.2 so, 2.9 without a face; 256^2 FP64 14.9 and 12.2, 64^3 FP32 second order
+// 46 and 30.
 
 // ---- TMA bulk-copy row ring (per warp).  Lane 0 issues one cp.async.bulk per row into a ring slot,
 // armed with mbarrier expect_tx; every lane waits on the slot's mbarrier phase before reading it.
@@ -547,33 +512,51 @@ __device__ __forceinline__ void x_characteristics(const Cx<T> (*s)[4], int lane,
     }
 }
 
-// One row of the face flux: the face lane's 8 values go to lane (row % 32) of the hand-off area; at every 32nd
-// row (or the segment's last) all lanes fold their rows: scale (|u14|^2 + |u23|^2) - scale (|w14|^2 + |w23|^2),
-// scale = 1/2 for a state at its true size, 2 for one held at half size.
+// The sum over a warp of values that are zero but on the lanes of cells face - 1 and face (cells consecutive in the lanes,
+// lane 0 holding cell x0): the two of them added, the same value as any tree over all lanes gives, in every lane.
+__device__ __forceinline__ double face_lanes_sum(double v, int64_t face, int64_t x0) {
+    const int l = (int)(face - x0);
+    const double a = __shfl_sync(0xffffffffu, v, l - 1), b = __shfl_sync(0xffffffffu, v, l);
+    return __dadd_rn(a, b);
+}
+
+// One row of the face flux: the face lane leaves the row's 8 values at place (row % 32) of the hand-off area; at every
+// 32nd row (or the segment's last) all lanes fold their rows: scale (|u14|^2 + |u23|^2) - scale (|w14|^2 + |w23|^2),
+// scale = 1/2 for a state at its true size, 2 for one held at half size.  The face's warps run as long as the launch does
+// when it is one wave, so what a row costs them counts whole: handing the values over by eight shuffles a row the launch
+// took 29.6 us a step against 23.3 without a face (FP32 k = 2 at 2048^2; second order 52.2 against 37.9), this way and
+// with the fold apart 25.3 (44.2).
 template <typename T, int P>
 __device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, const Cx<T> *w14, const Cx<T> *w23,
                                          int face_j, int face_lane, int lane, int64_t row_in_seg, bool last_row, T *g,
                                          double scale, double &facc) {
-    T v[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-        if (j == face_j) {
-            v[0] = lu14[j].re; v[1] = lu14[j].im; v[2] = lu23[j].re; v[3] = lu23[j].im;
-            v[4] = w14[j].re;  v[5] = w14[j].im;  v[6] = w23[j].re;  v[7] = w23[j].im;
-        }
-    }
     const int t = (int)(row_in_seg & 31);
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const T x = __shfl_sync(0xffffffffu, v[k], face_lane);
-        if (lane == t) g[k * 32 + t] = x;
+        for (int j = 0; j < P; ++j) {
+            const Cx<T> v[4] = {lu14[j], lu23[j], w14[j], w23[j]};
+            if (lane == face_lane && j == face_j) store_pt(g + t * 8, v);
+        }
+    } else if (lane == face_lane) {  // one branch: a store for each point costs registers (fixed point 112.6 against 107.3 us)
+        Cx<T> v[4] = {lu14[0], lu23[0], w14[0], w23[0]};
+#pragma unroll
+        for (int j = 1; j < P; ++j) {
+            if (j == face_j) {
+                v[0] = lu14[j];
+                v[1] = lu23[j];
+                v[2] = w14[j];
+                v[3] = w23[j];
+            }
+        }
+        store_pt(g + t * 8, v);
     }
     if (t == 31 || last_row) {
         __syncwarp();
         if (lane <= t) {
-            const T *gl = g + lane;
-            const double right = __dmul_rn(scale, __dadd_rn(abs2d(Cx<T>{gl[0], gl[32]}), abs2d(Cx<T>{gl[64], gl[96]})));
-            const double left = __dmul_rn(scale, __dadd_rn(abs2d(Cx<T>{gl[128], gl[160]}), abs2d(Cx<T>{gl[192], gl[224]})));
+            Cx<T> v[4];
+            load_pt(g + lane * 8, v);
+            const double right = __dmul_rn(scale, __dadd_rn(abs2d(v[0]), abs2d(v[1])));
+            const double left = __dmul_rn(scale, __dadd_rn(abs2d(v[2]), abs2d(v[3])));
             facc = __dadd_rn(facc, __dsub_rn(right, left));
         }
         __syncwarp();
@@ -995,16 +978,6 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
             if (lane == 0) a.flux_part[(int64_t)s * a.nsegs * a.nplanes + plane * a.nsegs + seg] = v;
-        }
-        if (a.ticket) {
-            // single-grid launches: the face strip's warps count themselves (one per partial, also one whose wait ran
-            // out) and the last one folds; the other warps have nothing to report and end
-            unsigned t = 0;
-            if (lane == 0) {
-                __threadfence();
-                t = atomicAdd(a.ticket, 1u);
-            }
-            if (__shfl_sync(0xffffffffu, t, 0) == (unsigned)(a.nsegs * a.nplanes) - 1) fold_flux(a, L, lane);
         }
     }
 }

@@ -247,9 +247,7 @@ __device__ __forceinline__ void strang_xy_block(const StrangXYArgs &A, const int
         const int64_t qi = (zseg * A.nytiles + ytile) * W + w;
 #pragma unroll
         for (int s2 = 0; s2 < NS; ++s2) {
-            double f = facc[s2];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) f = __dadd_rn(f, __shfl_xor_sync(0xffffffffu, f, o));
+            const double f = face_lanes_sum(facc[s2], face, x_own0 - HX);
             if (lane == 0) a.flux_part[s2 * nparts + qi] = __dmul_rn(A.fscale[s2], f);
         }
     }
@@ -280,7 +278,6 @@ __global__ void __launch_bounds__(32 * W, XYMinBlocks<T, W>::value) strang_xy_ke
         if (eblk) strang_xy_block<T, W, NH, false, true>(A, strip, ytile, zseg, ych);
         else strang_xy_block<T, W, NH, false, false>(A, strip, ytile, zseg, ych);
     }
-    if (face >= 0) finish_flux<2 * NH>(a);
 }
 
 template <typename T, bool FIELD>
