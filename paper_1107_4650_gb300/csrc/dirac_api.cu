@@ -25,6 +25,7 @@ constexpr int kObsBlocksMax = 1216;
 struct Plan {
     int K = 1, P = 2, wpb = 4;
     int64_t strip_w = 0, nstrips = 0, nsegs = 0, seg_h = 0;
+    const TileShape *tile = nullptr;  // 2-D small grids: the tile kernel's shape (tile_kernels.cuh); null: the row kernel
     int z_threads = 128;
     int64_t z_nsegs = 1, z_seg_h = 0;
     // 3-D: fused single-pass step (fused3d_kernels.cuh) instead of the x-y pass + z/phase pass
@@ -338,6 +339,7 @@ int resident_blocks(const dirac_grid *g, int K, int P) {
 // SM, or, with target 0, by the row-time model above.
 void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
     Plan &p = g->plan;
+    p.tile = nullptr;
     p.K = K;
     p.P = P;
     p.wpb = wpb;
@@ -413,6 +415,49 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         }
 }
 
+int precision_index(const dirac_grid *g) { return g->fx ? 2 : (g->fp32 ? 1 : 0); }
+
+// Launches of a tile shape's own step count (its remainders run with the same warps and rows).
+void tile_plan(dirac_grid *g, const TileShape *t) {
+    // the row kernel's (K, P) that a caller may ask for stands beside it, and is what dirac_get_info reports
+    make_plan(g, t->steps, t->steps > 1 ? 2 : 1, 4, 0);
+    g->plan.tile = t;
+}
+
+int64_t tiles_of(const dirac_grid *g, const TileShape &t) {
+    const int H = levels(g, t.steps);
+    const int64_t ox = 32 - 2 * H, oz = t.warps * t.rows - 2 * H;
+    return ((g->cfg.n[0] + ox - 1) / ox) * ((g->cfg.n[2] + oz - 1) / oz);
+}
+
+// The tile shape for a 2-D grid without a field, or null where the row kernel is faster: least modelled time a step.  The
+// row kernel's time is taken as linear in the cells (fitted from 128^2 to 4096^2), a launch of the tile kernel's as linear
+// in the tiles on the fullest SM.  The lines cross, us a step with rows / tiles, at about: FP64 640^2 (512^2 30.2 / 28.4,
+// 768^2 52.4 / 61), second order 900^2 (768^2 111 / 105, 1024^2 176 / 184), FP32 3500^2 (2048^2 25.2 / 24.0, 4096^2 88.8 /
+// 90.3), second order 1800^2 (1600^2 30.6 / 29.7, 2048^2 44.1 / 46.8), fixed point 768^2 (512^2 12.7 / 10.4, 1024^2 32.8 /
+// 36.5), second order 700^2 (512^2 21.9 / 17.0, 768^2 32.3 / 35.4).
+const TileShape *pick_tile(const dirac_grid *g) {
+    const int mode = sweep_mode(g);
+    if (ndim_of(g) != 2 || (mode != 0 && mode != 2) || g->inject_stall) return nullptr;
+    if (g->cfg.n[0] >= (1 << 30) || g->cfg.n[2] >= (1 << 30)) return nullptr;  // the tile kernel's 32-bit coordinates
+    static const double row[3][2][2] = {{{7.5, 7.8e-5}, {18.0, 1.5e-4}}, {{4.4, 5.0e-6}, {6.7, 9.3e-6}}, {{5.7, 2.67e-5}, {10.7, 3.9e-5}}};
+    const double *line = row[precision_index(g)][strang(g) ? 1 : 0];
+    double best = line[0] + line[1] * (double)g->ncells;
+    const TileShape *pick = nullptr;
+    int count = 0;
+    const TileShape *t = tile_shapes(&count);
+    for (; count > 0; --count, ++t) {
+        if (!t->plan || t->precision != precision_index(g) || t->strang != (strang(g) ? 1 : 0)) continue;
+        const int64_t per_sm = (tiles_of(g, *t) + g->sm_count - 1) / g->sm_count;
+        const double us = (t->base + t->per_tile * (double)per_sm) / t->steps;
+        if (us < best) {
+            best = us;
+            pick = t;
+        }
+    }
+    return pick;
+}
+
 // Grid of the single-sweep kernels (grid-stride): up to 8 blocks of 256 threads per SM.
 int axis_blocks(const dirac_grid *g) {
     const int64_t need = (g->ncells + 255) / 256;
@@ -427,6 +472,7 @@ dirac_status ensure_flux_part(dirac_grid *g) {
         if (g->plan.K == 2)
             need = std::max(need, (size_t)(2 * g->plan.f2_nzsegs * g->plan.f2_nytiles * g->plan.f2_warps));
     }
+    if (g->plan.tile) need = std::max(need, (size_t)(levels(g, g->plan.K) * g->cfg.n[2]));
     if (sweep_mode(g) >= 6) need = std::max(need, (size_t)axis_blocks(g));
     if (strang3d_fused(g))
         for (int nh = 1; nh <= 2; ++nh) {
@@ -672,6 +718,16 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
         g->launches++;
         return DIRAC_OK;
     }
+    if (p.tile) {
+        a.strip_w = 32 - 2 * levels(g, K);
+        a.nstrips = (a.nx + a.strip_w - 1) / a.strip_w;
+        dirac_status st = flux_place(g, levels(g, K), a.nr, s, &a.flux_part);
+        if (st != DIRAC_OK) return st;
+        cudaError_t e = launch_tile(a, *p.tile, K, s);
+        if (e != cudaSuccess) return cuda_fail(g, e, "tile kernel launch");
+        g->launches++;
+        return DIRAC_OK;
+    }
     dirac_status st = flux_place(g, mode == 4 ? 1 : levels(g, K), a.nsegs * planes, s, &a.flux_part);
     if (st != DIRAC_OK) return st;
     cudaError_t e = mode == 4 ? launch_shift(a, g->fp32, char_shift(g), p.P, p.wpb, s)
@@ -857,11 +913,13 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
         g->cur ^= block_flips(g);
         t += K;
     }
-    for (int64_t r = 0; r < rem; ++r) {
-        dirac_status st = enqueue_block(g, g->cur, 1, g->stream, t);
+    while (rem > 0) {
+        const int kk = g->plan.tile && rem >= 2 ? 2 : 1;  // the tile kernel has launches of 4, 2 and 1 steps
+        dirac_status st = enqueue_block(g, g->cur, kk, g->stream, t);
         if (st != DIRAC_OK) return st;
         g->cur ^= block_flips(g);
-        t += 1;
+        t += kk;
+        rem -= kk;
     }
     g->step += nsteps;
     return fold_flux(g, g->stream);
@@ -977,6 +1035,12 @@ void default_plan(dirac_grid *g) {
         return;
     }
     const int mode = sweep_mode(g);
+    if (k == 0 && pp == 0) {
+        if (const TileShape *t = pick_tile(g)) {
+            tile_plan(g, t);
+            return;
+        }
+    }
     if (g->fx) {
         // one cell per lane (128 registers: four blocks per SM) and enough segments to fill them
         int K = k > 0 ? k : 1, P = pp > 0 ? pp : 1;
@@ -1572,6 +1636,11 @@ dirac_status dirac_get_info(const dirac_grid *g, dirac_info *info) {
         info->strip_width = 24;
         info->segment_rows = q.zseg_h;
     }
+    if (p.tile) {
+        info->launch_warps = tiles_of(g, *p.tile) * p.tile->warps;
+        info->strip_width = 32 - 2 * levels(g, p.K);
+        info->segment_rows = p.tile->warps * p.tile->rows - 2 * levels(g, p.K);
+    }
     if (fused_pass(g)) {
         info->points_per_lane = 1;
         info->launch_warps = p.f_nstrips * p.f_nytiles * p.f_nzsegs * p.f_warps;
@@ -1600,6 +1669,7 @@ dirac_status dirac_autotune(dirac_grid *g) {
         int s3 = 0;     // 3-D second order: 0 = eight single sweeps, else warps per block of the x-y-x pass
         int s3z = 2;    // and the z-phase-z pass's threads per SM / 1024
         int s3zp = 0;   // 3-D second order, single sweeps: C D C as one z-phase-z pass
+        const TileShape *tile = nullptr;  // 2-D: the tile kernel in this shape
     };
     std::vector<Cand> cands;
     if (sweep_mode(g) >= 7) {
@@ -1648,6 +1718,15 @@ dirac_status dirac_autotune(dirac_grid *g) {
         for (auto &kp : KP)
             for (int wsm : {0, 8, 12, 16, 24}) cands.push_back({kp[0], kp[1], 4, wsm});
     }
+    if (pick_tile(g)) {  // small 2-D grids
+        int count = 0;
+        const TileShape *t = tile_shapes(&count);
+        for (; count > 0; --count, ++t)
+            if (t->plan && t->precision == precision_index(g) && t->strang == (strang(g) ? 1 : 0)) {
+                cands.push_back({t->steps});
+                cands.back().tile = t;
+            }
+    }
     // save state and counters
     const size_t bytes = (size_t)g->ncells * 8 * g->elem;
     void *backup = nullptr;
@@ -1676,7 +1755,10 @@ dirac_status dirac_autotune(dirac_grid *g) {
         if (c.s3) g->plan.s3_warps = c.s3;
         g->plan.s3_zfactor = c.s3z;
         g->plan.s3_zpass = c.s3zp;
-        make_plan(g, c.K, c.P, c.wpb, c.wsm);
+        if (c.tile)
+            tile_plan(g, c.tile);
+        else
+            make_plan(g, c.K, c.P, c.wpb, c.wsm);
         st = ensure_flux_part(g);
         if (st != DIRAC_OK) break;
         const int64_t nsteps = std::max<int64_t>(8, 8 * (int64_t)c.K);
@@ -1706,7 +1788,10 @@ dirac_status dirac_autotune(dirac_grid *g) {
         if (best.s3) g->plan.s3_warps = best.s3;
         g->plan.s3_zfactor = best.s3z;
         g->plan.s3_zpass = best.s3zp;
-        make_plan(g, best.K, best.P, best.wpb, best.wsm);
+        if (best.tile)
+            tile_plan(g, best.tile);
+        else
+            make_plan(g, best.K, best.P, best.wpb, best.wsm);
         st = ensure_flux_part(g);
     }
     g->cur = cur_saved;

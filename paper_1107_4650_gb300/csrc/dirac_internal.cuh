@@ -128,6 +128,17 @@ cudaError_t launch_flux_fold(const FluxFold &f, cudaStream_t s);
 // Instantiated (K, P) pairs of the sweep kernels.
 bool sweep_supported(int fp32, int mode, int K, int P);
 
+// Small 2-D grids: `steps` whole steps per launch of a 32 x (warps rows) tile a block (tile_kernels.cuh); a.nstrips tiles
+// along x, each owning 32 - 2 H columns and warps rows - 2 H rows, H = steps (second order 2 steps).  Flux parts: [x
+// sweeps][nr].  precision: 0 FP64, 1 FP32, 2 int64 fixed point.
+struct TileShape {
+    int precision, warps, rows, steps, strang;
+    int plan;               // chosen by the library (0: only runs the steps left over)
+    double base, per_tile;  // microseconds of a launch: base + per_tile x tiles on the fullest SM
+};
+const TileShape *tile_shapes(int *count);
+cudaError_t launch_tile(const SweepArgs &a, const TileShape &t, int steps, cudaStream_t s);
+
 // Characteristic-shift step kernel (mode 4: 2-D first-order step with c dt = S dx, one step per launch,
 // strips of 32 P - 2 S owned cells); S in 2..4, P in {1, 2}.
 cudaError_t launch_shift(const SweepArgs &a, int fp32, int S, int P, int warps_per_block, cudaStream_t s);

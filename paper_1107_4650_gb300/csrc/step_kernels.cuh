@@ -281,6 +281,38 @@ template <typename T> __device__ __forceinline__ void load_row_pt(const T *p, in
         load_pt(p, s);
     }
 }
+// The same for a load.
+template <typename T> __device__ __forceinline__ void load_cell(const T *p, Cx<T> s[4], bool wide) {
+    if (wide) {
+        if constexpr (sizeof(T) == 4) {
+            asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=f"(s[0].re), "=f"(s[0].im), "=f"(s[1].re), "=f"(s[1].im), "=f"(s[2].re), "=f"(s[2].im),
+                           "=f"(s[3].re), "=f"(s[3].im)
+                         : "l"(p)
+                         : "memory");
+        } else if constexpr (std::is_same<T, double>::value) {
+            asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                         : "=d"(s[0].re), "=d"(s[0].im), "=d"(s[1].re), "=d"(s[1].im)
+                         : "l"(p)
+                         : "memory");
+            asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                         : "=d"(s[2].re), "=d"(s[2].im), "=d"(s[3].re), "=d"(s[3].im)
+                         : "l"(p + 4)
+                         : "memory");
+        } else {
+            asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                         : "=l"(s[0].re), "=l"(s[0].im), "=l"(s[1].re), "=l"(s[1].im)
+                         : "l"(p)
+                         : "memory");
+            asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                         : "=l"(s[2].re), "=l"(s[2].im), "=l"(s[3].re), "=l"(s[3].im)
+                         : "l"(p + 4)
+                         : "memory");
+        }
+    } else {
+        load_pt(p, s);
+    }
+}
 // The two sums a level keeps of a row's point, in the warp's shared memory: consecutive lanes 16 bytes apart (no bank
 // conflict).  `p` is the pair's place for this lane: 4-byte types keep both sums there, 8-byte types 32 lanes apart.
 template <typename T> __device__ __forceinline__ Cx<T> *hist_at(Cx<T> *hist, int slot, int lane) {
