@@ -326,8 +326,8 @@ dirac_status dirac_batch_create(const dirac_klein_run *runs, int nruns, const di
             return bfail(nullptr, DIRAC_ERR_ARG, "run " + std::to_string(r) + " has an invalid field");
     }
     const int fp32 = cfg->precision == DIRAC_FP32;
-    // FP32: four steps a launch (196 against 168 G point-steps/s on 24 runs; four points a lane: two); FP64: one (9.8
-    // against 8.6 G on 12 runs)
+    // FP32: four steps a launch (254 against 181 G point-steps/s on 24 runs; four points a lane: two); FP64: one (10.3
+    // against 9.1 G)
     const int P = cfg->points_per_lane > 0 ? cfg->points_per_lane : 2;
     const int K = cfg->steps_per_launch > 0 ? cfg->steps_per_launch : (fp32 ? (P == 2 ? 4 : 2) : 1);
     if (!batch_supported(fp32, K, P) || !batch_supported(fp32, 1, P))

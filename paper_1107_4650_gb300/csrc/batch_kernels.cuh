@@ -71,14 +71,16 @@ static __global__ void batch_flux_fold_kernel(const __grid_constant__ BatchFluxF
 
 // FP32 with two points a lane and two or four steps a launch: the sweep history in shared memory and one row per
 // iteration (24 runs of sides 768 and 1024, four steps: 196 against 157 G point-steps/s with it in registers and two
-// rows per iteration; two steps: 168 against 167; sides 256 to 1024: 158 against 133 and 131 against 135).
+// rows per iteration), which with two adjacent cells a lane, the flux of the levels together and two ring slots
+// (step_kernels.cuh) leaves room for 16 warps an SM: 254 G, 260 with 96 rows a task.
 template <typename T, int K, int P> struct BatchHist {
     static constexpr bool value = sizeof(T) == 4 && P == 2 && K >= 2;
     static constexpr int unroll = value ? 1 : 2;
+    static constexpr int blocks = value ? 4 : 1;  // resident 4-warp blocks the registers are fitted to
 };
 
 template <typename T, int K, int P>
-__global__ void __launch_bounds__(128) batch_kernel(const BatchArgs b) {
+__global__ void __launch_bounds__(128, BatchHist<T, K, P>::blocks) batch_kernel(const BatchArgs b) {
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     const int lane = threadIdx.x & 31;
     unsigned char *wsmem = dyn_smem + (threadIdx.x >> 5) * Ring<T, K, P, BatchHist<T, K, P>::value>::WARP_BYTES;

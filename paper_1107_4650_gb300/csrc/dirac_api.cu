@@ -332,7 +332,7 @@ int resident_blocks(const dirac_grid *g, int K, int P) {
     if (sweep_mode(g) == 4) return g->fp32 ? 4 : (P == 1 ? 3 : 2);
     if (P == 1) return g->fp32 && K == 1 ? 5 : 4;
     if (P == 4) return 2;
-    return g->fp32 ? (levels(g, K) == 4 ? 3 : 4) : 2;  // FP32, four levels: 18.5 KB of shared memory a warp
+    return g->fp32 ? 4 : 2;
 }
 
 // Launch geometry for (K, P, warps per block): strips of 32P - 2K owned cells; segments for about `target` warps per
@@ -431,18 +431,19 @@ int64_t tiles_of(const dirac_grid *g, const TileShape &t) {
 }
 
 // The tile shape for a 2-D grid without a field, or null where the row kernel is faster: least modelled time a step.  The
-// row kernel's time is taken as linear in the cells (fitted from 128^2 to 4096^2), a launch of the tile kernel's as linear
-// in the tiles on the fullest SM.  The lines cross, us a step with rows / tiles, at about: FP64 640^2 (512^2 30.2 / 28.4,
-// 768^2 52.4 / 61), second order 900^2 (768^2 111 / 105, 1024^2 176 / 184), FP32 3500^2 (2048^2 25.2 / 24.0, 4096^2 88.8 /
-// 90.3), second order 1800^2 (1600^2 30.6 / 29.7, 2048^2 44.1 / 46.8), fixed point 768^2 (512^2 12.7 / 10.4, 1024^2 32.8 /
+// row kernel's time is taken as linear in its strips' cells (fitted from 128^2 to 4096^2), a launch of the tile kernel's as
+// linear in the tiles on the fullest SM.  The lines cross, us a step with rows / tiles, at about: FP64 640^2 (512^2 30.2 /
+// 28.4, 768^2 52.4 / 61), second order 900^2 (768^2 111 / 105, 1024^2 176 / 184), FP32 1500^2 (1024^2 9.5 / 6.3, 2048^2 21.2
+// / 23.7), second order 1200^2 (1024^2 16.3 / 12.2, 1600^2 26 / 29.5), fixed point 768^2 (512^2 12.7 / 10.4, 1024^2 32.8 /
 // 36.5), second order 700^2 (512^2 21.9 / 17.0, 768^2 32.3 / 35.4).
 const TileShape *pick_tile(const dirac_grid *g) {
     const int mode = sweep_mode(g);
     if (ndim_of(g) != 2 || (mode != 0 && mode != 2) || g->inject_stall) return nullptr;
     if (g->cfg.n[0] >= (1 << 30) || g->cfg.n[2] >= (1 << 30)) return nullptr;  // the tile kernel's 32-bit coordinates
-    static const double row[3][2][2] = {{{7.5, 7.8e-5}, {18.0, 1.5e-4}}, {{4.4, 5.0e-6}, {6.7, 9.3e-6}}, {{5.7, 2.67e-5}, {10.7, 3.9e-5}}};
+    static const double row[3][2][2] = {{{7.5, 7.8e-5}, {18.0, 1.5e-4}}, {{4.4, 4.0e-6}, {7.5, 7.0e-6}}, {{5.7, 2.67e-5}, {10.7, 3.9e-5}}};
     const double *line = row[precision_index(g)][strang(g) ? 1 : 0];
-    double best = line[0] + line[1] * (double)g->ncells;
+    const int64_t strip = g->fp32 ? 56 : 32 - 2 * levels(g, 1);
+    double best = line[0] + line[1] * (double)((g->cfg.n[0] + strip - 1) / strip * strip * g->cfg.n[2]);
     const TileShape *pick = nullptr;
     int count = 0;
     const TileShape *t = tile_shapes(&count);
@@ -914,7 +915,8 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
         t += K;
     }
     while (rem > 0) {
-        const int kk = g->plan.tile && rem >= 2 ? 2 : 1;  // the tile kernel has launches of 4, 2 and 1 steps
+        // the tile kernel and the FP32 one of four steps have launches of two and one besides
+        const int kk = rem >= 2 && K == 4 ? 2 : 1;
         dirac_status st = enqueue_block(g, g->cur, kk, g->stream, t);
         if (st != DIRAC_OK) return st;
         g->cur ^= block_flips(g);
@@ -1054,12 +1056,11 @@ void default_plan(dirac_grid *g) {
     // FP64: one point a lane, 16 warps an SM (four blocks of 128 registers): the sweeps' pairs split over the FP64 and
     // the integer pipe need warps to overlap (2048^2: 13.1 against 10.0 G with two points and 8 warps; second order
     // 6.35 against 5.1; in a laser field 7.6 against 6.4)
-    int K = g->fp32 ? 2 : 1, P = g->fp32 ? 2 : 1;
+    // FP32: four steps a launch (2048^2 21.2 us a step against 25.1 with two, 4096^2 70.6 against 87.2, where two move twice
+    // the bytes)
+    int K = g->fp32 ? (pp == 0 || pp == 2 ? 4 : 2) : 1, P = g->fp32 ? 2 : 1;
     if (mode == 3 || mode == 5) K = 1;  // measured: the field's phase matrix makes k = 2 register-bound
     if (mode == 2) K = g->fp32 ? 2 : 1;  // FP32 second order: two steps per pass with the history in shared memory
-    // small FP32 grids, second order: one step a launch with one cell a lane, whose short rows spread over the chip
-    // (300 x 257: 11.5 us a step against 13; 900 x 700: 25.4 against 26.2; 1400^2: 45.1 against 44.0)
-    if (mode == 2 && g->fp32 && k == 0 && pp == 0 && g->ncells < (1 << 20)) K = P = 1;
     if (k > 0) K = k;
     if (mode == 0 && g->fp32 && K == 1) P = 1;  // one step a launch: 84.9 against 76.8 G at 2048^2
     if (pp > 0) P = pp;

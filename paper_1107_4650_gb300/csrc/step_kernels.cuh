@@ -281,7 +281,31 @@ template <typename T> __device__ __forceinline__ void load_row_pt(const T *p, in
         load_pt(p, s);
     }
 }
-// The same for a load.
+// Two adjacent FP32 cells of a row in shared memory, the lanes' 64 bytes consecutive: each lane takes its four 16-byte
+// quarters in an order of its own, so that eight lanes read eight different bank groups (no conflict), and puts them in place.
+__device__ __forceinline__ void load_row_pair(const float *p, int lane, Cx<float> s0[4], Cx<float> s1[4]) {
+    const float4 *q = reinterpret_cast<const float4 *>(p);
+    const int f = (lane >> 1) & 3;
+    float4 v0 = q[f], v1 = q[1 ^ f], v2 = q[2 ^ f], v3 = q[3 ^ f];
+    const bool b0 = f & 1, b1 = f & 2;
+    auto pick = [](bool t, float4 a, float4 b) {
+        return make_float4(t ? a.x : b.x, t ? a.y : b.y, t ? a.z : b.z, t ? a.w : b.w);
+    };
+    const float4 c0 = pick(b0, v1, v0), c1 = pick(b0, v0, v1), c2 = pick(b0, v3, v2), c3 = pick(b0, v2, v3);
+    v0 = pick(b1, c2, c0);
+    v1 = pick(b1, c3, c1);
+    v2 = pick(b1, c0, c2);
+    v3 = pick(b1, c1, c3);
+    s0[0] = {v0.x, v0.y};
+    s0[1] = {v0.z, v0.w};
+    s0[2] = {v1.x, v1.y};
+    s0[3] = {v1.z, v1.w};
+    s1[0] = {v2.x, v2.y};
+    s1[1] = {v2.z, v2.w};
+    s1[2] = {v3.x, v3.y};
+    s1[3] = {v3.z, v3.w};
+}
+// The same pieces for a load.
 template <typename T> __device__ __forceinline__ void load_cell(const T *p, Cx<T> s[4], bool wide) {
     if (wide) {
         if constexpr (sizeof(T) == 4) {
@@ -402,7 +426,7 @@ template <int K, int MODE> struct Levels { static constexpr int value = (MODE ==
 // 150 registers and 3 blocks), lets them fit; FP64's shared magnitude sums need the warps to fill both pipes.
 template <typename T, int K, int P, int MODE> struct SweepMinBlocks {
     static constexpr int value = (IsFx<T>::value && K == 1 && P == 1 && (MODE == 0 || MODE == 2))             ? 4
-                                 : (sizeof(T) == 4 && P == 2 && ((K == 2 && MODE == 0) || (K == 1 && MODE == 2))) ? 4
+                                 : (sizeof(T) == 4 && P == 2 && (MODE == 0 || MODE == 2) && Levels<K, MODE>::value >= 2) ? 4
                                  : (IsF64<T>::value && K == 1 && P == 1)                                       ? 4
                                                                                                                : 1;
 };
@@ -485,13 +509,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return false;
 }
 
+// The face flux of several levels evaluated together (flux_row).
+template <typename T, int L> struct FluxTogether { static constexpr bool value = sizeof(T) == 4 && L >= 2; };
+
 // Per-warp shared memory: 128 B of mbarriers, the row ring, the flux hand-off area (K levels x 8 values x 32
 // lanes), then with HS the sweep history ([row parity 2][level K][point P][lane 32], two complex values each; the ring
 // keeps three rows so that four blocks fit, two of the 8-byte types, whose rows last long enough).
 template <typename T, int K, int P, bool HS> struct Ring {
     static constexpr int ROW_BYTES = 32 * P * 8 * (int)sizeof(T);  // one warp row: 32P cells
-    static constexpr int SLOTS = (HS && sizeof(T) == 8) ? 2 : (HS || ROW_BYTES >= 8192) ? 3 : 4;
-    static constexpr int FLUX_BYTES = K * 8 * 32 * (int)sizeof(T);
+    static constexpr int SLOTS = (HS && (sizeof(T) == 8 || K >= 4)) ? 2 : (HS || ROW_BYTES >= 8192) ? 3 : 4;
+    static constexpr int FLUX_BYTES = (FluxTogether<T, K>::value ? 1 : K) * 8 * 32 * (int)sizeof(T);
     static constexpr int HIST_BYTES = HS ? 2 * K * 32 * P * 2 * 2 * (int)sizeof(T) : 0;
     static constexpr int WARP_BYTES = 128 + SLOTS * ROW_BYTES + FLUX_BYTES + HIST_BYTES;
 };
@@ -516,15 +543,35 @@ __device__ __forceinline__ void push_row(Cx<T> (&s0)[2], Cx<T> (&s1)[2], Cx<T> (
     }
 }
 
+// Which cells a lane holds: two adjacent ones (2 lane, 2 lane + 1; FP32 with two points a lane), whose inner neighbours need
+// no shuffle, or one in each group of 32 (32 j + lane).  The FP32 step of several levels is bound by the shared-memory pipe, which
+// shuffles (8 words a cell and level, 4 so), the sweep history and the row reads share, and by its latency: 2048^2 k = 4 24.8
+// -> 23.4 us a step, second order 44.1 -> 40.8; one level 48.4 -> 50.4, so not there.
+template <typename T, int P, int L> struct PairedCells { static constexpr bool value = sizeof(T) == 4 && P == 2 && L >= 2; };
+template <typename T, int P, int L> __device__ __forceinline__ int cell_of(int lane, int j) {
+    return PairedCells<T, P, L>::value ? 2 * lane + j : 32 * j + lane;
+}
+
 // x characteristics of a row (u = a + b travels +x, w = a - b travels -x) and the neighbours the x sweep
-// takes: u of the left cell and w of the right cell (warp shuffles; lane 0 and lane 31 take them from the
-// adjacent point of lanes 31 and 0).
-template <bool HY, typename T, int P>
+// takes: u of the left cell and w of the right cell (warp shuffles; with one cell in each group of 32, lane 0 and lane 31
+// take them from the adjacent point of lanes 31 and 0).
+template <bool HY, int L, typename T, int P>
 __device__ __forceinline__ void x_characteristics(const Cx<T> (*s)[4], int lane, int src_prev, int src_next, Cx<T> *u14,
                                                   Cx<T> *u23, Cx<T> *w14, Cx<T> *w23, Cx<T> *lu14, Cx<T> *lu23,
                                                   Cx<T> *rw14, Cx<T> *rw23) {
 #pragma unroll
     for (int j = 0; j < P; ++j) x_chars<HY>(s[j], u14[j], w14[j], u23[j], w23[j]);
+    if constexpr (PairedCells<T, P, L>::value) {
+        lu14[0] = shfl_c(u14[1], src_prev);
+        lu23[0] = shfl_c(u23[1], src_prev);
+        rw14[1] = shfl_c(w14[0], src_next);
+        rw23[1] = shfl_c(w23[0], src_next);
+        lu14[1] = u14[0];
+        lu23[1] = u23[0];
+        rw14[0] = w14[1];
+        rw23[0] = w23[1];
+        return;
+    }
     Cx<T> pu14[P], pu23[P], nw14[P], nw23[P];
 #pragma unroll
     for (int j = 0; j < P; ++j) {
@@ -552,24 +599,17 @@ __device__ __forceinline__ double face_lanes_sum(double v, int64_t face, int64_t
     return __dadd_rn(a, b);
 }
 
-// One row of the face flux: the face lane leaves the row's 8 values at place (row % 32) of the hand-off area; at every
-// 32nd row (or the segment's last) all lanes fold their rows: scale (|u14|^2 + |u23|^2) - scale (|w14|^2 + |w23|^2),
-// scale = 1/2 for a state at its true size, 2 for one held at half size.  The face's warps run as long as the launch does
-// when it is one wave, so what a row costs them counts whole: handing the values over by eight shuffles a row the launch
-// took 29.6 us a step against 23.3 without a face (FP32 k = 2 at 2048^2; second order 52.2 against 37.9), this way and
-// with the fold apart 25.3 (44.2).
+// The face's 8 values of a row: u of the cell left of it and w of the cell right of it, left at `g` by the face lane.
 template <typename T, int P>
-__device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, const Cx<T> *w14, const Cx<T> *w23,
-                                         int face_j, int face_lane, int lane, int64_t row_in_seg, bool last_row, T *g,
-                                         double scale, double &facc) {
-    const int t = (int)(row_in_seg & 31);
+__device__ __forceinline__ void flux_put(const Cx<T> *lu14, const Cx<T> *lu23, const Cx<T> *w14, const Cx<T> *w23,
+                                         int face_j, bool on_face, T *g) {
     if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int j = 0; j < P; ++j) {
             const Cx<T> v[4] = {lu14[j], lu23[j], w14[j], w23[j]};
-            if (lane == face_lane && j == face_j) store_pt(g + t * 8, v);
+            if (on_face && j == face_j) store_pt(g, v);
         }
-    } else if (lane == face_lane) {  // one branch: a store for each point costs registers (fixed point 112.6 against 107.3 us)
+    } else if (on_face) {  // one branch: a store for each point costs registers (fixed point 112.6 against 107.3 us)
         Cx<T> v[4] = {lu14[0], lu23[0], w14[0], w23[0]};
 #pragma unroll
         for (int j = 1; j < P; ++j) {
@@ -580,17 +620,36 @@ __device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, c
                 v[3] = w23[j];
             }
         }
-        store_pt(g + t * 8, v);
+        store_pt(g, v);
     }
+}
+// scale (|u14|^2 + |u23|^2) - scale (|w14|^2 + |w23|^2) of the values at `g`
+template <typename T> __device__ __forceinline__ double flux_value(const T *g, double scale) {
+    Cx<T> v[4];
+    load_pt(g, v);
+    const double right = __dmul_rn(scale, __dadd_rn(abs2d(v[0]), abs2d(v[1])));
+    const double left = __dmul_rn(scale, __dadd_rn(abs2d(v[2]), abs2d(v[3])));
+    return __dsub_rn(right, left);
+}
+
+// Face flux: the face lane leaves each row's 8 values in the hand-off area, and 32 of them are evaluated at once, one per
+// lane, scale = 1/2 for a state at its true size, 2 for one held at half size.  The face's warps run as long as the launch
+// does when it is one wave, so what a row costs them counts whole: handing the values over by eight shuffles a row the
+// launch took 29.6 us a step against 23.3 without a face (FP32 k = 2 at 2048^2; second order 52.2 against 37.9), by a store
+// of the face lane and with the partials folded by a launch of their own 25.3 (44.2).
+// Several levels of 4-byte types: 32 / L rows of the L levels together, one sum a lane and 1 KB a warp instead of 4, which
+// with two ring slots lets four blocks of the k = 4 kernel on an SM instead of three (2048^2 23.4 -> 21.2 us a step).  The
+// 8-byte kernels are at the edge of their registers, where that form costs more (fixed point 39.1 -> 36.8 G): 32 rows of
+// each level.
+template <typename T, int P>
+__device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, const Cx<T> *w14, const Cx<T> *w23,
+                                         int face_j, int face_lane, int lane, int64_t row_in_seg, bool last_row, T *g,
+                                         double scale, double &facc) {
+    const int t = (int)(row_in_seg & 31);
+    flux_put<T, P>(lu14, lu23, w14, w23, face_j, lane == face_lane, g + t * 8);
     if (t == 31 || last_row) {
         __syncwarp();
-        if (lane <= t) {
-            Cx<T> v[4];
-            load_pt(g + lane * 8, v);
-            const double right = __dmul_rn(scale, __dadd_rn(abs2d(v[0]), abs2d(v[1])));
-            const double left = __dmul_rn(scale, __dadd_rn(abs2d(v[2]), abs2d(v[3])));
-            facc = __dadd_rn(facc, __dsub_rn(right, left));
-        }
+        if (lane <= t) facc = __dadd_rn(facc, flux_value(g + lane * 8, scale));
         __syncwarp();
     }
 }
@@ -612,9 +671,8 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     const int64_t x_own1 = min(x_own0 + a.strip_w, nx);
     const int64_t xa = x_own0 - L;
     // Row indices fit 32 bits (the host limits every grid dimension below 2^31): FP32 k = 2 105 against 94 G at
-    // 2048^2 with 64-bit ones.  The fixed-point first-order kernel on a zero-boundary grid keeps 64-bit ones, with
-    // which it runs 33.7 against 33.5 G.
-    using RI = typename std::conditional<IsFx<T>::value && MODE == 0 && !PER, int64_t, int>::type;
+    // 2048^2 with 64-bit ones, fixed point 39.4 against 37.5 G.
+    using RI = int;
     const RI nr32 = (RI)nr;
     const RI r_begin = (RI)(seg * a.seg_h);
     const RI r_end = (RI)min((int64_t)r_begin + a.seg_h, nr);
@@ -627,7 +685,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     bool xin[P], own[P];  // own: the cell is in this warp's strip (it stores it)
 #pragma unroll
     for (int j = 0; j < P; ++j) {
-        const int64_t x = xa + 32 * j + lane;
+        const int64_t x = xa + cell_of<T, P, L>(lane, j);
         xin[j] = (x >= 0 && x < nx);
         own[j] = x >= x_own0 && x < x_own1;
         xl[j] = per ? pmod(x, nx) : min(max(x, (int64_t)0), nx - 1);
@@ -658,15 +716,18 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         }
     }
     // Flux through the face (owned by this strip): per row, 1/2(|u14|^2+|u23|^2) at face-1 minus
-    // 1/2(|w14|^2+|w23|^2) at face.  The face lane's 8 values of row q are handed to lane (q - r_begin) % 32;
-    // every 32 rows all lanes evaluate their row at once, so the FP64 work runs SIMT-wide (1/32 of the FP64
-    // issue a single lane would need).  Each lane accumulates its rows in FP64; a fixed xor tree adds lanes.
+    // 1/2(|w14|^2+|w23|^2) at face, evaluated 32 rows (or rows of the levels) at once, so the FP64 work runs SIMT-wide (1/32
+    // of the FP64 issue a single lane would need).  Each lane accumulates its rows in FP64 (FT: lane lev FR + t those of
+    // level lev); a fixed xor tree adds lanes.
+    constexpr bool FT = FluxTogether<T, L>::value;
+    constexpr int FR = FT ? 32 / L : 32;
     const bool has_face = a.flux_face >= x_own0 && a.flux_face < x_own1;
     const int face_off = (int)(a.flux_face - xa);
-    const int face_lane = face_off & 31, face_j = face_off >> 5;
-    double facc[L];
+    const int face_lane = PairedCells<T, P, L>::value ? face_off >> 1 : face_off & 31;
+    const int face_j = PairedCells<T, P, L>::value ? face_off & 1 : face_off >> 5;
+    double facc[FT ? 1 : L];
 #pragma unroll
-    for (int s = 0; s < L; ++s) facc[s] = 0.0;
+    for (int s = 0; s < (FT ? 1 : L); ++s) facc[s] = 0.0;
 
     // "+" characteristic sums of the two previous rows per level: rows q-2 (A) and q-1 (B)
     // The two previous rows' sums per level sit in two register slots.  With rows taken in pairs (UNR = 2),
@@ -693,7 +754,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
 #pragma unroll
         for (int t = 0; t < 2 * L * P; ++t) hist_store(hist_at(hist, t, lane), Cx<T>{T(0), T(0)}, Cx<T>{T(0), T(0)});
     }
-    T *gsm = reinterpret_cast<T *>(wsmem + 128 + RG::SLOTS * RG::ROW_BYTES);  // flux hand-off [K][8][32]
+    T *gsm = reinterpret_cast<T *>(wsmem + 128 + RG::SLOTS * RG::ROW_BYTES);  // flux hand-off
     // span of grid cells a row copy brings: the strip clipped to the grid; periodic: all 32 P cells, wrapped, as
     // pieces that end at the grid's right edge (two at most where nx >= 32 P)
     const int64_t cx0 = per ? pmod(xa, nx) : max(xa, (int64_t)0), cx1 = per ? xa + 32 * P : min(xa + 32 * P, nx);
@@ -741,7 +802,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         for (int sl = 0; sl < RG::SLOTS; ++sl)
 #pragma unroll
             for (int j = 0; j < P; ++j)
-                if (!xin[j]) store_pt(reinterpret_cast<T *>(wsmem + 128 + sl * RG::ROW_BYTES) + (32 * j + lane) * 8, none);
+                if (!xin[j]) store_pt(reinterpret_cast<T *>(wsmem + 128 + sl * RG::ROW_BYTES) + cell_of<T, P, L>(lane, j) * 8, none);
     }
     __syncwarp();
     bool stall = a.inject_stall && wid == 0 && !per;
@@ -768,7 +829,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     // 42.0 -> 31.4 M warp instructions a launch with the packed adds, k = 4 125 -> 139 G point-steps/s, the batched
     // kernel 154 -> 164.  What then bounds the FP32 kernel is the shared-memory pipe (82 % busy at k = 2, half of it bank
     // conflicts of the history and the row reads): without the conflicts and with 32-byte stores 124 -> 145 G.
-    T *orow = out + ((int64_t)(r_first - L) * nx + xa + lane) * 8;       // this lane's cell of output row r - L
+    T *orow = out + ((int64_t)(r_first - L) * nx + xa) * 8;  // output row r - L
     const T *frow = in + ((int64_t)(r_first + RG::SLOTS) * nx + cx0) * 8;  // zero boundary: span of row r + SLOTS
     const RI f_end = per ? r_last : min(r_last, nr32);                   // rows [.., f_end) are fetched
     const int64_t row_step = nx * 8;
@@ -783,16 +844,41 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
             phase_bits ^= 1u << sl;
             pending &= ~(1u << sl);
         }
-        const T *srow = reinterpret_cast<const T *>(wsmem + 128 + sl * RG::ROW_BYTES) + lane * 8;
-#pragma unroll
-        for (int j = 0; j < P; ++j) {
-            if (row_ok) {
-                load_row_pt(srow + 32 * 8 * j, lane, st[j]);
+        const T *srow = reinterpret_cast<const T *>(wsmem + 128 + sl * RG::ROW_BYTES);
+        if (row_ok) {
+            if constexpr (PairedCells<T, P, L>::value) {
+                load_row_pair(srow + lane * 16, lane, st[0], st[1]);
             } else {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) st[j][c] = {T(0), T(0)};
+                for (int j = 0; j < P; ++j) load_row_pt(srow + cell_of<T, P, L>(lane, j) * 8, lane, st[j]);
             }
+        } else {
+#pragma unroll
+            for (int j = 0; j < P; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) st[j][c] = {T(0), T(0)};
         }
+        // refills this slot with row r + SLOTS once every lane has read it
+        auto refill = [&]() {
+            __syncwarp();
+            const RI rn = r + RG::SLOTS;
+            if (rn < f_end && (STEADY || per || rn >= 0)) {
+                if (per) {
+                    if (lane == 0) {
+                        fence_proxy_async();
+                        fetch_row(grid_row(rn), sl);
+                    }
+                } else {
+                    refill_row(lane == 0, slot0 + sl * RG::ROW_BYTES + dst_off, frow, copy_bytes, bar0 + 8 * sl);
+                }
+                pending |= 1u << sl;
+            }
+        };
+        // before the sweeps where rows last long (two or more levels; 2048^2 FP32 k = 4 with two slots), else after the stores
+        // (the 3-D x-y pass 521 us a step against 531 so)
+        constexpr bool EARLY = L >= 2;
+        if (EARLY) refill();
+        const int frow_t = (int)(r - r_first) & (FR - 1);
 #pragma unroll
         for (int lev = 0; lev < L; ++lev) {
             const RI q = r - lev;  // row of the level-lev state in st
@@ -829,10 +915,13 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                     continue;
                 }
                 Cx<T> u14[P], u23[P], w14[P], w23[P], lu14[P], lu23[P], rw14[P], rw23[P];
-                x_characteristics<HY, T, P>(zs, lane, src_prev, src_next, u14, u23, w14, w23, lu14, lu23, rw14, rw23);
-                if (has_face && q - 1 >= r_begin && q - 1 < r_end)
+                x_characteristics<HY, L, T, P>(zs, lane, src_prev, src_next, u14, u23, w14, w23, lu14, lu23, rw14, rw23);
+                if (FT) {
+                    if (has_face) flux_put<T, P>(lu14, lu23, w14, w23, face_j, lane == face_lane, gsm + (lev * FR + frow_t) * 8);
+                } else if (has_face && q - 1 >= r_begin && q - 1 < r_end) {
                     flux_row<T, P>(lu14, lu23, w14, w23, face_j, face_lane, lane, q - 1 - r_begin, q - 1 == r_end - 1,
-                                   gsm + lev * 8 * 32, 2.0 * a.flux_unit, facc[lev]);
+                                   gsm + lev * 8 * 32, 2.0 * a.flux_unit, facc[FT ? 0 : lev]);
+                }
 #pragma unroll
                 for (int j = 0; j < P; ++j) {
                     const bool keep = per || (zrow_ok && xin[j]);
@@ -843,30 +932,14 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                 }
                 continue;
             }
-            Cx<T> u14[P], u23[P], w14[P], w23[P];
-#pragma unroll
-            for (int j = 0; j < P; ++j) x_chars<HY>(st[j], u14[j], w14[j], u23[j], w23[j]);
-            Cx<T> pu14[P], pu23[P], nw14[P], nw23[P];
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-                pu14[j] = shfl_c(u14[j], src_prev);
-                pu23[j] = shfl_c(u23[j], src_prev);
-                nw14[j] = shfl_c(w14[j], src_next);
-                nw23[j] = shfl_c(w23[j], src_next);
-            }
-            Cx<T> lu14[P], lu23[P], rw14[P], rw23[P];
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-                const int jp = j > 0 ? j - 1 : 0;
-                const int jn = j < P - 1 ? j + 1 : P - 1;
-                lu14[j] = (lane == 0) ? pu14[jp] : pu14[j];
-                lu23[j] = (lane == 0) ? pu23[jp] : pu23[j];
-                rw14[j] = (lane == 31) ? nw14[jn] : nw14[j];
-                rw23[j] = (lane == 31) ? nw23[jn] : nw23[j];
-            }
-            if (has_face && q >= r_begin && q < r_end)
+            Cx<T> u14[P], u23[P], w14[P], w23[P], lu14[P], lu23[P], rw14[P], rw23[P];
+            x_characteristics<HY, L, T, P>(st, lane, src_prev, src_next, u14, u23, w14, w23, lu14, lu23, rw14, rw23);
+            if (FT) {
+                if (has_face) flux_put<T, P>(lu14, lu23, w14, w23, face_j, lane == face_lane, gsm + (lev * FR + frow_t) * 8);
+            } else if (has_face && q >= r_begin && q < r_end) {
                 flux_row<T, P>(lu14, lu23, w14, w23, face_j, face_lane, lane, q - r_begin, q == r_end - 1,
-                               gsm + lev * 8 * 32, 0.5 * a.flux_unit, facc[lev]);
+                               gsm + lev * 8 * 32, 0.5 * a.flux_unit, facc[FT ? 0 : lev]);
+            }
             const bool out_row_ok = STEADY || per || (q - 1 >= 0 && q - 1 < nr32);
 #pragma unroll
             for (int j = 0; j < P; ++j) {
@@ -951,25 +1024,21 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                 }
             }
         }
+        if (FT && has_face && (frow_t == FR - 1 || r == r_last - 1)) {
+            __syncwarp();
+            const int lev = lane / FR, t = lane & (FR - 1);
+            const bool half2 = (MODE == 2 || MODE == 5) && (lev & 1);  // a second-order step's second x sweep, a row later
+            const RI q = r - frow_t + t - lev - (half2 ? 1 : 0);       // the row that this lane's values belong to
+            if (t <= frow_t && q >= r_begin && q < r_end)
+                facc[0] = __dadd_rn(facc[0], flux_value(gsm + lane * 8, half2 ? 2.0 * a.flux_unit : 0.5 * a.flux_unit));
+            __syncwarp();
+        }
         if (STEADY || r >= r_first + 2 * L) {
 #pragma unroll
             for (int j = 0; j < P; ++j)
-                if (own[j]) store_cell(orow + 32 * 8 * j, st[j], a.wide != 0);
+                if (own[j]) store_cell(orow + cell_of<T, P, L>(lane, j) * 8, st[j], a.wide != 0);
         }
-        // refill this slot with row r + SLOTS once every lane has read it
-        __syncwarp();
-        const RI rn = r + RG::SLOTS;
-        if (rn < f_end && (STEADY || per || rn >= 0)) {
-            if (per) {
-                if (lane == 0) {
-                    fence_proxy_async();
-                    fetch_row(grid_row(rn), sl);
-                }
-            } else {
-                refill_row(lane == 0, slot0 + sl * RG::ROW_BYTES + dst_off, frow, copy_bytes, bar0 + 8 * sl);
-            }
-            pending |= 1u << sl;
-        }
+        if (!EARLY) refill();
         sl = (sl + 1 == RG::SLOTS) ? 0 : sl + 1;
         orow += row_step;
         frow += row_step;
@@ -1005,11 +1074,11 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     __syncwarp();
     if (has_face) {
 #pragma unroll
-        for (int s = 0; s < L; ++s) {
+        for (int s = 0; s < (FT ? 1 : L); ++s) {
             double v = facc[s];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (lane == 0) a.flux_part[(int64_t)s * a.nsegs * a.nplanes + plane * a.nsegs + seg] = v;
+            for (int o = FR / 2; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if ((lane & (FR - 1)) == 0) a.flux_part[(int64_t)(FT ? lane / FR : s) * a.nsegs * a.nplanes + plane * a.nsegs + seg] = v;
         }
     }
 }
