@@ -55,9 +55,11 @@ struct dirac_batch {
     unsigned *counters = nullptr;  // two task counters, err, pad
     int *d_order_main = nullptr, *d_order_rem = nullptr;
     int64_t *d_off_main = nullptr, *d_off_rem = nullptr;
-    std::vector<int> nact_main, nact_rem;
+    std::vector<int> nact_main, nact_rem;       // active runs of each launch
+    std::vector<int> height_main, height_rem;   // and the place of its rows per task in `heights`
+    std::vector<int64_t> heights;               // rows per task in use: the caller's, or the library's choices
     int K = 2, P = 2, blocks = 0, sm_count = 152;
-    int64_t seg_rows = 64, max_tasks = 0;
+    int64_t seg_rows = 0, max_tasks = 0;  // rows per task, 0: chosen for each launch
     cudaGraphExec_t graph = nullptr;
     bool ran = false;
     int64_t launches = 0;
@@ -94,26 +96,52 @@ void drop_graph(dirac_batch *b) {
     b->graph = nullptr;
 }
 
-// Tasks of run r for a launch with `k` steps per launch.
-int64_t run_tasks(const dirac_batch *b, int r, int k) {
+// The library's choices of rows per task.
+constexpr int kMaxHeights = 14;
+constexpr int64_t kHeights[kMaxHeights] = {128, 112, 96, 80, 64, 56, 48, 40, 32, 24, 20, 16, 12, 8};
+
+// Tasks of run r for a launch with `k` steps per launch and h rows a task.
+int64_t run_tasks(const dirac_batch *b, int r, int k, int64_t h) {
     const int64_t side = b->runs[r].side;
     const int64_t sw = 32 * b->P - 2 * k;
-    return ((side + sw - 1) / sw) * b->hrun[r].nsegs;
+    return ((side + sw - 1) / sw) * batch_segments(side, h);
+}
+
+// Rows per task of a launch, from the tasks that each height makes.  A launch's time in rows, n tasks a resident warp.  FP32:
+// a start of 8 rows, then rows and halo once as long as every task has its warp (a chip half full is hardly faster than a
+// full one), 1.3 times just beyond, n times from there on (20 ensembles of 3 to 24 runs, 8 to 128 rows: within 8 %).  FP64:
+// bound by its pipe, which a chip not full leaves faster rows, and with ends a third of a wave apart; 64 rows unless another
+// height is clearly better (8 runs 9.3 G, 24 runs 10.2, as before; 2 runs of 1024^2 4.6 -> 8.4 G).  Chosen for each launch's active runs, since the longest runs are alone at the end.  With 64 rows
+// throughout, 24 runs of sides 256 to 768 took 98.4 ms, now 77; one run of 1024^2 34 G point-steps/s, 104; 8 246, as before.
+int pick_height(const dirac_batch *b, const std::vector<int64_t> &tasks, int k) {
+    int pick = 0;
+    double best = 1e300;
+    for (size_t i = 0; i < b->heights.size(); ++i) {
+        const double n = (double)tasks[i] / (4.0 * b->blocks);
+        const double rows = (double)(b->heights[i] + 2 * k);
+        const double t = b->fp32 ? 8.0 + rows * (n <= 1.0 ? 0.9 + 0.1 * n : std::max(1.3, n + 0.05))
+                                 : rows * (n <= 1.0 ? 0.6 + 0.4 * n : n + 0.35) * (b->heights[i] == 64 ? 0.85 : 1.0);
+        if (t < best) {
+            best = t;
+            pick = (int)i;
+        }
+    }
+    return pick;
 }
 
 // (Re)builds the launch plan for the current (K, P, seg_rows): segments, orders, task offsets, active counts.
 dirac_status plan(dirac_batch *b) {
     drop_graph(b);
     const int n = b->nruns;
-    for (int r = 0; r < n; ++r) {
-        BatchRunDev &R = b->hrun[r];
-        R.seg_h = std::min<int64_t>(b->seg_rows, R.side);
-        R.nsegs = (R.side + R.seg_h - 1) / R.seg_h;
-        R.parity_base = b->runs[r].nsteps / b->K;
-    }
-    // flux partials: K x nsegs per run, for kBatchSlots launches between folds
+    int per_sm = 0;
+    BCK(b, batch_occupancy(b->fp32, b->K, b->P, &per_sm));
+    b->blocks = std::max(1, per_sm) * b->sm_count;
+    b->heights = b->seg_rows > 0 ? std::vector<int64_t>{b->seg_rows} : std::vector<int64_t>(kHeights, kHeights + kMaxHeights);
+    const int64_t h_min = b->heights.back();
+    for (int r = 0; r < n; ++r) b->hrun[r].parity_base = b->runs[r].nsteps / b->K;
+    // flux partials: K x segments per run, for kBatchSlots launches between folds
     size_t need = 0;
-    for (int r = 0; r < n; ++r) need += (size_t)b->K * b->hrun[r].nsegs;
+    for (int r = 0; r < n; ++r) need += (size_t)b->K * batch_segments(b->runs[r].side, h_min);
     b->flux_stride = (int64_t)need;
     need *= kBatchSlots;
     if (need > b->flux_part_n) {
@@ -129,7 +157,7 @@ dirac_status plan(dirac_batch *b) {
     size_t off = 0;
     for (int r = 0; r < n; ++r) {
         b->hrun[r].flux_part = b->flux_part_pool + off;
-        off += (size_t)b->K * b->hrun[r].nsegs;
+        off += (size_t)b->K * batch_segments(b->runs[r].side, h_min);
     }
     std::vector<int> om(n), orr(n);
     std::iota(om.begin(), om.end(), 0);
@@ -137,11 +165,28 @@ dirac_status plan(dirac_batch *b) {
     const int K = b->K;
     std::stable_sort(om.begin(), om.end(), [&](int x, int y) { return b->runs[x].nsteps / K > b->runs[y].nsteps / K; });
     std::stable_sort(orr.begin(), orr.end(), [&](int x, int y) { return b->runs[x].nsteps % K > b->runs[y].nsteps % K; });
-    std::vector<int64_t> offm(n + 1, 0), offr(n + 1, 0);
-    for (int i = 0; i < n; ++i) {
-        offm[i + 1] = offm[i] + run_tasks(b, om[i], K);
-        offr[i + 1] = offr[i] + run_tasks(b, orr[i], 1);
-    }
+    // task offsets along each order, one table of n + 1 per height
+    const int nh = (int)b->heights.size();
+    std::vector<int64_t> offm((size_t)nh * (n + 1), 0), offr((size_t)nh * (n + 1), 0);
+    for (int h = 0; h < nh; ++h)
+        for (int i = 0; i < n; ++i) {
+            const size_t at = (size_t)h * (n + 1) + i;
+            offm[at + 1] = offm[at] + run_tasks(b, om[i], K, b->heights[h]);
+            offr[at + 1] = offr[at] + run_tasks(b, orr[i], 1, b->heights[h]);
+        }
+    auto heights_for = [&](const std::vector<int> &nact, const std::vector<int64_t> &off, int k) {
+        std::vector<int> out(nact.size());
+        std::vector<int64_t> tasks(nh);
+        for (size_t l = 0; l < nact.size(); ++l) {
+            if (l > 0 && nact[l] == nact[l - 1]) {
+                out[l] = out[l - 1];
+                continue;
+            }
+            for (int h = 0; h < nh; ++h) tasks[h] = off[(size_t)h * (n + 1) + nact[l]];
+            out[l] = pick_height(b, tasks, k);
+        }
+        return out;
+    };
     const int64_t Lmain = n ? b->runs[om[0]].nsteps / K : 0;
     b->nact_main.assign(Lmain, 0);
     for (int64_t l = 0; l < Lmain; ++l) {
@@ -155,16 +200,15 @@ dirac_status plan(dirac_batch *b) {
         while (c < n && b->runs[orr[c]].nsteps % K > j) ++c;
         if (c > 0) b->nact_rem.push_back(c);
     }
-    b->max_tasks = offm[n];
+    b->height_main = heights_for(b->nact_main, offm, K);
+    b->height_rem = heights_for(b->nact_rem, offr, 1);
+    b->max_tasks = offm[(size_t)(b->height_main.empty() ? 0 : b->height_main[0]) * (n + 1) + n];
     BCK(b, cudaMemcpyAsync(b->d_order_main, om.data(), n * sizeof(int), cudaMemcpyHostToDevice, b->stream));
     BCK(b, cudaMemcpyAsync(b->d_order_rem, orr.data(), n * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-    BCK(b, cudaMemcpyAsync(b->d_off_main, offm.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, b->stream));
-    BCK(b, cudaMemcpyAsync(b->d_off_rem, offr.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, b->stream));
+    BCK(b, cudaMemcpyAsync(b->d_off_main, offm.data(), offm.size() * sizeof(int64_t), cudaMemcpyHostToDevice, b->stream));
+    BCK(b, cudaMemcpyAsync(b->d_off_rem, offr.data(), offr.size() * sizeof(int64_t), cudaMemcpyHostToDevice, b->stream));
     BCK(b, cudaMemcpyAsync(b->drun, b->hrun.data(), n * sizeof(BatchRunDev), cudaMemcpyHostToDevice, b->stream));
     BCK(b, cudaStreamSynchronize(b->stream));
-    int per_sm = 0;
-    BCK(b, batch_occupancy(b->fp32, b->K, b->P, &per_sm));
-    b->blocks = std::max(1, per_sm) * b->sm_count;
     return DIRAC_OK;
 }
 
@@ -222,8 +266,11 @@ dirac_status enqueue_schedule(dirac_batch *b, cudaStream_t s, int64_t max_main =
         f.count = 0;
         return DIRAC_OK;
     };
-    auto launch = [&](int K) -> dirac_status {
+    auto launch = [&](int K, int height, const int64_t *off) -> dirac_status {
+        a.seg_rows = b->heights[height];
+        a.task_off = off + (size_t)height * (b->nruns + 1);
         a.flux_off = f.count * b->flux_stride;
+        f.seg_rows[f.count] = a.seg_rows;
         f.n_active[f.count++] = a.n_active;
         BCK(b, launch_batch(a, b->fp32, K, b->P, b->blocks, s));
         b->launches++;
@@ -232,25 +279,23 @@ dirac_status enqueue_schedule(dirac_batch *b, cudaStream_t s, int64_t max_main =
     };
     const int64_t Lm = (max_main >= 0) ? std::min<int64_t>(max_main, b->nact_main.size()) : (int64_t)b->nact_main.size();
     a.order = f.order = b->d_order_main;
-    a.task_off = b->d_off_main;
     a.parity_mode = 0;
     f.K = b->K;
     dirac_status st = DIRAC_OK;
     for (int64_t l = 0; l < Lm && st == DIRAC_OK; ++l) {
         a.n_active = b->nact_main[l];
         a.launch = l;
-        st = launch(b->K);
+        st = launch(b->K, b->height_main[l], b->d_off_main);
     }
     if (st == DIRAC_OK) st = fold();
     if (max_main >= 0 || st != DIRAC_OK) return st;
     a.order = f.order = b->d_order_rem;
-    a.task_off = b->d_off_rem;
     a.parity_mode = 1;
     f.K = 1;
     for (size_t j = 0; j < b->nact_rem.size() && st == DIRAC_OK; ++j) {
         a.n_active = b->nact_rem[j];
         a.launch = (int64_t)j;
-        st = launch(1);
+        st = launch(1, b->height_rem[j], b->d_off_rem);
     }
     return st == DIRAC_OK ? fold() : st;
 }
@@ -342,7 +387,7 @@ dirac_status dirac_batch_create(const dirac_klein_run *runs, int nruns, const di
     b->runs.assign(runs, runs + nruns);
     b->K = K;
     b->P = P;
-    b->seg_rows = cfg->segment_rows > 0 ? cfg->segment_rows : 64;
+    b->seg_rows = std::max<int64_t>(0, cfg->segment_rows);
     auto fail_release = [&](dirac_status st) {
         std::string m = b->err;
         release(b);
@@ -371,8 +416,8 @@ dirac_status dirac_batch_create(const dirac_klein_run *runs, int nruns, const di
     if ((st = balloc(b, &b->counters, 4 * sizeof(unsigned))) != DIRAC_OK) return fail_release(st);
     if ((st = balloc(b, &b->d_order_main, nruns * sizeof(int))) != DIRAC_OK) return fail_release(st);
     if ((st = balloc(b, &b->d_order_rem, nruns * sizeof(int))) != DIRAC_OK) return fail_release(st);
-    if ((st = balloc(b, &b->d_off_main, (nruns + 1) * sizeof(int64_t))) != DIRAC_OK) return fail_release(st);
-    if ((st = balloc(b, &b->d_off_rem, (nruns + 1) * sizeof(int64_t))) != DIRAC_OK) return fail_release(st);
+    if ((st = balloc(b, &b->d_off_main, kMaxHeights * (nruns + 1) * sizeof(int64_t))) != DIRAC_OK) return fail_release(st);
+    if ((st = balloc(b, &b->d_off_rem, kMaxHeights * (nruns + 1) * sizeof(int64_t))) != DIRAC_OK) return fail_release(st);
     if ((st = balloc(b, &b->d_cell_off, (nruns + 1) * sizeof(int64_t))) != DIRAC_OK) return fail_release(st);
     if ((st = balloc(b, &b->d_chunk_off, (nruns + 1) * sizeof(int64_t))) != DIRAC_OK) return fail_release(st);
     if ((st = balloc(b, &b->d_init, 4 * nruns * sizeof(double))) != DIRAC_OK) return fail_release(st);
@@ -572,7 +617,7 @@ dirac_status dirac_batch_autotune(dirac_batch *b) {
     struct Cand { int K, P; int64_t seg; };
     std::vector<Cand> cands;
     const int Ks[] = {1, 2, 4}, Ps[] = {2, 4};
-    const int64_t segs[] = {64, 128, 256};
+    const int64_t segs[] = {0, 64, 128, 256};
     for (int K : Ks)
         for (int P : Ps)
             for (int64_t sg : segs)
@@ -604,7 +649,8 @@ dirac_status dirac_batch_autotune(dirac_batch *b) {
             ps += act * c.K * b->runs[r].side * b->runs[r].side;
         }
         const double per = ps > 0 ? ms / (double)ps : 1e300;
-        if (per < best_t) {
+        // a fixed height has to be clearly better here, where all runs are active, to be kept for the launches where few are
+        if (per * (c.seg ? 1.05 : 1.0) < best_t) {
             best_t = per;
             best = c;
         }
@@ -625,7 +671,7 @@ dirac_status dirac_batch_get_info(const dirac_batch *b, dirac_batch_info *info) 
     if (!b || !info) return bfail(nullptr, DIRAC_ERR_ARG, "null argument");
     info->steps_per_launch = b->K;
     info->points_per_lane = b->P;
-    info->segment_rows = b->seg_rows;
+    info->segment_rows = b->heights[b->height_main.empty() ? 0 : b->height_main[0]];  // of the first launch
     info->launches = run_launches(b);
     info->max_tasks = b->max_tasks;
     int64_t ps = 0;

@@ -21,8 +21,7 @@ struct BatchRunDev {
     const void *table;      // x-only phase table, 4 values per column (pre-scaled by 1/4)
     int64_t side;           // nx = nz = side
     int64_t face;           // flux face index
-    int64_t nsegs, seg_h;   // row segments
-    double *flux_part;      // [slot][K][nsegs], slots flux_stride apart
+    double *flux_part;      // [slot][K][the launch's segments], slots flux_stride apart
     double *flux_cum;       // cumulative flux of this run
     int64_t parity_base;    // parity offset of the remainder phase (number of K-step launches)
 };
@@ -36,6 +35,7 @@ struct BatchArgs {
     int64_t launch;
     unsigned *counter;      // two task counters: a launch takes from [turn] and clears the other for the next one
     int turn;
+    int64_t seg_rows;       // rows per task of this launch
     int64_t flux_off;       // this launch's slot of the flux partials
     unsigned *err;
 };
@@ -44,6 +44,10 @@ struct BatchArgs {
 // runs' cumulative fluxes, one warp per run, launch by launch and step by step (lane l adds segments l, l + 32, ..., then
 // an xor tree).
 constexpr int kBatchSlots = 16;
+__host__ __device__ inline int64_t batch_segments(int64_t side, int64_t seg_rows) {
+    const int64_t h = seg_rows < side ? seg_rows : side;
+    return (side + h - 1) / h;
+}
 struct BatchFluxFold {
     const BatchRunDev *runs;
     const int *order;
@@ -51,21 +55,24 @@ struct BatchFluxFold {
     int64_t stride;
     double vol;
     int n_active[kBatchSlots];
+    int64_t seg_rows[kBatchSlots];
 };
 static __global__ void batch_flux_fold_kernel(const __grid_constant__ BatchFluxFold f) {
     const int lane = threadIdx.x & 31, i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (i >= f.n_active[0]) return;  // the active set only shrinks
     const BatchRunDev &R = f.runs[f.order[i]];
     double F = *R.flux_cum;
-    for (int l = 0; l < f.count && i < f.n_active[l]; ++l)
+    for (int l = 0; l < f.count && i < f.n_active[l]; ++l) {
+        const int64_t nsegs = batch_segments(R.side, f.seg_rows[l]);
         for (int s = 0; s < f.K; ++s) {
-            const double *part = R.flux_part + l * f.stride + s * R.nsegs;
+            const double *part = R.flux_part + l * f.stride + s * nsegs;
             double v = 0.0;
-            for (int64_t q = lane; q < R.nsegs; q += 32) v = __dadd_rn(v, part[q]);
+            for (int64_t q = lane; q < nsegs; q += 32) v = __dadd_rn(v, part[q]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
             F = __dadd_rn(F, __dmul_rn(v, f.vol));
         }
+    }
     if (lane == 0) *R.flux_cum = F;
 }
 
@@ -107,8 +114,8 @@ __global__ void __launch_bounds__(128, BatchHist<T, K, P>::blocks) batch_kernel(
         a.nplanes = 1;
         a.strip_w = 32 * P - 2 * K;
         a.nstrips = (R.side + a.strip_w - 1) / a.strip_w;
-        a.nsegs = R.nsegs;
-        a.seg_h = R.seg_h;
+        a.seg_h = min(b.seg_rows, R.side);
+        a.nsegs = (R.side + a.seg_h - 1) / a.seg_h;
         a.flux_face = R.face;
         a.flux_part = R.flux_part + b.flux_off;
         a.err = b.err;
