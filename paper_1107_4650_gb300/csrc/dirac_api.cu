@@ -31,7 +31,7 @@ struct Plan {
     // 3-D: fused single-pass step (fused3d_kernels.cuh) instead of the x-y pass + z/phase pass
     int fused3d = 0, f_warps = 16;
     int64_t f_nstrips = 0, f_nytiles = 0, f_nzsegs = 0, f_zseg_h = 0;
-    // two steps per fused pass (K = 2): 28-cell strips x (f2_warps - 4)-row tiles
+    // two steps per fused pass (K = 2): 28-cell strips x tiles of one or two rows a warp, four of them halo
     int f2_warps = 16;
     int64_t f2_nstrips = 0, f2_nytiles = 0, f2_nzsegs = 0, f2_zseg_h = 0;
     // 3-D second-order step: three fused passes (strang3d_kernels.cuh) instead of eight single sweeps
@@ -382,13 +382,27 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         const int f_resident = !g->fp32 && p.f_warps == 8 ? 2 : 1;
         p.f_zseg_h = pick_rows(nz, tiles, 1, g->sm_count, f_resident, 3.0, 0.5, whole);
         p.f_nzsegs = (nz + p.f_zseg_h - 1) / p.f_zseg_h;
-        // two steps per fused pass: 28-cell strips x (warps - 4)-row tiles (16 warps in FP32, 8 in FP64), z
-        // segments as above (each carries two halo planes a side)
-        p.f2_warps = g->fp32 ? 16 : 8;
+        // two steps per fused pass: 28-cell strips x (rows - 4)-row tiles, z segments as above (each carries two halo
+        // planes a side).  FP32: 24 rows, two a warp, or 16, one a warp, where those fit a small grid better, whose planes take
+        // 1.68 and 1.23 of the time (256^3: 219 us a step with 24, 271 with 16; 64^3 13.0 and 12.2); with the field's phase
+        // matrices 16 rows; FP64 8 rows
+        const bool two_rows = g->fp32 && !field_on(g);
         p.f2_nstrips = (g->cfg.n[0] + 27) / 28;
-        p.f2_nytiles = (g->cfg.n[1] + (p.f2_warps - 4) - 1) / (p.f2_warps - 4);
-        const int64_t tiles2 = p.f2_nstrips * p.f2_nytiles;
-        p.f2_zseg_h = pick_rows(nz, tiles2, 1, g->sm_count, 1, 5.0, 0.0, whole);
+        double best = 1e300;
+        for (int warps : {12, 16}) {
+            if (!two_rows) warps = g->fp32 ? 16 : 8;
+            const int64_t own = (warps == 12 ? 2 : 1) * warps - 4;
+            const int64_t nytiles = (g->cfg.n[1] + own - 1) / own, tiles2 = p.f2_nstrips * nytiles;
+            const int64_t h = pick_rows(nz, tiles2, 1, g->sm_count, 1, 5.0, 0.0, whole);
+            const int64_t waves = (tiles2 * ((nz + h - 1) / h) + g->sm_count - 1) / g->sm_count;
+            const double t = (warps == 12 ? 1.68 : 1.23) * (double)((h + 5) * waves);
+            if (t < best) {
+                best = t;
+                p.f2_warps = warps;
+                p.f2_nytiles = nytiles;
+                p.f2_zseg_h = h;
+            }
+        }
         p.f2_nzsegs = (nz + p.f2_zseg_h - 1) / p.f2_zseg_h;
         // second-order passes: x-y-x(-x-y-x) blocks over (32 - 4 nh)-cell strips x (warps - 4 nh)-row tiles x
         // z segments (planes are independent; whole waves); z-phase-z columns x 2 plane parities

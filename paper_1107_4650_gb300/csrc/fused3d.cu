@@ -1,6 +1,6 @@
 // Instantiations of the fused 3-D step kernels: one step per pass (8 or 16 warps per block: 6 or 14 owned
-// rows per tile) and two steps per pass (FP32: 16 warps, 12 owned rows; FP64: 8 warps, 4 owned rows), with
-// and without a uniform vector potential.
+// rows per tile) and two steps per pass (FP32: 12 warps of two rows, 20 owned rows, or 16 of one, 12 owned rows;
+// FP64: 8 of one, 4 owned rows), with and without a uniform vector potential.
 #include "fused3d_kernels.cuh"
 
 namespace dirac {
@@ -24,11 +24,12 @@ cudaError_t launch_fused3d(const SweepArgs &a, int precision, int warps, int ste
         return cudaErrorInvalidValue;
     }
     if (steps == 2) {
-        // two steps per pass: FP32 with 16-warp blocks, FP64 with 8 (its register budget)
+        // two steps per pass (warps: rows of the tile / rows a warp)
         if (fp32 && warps == 16)
-            return field ? launch_fused3d2_one<float, 16, true>(A, s) : launch_fused3d2_one<float, 16, false>(A, s);
+            return field ? launch_fused3d2_one<float, 16, 1, true>(A, s) : launch_fused3d2_one<float, 16, 1, false>(A, s);
+        if (fp32 && !field && warps == 12) return launch_fused3d2_one<float, 12, 2, false>(A, s);
         if (!fp32 && warps == 8)
-            return field ? launch_fused3d2_one<double, 8, true>(A, s) : launch_fused3d2_one<double, 8, false>(A, s);
+            return field ? launch_fused3d2_one<double, 8, 1, true>(A, s) : launch_fused3d2_one<double, 8, 1, false>(A, s);
         return cudaErrorInvalidValue;
     }
     if (steps != 1) return cudaErrorInvalidValue;

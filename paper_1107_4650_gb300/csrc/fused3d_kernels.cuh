@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(32 * W, Fused3DMinBlocks<T, W>::value) fused3d
         for (int e = 0; e < (FIELD ? 6 : 1); ++e) UM[e] = Cx<T>{(T)__ldg(u + 2 * e), (T)__ldg(u + 2 * e + 1)};
     }
     const int64_t face = a.flux_face;
-    const bool face_lane = owned_row && face >= x_own0 && face < x_own1 && (x == face - 1 || x == face);
+    const bool face_warp = owned_row && face >= x_own0 && face < x_own1;  // warp-uniform
+    const bool face_lane = face_warp && (x == face - 1 || x == face);
     double facc = 0.0;
     typename FaceAcc<T>::type fpart = 0;
 
@@ -151,10 +152,16 @@ __global__ void __launch_bounds__(32 * W, Fused3DMinBlocks<T, W>::value) fused3d
             using F = typename FaceAcc<T>::type;
             const F v = (x == face - 1) ? face_sq(u14, u23) : -face_sq(w14, w23);
             fpart = Ar<F>::add(fpart, v);
-            if (((k - z_begin) & 31) == 31 || k == z_end - 1) {
+            if (IsFx<T>::value && (((k - z_begin) & 31) == 31 || k == z_end - 1)) {
                 facc = __dadd_rn(facc, (double)fpart);
                 fpart = 0;
             }
+        }
+        // by the whole warp, a branch (see the two-step kernel); fixed point, with FP64 idle, is 1 % faster the other way
+        if (!IsFx<T>::value && face_warp && k >= z_begin && (((k - z_begin) & 31) == 31 || k == z_end - 1)) {
+            __syncwarp();
+            facc = __dadd_rn(facc, (double)fpart);
+            fpart = 0;
         }
         const Cx<T> lu14 = shfl_c(u14, (lane + 31) & 31), lu23 = shfl_c(u23, (lane + 31) & 31);
         const Cx<T> rw14 = shfl_c(w14, (lane + 1) & 31), rw23 = shfl_c(w23, (lane + 1) & 31);
@@ -224,8 +231,11 @@ __global__ void __launch_bounds__(32 * W, Fused3DMinBlocks<T, W>::value) fused3d
 }
 
 // Two first-order steps per pass (temporal block k = 2): HBM is read and written once per two steps.
-// The block's strip is 28 cells (two halo lanes each side) by W - 4 rows (two halo rows each side), and
-// the block streams its z segment plus two halo planes each side.  Per input plane k:
+// The block's strip is 28 cells (two halo lanes each side) by W R - 4 rows (two halo rows each side; R rows a warp), and
+// the block streams its z segment plus two halo planes each side.  Two rows a warp (FP32) halve the rows that go through
+// shared memory, give each warp two chains, and let 12 warps of 168 registers hold 24 rows (20 owned) where 16 of 122 hold 16
+// (12 owned), which fits small grids better: bound by latency between the two barriers of a plane (issue slots half used, memory 31 % of its peak), 256^3
+// 271 -> 218 us a step, 384^3 786 -> 674.  Per input plane k:
 //   * step 1: every warp x-sweeps its row and writes its y characteristics to shared memory; after a
 //     barrier the rows one inside the halo y-sweep, z-sweep (register history of the "+z" sums of the
 //     previous two planes) and take the phase: the state after step 1 at plane k - 1, zeroed outside the
@@ -235,9 +245,9 @@ __global__ void __launch_bounds__(32 * W, Fused3DMinBlocks<T, W>::value) fused3d
 // Each step's arithmetic is that of the one-step kernel, so the result equals two one-step launches bit for
 // bit.  Both steps' face flux is taken on the state entering their x sweep (parts [2][nzsegs nytiles W]).
 // FIELD: the phase matrices of steps step0 and step0 + 1.
-template <typename T, int W, bool FIELD>
+template <typename T, int W, int R, bool FIELD>
 __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A) {
-    constexpr int H = W - 4;
+    constexpr int ROWS = W * R, H = ROWS - 4;
     const SweepArgs &a = A.s;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t b = blockIdx.x;
@@ -249,22 +259,23 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A
     const bool per = a.periodic != 0;
     const int64_t x_own0 = strip * 28, x_own1 = min(x_own0 + 28, nx);
     const int64_t x = x_own0 - 2 + lane;
-    const int64_t y = ytile * H - 2 + w;
-    const bool owned_row = w >= 2 && w < W - 2 && y < ny;
-    const bool mid_row = w >= 1 && w < W - 1;
+    const int64_t y0 = ytile * H - 2 + w * R;  // this warp's rows are y0 .. y0 + R - 1
+    // warps with a row one inside the halo (step 1's output), and with rows of their own (step 2's)
+    const bool mid_warp = w * R + R - 1 >= 1 && w * R < ROWS - 1;
+    const bool own_warp = w * R + R - 1 >= 2 && w * R < ROWS - 2 && y0 < ny;
     const bool own_lane = x >= x_own0 && x < x_own1;
     using ZI = typename PlaneIdx<T>::type;
     const ZI z_begin = (ZI)(zseg * A.zseg_h), z_end = (ZI)min((int64_t)z_begin + A.zseg_h, nz);
-    const bool xin = x >= 0 && x < nx, yin = y >= 0 && y < ny;
-    const bool ghost_xy = !per && !(xin && yin);
+    const bool xin = x >= 0 && x < nx;
     const int64_t xl = per ? pmod(x, nx) : min(max(x, (int64_t)0), nx - 1);
-    const int64_t yl = per ? pmod(y, ny) : min(max(y, (int64_t)0), ny - 1);
+    auto owned_row = [&](int r) { return w * R + r >= 2 && w * R + r < ROWS - 2 && y0 + r < ny; };
+    auto in_xy = [&](int r) { return per || (xin && y0 + r >= 0 && y0 + r < ny); };
     const T *in = static_cast<const T *>(a.in);
     T *out = static_cast<T *>(a.out);
     const T *tab = static_cast<const T *>(a.table);
 
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    Cx<T> *buf1 = reinterpret_cast<Cx<T> *>(dyn_smem);  // [W][4][32] step 1's y characteristics
+    Cx<T> *buf1 = reinterpret_cast<Cx<T> *>(dyn_smem);  // [W][4][32] step 1's y characteristics of the warps' outermost rows
     Cx<T> *buf2 = buf1 + W * 4 * 32;                    // [W][4][32] step 2's
 
     Cx<T> pu = {T(0), T(0)}, pd = {T(0), T(0)};
@@ -280,138 +291,189 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A
         }
     }
     const int64_t face = a.flux_face;
-    const bool face_warp = owned_row && face >= x_own0 && face < x_own1;
-    const bool fl_u = face_warp && x == face - 1, fl_w = face_warp && x == face;
+    const bool has_face = face >= x_own0 && face < x_own1;  // block-uniform
+    const bool on_u = x == face - 1, on_w = x == face;
     double facc[2] = {0.0, 0.0};
     T fp[2] = {T(0), T(0)};
 
     // cell (xl, yl) of a plane: plane k at (k nx ny + cell) (periodic: halo planes wrap)
-    const int64_t plane_cells = nx * ny, cell = yl * nx + xl;
+    const int64_t plane_cells = nx * ny;
+    int64_t cell[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        cell[r] = (per ? pmod(y0 + r, ny) : min(max(y0 + r, (int64_t)0), ny - 1)) * nx + xl;
     auto wrap_z = [&](ZI k) -> int64_t {
         if (per && (k < 0 || k >= nz)) return pmod((int64_t)k, nz);
         return k;
     };
-    auto load_row = [&](ZI k, Cx<T> s[4]) {
-        const bool ok = per || (yin && k >= 0 && k < nz && xin);
-        if (ok) {
-            load_pt(in + (wrap_z(k) * plane_cells + cell) * 8, s);
-        } else {
+    auto load_rows = [&](ZI k, Cx<T> (&v)[R][4]) {
+        const bool zin = per || (k >= 0 && k < nz);
+        const int64_t plane = wrap_z(k) * plane_cells;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) s[c] = {T(0), T(0)};
+        for (int r = 0; r < R; ++r) {
+            if (zin && in_xy(r)) {
+                load_cell(in + (plane + cell[r]) * 8, v[r], a.wide != 0);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[r][c] = {T(0), T(0)};
+            }
         }
     };
     auto face_term = [&](Cx<T> p14, Cx<T> p23) -> T {
         return Ar<T>::fma(p14.re, p14.re, Ar<T>::fma(p14.im, p14.im, Ar<T>::fma(p23.re, p23.re, Ar<T>::mul(p23.im, p23.im))));
     };
-    // x sweep of a row held one cell per lane (valid where both neighbours are); face terms of its input
-    auto xsweep = [&](const Cx<T> s[4], Cx<T> o[4], T &acc, bool count) {
-        Cx<T> u14, w14, u23, w23;
-        x_chars<false>(s, u14, w14, u23, w23);
-        if (count && fl_u) acc = Ar<T>::add(acc, face_term(u14, u23));
-        if (count && fl_w) acc = Ar<T>::sub(acc, face_term(w14, w23));
-        const Cx<T> lu14 = shfl_c(u14, (lane + 31) & 31), lu23 = shfl_c(u23, (lane + 31) & 31);
-        const Cx<T> rw14 = shfl_c(w14, (lane + 1) & 31), rw23 = shfl_c(w23, (lane + 1) & 31);
-        x_join<false>(lu14, rw14, lu23, rw23, o);
+    // x sweep of rows held one cell per lane (valid where both neighbours are); face terms of its input
+    auto xsweep = [&](const Cx<T> (&v)[R][4], Cx<T> (&o)[R][4], T &acc, bool count) {
+        Cx<T> u14[R], w14[R], u23[R], w23[R], lu14[R], lu23[R], rw14[R], rw23[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) x_chars<false>(v[r], u14[r], w14[r], u23[r], w23[r]);
+        if (has_face && own_warp && count) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (on_u && owned_row(r)) acc = Ar<T>::add(acc, face_term(u14[r], u23[r]));
+                if (on_w && owned_row(r)) acc = Ar<T>::sub(acc, face_term(w14[r], w23[r]));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            lu14[r] = shfl_c(u14[r], (lane + 31) & 31);
+            lu23[r] = shfl_c(u23[r], (lane + 31) & 31);
+            rw14[r] = shfl_c(w14[r], (lane + 1) & 31);
+            rw23[r] = shfl_c(w23[r], (lane + 1) & 31);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) x_join<false>(lu14[r], rw14[r], lu23[r], rw23[r], o[r]);
     };
     // y characteristics (Eq. sol_dis_2): "+y" movers (b1 - i b4, b2 + i b3), "-y" movers (b1 + i b4, b2 - i b3)
-    auto ywrite = [&](Cx<T> *buf, const Cx<T> b4[4]) {
-        Cx<T> U14, W14, U23, W23;
-        y_chars<false>(b4, U14, W14, U23, W23);
-        buf[(w * 4 + 0) * 32 + lane] = U14;
-        buf[(w * 4 + 1) * 32 + lane] = U23;
-        buf[(w * 4 + 2) * 32 + lane] = W14;
-        buf[(w * 4 + 3) * 32 + lane] = W23;
-    };
-    // y sweep from rows w - 1 and w + 1, z sweep against the history (output plane = input plane - 1), phase
-    auto yz_phase = [&](const Cx<T> *buf, Cx<T> (&HA)[2], Cx<T> (&HB)[2], Cx<T> qu, Cx<T> qd, int st, Cx<T> o[4]) {
-        const Cx<T> U14 = buf[((w - 1) * 4 + 0) * 32 + lane], U23 = buf[((w - 1) * 4 + 1) * 32 + lane];
-        const Cx<T> W14 = buf[((w + 1) * 4 + 2) * 32 + lane], W23 = buf[((w + 1) * 4 + 3) * 32 + lane];
-        Cx<T> s[4], U13, W13, U24, W24;
-        y_join<false>(U14, W14, U23, W23, s);
-        z_chars<false>(s, U13, W13, U24, W24);
-        z_join<false>(HA[0], W13, HA[1], W24, o);
-        HA[0] = HB[0];
-        HA[1] = HB[1];
-        HB[0] = U13;
-        HB[1] = U24;
-        if (FIELD) {
-            Cx<T> m6[FIELD ? 6 : 1];
+    Cx<T> U14[R], W14[R], U23[R], W23[R];
+    auto ywrite = [&](Cx<T> *buf, const Cx<T> (&v)[R][4]) {
 #pragma unroll
-            for (int e = 0; e < (FIELD ? 6 : 1); ++e) m6[e] = cmulp(UM[st][e], qu);
-            const Cx<T> z0 = {T(0), T(0)};
-            const Cx<T> n0 = cmac(cmac(cmac(z0, o[0], m6[0]), o[2], m6[2]), o[3], m6[4]);
-            const Cx<T> n1 = cmac(cmac(cmac(z0, o[1], m6[0]), o[2], m6[5]), o[3], m6[3]);
-            const Cx<T> n2 = cmac(cmac(cmac(z0, o[0], m6[2]), o[1], m6[4]), o[2], m6[1]);
-            const Cx<T> n3 = cmac(cmac(cmac(z0, o[0], m6[5]), o[1], m6[3]), o[3], m6[1]);
-            o[0] = n0;
-            o[1] = n1;
-            o[2] = n2;
-            o[3] = n3;
-        } else {
-            o[0] = cmulp(o[0], qu);
-            o[1] = cmulp(o[1], qu);
-            o[2] = cmulp(o[2], qd);
-            o[3] = cmulp(o[3], qd);
+        for (int r = 0; r < R; ++r) y_chars<false>(v[r], U14[r], W14[r], U23[r], W23[r]);
+        buf[(w * 4 + 0) * 32 + lane] = U14[R - 1];
+        buf[(w * 4 + 1) * 32 + lane] = U23[R - 1];
+        buf[(w * 4 + 2) * 32 + lane] = W14[0];
+        buf[(w * 4 + 3) * 32 + lane] = W23[0];
+    };
+    // y sweep from the rows below and above, z sweep against the history (output plane = input plane - 1), phase
+    auto yz_phase = [&](const Cx<T> *buf, Cx<T> (&HA)[R][2], Cx<T> (&HB)[R][2], const Cx<T> (&qu)[R], const Cx<T> (&qd)[R], int st,
+                        Cx<T> (&out4)[R][4]) {
+        const int lo = R > 1 ? max(w - 1, 0) : w - 1, hi = R > 1 ? min(w + 1, W - 1) : w + 1;  // beyond them: rows past use
+        const Cx<T> l14 = buf[(lo * 4 + 0) * 32 + lane], l23 = buf[(lo * 4 + 1) * 32 + lane];
+        const Cx<T> h14 = buf[(hi * 4 + 2) * 32 + lane], h23 = buf[(hi * 4 + 3) * 32 + lane];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int rl = r > 0 ? r - 1 : 0, rh = r < R - 1 ? r + 1 : r;
+            Cx<T> s[4], U13, W13, U24, W24;
+            Cx<T> *o = out4[r];
+            y_join<false>(r > 0 ? U14[rl] : l14, r < R - 1 ? W14[rh] : h14, r > 0 ? U23[rl] : l23, r < R - 1 ? W23[rh] : h23, s);
+            z_chars<false>(s, U13, W13, U24, W24);
+            z_join<false>(HA[r][0], W13, HA[r][1], W24, out4[r]);
+            HA[r][0] = HB[r][0];
+            HA[r][1] = HB[r][1];
+            HB[r][0] = U13;
+            HB[r][1] = U24;
+            if (FIELD) {
+                Cx<T> m6[FIELD ? 6 : 1];
+#pragma unroll
+                for (int e = 0; e < (FIELD ? 6 : 1); ++e) m6[e] = cmulp(UM[st][e], qu[r]);
+                const Cx<T> z0 = {T(0), T(0)};
+                const Cx<T> n0 = cmac(cmac(cmac(z0, o[0], m6[0]), o[2], m6[2]), o[3], m6[4]);
+                const Cx<T> n1 = cmac(cmac(cmac(z0, o[1], m6[0]), o[2], m6[5]), o[3], m6[3]);
+                const Cx<T> n2 = cmac(cmac(cmac(z0, o[0], m6[2]), o[1], m6[4]), o[2], m6[1]);
+                const Cx<T> n3 = cmac(cmac(cmac(z0, o[0], m6[5]), o[1], m6[3]), o[3], m6[1]);
+                o[0] = n0;
+                o[1] = n1;
+                o[2] = n2;
+                o[3] = n3;
+            } else {
+                o[0] = cmulp(o[0], qu[r]);
+                o[1] = cmulp(o[1], qu[r]);
+                o[2] = cmulp(o[2], qd[r]);
+                o[3] = cmulp(o[3], qd[r]);
+            }
         }
     };
 
-    constexpr int LA = sizeof(T) == 4 ? 2 : 1;
+    constexpr int LA = sizeof(T) == 4 && R == 1 ? 2 : 1;
     const ZI k_first = z_begin - 2, k_last = z_end + 1;
-    Cx<T> ring[LA][4];
+    Cx<T> ring[LA][R][4];
 #pragma unroll
     for (int j = 0; j < LA; ++j)
-        if (k_first + j <= k_last) load_row(k_first + j, ring[j]);
-    Cx<T> H1A[2] = {{T(0), T(0)}, {T(0), T(0)}}, H1B[2] = {{T(0), T(0)}, {T(0), T(0)}};
-    Cx<T> H2A[2] = {{T(0), T(0)}, {T(0), T(0)}}, H2B[2] = {{T(0), T(0)}, {T(0), T(0)}};
+        if (k_first + j <= k_last) load_rows(k_first + j, ring[j]);
+    Cx<T> H1A[R][2], H1B[R][2], H2A[R][2], H2B[R][2];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) H1A[r][h] = H1B[r][h] = H2A[r][h] = H2B[r][h] = {T(0), T(0)};
     // per-cell table entries (full table): step 1 at plane k - 1 (rows one inside the halo), step 2 at k - 2
-    auto table_at = [&](ZI j, Cx<T> &qu, Cx<T> &qd) {
-        qu = pu;
-        qd = pd;
-        if (a.full_table && (per || (j >= 0 && j < nz)))
-            load_tab(tab + (wrap_z(j) * plane_cells + cell) * 4, qu, qd);
+    auto table_at = [&](ZI j, Cx<T> (&qu)[R], Cx<T> (&qd)[R]) {
+        const bool there = a.full_table && (per || (j >= 0 && j < nz));
+        const int64_t plane = wrap_z(j) * plane_cells;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            qu[r] = pu;
+            qd[r] = pd;
+            if (there) load_tab(tab + (plane + cell[r]) * 4, qu[r], qd[r]);
+        }
     };
-    Cx<T> t1u, t1d, t2u, t2d;
+    Cx<T> t1u[R], t1d[R], t2u[R], t2d[R];
     table_at(k_first - 1, t1u, t1d);
     table_at(k_first - 2, t2u, t2d);
 
     for (ZI k = k_first; k <= k_last; ++k) {
-        Cx<T> st[4];
+        Cx<T> st[R][4], q1u[R], q1d[R], q2u[R], q2d[R];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) st[c] = ring[0][c];
+        for (int r = 0; r < R; ++r) {
 #pragma unroll
-        for (int j = 0; j + 1 < LA; ++j)
+            for (int c = 0; c < 4; ++c) st[r][c] = ring[0][r][c];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) ring[j][c] = ring[j + 1][c];
-        if (k + LA <= k_last) load_row(k + LA, ring[LA - 1]);
-        const Cx<T> q1u = t1u, q1d = t1d, q2u = t2u, q2d = t2d;
-        if (mid_row) table_at(k, t1u, t1d);            // step 1's next plane
-        if (owned_row) table_at(k - 1, t2u, t2d);      // step 2's next plane
+            for (int j = 0; j + 1 < LA; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ring[j][r][c] = ring[j + 1][r][c];
+            q1u[r] = t1u[r];
+            q1d[r] = t1d[r];
+            q2u[r] = t2u[r];
+            q2d[r] = t2d[r];
+        }
+        if (k + LA <= k_last) load_rows(k + LA, ring[LA - 1]);
+        if (mid_warp) table_at(k, t1u, t1d);      // step 1's next plane
+        if (own_warp) table_at(k - 1, t2u, t2d);  // step 2's next plane
 
         // step 1: x sweep of input plane k
-        Cx<T> b4[4];
+        Cx<T> b4[R][4];
         xsweep(st, b4, fp[0], k >= z_begin && k < z_end);
         ywrite(buf1, b4);
         __syncthreads();
         const ZI j1 = k - 1;  // step 1's output plane
-        if (mid_row) {
-            Cx<T> o[4];
+        if (mid_warp) {
+            Cx<T> o[R][4];
             yz_phase(buf1, H1A, H1B, q1u, q1d, 0, o);
-            if (ghost_xy || (!per && (j1 < 0 || j1 >= nz))) {
+            const bool zout = !per && (j1 < 0 || j1 >= nz);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) o[c] = {T(0), T(0)};
-            }
+            for (int r = 0; r < R; ++r)
+                if (zout || !in_xy(r)) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) o[r][c] = {T(0), T(0)};
+                }
             // step 2: x sweep of plane j1
             xsweep(o, b4, fp[1], j1 >= z_begin && j1 < z_end);
             ywrite(buf2, b4);
         }
         __syncthreads();
         const ZI m = k - 2;  // step 2's output plane
-        if (owned_row) {
-            Cx<T> o[4];
+        if (own_warp) {
+            Cx<T> o[R][4];
             yz_phase(buf2, H2A, H2B, q2u, q2d, 1, o);
-            if (own_lane && m >= z_begin && m < z_end) store_pt(out + ((int64_t)m * plane_cells + cell) * 8, o);
+            if (own_lane && m >= z_begin && m < z_end) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (owned_row(r)) store_cell(out + ((int64_t)m * plane_cells + cell[r]) * 8, o[r], a.wide != 0);
+            }
         }
-        if ((fl_u || fl_w) && (((k - k_first) & 31) == 31 || k == k_last)) {
+        // every 32 terms into the FP64 sums, by the whole warp: under a condition on the lane the additions and conversions
+        // were issued for every plane of every warp, predicated (37 % of the FP64 pipe's time)
+        if (has_face && own_warp && (((k - k_first) & (32 / R - 1)) == 32 / R - 1 || k == k_last)) {
+            __syncwarp();
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 facc[q] = __dadd_rn(facc[q], (double)fp[q]);
@@ -419,7 +481,7 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A
             }
         }
     }
-    if (face >= 0 && face >= x_own0 && face < x_own1) {
+    if (has_face) {
         // one part per (step, z segment, y tile, warp) of the strip that owns the face; other warps write 0
         const int64_t nparts = A.nzsegs * A.nytiles * W;
         const int64_t q = (zseg * A.nytiles + ytile) * W + w;
@@ -431,15 +493,15 @@ __global__ void __launch_bounds__(32 * W, 1) fused3d2_kernel(const Fused3DArgs A
     }
 }
 
-template <typename T, int W, bool FIELD>
+template <typename T, int W, int R, bool FIELD>
 static cudaError_t launch_fused3d2_one(const Fused3DArgs &A, cudaStream_t s) {
     const int64_t blocks = A.nstrips * A.nytiles * A.nzsegs;
     if (blocks <= 0) return cudaSuccess;
     const int smem = 2 * W * 4 * 32 * (int)sizeof(Cx<T>);
     static std::atomic<unsigned long long> done{0};
-    cudaError_t e = optin_smem(fused3d2_kernel<T, W, FIELD>, smem, done);
+    cudaError_t e = optin_smem(fused3d2_kernel<T, W, R, FIELD>, smem, done);
     if (e != cudaSuccess) return e;
-    fused3d2_kernel<T, W, FIELD><<<(unsigned)blocks, 32 * W, smem, s>>>(A);
+    fused3d2_kernel<T, W, R, FIELD><<<(unsigned)blocks, 32 * W, smem, s>>>(A);
     return cudaGetLastError();
 }
 

@@ -146,6 +146,7 @@ __device__ __forceinline__ void shift_warp(const SweepArgs &a, const int64_t wid
                     fpart = Ar<T>::add(fpart, Ar<T>::sub(vr, vl));
                 }
                 if (((r - r_begin) & 31) == 31 || r == r_end - 1) {
+                    __syncwarp();  // a branch, not predicated FP64 work in every row (see fused3d2_kernel)
                     facc = __dadd_rn(facc, (double)fpart);
                     fpart = T(0);
                 }

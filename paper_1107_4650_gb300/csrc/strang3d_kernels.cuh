@@ -233,7 +233,8 @@ __device__ __forceinline__ void strang_xy_block(const StrangXYArgs &A, const int
                 if (own_lane) store_pt(dst, t);
             }
         }
-        if (FLUX && fw && (fl_u || fl_w) && (((k - z_begin) & 31) == 31 || k == z_end - 1)) {
+        if (FLUX && fw && (((k - z_begin) & 31) == 31 || k == z_end - 1)) {
+            __syncwarp();  // by the whole warp (a branch: see fused3d2_kernel)
 #pragma unroll
             for (int s2 = 0; s2 < NS; ++s2) {
                 facc[s2] = __dadd_rn(facc[s2], (double)fp[s2]);
