@@ -1073,7 +1073,9 @@ void default_plan(dirac_grid *g) {
     // FP32: four steps a launch (2048^2 21.2 us a step against 25.1 with two, 4096^2 70.6 against 87.2, where two move twice
     // the bytes)
     int K = g->fp32 ? (pp == 0 || pp == 2 ? 4 : 2) : 1, P = g->fp32 ? 2 : 1;
-    if (mode == 3 || mode == 5) K = 1;  // measured: the field's phase matrix makes k = 2 register-bound
+    // with a field FP32 first order two (2048^2 43.9 us a step against 61.0 with one, 1000 x 777 12.0 and 17.0, 300^2 6.8 and
+    // 9.0; the kernels of four would not fit the registers), else one
+    if (mode == 3 || mode == 5) K = mode == 3 && g->fp32 && (pp == 0 || pp == 2) ? 2 : 1;
     if (mode == 2) K = g->fp32 ? 2 : 1;  // FP32 second order: two steps per pass with the history in shared memory
     if (k > 0) K = k;
     if (mode == 0 && g->fp32 && K == 1) P = 1;  // one step a launch: 84.9 against 76.8 G at 2048^2
