@@ -444,25 +444,29 @@ int64_t tiles_of(const dirac_grid *g, const TileShape &t) {
     return ((g->cfg.n[0] + ox - 1) / ox) * ((g->cfg.n[2] + oz - 1) / oz);
 }
 
-// The tile shape for a 2-D grid without a field, or null where the row kernel is faster: least modelled time a step.  The
+// The tile shape for a 2-D grid, or null where the row kernel is faster: least modelled time a step.  The
 // row kernel's time is taken as linear in its strips' cells (fitted from 128^2 to 4096^2), a launch of the tile kernel's as
 // linear in the tiles on the fullest SM.  The lines cross, us a step with rows / tiles, at about: FP64 640^2 (512^2 30.2 /
 // 28.4, 768^2 52.4 / 61), second order 900^2 (768^2 111 / 105, 1024^2 176 / 184), FP32 1500^2 (1024^2 9.5 / 6.3, 2048^2 21.2
 // / 23.7), second order 1200^2 (1024^2 16.3 / 12.2, 1600^2 26 / 29.5), fixed point 768^2 (512^2 12.7 / 10.4, 1024^2 32.8 /
 // 36.5), second order 700^2 (512^2 21.9 / 17.0, 768^2 32.3 / 35.4).
+// With a uniform field (and an x-only table): FP64 350^2 (300^2 25.0 / 22.1, second order 45.8 / 33.6), FP32 1000^2 (300^2 6.6
+// / 3.0), second order 1400^2 (300^2 10.9 / 5.1).
 const TileShape *pick_tile(const dirac_grid *g) {
     const int mode = sweep_mode(g);
-    if (ndim_of(g) != 2 || (mode != 0 && mode != 2) || g->inject_stall) return nullptr;
+    const bool field = mode == 3 || mode == 5;
+    if (ndim_of(g) != 2 || (mode != 0 && mode != 2 && !field) || g->inject_stall) return nullptr;
     if (g->cfg.n[0] >= (1 << 30) || g->cfg.n[2] >= (1 << 30)) return nullptr;  // the tile kernel's 32-bit coordinates
     static const double row[3][2][2] = {{{7.5, 7.8e-5}, {18.0, 1.5e-4}}, {{4.4, 4.0e-6}, {7.5, 7.0e-6}}, {{5.7, 2.67e-5}, {10.7, 3.9e-5}}};
-    const double *line = row[precision_index(g)][strang(g) ? 1 : 0];
+    static const double frow[2][2][2] = {{{12.0, 1.31e-4}, {25.0, 2.1e-4}}, {{5.6, 8.2e-6}, {10.3, 1.25e-5}}};  // with a field
+    const double *line = field ? frow[precision_index(g)][strang(g) ? 1 : 0] : row[precision_index(g)][strang(g) ? 1 : 0];
     const int64_t strip = g->fp32 ? 56 : 32 - 2 * levels(g, 1);
     double best = line[0] + line[1] * (double)((g->cfg.n[0] + strip - 1) / strip * strip * g->cfg.n[2]);
     const TileShape *pick = nullptr;
     int count = 0;
     const TileShape *t = tile_shapes(&count);
     for (; count > 0; --count, ++t) {
-        if (!t->plan || t->precision != precision_index(g) || t->strang != (strang(g) ? 1 : 0)) continue;
+        if (!t->plan || t->precision != precision_index(g) || t->strang != (strang(g) ? 1 : 0) || t->field != (field ? 1 : 0)) continue;
         const int64_t per_sm = (tiles_of(g, *t) + g->sm_count - 1) / g->sm_count;
         const double us = (t->base + t->per_tile * (double)per_sm) / t->steps;
         if (us < best) {
@@ -733,7 +737,7 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
         g->launches++;
         return DIRAC_OK;
     }
-    if (p.tile) {
+    if (p.tile && !(p.tile->field && g->table_full)) {  // (a field over a full table: the row kernel of the same K)
         a.strip_w = 32 - 2 * levels(g, K);
         a.nstrips = (a.nx + a.strip_w - 1) / a.strip_w;
         dirac_status st = flux_place(g, levels(g, K), a.nr, s, &a.flux_part);
@@ -1653,7 +1657,7 @@ dirac_status dirac_get_info(const dirac_grid *g, dirac_info *info) {
         info->strip_width = 24;
         info->segment_rows = q.zseg_h;
     }
-    if (p.tile) {
+    if (p.tile && !(p.tile->field && g->table_full)) {
         info->launch_warps = tiles_of(g, *p.tile) * p.tile->warps;
         info->strip_width = 32 - 2 * levels(g, p.K);
         info->segment_rows = p.tile->warps * p.tile->rows - 2 * levels(g, p.K);
@@ -1739,7 +1743,8 @@ dirac_status dirac_autotune(dirac_grid *g) {
         int count = 0;
         const TileShape *t = tile_shapes(&count);
         for (; count > 0; --count, ++t)
-            if (t->plan && t->precision == precision_index(g) && t->strang == (strang(g) ? 1 : 0)) {
+            if (t->plan && t->precision == precision_index(g) && t->strang == (strang(g) ? 1 : 0) &&
+                t->field == (field_on(g) ? 1 : 0)) {
                 cands.push_back({t->steps});
                 cands.back().tile = t;
             }

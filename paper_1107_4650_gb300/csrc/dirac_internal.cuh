@@ -133,6 +133,7 @@ bool sweep_supported(int fp32, int mode, int K, int P);
 // sweeps][nr].  precision: 0 FP64, 1 FP32, 2 int64 fixed point.
 struct TileShape {
     int precision, warps, rows, steps, strang;
+    int field;              // with a uniform vector potential (x-only tables)
     int plan;               // chosen by the library (0: only runs the steps left over)
     double base, per_tile;  // microseconds of a launch: base + per_tile x tiles on the fullest SM
 };

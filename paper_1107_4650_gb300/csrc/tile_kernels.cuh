@@ -14,7 +14,7 @@
 // through shared memory and the more chains a warp has, the better; two cells a lane gave nothing more).
 // Measured, us a step with the face flux, row kernel -> this: FP64 128^2 9.1 -> 4.9, 256^2 12.2 -> 9.0 (second order 32.8 ->
 // 14.9); FP32 128^2 4.2 -> 1.1, 512^2 5.9 -> 2.6, 1024^2 10.2 -> 6.3 (second order 256^2 7.8 -> 2.5); fixed point 256^2 7.2 ->
-// 3.6.  A launch may begin while the one before it drains (256^2 FP32 1.5 -> 1.3 us a step).
+// 3.6; in a uniform field, 300^2, FP64 25.0 -> 22.1 (second order 45.8 -> 33.6), FP32 6.6 -> 2.9 (10.9 -> 5.1).  A launch may begin while the one before it drains (256^2 FP32 1.5 -> 1.3 us a step).
 // Face flux: the two lanes at the face leave each row's sums in shared memory, and after the last step one warp takes all
 // rows of a sweep at once, lane = row (evaluated in each row's warp it cost 7 FP64 instructions a row and sweep: FP32 at
 // 256^2, K = 4, 4.0 us a step against 1.6).  Parts: [x sweeps][rows of the grid].
@@ -24,7 +24,7 @@
 
 namespace dirac {
 
-template <typename T, int W, int R, int K, bool STRANG, bool PER>
+template <typename T, int W, int R, int K, bool STRANG, bool PER, bool FIELD>
 __global__ void __launch_bounds__(32 * W, 1) tile_kernel(const SweepArgs a) {
     constexpr int ROWS = W * R;         // warp w holds rows w R .. w R + R - 1 of the tile
     constexpr int ZS = STRANG ? 2 : 1;  // x sweeps, and z sweeps, a step
@@ -53,6 +53,16 @@ __global__ void __launch_bounds__(32 * W, 1) tile_kernel(const SweepArgs a) {
         } else {
             pu[r] = pu[0];
             pd[r] = pd[0];
+        }
+    }
+    // with a uniform field the phase is the matrix M = U g, U of the step and g (x-only) of the column: its non-zero entries
+    Cx<T> M[FIELD ? K : 1][FIELD ? 6 : 1];
+    if (FIELD) {
+#pragma unroll
+        for (int k = 0; k < (FIELD ? K : 1); ++k) {
+            const double *u = a.ucoef + ((a.step0 + k) % a.ucoef_n) * 12;
+#pragma unroll
+            for (int e = 0; e < (FIELD ? 6 : 1); ++e) M[k][e] = cmulp(Cx<T>{(T)__ldg(u + 2 * e), (T)__ldg(u + 2 * e + 1)}, pu[0]);
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -143,10 +153,24 @@ __global__ void __launch_bounds__(32 * W, 1) tile_kernel(const SweepArgs a) {
             z_get(bz, st);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                st[r][0] = cmulp(st[r][0], pu[r]);
-                st[r][1] = cmulp(st[r][1], pu[r]);
-                st[r][2] = cmulp(st[r][2], pd[r]);
-                st[r][3] = cmulp(st[r][3], pd[r]);
+                Cx<T> *o = st[r];
+                if (FIELD) {
+                    const Cx<T> *m = M[FIELD ? k : 0], z0 = {T(0), T(0)};
+                    constexpr int m1 = FIELD ? 1 : 0, m2 = FIELD ? 2 : 0, m3 = FIELD ? 3 : 0, m4 = FIELD ? 4 : 0, m5 = FIELD ? 5 : 0;
+                    const Cx<T> n0 = cmac(cmac(cmac(z0, o[0], m[0]), o[2], m[m2]), o[3], m[m4]);
+                    const Cx<T> n1 = cmac(cmac(cmac(z0, o[1], m[0]), o[2], m[m5]), o[3], m[m3]);
+                    const Cx<T> n2 = cmac(cmac(cmac(z0, o[0], m[m2]), o[1], m[m4]), o[2], m[m1]);
+                    const Cx<T> n3 = cmac(cmac(cmac(z0, o[0], m[m5]), o[1], m[m3]), o[3], m[m1]);
+                    o[0] = n0;
+                    o[1] = n1;
+                    o[2] = n2;
+                    o[3] = n3;
+                } else {
+                    o[0] = cmulp(o[0], pu[r]);
+                    o[1] = cmulp(o[1], pu[r]);
+                    o[2] = cmulp(o[2], pd[r]);
+                    o[3] = cmulp(o[3], pd[r]);
+                }
             }
             clear_ghosts(st);
             if (STRANG) z_put(st, buf1);
@@ -183,12 +207,12 @@ __global__ void __launch_bounds__(32 * W, 1) tile_kernel(const SweepArgs a) {
     }
 }
 
-template <typename T, int W, int R, int K, bool STRANG, bool PER>
+template <typename T, int W, int R, int K, bool STRANG, bool PER, bool FIELD>
 static cudaError_t launch_tile_per(const SweepArgs &a, cudaStream_t s) {
     constexpr int H = STRANG ? 2 * K : K, OWNZ = W * R - 2 * H;
     const int smem = (2 * 32 + R * H) * W * 4 * (int)sizeof(Cx<T>);
     static std::atomic<unsigned long long> done{0};
-    cudaError_t e = optin_smem(tile_kernel<T, W, R, K, STRANG, PER>, smem, done);
+    cudaError_t e = optin_smem(tile_kernel<T, W, R, K, STRANG, PER, FIELD>, smem, done);
     if (e != cudaSuccess) return e;
     // may start while the launch before it drains, and waits for it before it reads the state
     cudaLaunchAttribute at{};
@@ -201,7 +225,7 @@ static cudaError_t launch_tile_per(const SweepArgs &a, cudaStream_t s) {
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tile_kernel<T, W, R, K, STRANG, PER>, a);
+    return cudaLaunchKernelEx(&cfg, tile_kernel<T, W, R, K, STRANG, PER, FIELD>, a);
 }
 
 }  // namespace dirac

@@ -53,6 +53,37 @@ def test_tiles_equal_rows(n, precision, strang, periodic):
     assert abs(ogot[key] - owant[key]) <= tol, (ogot[key], owant[key], tol)
 
 
+@pytest.mark.parametrize("periodic", [0, 1])
+@pytest.mark.parametrize("precision,strang", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("n,full", [((5, 3), False), ((28, 12), False), ((57, 41), False), ((57, 41), True), ((200, 150), False),
+                                    ((301, 257), False), ((520, 384), False)])
+def test_tiles_in_a_field_equal_rows(n, full, precision, strang, periodic):
+    import paper_1107_4650_gb300 as D
+    from paper_1107_4650_gb300 import workloads as W
+    nx, nz = n
+    rng = np.random.default_rng(nx + nz)
+    psi = W.random_state(nz, 1, nx, nx + 3 * nz).astype(np.complex64 if precision else np.complex128)
+    V = rng.uniform(-1, 1, (nz, 1, nx) if full else nx) * W.C_AU ** 2
+    A = rng.uniform(-1, 1, (9, 3))  # another matrix each step
+
+    def run(k, p):
+        h = D.dirac_create_grid(D.make_config((nx, 1, nz), precision=precision, splitting=strang, boundary=periodic,
+                                              steps_per_launch=k, points_per_lane=p))
+        try:
+            D.dirac_set_vector_potential(h, A)
+            D.dirac_set_potential(h, V, D.DIRAC_V_FULL if full else D.DIRAC_V_X_ONLY)
+            D.dirac_set_state(h, psi)
+            D.dirac_step(h, 4)
+            D.dirac_step(h, 5)
+            out = np.empty_like(psi)
+            D.dirac_get_state(h, out)
+            return out
+        finally:
+            D.dirac_destroy(h)
+
+    assert np.array_equal(run(0, 0).view(np.uint8), run(1, 2).view(np.uint8))
+
+
 def test_tiles_inside_a_callers_capture():
     """A copy and the steps captured in a caller's graph and replayed: the same state as the calls made directly."""
     import torch
