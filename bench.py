@@ -42,21 +42,23 @@ import numpy as np  # noqa: E402
 FP64_BYTES_PER_POINT_STEP = 128  # 2-D, x-only table: 64 B read + 64 B written
 FP32_BYTES_PER_POINT_STEP = 64
 FLOPS_PER_POINT_STEP_2D = 56    # 32 adds (two sweeps) + 4 complex products of 6 flops
-FP64_INSTR_PER_POINT_STEP_2D = 48  # 32 DADD + 8 DMUL + 8 DFMA: what the FP64 pipe issues per 2-D point-step
-FP64_INSTR_PER_POINT_STEP_2D_FIELD = 80  # with a vector potential: 32 DADD + 12 complex multiply-adds of 4 DFMA
+# What the FP64 pipe issues per 2-D point-step: 16 of the 32 additions (the other half of each pair of sums runs on the
+# integer pipe, bit for bit; butterfly.cuh) + 8 DMUL + 8 DFMA.
+FP64_INSTR_PER_POINT_STEP_2D = 32
+FP64_INSTR_PER_POINT_STEP_2D_FIELD = 64  # with a vector potential: 16 DADD + 12 complex multiply-adds of 4 DFMA
 # FP64 issue roof from GB300's unit counts and clock: 1.25 TFLOP/s FP64 with a DFMA counted as two flops is two
 # FP64 instructions per SM per clock (DADD and DMUL issue at the DFMA rate): 2 x 152 SMs x 2.07 GHz.
 FP64_INSTR_PER_SM_CLOCK = 2
 SM_COUNT = 152
 FP64_ISSUE_PEAK_NOMINAL = FP64_INSTR_PER_SM_CLOCK * SM_COUNT * 2.07e9 / 1e12  # 0.629 T FP64 instructions/s
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of the step kernel on the 2048^2 workload, keyed
-# by (steps per launch, points per lane) of the captured variant (profiles/step_kernel_fp64_klein2048.md,
-# profiles/step_kernel_fp32_klein2048.md).  A variant without a capture reports null.
-MEASURED_TRAFFIC_PER_LAUNCH = {"fp64": {(1, 2): 277.539584e6 + 216.977408e6, (1, 4): 287.031808e6 + 217.295616e6},
-                               "fp32": {(2, 2): 152.147456e6 + 83.809024e6},
-                               "fx64": {(1, 1): 277.640448e6 + 217.100288e6}}
+# by (steps per launch, points per lane) of the captured variant
+# (profiles/step_kernels_two_pipes_pairs_tiles.md).  A variant without a capture reports null.
+MEASURED_TRAFFIC_PER_LAUNCH = {"fp64": {(1, 1): 277.649248e6 + 222.500720e6},
+                               "fp32": {(4, 2): 167.320192e6 + 88.742166e6},
+                               "fx64": {(1, 1): 277.561088e6 + 219.967744e6}}
 # ncu sm__pipe_fp64_cycles_active of the same captures (fraction of active cycles)
-MEASURED_FP64_PIPE = {(1, 2): 0.8311, (1, 4): 0.8297}
+MEASURED_FP64_PIPE = {(1, 1): 0.7937}
 
 
 def parse():
@@ -508,7 +510,7 @@ def main():
                                 "dT": (o32["flux_cum"] - fp64_flux) / n0}}
         D.dirac_destroy(h32)
         # the same FP32 step at one step per launch (k = 1, P = 2): it moves the full 64 B per point-step, so
-        # its HBM fraction is on its own traffic (the k = 2 plan above moves half of that and runs faster)
+        # its HBM fraction is on its own traffic (the plan above, several steps a launch, moves less and runs faster)
         c1 = D.make_config((args.side, 1, args.side), x_min=(x_min, 0.0, z_min), flux_face=face,
                            stream=stream.cuda_stream, device=local, precision=D.DIRAC_FP32, steps_per_launch=1,
                            points_per_lane=2)
@@ -587,7 +589,8 @@ def main():
             iv = D.dirac_get_info(hv)
             D.dirac_destroy(hv)
             vv = ncell * nv * world / (tv / 1e3)
-            instr = 80 if vname == "fp64_strang2d" else FP64_INSTR_PER_POINT_STEP_2D  # Strang: 4 sweeps + phase
+            # Strang: 4 sweeps + phase; shifts with two points a lane: all additions on the FP64 pipe
+            instr = 48 if vname == "fp64_strang2d" or iv["points_per_lane"] > 1 else FP64_INSTR_PER_POINT_STEP_2D
             if vname.startswith("fx64"):
                 variants[vname] = {
                     "value": vv, "unit": "point-steps/s", "steps": nv, "ms_per_step": tv / nv,
@@ -652,7 +655,7 @@ def main():
                         del fin, ref
                 D.dirac_destroy(h3)
                 v3 = n3 ** 3 * n_steps3 * world / (t3 / 1e3)
-                instr = 64 if split == D.DIRAC_LIE else 144
+                instr = 40 if split == D.DIRAC_LIE else 144  # first order: 24 of the 48 additions + phase
                 entry = {"value": v3, "unit": "point-steps/s", "steps": n_steps3, "ms_per_step": t3 / n_steps3,
                          "physical_time_per_step_dx_over_c": per_step,
                          "first_order_equivalent_point_steps_per_s": v3 * per_step,

@@ -78,7 +78,9 @@ typedef struct {
     int steps_per_launch; /* steps fused in one kernel launch (temporal block depth).  2-D: 1 or 2 for FP64,
                              1, 2 or 4 for FP32.  3-D first order: 1 or 2, 2 only in the fused pass
                              (points_per_lane 0); 3-D second order: 1.  0 = library choice (3-D: 2 for FP32
-                             storage, 1 for FP64) */
+                             storage, 1 for FP64; 2-D: with points_per_lane 0 too, small grids advance several
+                             steps of a tile per launch where that is faster; else 4, second order 2, for FP32
+                             and 1 for FP64 and fixed point) */
     int use_graphs;       /* 1: replay dirac_step's steady-state launches from a captured CUDA graph */
     int points_per_lane;  /* x cells per lane of the step kernel: 1, 2 or 4 (K = 2 needs 2 in FP64);
                              0 = library choice */
@@ -237,7 +239,7 @@ typedef struct {
     int points_per_lane;    /* x cells per lane in the step kernel */
     int64_t launch_warps;   /* warps in one step launch */
     int64_t strip_width;    /* x cells written by one warp */
-    int64_t segment_rows;   /* rows written by one warp */
+    int64_t segment_rows;   /* rows written by one warp (small 2-D grids: by one block's tile) */
     int graphs;             /* 1 when dirac_step replays a CUDA graph */
     int64_t kernel_launches;/* kernels enqueued by this grid so far (all kinds) */
     size_t device_bytes;    /* device memory owned by the grid */
@@ -302,7 +304,7 @@ typedef struct {
     int device;
     int steps_per_launch;   /* 0 = library choice */
     int points_per_lane;    /* 0 = library choice */
-    int64_t segment_rows;   /* rows per task; 0 = library choice */
+    int64_t segment_rows;   /* rows per task; 0 = library choice, for each launch's active runs */
     int use_graphs;         /* 1: the launch sequence of dirac_batch_run is captured once and replayed */
 } dirac_batch_config;
 

@@ -1015,6 +1015,8 @@ void default_plan(dirac_grid *g) {
         // the x-y pass + z/phase pass with that P; second order: points_per_lane 1 = eight single sweeps, 0 or 2 =
         // the fused passes (bandwidth-bound integer sweeps: the passes move a seventh of the single sweeps' bytes),
         // 4 = single x and y sweeps with one z-phase-z pass
+        // (64^3 and 96^3 the two passes with P = 1 are faster, 32.0 and 61 us a step against 40.3 and 74; the autotuner finds
+        // them)
         g->plan.fused3d = pp > 0 ? 0 : 1;
         g->plan.f_warps = 8;  // two blocks an SM (fused3d_kernels.cuh)
         g->plan.s3_fused = (strang(g) && pp != 1 && pp != 4) ? 1 : 0;
@@ -1025,8 +1027,12 @@ void default_plan(dirac_grid *g) {
         return;
     }
     if (ndim_of(g) == 3) {
-        // points_per_lane 0: the fused single-pass step; 1, 2 or 4: the x-y pass + z/phase pass with that P
-        g->plan.fused3d = pp > 0 ? 0 : 1;
+        // points_per_lane 0: the fused single-pass step; 1, 2 or 4: the x-y pass + z/phase pass with that P.  FP64, bound by
+        // its pipe, recomputes no halo rows in the two passes, whose one point a lane splits its sums over both pipes: the
+        // library's choice from about 60^3 (64^3 66.9 us a step against 81.4 fused, 256^3 1855 against 2330, 384^3 6301
+        // against 7281; 48^3 46.5 against 38.1)
+        const bool two64 = !g->fp32 && !strang(g) && !field_on(g) && k == 0 && pp == 0 && g->ncells > 200000;
+        g->plan.fused3d = pp > 0 || two64 ? 0 : 1;
         // FP64: 8-warp blocks, two on an SM (fused3d_kernels.cuh); FP32: 16, short y extents 8 (6-row tiles waste fewer
         // halo rows)
         g->plan.f_warps = !g->fp32 || g->cfg.n[1] <= 12 ? 8 : 16;
@@ -1042,7 +1048,7 @@ void default_plan(dirac_grid *g) {
         int K3 = 1;
         if (!strang(g) && (pp == 0 || field_on(g))) K3 = k == 2 ? 2 : (k == 1 ? 1 : (g->fp32 ? 2 : 1));
         // FP64 two-pass plan: 32 warps an SM of segments (8.75 against 8.2 G at 256^3 with 16)
-        make_plan(g, K3, pp > 0 ? pp : 2, 4, g->fp32 ? 16 : 32);
+        make_plan(g, K3, pp > 0 ? pp : (two64 ? 1 : 2), 4, g->fp32 ? 16 : 32);
         return;
     }
     if (sweep_mode(g) == 4) {

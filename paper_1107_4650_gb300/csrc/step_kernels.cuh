@@ -1,15 +1,16 @@
 // Fused sweep kernels of the split-operator Dirac scheme (Sec. 2.3, Eqs. sol_dis_1-sol_dis_4).
 //
-// Design (one warp = one independent strip, no shared memory, no block barrier):
-//   * a warp owns `strip_w` consecutive x cells of one plane and a segment of rows; it loads
-//     32*P cells per row (lane l holds cells xa + 32 j + l, j < P), i.e. K halo cells on each side;
+// Design (one warp = one independent strip with shared memory of its own, no block barrier):
+//   * a warp owns `strip_w` consecutive x cells of one plane and a segment of rows; it takes
+//     32*P cells per row (which of them a lane holds: PairedCells below), i.e. K halo cells on each side, from a
+//     ring of rows that bulk copies fill ahead of it;
 //   * it streams the rows of its segment (plus K halo rows at each end) through K pipelined
 //     levels held in registers: level s turns the step-(s-1) state of row q into the step-s state
 //     of row q-1, so one pass over HBM advances K steps (temporal blocking);
 //   * the x sweep needs cells x-1 and x+1: the characteristic sums u = a+b of the left neighbour
 //     and w = a-b of the right neighbour come from warp shuffles;
 //   * the second sweep (z in 2-D, y in the 3-D x-y pass) needs rows q-1 and q+1: each level keeps
-//     the "+" characteristic sums of the two previous rows in registers;
+//     the "+" characteristic sums of the two previous rows in registers or shared memory (HistSmem);
 //   * the ghost-zero boundary is imposed on every level's output (cells outside the grid are 0
 //     at every sub-step); a zero row stays zero through the x sweep, so one mask per level is
 //     exact.
@@ -423,7 +424,8 @@ template <int K, int MODE> struct Levels { static constexpr int value = (MODE ==
 //         table holding g = exp(-i V dt) / 16).
 // Resident 4-warp blocks per SM the register budget is fitted to (1: the compiler's choice).  Four (128 registers)
 // where the history in shared memory, or two rows per iteration (fixed point first order: 33.1 against 26.7 G at
-// 150 registers and 3 blocks), lets them fit; FP64's shared magnitude sums need the warps to fill both pipes.
+// 150 registers and 3 blocks), lets them fit; FP64's shared magnitude sums need the warps to fill both pipes, and the FP32
+// kernels of two and four levels to cover their latency (k = 4 at 2048^2 22.2 us a step with three blocks, 21.2 with four).
 template <typename T, int K, int P, int MODE> struct SweepMinBlocks {
     static constexpr int value = (IsFx<T>::value && K == 1 && P == 1 && (MODE == 0 || MODE == 2))             ? 4
                                  : (sizeof(T) == 4 && P == 2 && (MODE == 0 || MODE == 2) && Levels<K, MODE>::value >= 2) ? 4
@@ -544,9 +546,9 @@ __device__ __forceinline__ void push_row(Cx<T> (&s0)[2], Cx<T> (&s1)[2], Cx<T> (
 }
 
 // Which cells a lane holds: two adjacent ones (2 lane, 2 lane + 1; FP32 with two points a lane), whose inner neighbours need
-// no shuffle, or one in each group of 32 (32 j + lane).  The FP32 step of several levels is bound by the shared-memory pipe, which
-// shuffles (8 words a cell and level, 4 so), the sweep history and the row reads share, and by its latency: 2048^2 k = 4 24.8
-// -> 23.4 us a step, second order 44.1 -> 40.8; one level 48.4 -> 50.4, so not there.
+// no shuffle, or one in each group of 32 (32 j + lane).  The FP32 step of several levels is bound by the shared-memory pipe,
+// which shuffles (8 words a cell and level, 4 so), the sweep history and the row reads share, and by its latency: 2048^2
+// k = 4 24.8 -> 23.4 us a step, second order 44.1 -> 40.8; one level 48.4 -> 50.4, so not there.
 template <typename T, int P, int L> struct PairedCells { static constexpr bool value = sizeof(T) == 4 && P == 2 && L >= 2; };
 template <typename T, int P, int L> __device__ __forceinline__ int cell_of(int lane, int j) {
     return PairedCells<T, P, L>::value ? 2 * lane + j : 32 * j + lane;

@@ -14,7 +14,8 @@
 // through shared memory and the more chains a warp has, the better; two cells a lane gave nothing more).
 // Measured, us a step with the face flux, row kernel -> this: FP64 128^2 9.1 -> 4.9, 256^2 12.2 -> 9.0 (second order 32.8 ->
 // 14.9); FP32 128^2 4.2 -> 1.1, 512^2 5.9 -> 2.6, 1024^2 10.2 -> 6.3 (second order 256^2 7.8 -> 2.5); fixed point 256^2 7.2 ->
-// 3.6; in a uniform field, 300^2, FP64 25.0 -> 22.1 (second order 45.8 -> 33.6), FP32 6.6 -> 2.9 (10.9 -> 5.1).  A launch may begin while the one before it drains (256^2 FP32 1.5 -> 1.3 us a step).
+// 3.6; in a uniform field, 300^2, FP64 25.0 -> 22.1 (second order 45.8 -> 33.6), FP32 6.6 -> 2.9 (10.9 -> 5.1).  A launch may
+// begin while the one before it drains (256^2 FP32 1.5 -> 1.3 us a step).
 // Face flux: the two lanes at the face leave each row's sums in shared memory, and after the last step one warp takes all
 // rows of a sweep at once, lane = row (evaluated in each row's warp it cost 7 FP64 instructions a row and sweep: FP32 at
 // 256^2, K = 4, 4.0 us a step against 1.6).  Parts: [x sweeps][rows of the grid].
