@@ -447,8 +447,8 @@ int64_t tiles_of(const dirac_grid *g, const TileShape &t) {
 // The tile shape for a 2-D grid, or null where the row kernel is faster: least modelled time a step.  The
 // row kernel's time is taken as linear in its strips' cells (fitted from 128^2 to 4096^2), a launch of the tile kernel's as
 // linear in the tiles on the fullest SM.  The lines cross, us a step with rows / tiles, at about: FP64 640^2 (512^2 30.2 /
-// 28.4, 768^2 52.4 / 61), second order 900^2 (768^2 111 / 105, 1024^2 176 / 184), FP32 1500^2 (1024^2 9.5 / 6.3, 2048^2 21.2
-// / 23.7), second order 1200^2 (1024^2 16.3 / 12.2, 1600^2 26 / 29.5), fixed point 768^2 (512^2 12.7 / 10.4, 1024^2 32.8 /
+// 28.4, 768^2 52.4 / 61), second order 900^2 (768^2 111 / 105, 1024^2 176 / 184), FP32 1900^2 (1024^2 9.5 / 6.0, 2048^2 21.2
+// / 23), second order 1700^2 (1024^2 16.3 / 11.3, 1300^2 20.2 / 17), fixed point 768^2 (512^2 12.7 / 10.4, 1024^2 32.8 /
 // 36.5), second order 700^2 (512^2 21.9 / 17.0, 768^2 32.3 / 35.4).
 // With a uniform field (and an x-only table): FP64 350^2 (300^2 25.0 / 22.1, second order 45.8 / 33.6), FP32 1000^2 (300^2 6.6
 // / 3.0), second order 1400^2 (300^2 10.9 / 5.1).
@@ -742,7 +742,7 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
         a.nstrips = (a.nx + a.strip_w - 1) / a.strip_w;
         dirac_status st = flux_place(g, levels(g, K), a.nr, s, &a.flux_part);
         if (st != DIRAC_OK) return st;
-        cudaError_t e = launch_tile(a, *p.tile, K, s);
+        cudaError_t e = launch_tile(a, *p.tile, K, g->sm_count, s);
         if (e != cudaSuccess) return cuda_fail(g, e, "tile kernel launch");
         g->launches++;
         return DIRAC_OK;

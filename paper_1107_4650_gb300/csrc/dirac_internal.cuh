@@ -138,7 +138,7 @@ struct TileShape {
     double base, per_tile;  // microseconds of a launch: base + per_tile x tiles on the fullest SM
 };
 const TileShape *tile_shapes(int *count);
-cudaError_t launch_tile(const SweepArgs &a, const TileShape &t, int steps, cudaStream_t s);
+cudaError_t launch_tile(const SweepArgs &a, const TileShape &t, int steps, int sms, cudaStream_t s);
 
 // Characteristic-shift step kernel (mode 4: 2-D first-order step with c dt = S dx, one step per launch,
 // strips of 32 P - 2 S owned cells); S in 2..4, P in {1, 2}.

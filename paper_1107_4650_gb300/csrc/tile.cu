@@ -9,9 +9,9 @@ namespace dirac {
 // FP64 second order, bound by the FP64 pipe, does not.  Shapes that are no plan's run the steps that a plan's do not divide.
 #define DIRAC_TILE_SHAPES(X)                                                                                            \
     X(float, 16, 1, 4, false, 0, 1, 4.2, 1.12) X(float, 16, 1, 2, false, 0, 0, 0, 0) X(float, 16, 1, 1, false, 0, 0, 0, 0)       \
-    X(float, 8, 4, 4, false, 0, 1, 4.2, 1.85) X(float, 8, 4, 2, false, 0, 0, 0, 0) X(float, 8, 4, 1, false, 0, 0, 0, 0)          \
+    X(float, 8, 4, 4, false, 0, 1, 4.2, 1.68) X(float, 8, 4, 2, false, 0, 0, 0, 0) X(float, 8, 4, 1, false, 0, 0, 0, 0)          \
     X(float, 16, 1, 2, true, 0, 1, 3.1, 1.06) X(float, 16, 1, 1, true, 0, 0, 0, 0)                                            \
-    X(float, 8, 4, 2, true, 0, 1, 3.55, 1.8) X(float, 8, 4, 1, true, 0, 0, 0, 0)                                              \
+    X(float, 8, 4, 2, true, 0, 1, 3.55, 1.57) X(float, 8, 4, 1, true, 0, 0, 0, 0)                                              \
     X(double, 8, 1, 2, false, 0, 1, 3.1, 4.25) X(double, 8, 1, 1, false, 0, 0, 0, 0)                                           \
     X(double, 12, 1, 2, false, 0, 1, 2.2, 8.2) X(double, 12, 1, 1, false, 0, 0, 0, 0)                                         \
     X(double, 16, 1, 2, false, 0, 1, 2.3, 10.7) X(double, 16, 1, 1, false, 0, 0, 0, 0)                                        \
@@ -42,10 +42,10 @@ const TileShape *tile_shapes(int *count) {
     return shapes;
 }
 
-cudaError_t launch_tile(const SweepArgs &a, const TileShape &t, int steps, cudaStream_t s) {
+cudaError_t launch_tile(const SweepArgs &a, const TileShape &t, int steps, int sms, cudaStream_t s) {
 #define X(T, w, r, k, st, fld, plan, base, per)                                                                             \
     if (t.precision == precision_of<T>() && t.warps == w && t.rows == r && steps == k && (t.strang != 0) == st && t.field == fld) \
-        return a.periodic ? launch_tile_per<T, w, r, k, st, true, fld>(a, s) : launch_tile_per<T, w, r, k, st, false, fld>(a, s);
+        return a.periodic ? launch_tile_per<T, w, r, k, st, true, fld>(a, sms, s) : launch_tile_per<T, w, r, k, st, false, fld>(a, sms, s);
     DIRAC_TILE_SHAPES(X)
 #undef X
     return cudaErrorInvalidValue;

@@ -11,9 +11,10 @@
 // What bounds it: FP64 the FP64 pipe (0.33 us per row and step on an SM, 32 DADD-class instructions at about 20 clocks);
 // FP32 at one tile an SM the latency of a launch and of K dependent steps (5.3 us for four steps of 128^2), at several the
 // issue of about 60 instructions a cell and step (0.0135 us per row and step with R = 4, 0.018 with R = 1: the fewer rows go
-// through shared memory and the more chains a warp has, the better; two cells a lane gave nothing more).
+// through shared memory and the more chains a warp has, the better; two cells a lane gave nothing more), with three blocks of
+// 80 registers an SM (1024^2 6.3 -> 6.0 us a step against two, 1300^2 10.5 -> 9.2).
 // Measured, us a step with the face flux, row kernel -> this: FP64 128^2 9.1 -> 4.9, 256^2 12.2 -> 9.0 (second order 32.8 ->
-// 14.9); FP32 128^2 4.2 -> 1.1, 512^2 5.9 -> 2.6, 1024^2 10.2 -> 6.3 (second order 256^2 7.8 -> 2.5); fixed point 256^2 7.2 ->
+// 14.9); FP32 128^2 4.2 -> 1.1, 512^2 5.9 -> 2.5, 1024^2 10.2 -> 6.0 (second order 256^2 7.8 -> 2.5); fixed point 256^2 7.2 ->
 // 3.6; in a uniform field, 300^2, FP64 25.0 -> 22.1 (second order 45.8 -> 33.6), FP32 6.6 -> 2.9 (10.9 -> 5.1).  A launch may
 // begin while the one before it drains (256^2 FP32 1.5 -> 1.3 us a step).
 // Face flux: the two lanes at the face leave each row's sums in shared memory, and after the last step one warp takes all
@@ -26,7 +27,7 @@
 namespace dirac {
 
 template <typename T, int W, int R, int K, bool STRANG, bool PER, bool FIELD>
-__global__ void __launch_bounds__(32 * W, 1) tile_kernel(const SweepArgs a) {
+__global__ void __launch_bounds__(32 * W, (R == 4 ? 3 : 1)) tile_kernel(const SweepArgs a) {
     constexpr int ROWS = W * R;         // warp w holds rows w R .. w R + R - 1 of the tile
     constexpr int ZS = STRANG ? 2 : 1;  // x sweeps, and z sweeps, a step
     constexpr int H = ZS * K;
@@ -209,18 +210,22 @@ __global__ void __launch_bounds__(32 * W, 1) tile_kernel(const SweepArgs a) {
 }
 
 template <typename T, int W, int R, int K, bool STRANG, bool PER, bool FIELD>
-static cudaError_t launch_tile_per(const SweepArgs &a, cudaStream_t s) {
+static cudaError_t launch_tile_per(const SweepArgs &a, int sms, cudaStream_t s) {
     constexpr int H = STRANG ? 2 * K : K, OWNZ = W * R - 2 * H;
-    const int smem = (2 * 32 + R * H) * W * 4 * (int)sizeof(Cx<T>);
+    constexpr int need = (2 * 32 + R * H) * W * 4 * (int)sizeof(Cx<T>), two = 80 << 10, one = 120 << 10;
+    const int64_t tiles = a.nstrips * ((a.nr + OWNZ - 1) / OWNZ);
+    // Two tiles an SM: shared memory that keeps a third out, so that a launch which starts beside the one before it spreads
+    // over the chip instead of filling the SMs that drain first (384^2 FP32 2.08 us a step, 1.75 so).
+    const int smem = tiles <= 2 * (int64_t)sms && tiles > sms ? (need > two ? need : two) : need;
     static std::atomic<unsigned long long> done{0};
-    cudaError_t e = optin_smem(tile_kernel<T, W, R, K, STRANG, PER, FIELD>, smem, done);
+    cudaError_t e = optin_smem(tile_kernel<T, W, R, K, STRANG, PER, FIELD>, need > one ? need : one, done);
     if (e != cudaSuccess) return e;
     // may start while the launch before it drains, and waits for it before it reads the state
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(a.nstrips * ((a.nr + OWNZ - 1) / OWNZ)));
+    cfg.gridDim = dim3((unsigned)tiles);
     cfg.blockDim = dim3(32 * W);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
