@@ -161,6 +161,16 @@ double cell_volume(const dirac_grid *g) {
     return ndim_of(g) == 3 ? dx * dx * dx : dx * dx;
 }
 
+// A graph holds the arguments of its launches: the plan, the buffers' addresses, the kind of the table.  Called wherever one of
+// them changes.
+void drop_graphs(dirac_grid *g) {
+    for (auto &x : g->graph)
+        if (x) {
+            cudaGraphExecDestroy(x);
+            x = nullptr;
+        }
+}
+
 dirac_status ensure_table(dirac_grid *g, size_t bytes) {
     if (bytes <= g->table_cap) return DIRAC_OK;
     if (g->table) {
@@ -172,11 +182,7 @@ dirac_status ensure_table(dirac_grid *g, size_t bytes) {
     CK(g, cudaMalloc(&g->table, bytes));
     g->table_cap = bytes;
     g->device_bytes += bytes;
-    for (auto &x : g->graph)
-        if (x) {
-            cudaGraphExecDestroy(x);
-            x = nullptr;
-        }
+    drop_graphs(g);
     return DIRAC_OK;
 }
 
@@ -244,6 +250,7 @@ dirac_status upload_table(dirac_grid *g, const double *V, int layout, int64_t co
         CK(g, cudaMemcpyAsync(g->table, h.data(), bytes, cudaMemcpyHostToDevice, g->stream));
         CK(g, cudaStreamSynchronize(g->stream));
     }
+    if (g->table_full != (layout == DIRAC_V_FULL)) drop_graphs(g);
     g->table_full = (layout == DIRAC_V_FULL);
     return cellfield_on(g) ? upload_field_aux(g) : DIRAC_OK;
 }
@@ -422,11 +429,7 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         p.s3_z_seg_h = (nz + zz - 1) / zz;
         p.s3_z_nsegs = (nz + p.s3_z_seg_h - 1) / p.s3_z_seg_h;
     }
-    for (auto &x : g->graph)
-        if (x) {
-            cudaGraphExecDestroy(x);
-            x = nullptr;
-        }
+    drop_graphs(g);
 }
 
 int precision_index(const dirac_grid *g) { return g->fx ? 2 : (g->fp32 ? 1 : 0); }
@@ -948,8 +951,7 @@ dirac_status run_steps(dirac_grid *g, int64_t nsteps) {
 void release(dirac_grid *g) {
     if (!g) return;
     if (g->stream || g->cap_stream) cudaStreamSynchronize(g->stream);
-    for (auto &x : g->graph)
-        if (x) cudaGraphExecDestroy(x);
+    drop_graphs(g);
     if (!g->ext)
         for (auto &p : g->psi)
             if (p) cudaFree(p);
@@ -1485,11 +1487,7 @@ dirac_status dirac_set_field(dirac_grid *g, const double *a, const double *w, co
         if (st == DIRAC_OK) st = upload_field_aux(g);
     }
     if (st != DIRAC_OK) return st;
-    for (auto &x : g->graph)
-        if (x) {
-            cudaGraphExecDestroy(x);
-            x = nullptr;
-        }
+    drop_graphs(g);
     default_plan(g);
     return ensure_flux_part(g);
 }
