@@ -161,8 +161,8 @@ double cell_volume(const dirac_grid *g) {
     return ndim_of(g) == 3 ? dx * dx * dx : dx * dx;
 }
 
-// A graph holds the arguments of its launches: the plan, the buffers' addresses, the kind of the table.  Called wherever one of
-// them changes.
+// A graph holds the arguments of its launches: the plan, the buffers' addresses, the kind of the table, a fixed-point state's
+// scale (which multiplies the flux).  Called wherever one of them changes.
 void drop_graphs(dirac_grid *g) {
     for (auto &x : g->graph)
         if (x) {
@@ -970,6 +970,11 @@ void release(dirac_grid *g) {
     delete g;
 }
 
+void set_fx_shift(dirac_grid *g, int shift) {
+    if (g->fx_shift != shift) drop_graphs(g);
+    g->fx_shift = shift;
+}
+
 // DIRAC_FX64 state in: the complex128 state is copied to the idle ping-pong buffer, its discrete L2 norm A
 // (square root of the sum of |psi_c|^2 over all cells and components) reduced there, the shift chosen as
 // S = 60 - e in 2-D, 59 - e in 3-D, with A = m 2^e, m in [0.5, 1): each sweep (with its 1/2) and the phase
@@ -998,7 +1003,7 @@ dirac_status fx_load_state(dirac_grid *g, const void *psi, int on_device) {
     if (!std::isfinite(sumsq)) return fail(g, DIRAC_ERR_NONFINITE, "dirac_set_state: state holds NaN or Inf");
     int e = 0;
     if (sumsq > 0) std::frexp(std::sqrt(sumsq), &e);
-    g->fx_shift = (ndim_of(g) == 3 ? (strang(g) ? 57 : 59) : 60) - e;
+    set_fx_shift(g, (ndim_of(g) == 3 ? (strang(g) ? 57 : 59) : 60) - e);
     CK(g, launch_fx_encode(tmp, static_cast<long long *>(g->psi[g->cur]), g->ncells * 8, g->fx_shift, g->stream));
     return DIRAC_OK;
 }
@@ -1541,7 +1546,7 @@ dirac_status dirac_set_state_fx(dirac_grid *g, const int64_t *q, int shift, int 
     CK(g, cudaMemsetAsync(g->flux_dev, 0, sizeof(double), g->stream));
     CK(g, cudaMemsetAsync(g->ticket + 1, 0, sizeof(unsigned), g->stream));
     if (!on_device) CK(g, cudaStreamSynchronize(g->stream));
-    g->fx_shift = shift;
+    set_fx_shift(g, shift);
     g->step = 0;
     return DIRAC_OK;
 }

@@ -4,6 +4,7 @@
 // that it would touch has to be allocated still.
 #include <cuda_runtime.h>
 
+#include <cstdio>
 #include <cstdlib>
 #include <map>
 #include <string>
@@ -50,10 +51,15 @@ cudaError_t enqueue(std::string line, std::vector<Range> touched) {
     return cudaSuccess;
 }
 std::string n(long long v) { return " " + std::to_string(v); }
+std::string x(double v) {
+    char s[32];
+    snprintf(s, sizeof s, " %.17g", v);
+    return s;
+}
 // a step launch of any kernel: `parts` flux partials a step or sweep, `sums` of them, entries of `elem` bytes
 cudaError_t step(const std::string &what, const SweepArgs &a, int K, int64_t cells, int64_t parts, int sums, int elem) {
     std::string line = what + n(K) + n(a.strip_w) + n(a.nstrips) + n(a.nsegs) + n(a.seg_h) + n(a.full_table) + n(a.periodic) +
-                       n(a.ucoef_n ? a.step0 : -1) + " " + std::to_string(a.flux_unit * 1e12);
+                       n(a.ucoef_n ? a.step0 : -1) + x(a.flux_unit);
     std::vector<Range> t = {{a.in, (size_t)cells * 8 * elem}, {a.out, (size_t)cells * 8 * elem},
                             {a.table, (size_t)(a.full_table ? cells : a.nx) * 4 * elem},
                             {a.ucoef, (size_t)a.ucoef_n * 96}};
@@ -192,8 +198,8 @@ cudaError_t launch_fused3d(const SweepArgs &a, int precision, int warps, int ste
     return step("fused3d" + n(warps), a, steps, a.nx * ny * nz, a.nsegs, steps, precision == 1 ? 4 : 8);
 }
 cudaError_t launch_strang_xy(const SweepArgs &a, int precision, int warps, int nh, int64_t ny, int64_t nz, int64_t, int64_t, int64_t,
-                             int64_t, const double *, int, int, cudaStream_t) {
-    return step("strang_xy" + n(warps) + n(nh), a, 1, a.nx * ny * nz, a.nsegs, 2 * nh, precision == 1 ? 4 : 8);
+                             int64_t, const double *fscale, int, int, cudaStream_t) {
+    return step("strang_xy" + n(warps) + n(nh) + x(fscale[0]) + x(fscale[1]), a, 1, a.nx * ny * nz, a.nsegs, 2 * nh, precision == 1 ? 4 : 8);
 }
 cudaError_t launch_strang_z(const void *in, void *out, const void *table, int64_t nx, int64_t ny, int64_t nz, int, int full, const double *,
                             int64_t, int64_t, int64_t, int64_t, int precision, cudaStream_t) {
@@ -201,10 +207,10 @@ cudaError_t launch_strang_z(const void *in, void *out, const void *table, int64_
     return enqueue("strang_z" + n(full), {{in, c * 8 * e}, {out, c * 8 * e}, {table, (full ? c : (size_t)nx) * 4 * e}});
 }
 cudaError_t launch_axis(const void *in, void *out, const void *table, int64_t nx, int64_t ny, int64_t nz, int axis, int64_t, int, int full,
-                        int phase, int64_t flux_face, double, double *flux_part, const double *, int64_t, int64_t, int precision, int,
+                        int phase, int64_t flux_face, double fscale, double *flux_part, const double *, int64_t, int64_t, int precision, int,
                         int blocks, cudaStream_t) {
     const size_t e = precision == 1 ? 4 : 8, c = (size_t)(nx * ny * nz);
-    return enqueue("axis" + n(axis) + n(phase) + n(full), {{in, c * 8 * e}, {out, c * 8 * e}, {table, (full ? c : (size_t)nx) * 4 * e},
+    return enqueue("axis" + n(axis) + n(phase) + n(full) + x(fscale), {{in, c * 8 * e}, {out, c * 8 * e}, {table, (full ? c : (size_t)nx) * 4 * e},
                                                            {flux_part, flux_face >= 0 ? blocks * sizeof(double) : 0}});
 }
 cudaError_t launch_axis_cellfield(const AxisArgs &, int, int, cudaStream_t) { return enqueue("cellfield", {}); }

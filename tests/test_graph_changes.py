@@ -70,3 +70,18 @@ def test_potential_of_another_kind(fake, precision, n, splitting):
 
     _same_with_and_without(fake, change, n=n, ndim=3 if n[1] > 1 else 2, precision=precision, splitting=splitting,
                            flux_face=n[0] // 2)
+
+
+@pytest.mark.parametrize("splitting", [0, 1])
+@pytest.mark.parametrize("n,points", [((40, 1, 33), 0), ((2000, 1, 1500), 0), ((20, 12, 16), 0), ((20, 12, 16), 1)])
+def test_fixed_point_state_of_another_scale(fake, n, points, splitting):
+    q = np.zeros(n[::-1] + (4, 2), dtype=np.int64)
+    psi = np.zeros(n[::-1] + (4,), dtype=np.complex128)
+
+    def change(h):
+        for shift in (50, 43, None, 50):
+            D.dirac_set_state(h, psi) if shift is None else D.dirac_set_state_fx(h, q, shift)
+            D.dirac_step(h, 32 * D.dirac_get_info(h)["steps_per_launch"])
+
+    _same_with_and_without(fake, change, n=n, ndim=3 if n[1] > 1 else 2, precision=2, splitting=splitting, points_per_lane=points,
+                           flux_face=n[0] // 2)

@@ -37,3 +37,18 @@ def test_potential_of_another_kind(n, precision):
             D.dirac_step(h, 32 * D.dirac_get_info(h)["steps_per_launch"])
 
     _same_with_and_without(change, psi, ndim=3 if n[1] > 1 else 2, precision=precision)
+
+
+@pytest.mark.parametrize("splitting", [0, 1])
+@pytest.mark.parametrize("n", [(96, 1, 80), (20, 12, 16)])
+def test_fixed_point_state_of_another_norm(n, splitting):
+    from paper_1107_4650_gb300 import workloads as W
+    psi = W.random_state(n[2], n[1], n[0], 3)
+
+    def change(D, h):
+        steps = 32 * D.dirac_get_info(h)["steps_per_launch"]
+        D.dirac_step(h, steps)
+        D.dirac_set_state(h, psi * 37.0)
+        D.dirac_step(h, steps)
+
+    _same_with_and_without(change, psi, ndim=3 if n[1] > 1 else 2, precision=2, splitting=splitting)
