@@ -171,19 +171,24 @@ void drop_graphs(dirac_grid *g) {
         }
 }
 
+// Grows a device buffer of the grid to `bytes` (its contents are lost).  The new one is allocated before the old one is freed,
+// so that a call that runs out of memory leaves the grid with the buffer that its next steps use.
+template <typename T> dirac_status grow(dirac_grid *g, T *&dev, size_t &cap, size_t bytes) {
+    if (bytes <= cap) return DIRAC_OK;
+    T *fresh = nullptr;
+    CK(g, cudaMalloc((void **)&fresh, bytes));
+    if (dev) cudaFree(dev);
+    g->device_bytes += bytes - cap;
+    dev = fresh;
+    cap = bytes;
+    return DIRAC_OK;
+}
+
 dirac_status ensure_table(dirac_grid *g, size_t bytes) {
     if (bytes <= g->table_cap) return DIRAC_OK;
-    if (g->table) {
-        cudaFree(g->table);
-        g->device_bytes -= g->table_cap;
-        g->table = nullptr;
-        g->table_cap = 0;
-    }
-    CK(g, cudaMalloc(&g->table, bytes));
-    g->table_cap = bytes;
-    g->device_bytes += bytes;
-    drop_graphs(g);
-    return DIRAC_OK;
+    dirac_status st = grow(g, g->table, g->table_cap, bytes);
+    if (st == DIRAC_OK) drop_graphs(g);
+    return st;
 }
 
 dirac_status upload_field_aux(dirac_grid *g);
@@ -258,18 +263,15 @@ dirac_status upload_table(dirac_grid *g, const double *V, int layout, int64_t co
 // Copies n doubles from the host to a device array of the grid, (re)allocating it to fit; n = 0 frees it.
 dirac_status put_doubles(dirac_grid *g, double *&dev, size_t &bytes, const double *host, size_t n) {
     const size_t need = n * sizeof(double);
-    if (need == 0 || need > bytes) {
-        if (dev) {
-            cudaFree(dev);
-            g->device_bytes -= bytes;
-        }
+    if (need == 0) {
+        if (dev) cudaFree(dev);
+        g->device_bytes -= bytes;
         dev = nullptr;
         bytes = 0;
-        if (need == 0) return DIRAC_OK;
-        CK(g, cudaMalloc(&dev, need));
-        bytes = need;
-        g->device_bytes += need;
+        return DIRAC_OK;
     }
+    dirac_status st = grow(g, dev, bytes, need);
+    if (st != DIRAC_OK) return st;
     CK(g, cudaMemcpyAsync(dev, host, need, cudaMemcpyHostToDevice, g->stream));
     CK(g, cudaStreamSynchronize(g->stream));
     return DIRAC_OK;
@@ -503,16 +505,10 @@ dirac_status ensure_flux_part(dirac_grid *g) {
         }
     // room for 32 launches between folds, within 4 MB (a launch that leaves more is folded by itself)
     need = std::max(need, std::min<size_t>(32 * need, (size_t)1 << 19));
-    if (need <= g->flux_part_cap) return DIRAC_OK;
-    if (g->flux_part) {
-        cudaFree(g->flux_part);
-        g->device_bytes -= g->flux_part_cap * sizeof(double);
-    }
-    g->flux_part = nullptr;
-    CK(g, cudaMalloc(&g->flux_part, need * sizeof(double)));
-    g->flux_part_cap = need;
-    g->device_bytes += need * sizeof(double);
-    return DIRAC_OK;
+    size_t bytes = g->flux_part_cap * sizeof(double);
+    dirac_status st = grow(g, g->flux_part, bytes, need * sizeof(double));
+    g->flux_part_cap = bytes / sizeof(double);
+    return st;
 }
 
 // Folds what the launches since the last fold have left.
@@ -1393,9 +1389,15 @@ dirac_status dirac_set_potential(dirac_grid *g, const double *V, int layout, int
     }
     for (int64_t i = 0; i < count; ++i)
         if (!std::isfinite(V[i])) return fail(g, DIRAC_ERR_ARG, "potential holds a non-finite value");
-    g->v_host.assign(V, V + count);
-    g->v_layout = layout;
-    return upload_table(g, V, layout, count);
+    std::vector<double> before(V, V + count);
+    before.swap(g->v_host);
+    std::swap(g->v_layout, layout);
+    dirac_status st = upload_table(g, V, g->v_layout, count);
+    if (st != DIRAC_OK) {  // the potential that the table holds still
+        g->v_host.swap(before);
+        g->v_layout = layout;
+    }
+    return st;
 }
 
 dirac_status dirac_set_absorber(dirac_grid *g, const double *a, int64_t count) {
@@ -1426,22 +1428,13 @@ dirac_status dirac_set_vector_potential(dirac_grid *g, const double *A_tilde, in
         for (int64_t i = 0; i < 3 * nsteps_table; ++i)
             if (!std::isfinite(A_tilde[i])) return fail(g, DIRAC_ERR_ARG, "vector-potential table holds a non-finite value");
     CK(g, cudaSetDevice(g->cfg.device));
-    const bool field_before = field_on(g);
+    const std::vector<double> before = g->avec;
     if (clear) {
         g->avec.clear();
     } else {
         const size_t bytes = (size_t)nsteps_table * 12 * sizeof(double);
-        if (bytes > g->ucoef_cap) {
-            if (g->ucoef) {
-                cudaFree(g->ucoef);
-                g->device_bytes -= g->ucoef_cap;
-                g->ucoef = nullptr;
-                g->ucoef_cap = 0;
-            }
-            CK(g, cudaMalloc(&g->ucoef, bytes));
-            g->ucoef_cap = bytes;
-            g->device_bytes += bytes;
-        }
+        dirac_status st = grow(g, g->ucoef, g->ucoef_cap, bytes);
+        if (st != DIRAC_OK) return st;
         const double mu = g->cfg.m * g->cfg.c * g->cfg.c * g->dt;
         std::vector<double> h((size_t)nsteps_table * 12);
         for (int64_t n = 0; n < nsteps_table; ++n) u_entries(mu, A_tilde + 3 * n, &h[(size_t)n * 12]);
@@ -1449,10 +1442,14 @@ dirac_status dirac_set_vector_potential(dirac_grid *g, const double *A_tilde, in
         CK(g, cudaStreamSynchronize(g->stream));
         g->avec.assign(A_tilde, A_tilde + 3 * nsteps_table);
     }
-    if (field_on(g) != field_before) {
+    if (field_on(g) == before.empty()) {
         default_plan(g);
         dirac_status st = ensure_flux_part(g);
-        if (st != DIRAC_OK) return st;
+        if (st != DIRAC_OK) {
+            g->avec = before;
+            default_plan(g);
+            return st;
+        }
         const bool have_v = g->v_layout != DIRAC_V_NONE && !g->v_host.empty();
         return upload_table(g, have_v ? g->v_host.data() : nullptr, have_v ? g->v_layout : DIRAC_V_NONE,
                             have_v ? (int64_t)g->v_host.size() : 0);
@@ -1775,6 +1772,7 @@ dirac_status dirac_autotune(dirac_grid *g) {
     Cand best = {g->plan.K, g->plan.P, g->plan.wpb, 0, g->plan.fused3d ? g->plan.f_warps : 0,
                  g->plan.s3_fused ? g->plan.s3_warps : 0, g->plan.s3_zfactor, g->plan.s3_zpass};
     double best_t = 1e300;
+    const Plan plan_saved = g->plan;
     const int use_graphs = g->cfg.use_graphs;
     g->cfg.use_graphs = 0;
     g->tuning = true;
@@ -1825,6 +1823,7 @@ dirac_status dirac_autotune(dirac_grid *g) {
             make_plan(g, best.K, best.P, best.wpb, best.wsm);
         st = ensure_flux_part(g);
     }
+    if (st != DIRAC_OK) g->plan = plan_saved;  // the scratch has not shrunk
     g->cur = cur_saved;
     cudaMemcpyAsync(g->psi[g->cur], backup, bytes, cudaMemcpyDeviceToDevice, g->stream);
     g->host_obs[6] = flux_saved;

@@ -85,3 +85,27 @@ def test_fixed_point_state_of_another_scale(fake, n, points, splitting):
 
     _same_with_and_without(fake, change, n=n, ndim=3 if n[1] > 1 else 2, precision=2, splitting=splitting, points_per_lane=points,
                            flux_face=n[0] // 2)
+
+
+@pytest.mark.parametrize("precision,n,what", [(1, (2048, 1, 2048), "scratch"), (0, (1536, 1, 1536), "scratch"), (0, (40, 1, 40), "field"),
+                                              (1, (24, 24, 24), "field"), (1, (2048, 1, 2048), "table"), (0, (40, 1, 40), "table")])
+def test_steps_after_a_failed_allocation(fake, precision, n, what):
+    """A call that runs out of memory leaves a grid whose next steps touch nothing that was freed."""
+    def change(h):
+        steps = 32 * D.dirac_get_info(h)["steps_per_launch"]
+        if what == "field":
+            D.dirac_set_vector_potential(h, np.zeros((2 * steps, 3)))
+        D.dirac_step(h, steps)
+        fake.fake_limit(96 * 600 if what == "scratch" else 0)  # (room for the field's table alone)
+        with pytest.raises(D.DiracError) as e:
+            if what == "table":
+                D.dirac_set_potential(h, np.zeros(n[::-1]), D.DIRAC_V_FULL)
+            else:
+                D.dirac_set_vector_potential(h, np.zeros((600 if what == "scratch" else 5 * steps, 3)))
+        assert e.value.status == D.DIRAC_ERR_OOM
+        fake.fake_limit(2 ** 64 - 1)
+        D.dirac_step(h, steps)
+
+    for graphs in (0, 1):
+        log, bad = _launches(fake, change, graphs, n=n, ndim=3 if n[1] > 1 else 2, precision=precision, flux_face=n[0] // 2)
+        assert bad == 0, [l for l in log if "freed" in l][:2]
