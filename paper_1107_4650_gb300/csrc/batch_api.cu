@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <numeric>
 #include <string>
@@ -85,7 +86,8 @@ dirac_status bcuda(dirac_batch *b, cudaError_t e, const char *where) {
 
 template <typename P>
 dirac_status balloc(dirac_batch *b, P **p, size_t bytes) {
-    cudaError_t e = cudaMalloc((void **)p, std::max<size_t>(bytes, 16));
+    // (failure-detection test hook: allocations fail under DIRAC_INJECT_OOM)
+    cudaError_t e = std::getenv("DIRAC_INJECT_OOM") ? cudaErrorMemoryAllocation : cudaMalloc((void **)p, std::max<size_t>(bytes, 16));
     if (e != cudaSuccess) return bcuda(b, e, "cudaMalloc");
     b->device_bytes += std::max<size_t>(bytes, 16);
     return DIRAC_OK;
@@ -145,13 +147,14 @@ dirac_status plan(dirac_batch *b) {
     b->flux_stride = (int64_t)need;
     need *= kBatchSlots;
     if (need > b->flux_part_n) {
+        double *fresh = nullptr;  // before the old pool goes: a plan made earlier fits it still
+        dirac_status st = balloc(b, &fresh, need * sizeof(double));
+        if (st != DIRAC_OK) return st;
         if (b->flux_part_pool) {
             cudaFree(b->flux_part_pool);
             b->device_bytes -= b->flux_part_n * sizeof(double);
         }
-        b->flux_part_pool = nullptr;
-        dirac_status st = balloc(b, &b->flux_part_pool, need * sizeof(double));
-        if (st != DIRAC_OK) return st;
+        b->flux_part_pool = fresh;
         b->flux_part_n = need;
     }
     size_t off = 0;
@@ -657,14 +660,16 @@ dirac_status dirac_batch_autotune(dirac_batch *b) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    b->K = best.K;
-    b->P = best.P;
-    b->seg_rows = best.seg;
+    // after a failure the plan that was there, whose scratch is allocated; the states are new either way
+    const Cand &use = st == DIRAC_OK ? best : keep;
+    b->K = use.K;
+    b->P = use.P;
+    b->seg_rows = use.seg;
+    const std::string failed = b->err;
     dirac_status st2 = plan(b);
-    if (st == DIRAC_OK) st = st2;
-    if (st == DIRAC_OK) st = upload_tables(b);
-    if (st == DIRAC_OK) st = init_states(b);
-    return st;
+    if (st2 == DIRAC_OK) st2 = upload_tables(b);
+    if (st2 == DIRAC_OK) st2 = init_states(b);
+    return st == DIRAC_OK ? st2 : bfail(b, st, failed);
 }
 
 dirac_status dirac_batch_get_info(const dirac_batch *b, dirac_batch_info *info) {
