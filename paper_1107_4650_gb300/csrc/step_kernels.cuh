@@ -808,7 +808,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     }
     __syncwarp();
     if (lane == 0) fence_proxy_async();  // the previous task's reads of the slots (batch_kernels.cuh) before this one's copies
-    bool stall = a.inject_stall && wid == 0 && !per;
+    bool stall = a.inject_stall && wid == 0;
 #pragma unroll
     for (int sl = 0; sl < RG::SLOTS; ++sl) {
         const RI r = r_first + sl;
