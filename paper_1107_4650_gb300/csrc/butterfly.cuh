@@ -25,12 +25,20 @@ namespace dirac {
 
 // |x| + |y| with x's sign, as bits.  The larger mantissa's leading bit sits at bit 62 with ten guard bits below; the
 // smaller one is shifted down by the exponents' difference, its lost bits jammed into bit 0; the sum's leading bit is
-// bit 62 or 63 (or lower for subnormals), so the rounding position is bit 10 or 11.  A NaN whose payload lies in its
-// low word alone may come out as infinity; the pair's other result, formed by the FP64 pipe, is then a NaN.
+// bit 62 or 63 (or lower for subnormals), so the rounding position is bit 10 or 11.
 DIRAC_HD uint64_t magnitude_sum_bits(uint64_t x, uint64_t y) {
     const uint32_t xh = (uint32_t)(x >> 32), xl = (uint32_t)x, yh = (uint32_t)(y >> 32), yl = (uint32_t)y;
     const uint32_t xa = xh & 0x7fffffffu, ya = yh & 0x7fffffffu;
-    const bool sw = xa < ya;  // equal high words: the exponents agree and the order does not matter
+    // The larger magnitude by all 63 bits: with equal high words the order matters to an infinity and a NaN alone (the NaN is
+    // the larger).  By a subtraction with borrow: FP64 2048^2 303 us a step, 580 by a comparison of 64-bit integers, 303 by
+    // one of the high words, which took such a NaN for the smaller.
+    int borrow;
+#ifdef __CUDA_ARCH__
+    asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %2;\n\tsubc.u32 %0, %3, %4;\n\t}" : "=r"(borrow) : "r"(xl), "r"(yl), "r"(xa), "r"(ya));
+#else
+    borrow = -(((uint64_t)xa << 32 | xl) < ((uint64_t)ya << 32 | yl));
+#endif
+    const bool sw = borrow < 0;
     const uint32_t bh = sw ? ya : xa, bl = sw ? yl : xl, sh = sw ? xa : ya, sl = sw ? xl : yl;
     // exponents less one, zero for subnormals too: high word - (e << 20) is the mantissa with its hidden bit
     const int be = (int)(bh >> 20) - 1 > 0 ? (int)(bh >> 20) - 1 : 0, se = (int)(sh >> 20) - 1 > 0 ? (int)(sh >> 20) - 1 : 0;
