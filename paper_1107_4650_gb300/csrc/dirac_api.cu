@@ -332,8 +332,12 @@ RowTime row_time_of(const dirac_grid *g, int K, int P) {
     // the second level of a second-order step has no phase (FP64: the phase is a third of the first's FP64 work)
     const double lv = strang(g) ? (g->fp32 || g->fx ? 1.5 : 2.0) * K : K;
     RowTime t = g->fx ? RowTime{1.03, 0.129} : (g->fp32 ? RowTime{0.5, 0.033} : RowTime{2.1, 0.31});
+    // FP64, two points a lane: a row is one long chain whoever else runs (9.1 us a row of the second-order step with one block
+    // on an SM, 11.5 with two), so a wave of short segments beats half a wave of long ones (1024^2 in a uniform field, second
+    // order: 16 rows 292 us a step, 32 rows 381; 777 x 1000 11 rows 164, 22 rows 235)
+    if (!g->fp32 && !g->fx && P == 2) t = RowTime{5.0, 0.21};
     t.lat *= lv * (matrix ? 1.4 : 1.0);
-    t.thr *= lv * P * (matrix ? 1.7 : 1.0) * (!g->fp32 && !g->fx && P > 1 ? 1.4 : 1.0);
+    t.thr *= lv * P * (matrix ? 1.7 : 1.0) * (!g->fp32 && !g->fx && P > 2 ? 1.4 : 1.0);
     return t;
 }
 // 4-warp blocks of the 2-D step resident on an SM (SweepMinBlocks; FP32 with one point a lane and one step fits five).
@@ -363,8 +367,10 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
     if (model) {
         const RowTime rt = row_time_of(g, K, P);
         // a wave's blocks end apart: FP32 at 4096^2, k = 2, 165 G point-steps/s in one wave, 170-175 in two to four; at
-        // 2048^2 145 in one, 130 in two; fixed point at 2048^2 33.7 in one, 32.8 in two
-        p.seg_h = pick_rows(nr, p.nstrips * planes, wpb, g->sm_count, resident_blocks(g, K, P), 2.0 * Lv, g->fp32 ? 0.2 : 0.1,
+        // 2048^2 145 in one, 130 in two; fixed point at 2048^2 33.7 in one, 32.8 in two; FP64 with two points a lane, second
+        // order at 2048^2: 767 us a step in one wave of 61 rows, 805 in two of 30
+        const double uneven = g->fp32 ? 0.2 : (!g->fx && P == 2 ? 0.0 : 0.1);
+        p.seg_h = pick_rows(nr, p.nstrips * planes, wpb, g->sm_count, resident_blocks(g, K, P), 2.0 * Lv, uneven,
                             [&](int64_t blocks) { return rt(blocks * wpb); });
     } else {
         int64_t nsegs = std::max<int64_t>(1, want / std::max<int64_t>(1, p.nstrips * planes));
