@@ -1088,7 +1088,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
 
 // 3-D z sweep + phase: one thread per (x, y) column and z segment; the input is 4x the x-y swept
 // state, the table carries 1/8, so the output is the state after the full step.
-template <typename T>
+template <typename T, bool FULL>
 __global__ void __launch_bounds__(128) zphase_kernel(const ZArgs a) {
     const int64_t ncol = a.nx * a.ny;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1104,16 +1104,17 @@ __global__ void __launch_bounds__(128) zphase_kernel(const ZArgs a) {
     T *out = static_cast<T *>(a.out);
     const T *tab = static_cast<const T *>(a.table);
     Cx<T> pu, pd;
-    if (!a.full_table) load_tab(tab + x * 4, pu, pd);
+    if (!FULL) load_tab(tab + x * 4, pu, pd);
     Cx<T> UA[2] = {{T(0), T(0)}, {T(0), T(0)}}, UB[2] = {{T(0), T(0)}, {T(0), T(0)}};
     for (int64_t z = z_begin - 1; z <= z_end; ++z) {
         Cx<T> s[4];
         const bool ok = per || (z >= 0 && z < nz);
         const int64_t zo = z - 1;
         // the table's entry asked for before the state: at its use below, each plane waited for it in turn (200^3 with a full
-        // table, two-pass plan, FP32 332 us a step, 249 so; fixed point 610 and 525)
+        // table, two-pass plan, FP32 332 us a step, 249 so; fixed point 610 and 525; in a variant of its own, since the
+        // per-column one is 2 % slower with it)
         Cx<T> qu = pu, qd = pd;
-        if (a.full_table && zo >= z_begin && zo < z_end) load_tab(tab + (zo * ncol + col) * 4, qu, qd);
+        if (FULL && zo >= z_begin && zo < z_end) load_tab(tab + (zo * ncol + col) * 4, qu, qd);
         if (ok) {
             const int64_t zl = per ? pmod(z, nz) : z;
             load_pt(in + (zl * ncol + col) * 8, s);

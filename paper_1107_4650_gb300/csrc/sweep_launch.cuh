@@ -30,7 +30,10 @@ static cudaError_t launch_zphase(const ZArgs &a, int threads, cudaStream_t s) {
     const int64_t n = a.nx * a.ny * a.nsegs;
     const int64_t blocks = (n + threads - 1) / threads;
     if (blocks <= 0) return cudaSuccess;
-    zphase_kernel<T><<<(unsigned)blocks, threads, 0, s>>>(a);
+    if (a.full_table)
+        zphase_kernel<T, true><<<(unsigned)blocks, threads, 0, s>>>(a);
+    else
+        zphase_kernel<T, false><<<(unsigned)blocks, threads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
