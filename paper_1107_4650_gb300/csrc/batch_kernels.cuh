@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(128, BatchHist<T, K, P>::blocks) batch_kernel(
         a.flux_unit = 1.0;  // floating-point states
         a.wide = 1;         // the pool is the library's own, a cell 32 or 64 bytes
         sweep_warp<T, K, P, 0, false, BatchHist<T, K, P>::unroll, BatchHist<T, K, P>::value>(a, (int64_t)task - b.task_off[lo], lane, wsmem);
+        if (lane == 0) fence_proxy_async();  // this task's reads of the row slots before the next one's first copies into them
     }
 }
 

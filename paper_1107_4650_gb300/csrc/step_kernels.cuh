@@ -807,7 +807,6 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                 if (!xin[j]) store_pt(reinterpret_cast<T *>(wsmem + 128 + sl * RG::ROW_BYTES) + cell_of<T, P, L>(lane, j) * 8, none);
     }
     __syncwarp();
-    if (lane == 0) fence_proxy_async();  // the previous task's reads of the slots (batch_kernels.cuh) before this one's copies
     bool stall = a.inject_stall && wid == 0;
 #pragma unroll
     for (int sl = 0; sl < RG::SLOTS; ++sl) {
