@@ -335,14 +335,21 @@ RowTime row_time_of(const dirac_grid *g, int K, int P) {
     // FP64, two points a lane: a row is one long chain whoever else runs (9.1 us a row of the second-order step with one block
     // on an SM, 11.5 with two), so a wave of short segments beats half a wave of long ones (1024^2 in a uniform field, second
     // order: 16 rows 292 us a step, 32 rows 381; 777 x 1000 11 rows 164, 22 rows 235)
-    if (!g->fp32 && !g->fx && P == 2) t = RowTime{5.0, 0.21};
+    // (a shift step: 3.3 and 4.9)
+    if (!g->fp32 && !g->fx && P == 2) t = mode == 4 ? RowTime{2.9, 0.24} : RowTime{5.0, 0.21};
     t.lat *= lv * (matrix ? 1.4 : 1.0);
     t.thr *= lv * P * (matrix ? 1.7 : 1.0) * (!g->fp32 && !g->fx && P > 2 ? 1.4 : 1.0);
     return t;
 }
 // 4-warp blocks of the 2-D step resident on an SM (SweepMinBlocks; FP32 with one point a lane and one step fits five).
 int resident_blocks(const dirac_grid *g, int K, int P) {
-    if (sweep_mode(g) == 4) return g->fp32 ? 4 : (P == 1 ? 3 : 2);
+    if (sweep_mode(g) == 4) {
+        // by their registers, [FP32][shift - 2][P - 1][field] (FP32 taken for four blocks, shift 4 at 2048^2 ran two waves of 32
+        // rows, 77.5 us a step, where one of 64 takes 70.6)
+        static const int blocks[2][3][2][2] = {{{{3, 3}, {2, 2}}, {{3, 2}, {2, 2}}, {{2, 2}, {2, 2}}},
+                                               {{{4, 4}, {3, 2}}, {{4, 3}, {2, 2}}, {{3, 3}, {2, 2}}}};
+        return blocks[g->fp32][char_shift(g) - 2][P - 1][field_on(g) ? 1 : 0];
+    }
     if (P == 1) return g->fp32 && K == 1 ? 5 : 4;
     if (P == 4) return 2;
     return g->fp32 ? 4 : 2;
@@ -369,7 +376,7 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         // a wave's blocks end apart: FP32 at 4096^2, k = 2, 165 G point-steps/s in one wave, 170-175 in two to four; at
         // 2048^2 145 in one, 130 in two; fixed point at 2048^2 33.7 in one, 32.8 in two; FP64 with two points a lane, second
         // order at 2048^2: 767 us a step in one wave of 61 rows, 805 in two of 30
-        const double uneven = g->fp32 ? 0.2 : (!g->fx && P == 2 ? 0.0 : 0.1);
+        const double uneven = sweep_mode(g) == 4 ? 0.1 : (g->fp32 ? 0.2 : (!g->fx && P == 2 ? 0.0 : 0.1));
         p.seg_h = pick_rows(nr, p.nstrips * planes, wpb, g->sm_count, resident_blocks(g, K, P), 2.0 * Lv, uneven,
                             [&](int64_t blocks) { return rt(blocks * wpb); });
     } else {

@@ -21,3 +21,10 @@ def _rows(field=False, **cfg):
                                            ((777, 1, 1000), False, 11, 12), ((1500, 1, 1100), False, 22, 24)])
 def test_fp64_second_order_two_points_a_lane(fake, n, field, lo, hi):  # noqa: F811
     assert lo <= _rows(field, n=n, splitting=D.DIRAC_STRANG, points_per_lane=2, steps_per_launch=1) <= hi
+
+
+@pytest.mark.parametrize("shift,n,lo,hi", [(3, (2048, 1, 2048), 63, 66), (4, (2048, 1, 2048), 63, 66), (3, (1800, 1, 1700), 45, 48),
+                                           (4, (1800, 1, 1700), 48, 52)])
+def test_fp32_shifts_fill_one_wave(fake, shift, n, lo, hi):  # noqa: F811
+    """Two blocks of four warps fit an SM: segments whose warps fill 2 x 152 blocks once."""
+    assert lo <= _rows(n=n, precision=D.DIRAC_FP32, char_shift=shift) <= hi
