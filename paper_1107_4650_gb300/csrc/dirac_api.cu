@@ -337,6 +337,8 @@ RowTime row_time_of(const dirac_grid *g, int K, int P) {
     // order: 16 rows 292 us a step, 32 rows 381; 777 x 1000 11 rows 164, 22 rows 235)
     // (a shift step: 3.3 and 4.9)
     if (!g->fp32 && !g->fx && P == 2) t = mode == 4 ? RowTime{2.9, 0.24} : RowTime{5.0, 0.21};
+    // (fixed point, four: 4.3 us a row; 1024^2 16 rows 98 us a step, 8 rows 74)
+    if (g->fx && P == 4) t = RowTime{4.2, 0.116};
     t.lat *= lv * (matrix ? 1.4 : 1.0);
     t.thr *= lv * P * (matrix ? 1.7 : 1.0) * (!g->fp32 && !g->fx && P > 2 ? 1.4 : 1.0);
     return t;

@@ -28,3 +28,8 @@ def test_fp64_second_order_two_points_a_lane(fake, n, field, lo, hi):  # noqa: F
 def test_fp32_shifts_fill_one_wave(fake, shift, n, lo, hi):  # noqa: F811
     """Two blocks of four warps fit an SM: segments whose warps fill 2 x 152 blocks once."""
     assert lo <= _rows(n=n, precision=D.DIRAC_FP32, char_shift=shift) <= hi
+
+
+@pytest.mark.parametrize("n,lo,hi", [((1024, 1, 1024), 8, 11), ((520, 1, 384), 2, 3)])
+def test_fixed_point_four_points_a_lane(fake, n, lo, hi):  # noqa: F811
+    assert lo <= _rows(n=n, precision=D.DIRAC_FX64, points_per_lane=4, steps_per_launch=1) <= hi
