@@ -659,9 +659,12 @@ __device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, c
 template <typename T, int K, int P, int MODE, bool PER, int UNR, bool HS>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem) {
     constexpr int L = Levels<K, MODE>::value;  // pipelined levels (one row and one x cell of halo each)
-    // FP64 pairs over two pipes, except where the registers run out: four points a lane (8.5 against 9.6 G at 2048^2)
-    // and the batched kernel's two steps a launch (6.2 against 8.6 G on 12 runs; one step: 9.8 against 8.9 G)
-    constexpr bool HY = P <= 2 && !(K == 2 && UNR == 2);
+    // FP64 pairs over two pipes, except where the registers run out: four points a lane (8.5 against 9.6 G at 2048^2),
+    // the batched kernel's two steps a launch (6.2 against 8.6 G on 12 runs; one step: 9.8 against 8.9 G), and with two points
+    // a lane, whose 8 warps an SM wait longer for the integer sums, the 3-D x-y pass (24^3 127 us a step so, 91.5 on the
+    // FP64 pipe alone; 256^3 2471 and 2397) and the zero-boundary second-order step (2048^2 794 and 760, 200 x 150 38 and
+    // 27; 1024^2 221 and 225)
+    constexpr bool HY = P == 1 || (P == 2 && !(K == 2 && UNR == 2) && MODE != 1 && !(MODE == 2 && !PER));
     const int64_t per_plane = a.nstrips * a.nsegs;
     const int64_t plane = wid / per_plane;
     const int64_t rem = wid - plane * per_plane;
