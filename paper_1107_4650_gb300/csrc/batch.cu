@@ -5,20 +5,20 @@
 namespace dirac {
 
 namespace {
-template <typename T, int K, int P>
-cudaError_t launch_batch_t(const BatchArgs &b, int blocks, cudaStream_t s) {
-    const int smem = ring_smem_bytes<T, K, P, BatchHist<T, K, P>::value>(4);
-    cudaError_t e = cudaFuncSetAttribute(batch_kernel<T, K, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+template <typename T, int K, int P, bool ONEPIPE = false>
+cudaError_t launch_batch_t(const BatchArgs &b, int blocks, int warps, cudaStream_t s) {
+    const int smem = ring_smem_bytes<T, K, P, BatchHist<T, K, P>::value>(warps);
+    cudaError_t e = cudaFuncSetAttribute(batch_kernel<T, K, P, ONEPIPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    batch_kernel<T, K, P><<<blocks, 128, smem, s>>>(b);
+    batch_kernel<T, K, P, ONEPIPE><<<blocks, 32 * warps, smem, s>>>(b);
     return cudaGetLastError();
 }
 template <typename T, int K, int P>
 cudaError_t occupancy_t(int *blocks_per_sm) {
     const int smem = ring_smem_bytes<T, K, P, BatchHist<T, K, P>::value>(4);
-    cudaError_t e = cudaFuncSetAttribute(batch_kernel<T, K, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(batch_kernel<T, K, P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<T, K, P>, 128, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, batch_kernel<T, K, P, false>, 128, smem);
 }
 }  // namespace
 
@@ -33,8 +33,10 @@ bool batch_supported(int fp32, int K, int P) {
     return false;
 }
 
-cudaError_t launch_batch(const BatchArgs &b, int fp32, int K, int P, int blocks, cudaStream_t s) {
-#define X(T, k, p) if ((fp32 != 0) == (sizeof(T) == 4) && K == k && P == p) return launch_batch_t<T, k, p>(b, blocks, s);
+cudaError_t launch_batch(const BatchArgs &b, int fp32, int K, int P, int few, int blocks, cudaStream_t s) {
+    // as many one-warp blocks as tasks, which the hardware spreads over the SMs (4-warp blocks leave four tasks on one)
+    if (few && !fp32 && K == 1 && P == 2) return launch_batch_t<double, 1, 2, true>(b, few, 1, s);
+#define X(T, k, p) if ((fp32 != 0) == (sizeof(T) == 4) && K == k && P == p) return launch_batch_t<T, k, p>(b, blocks, 4, s);
     DIRAC_BATCH_CASES(X)
 #undef X
     return cudaErrorInvalidValue;

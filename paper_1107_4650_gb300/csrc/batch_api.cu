@@ -58,6 +58,7 @@ struct dirac_batch {
     int64_t *d_off_main = nullptr, *d_off_rem = nullptr;
     std::vector<int> nact_main, nact_rem;       // active runs of each launch
     std::vector<int> height_main, height_rem;   // and the place of its rows per task in `heights`
+    std::vector<int64_t> tasks_main, tasks_rem;  // and its tasks
     std::vector<int64_t> heights;               // rows per task in use: the caller's, or the library's choices
     int K = 2, P = 2, blocks = 0, sm_count = 152;
     int64_t seg_rows = 0, max_tasks = 0;  // rows per task, 0: chosen for each launch
@@ -177,7 +178,7 @@ dirac_status plan(dirac_batch *b) {
             offm[at + 1] = offm[at] + run_tasks(b, om[i], K, b->heights[h]);
             offr[at + 1] = offr[at] + run_tasks(b, orr[i], 1, b->heights[h]);
         }
-    auto heights_for = [&](const std::vector<int> &nact, const std::vector<int64_t> &off, int k) {
+    auto heights_for = [&](const std::vector<int> &nact, const std::vector<int64_t> &off, int k, std::vector<int64_t> &launch_tasks) {
         std::vector<int> out(nact.size());
         std::vector<int64_t> tasks(nh);
         for (size_t l = 0; l < nact.size(); ++l) {
@@ -188,6 +189,8 @@ dirac_status plan(dirac_batch *b) {
             for (int h = 0; h < nh; ++h) tasks[h] = off[(size_t)h * (n + 1) + nact[l]];
             out[l] = pick_height(b, tasks, k);
         }
+        launch_tasks.resize(nact.size());
+        for (size_t l = 0; l < nact.size(); ++l) launch_tasks[l] = off[(size_t)out[l] * (n + 1) + nact[l]];
         return out;
     };
     const int64_t Lmain = n ? b->runs[om[0]].nsteps / K : 0;
@@ -203,8 +206,8 @@ dirac_status plan(dirac_batch *b) {
         while (c < n && b->runs[orr[c]].nsteps % K > j) ++c;
         if (c > 0) b->nact_rem.push_back(c);
     }
-    b->height_main = heights_for(b->nact_main, offm, K);
-    b->height_rem = heights_for(b->nact_rem, offr, 1);
+    b->height_main = heights_for(b->nact_main, offm, K, b->tasks_main);
+    b->height_rem = heights_for(b->nact_rem, offr, 1, b->tasks_rem);
     b->max_tasks = offm[(size_t)(b->height_main.empty() ? 0 : b->height_main[0]) * (n + 1) + n];
     BCK(b, cudaMemcpyAsync(b->d_order_main, om.data(), n * sizeof(int), cudaMemcpyHostToDevice, b->stream));
     BCK(b, cudaMemcpyAsync(b->d_order_rem, orr.data(), n * sizeof(int), cudaMemcpyHostToDevice, b->stream));
@@ -269,13 +272,13 @@ dirac_status enqueue_schedule(dirac_batch *b, cudaStream_t s, int64_t max_main =
         f.count = 0;
         return DIRAC_OK;
     };
-    auto launch = [&](int K, int height, const int64_t *off) -> dirac_status {
+    auto launch = [&](int K, int height, int64_t tasks, const int64_t *off) -> dirac_status {
         a.seg_rows = b->heights[height];
         a.task_off = off + (size_t)height * (b->nruns + 1);
         a.flux_off = f.count * b->flux_stride;
         f.seg_rows[f.count] = a.seg_rows;
         f.n_active[f.count++] = a.n_active;
-        BCK(b, launch_batch(a, b->fp32, K, b->P, b->blocks, s));
+        BCK(b, launch_batch(a, b->fp32, K, b->P, tasks <= b->sm_count ? (int)tasks : 0, b->blocks, s));
         b->launches++;
         a.turn ^= 1;
         return f.count == kBatchSlots ? fold() : DIRAC_OK;
@@ -288,7 +291,7 @@ dirac_status enqueue_schedule(dirac_batch *b, cudaStream_t s, int64_t max_main =
     for (int64_t l = 0; l < Lm && st == DIRAC_OK; ++l) {
         a.n_active = b->nact_main[l];
         a.launch = l;
-        st = launch(b->K, b->height_main[l], b->d_off_main);
+        st = launch(b->K, b->height_main[l], b->tasks_main[l], b->d_off_main);
     }
     if (st == DIRAC_OK) st = fold();
     if (max_main >= 0 || st != DIRAC_OK) return st;
@@ -298,7 +301,7 @@ dirac_status enqueue_schedule(dirac_batch *b, cudaStream_t s, int64_t max_main =
     for (size_t j = 0; j < b->nact_rem.size() && st == DIRAC_OK; ++j) {
         a.n_active = b->nact_rem[j];
         a.launch = (int64_t)j;
-        st = launch(1, b->height_rem[j], b->d_off_rem);
+        st = launch(1, b->height_rem[j], b->tasks_rem[j], b->d_off_rem);
     }
     return st == DIRAC_OK ? fold() : st;
 }

@@ -9,7 +9,8 @@ struct InitArgs;
 struct NormArgs;
 struct BatchFluxFold;
 bool batch_supported(int fp32, int K, int P);
-cudaError_t launch_batch(const BatchArgs &b, int fp32, int K, int P, int blocks, cudaStream_t s);
+// few: the tasks of a launch that has no more of them than the chip has SMs, else 0
+cudaError_t launch_batch(const BatchArgs &b, int fp32, int K, int P, int few, int blocks, cudaStream_t s);
 cudaError_t launch_batch_flux_fold(const BatchFluxFold &f, cudaStream_t s);
 cudaError_t batch_occupancy(int fp32, int K, int P, int *blocks_per_sm);
 cudaError_t launch_batch_init(const InitArgs &ia, int fp32, cudaStream_t s);

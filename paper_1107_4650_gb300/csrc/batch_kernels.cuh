@@ -86,7 +86,10 @@ template <typename T, int K, int P> struct BatchHist {
     static constexpr int blocks = value ? 4 : 1;  // resident 4-warp blocks the registers are fitted to
 };
 
-template <typename T, int K, int P>
+// ONEPIPE (FP64): the pairs on the FP64 pipe alone, for launches of no more tasks than SMs, one to a one-warp block, where the
+// integer sums only lengthen a warp's chain.  Such launches come from rows per task that the caller sets, and from single
+// small runs: one run of 64^2, 64 to 96 steps, 3.3 -> 2.5 ms, in 128 rows 20.0 -> 15.8; of 1024^2 in 128 rows 51 -> 31.
+template <typename T, int K, int P, bool ONEPIPE>
 __global__ void __launch_bounds__(128, BatchHist<T, K, P>::blocks) batch_kernel(const BatchArgs b) {
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     const int lane = threadIdx.x & 31;
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(128, BatchHist<T, K, P>::blocks) batch_kernel(
         a.full_table = 0;
         a.flux_unit = 1.0;  // floating-point states
         a.wide = 1;         // the pool is the library's own, a cell 32 or 64 bytes
-        sweep_warp<T, K, P, 0, false, BatchHist<T, K, P>::unroll, BatchHist<T, K, P>::value>(a, (int64_t)task - b.task_off[lo], lane, wsmem);
+        sweep_warp<T, K, P, 0, false, BatchHist<T, K, P>::unroll, BatchHist<T, K, P>::value, ONEPIPE>(a, (int64_t)task - b.task_off[lo], lane, wsmem);
         if (lane == 0) fence_proxy_async();  // this task's reads of the row slots before the next one's first copies into them
     }
 }

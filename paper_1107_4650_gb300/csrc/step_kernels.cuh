@@ -407,7 +407,7 @@ template <typename T, int K, int P, int MODE, bool PER> struct HistSmem {
         (IsFx<T>::value && P == 1 && K == 1 && (MODE == 2 || (MODE == 0 && PER))) ||
         (sizeof(T) == 4 && P == 2 && ((MODE == 0 && (K == 2 || K == 4)) || (MODE == 2 && (K == 1 || K == 2))));
 };
-template <typename T, int K, int P, int MODE, bool PER, int UNR = RowUnroll<T, K, MODE>::value, bool HS = false>
+template <typename T, int K, int P, int MODE, bool PER, int UNR = RowUnroll<T, K, MODE>::value, bool HS = false, bool ONEPIPE = false>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem);
 template <typename T, int K, int P, bool HS = false> struct Ring;
 
@@ -656,7 +656,7 @@ __device__ __forceinline__ void flux_row(const Cx<T> *lu14, const Cx<T> *lu23, c
     }
 }
 
-template <typename T, int K, int P, int MODE, bool PER, int UNR, bool HS>
+template <typename T, int K, int P, int MODE, bool PER, int UNR, bool HS, bool ONEPIPE>
 __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid, const int lane, unsigned char *wsmem) {
     constexpr int L = Levels<K, MODE>::value;  // pipelined levels (one row and one x cell of halo each)
     // FP64 pairs over two pipes, except where the registers run out: four points a lane (8.5 against 9.6 G at 2048^2),
@@ -664,7 +664,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     // a lane, whose 8 warps an SM wait longer for the integer sums, the 3-D x-y pass (24^3 127 us a step so, 91.5 on the
     // FP64 pipe alone; 256^3 2471 and 2397) and the zero-boundary second-order step (2048^2 794 and 760, 200 x 150 38 and
     // 27; 1024^2 221 and 225)
-    constexpr bool HY = P == 1 || (P == 2 && !(K == 2 && UNR == 2) && MODE != 1 && !(MODE == 2 && !PER));
+    constexpr bool HY = !ONEPIPE && (P == 1 || (P == 2 && !(K == 2 && UNR == 2) && MODE != 1 && !(MODE == 2 && !PER)));
     const int64_t per_plane = a.nstrips * a.nsegs;
     const int64_t plane = wid / per_plane;
     const int64_t rem = wid - plane * per_plane;
