@@ -1106,17 +1106,21 @@ __global__ void __launch_bounds__(128) zphase_kernel(const ZArgs a) {
     T *out = static_cast<T *>(a.out);
     const T *tab = static_cast<const T *>(a.table);
     Cx<T> pu, pd;
+    constexpr bool AHEAD = FULL && !IsF64<T>::value;
+    Cx<T> tu, td;
     if (!FULL) load_tab(tab + x * 4, pu, pd);
     Cx<T> UA[2] = {{T(0), T(0)}, {T(0), T(0)}}, UB[2] = {{T(0), T(0)}, {T(0), T(0)}};
     for (int64_t z = z_begin - 1; z <= z_end; ++z) {
         Cx<T> s[4];
         const bool ok = per || (z >= 0 && z < nz);
         const int64_t zo = z - 1;
-        // the table's entry asked for before the state: at its use below, each plane waited for it in turn (200^3 with a full
-        // table, two-pass plan, FP32 332 us a step, 249 so; fixed point 610 and 525; in a variant of its own, since the
-        // per-column one is 2 % slower with it)
-        Cx<T> qu = pu, qd = pd;
-        if (FULL && zo >= z_begin && zo < z_end) load_tab(tab + (zo * ncol + col) * 4, qu, qd);
+        // The table's entry is asked for a plane ahead, in FP64, which the pipe binds, just before the state: at its use below
+        // each plane waited for it in turn (two-pass plan at 200^3 with a full table, us a step at the use, before the state, a
+        // plane ahead: FP32 332, 285, 244; fixed point 610, 523, 521; FP64 1159, 1147, 1165).  The per-column table's variant
+        // is 2 % slower with the entries held so.
+        Cx<T> qu = AHEAD ? tu : pu, qd = AHEAD ? td : pd;
+        const int64_t zt = AHEAD ? z : zo;
+        if (FULL && zt >= z_begin && zt < z_end) load_tab(tab + (zt * ncol + col) * 4, AHEAD ? tu : qu, AHEAD ? td : qd);
         if (ok) {
             const int64_t zl = per ? pmod(z, nz) : z;
             load_pt(in + (zl * ncol + col) * 8, s);
