@@ -12,6 +12,7 @@
 
 #include "../../include/dirac.h"
 #include "dirac_internal.cuh"
+#include "rows.cuh"
 
 using namespace dirac;
 
@@ -388,6 +389,7 @@ void make_plan(dirac_grid *g, int K, int P, int wpb, int target_warps_per_sm) {
         nsegs = std::min<int64_t>(nsegs, std::max<int64_t>(1, nr / min_rows));
         p.seg_h = (nr + nsegs - 1) / nsegs;
     }
+    p.seg_h = std::min(p.seg_h, kMaxSegRows);
     p.nsegs = (nr + p.seg_h - 1) / p.seg_h;
     // 3-D z pass: one thread per column, segments until ~target warps per SM
     if (ndim_of(g) == 3) {

@@ -28,6 +28,7 @@
 
 #include "butterfly.cuh"
 #include "dirac_internal.cuh"
+#include "rows.cuh"
 
 namespace dirac {
 
@@ -675,12 +676,14 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     const int64_t x_own0 = strip * a.strip_w;
     const int64_t x_own1 = min(x_own0 + a.strip_w, nx);
     const int64_t xa = x_own0 - L;
-    // Row indices fit 32 bits (the host limits every grid dimension below 2^31): FP32 k = 2 105 against 94 G at
-    // 2048^2 with 64-bit ones, fixed point 39.4 against 37.5 G.
+    // Rows are counted from the segment's first in 32 bits (FP32 k = 2 105 against 94 G at 2048^2 with 64-bit ones, fixed
+    // point 39.4 against 37.5 G; the grid's own numbers run out of them near 2^31 rows).
     using RI = int;
-    const RI nr32 = (RI)nr;
-    const RI r_begin = (RI)(seg * a.seg_h);
-    const RI r_end = (RI)min((int64_t)r_begin + a.seg_h, nr);
+    const SegRows sr = seg_rows(seg, a.seg_h, nr);
+    const uint32_t row0 = (uint32_t)sr.row0, nr32 = (uint32_t)nr;
+    auto in_grid = [&](RI r) { return row_in_grid(row0, r, nr32); };
+    constexpr RI r_begin = 0;
+    const RI r_end = sr.end;
     const T *in = static_cast<const T *>(a.in) + plane * nr * nx * 8;
     T *out = static_cast<T *>(a.out) + plane * nr * nx * 8;
 
@@ -769,7 +772,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     const uint32_t slot0 = smem_u32(wsmem + 128);
     const uint32_t dst_off = per ? 0u : (uint32_t)(cx0 - xa) * CELL;
     // lane 0: row r of the grid into slot sl
-    auto fetch_row = [&](RI r, int sl) {
+    auto fetch_row = [&](uint32_t r, int sl) {
         const T *row = in + (int64_t)r * nx * 8;
         const uint32_t bar = bar0 + 8 * sl, dst = slot0 + sl * RG::ROW_BYTES + dst_off;
         bar_expect(bar, copy_bytes);
@@ -786,12 +789,8 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         }
     };
     // a row of the segment or its halo in the grid's own numbering (periodic: wrapped)
-    auto grid_row = [&](RI r) -> RI {
-        if (per) {
-            while (r < 0) r += nr32;
-            while (r >= nr32) r -= nr32;
-        }
-        return r;
+    auto grid_row = [&](RI r) -> uint32_t {
+        return per ? wrap_row(row0, r, nr32) : row0 + (uint32_t)r;
     };
     const RI r_first = r_begin - L, r_last = r_end + L;  // rows [r_first, r_last) are read
     uint32_t phase_bits = 0, pending = 0;
@@ -814,7 +813,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
 #pragma unroll
     for (int sl = 0; sl < RG::SLOTS; ++sl) {
         const RI r = r_first + sl;
-        if (r < r_last && (per || (r >= 0 && r < nr32))) {
+        if (r < r_last && (per || in_grid(r))) {
             if (lane == 0) {
                 // failure-detection test hook: the first warp of the launch announces 16 bytes more than
                 // its first row copy delivers, so that slot's phase never completes and its bounded wait
@@ -834,16 +833,16 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
     // 42.0 -> 31.4 M warp instructions a launch with the packed adds, k = 4 125 -> 139 G point-steps/s, the batched
     // kernel 154 -> 164.  What then bounds the FP32 kernel is the shared-memory pipe (82 % busy at k = 2, half of it bank
     // conflicts of the history and the row reads): without the conflicts and with 32-byte stores 124 -> 145 G.
-    T *orow = out + ((int64_t)(r_first - L) * nx + xa) * 8;  // output row r - L
-    const T *frow = in + ((int64_t)(r_first + RG::SLOTS) * nx + cx0) * 8;  // zero boundary: span of row r + SLOTS
-    const RI f_end = per ? r_last : min(r_last, nr32);                   // rows [.., f_end) are fetched
+    T *orow = out + ((sr.row0 + r_first - L) * nx + xa) * 8;  // output row r - L
+    const T *frow = in + ((sr.row0 + r_first + RG::SLOTS) * nx + cx0) * 8;  // zero boundary: span of row r + SLOTS
+    const RI f_end = per ? r_last : min(r_last, sr.top);                  // rows [.., f_end) are fetched
     const int64_t row_step = nx * 8;
     int sl = 0;
     auto do_row = [&](auto steady_c, auto par_c, const RI r) -> bool {
         constexpr bool STEADY = decltype(steady_c)::value;
         constexpr int par = decltype(par_c)::value;
         Cx<T> st[P][4];
-        const bool row_ok = STEADY || per || (r >= 0 && r < nr32);
+        const bool row_ok = STEADY || per || in_grid(r);
         if (row_ok) {
             if (!mbar_wait(bar0 + 8 * sl, (phase_bits >> sl) & 1u)) return false;
             phase_bits ^= 1u << sl;
@@ -867,7 +866,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
         auto refill = [&]() {
             __syncwarp();
             const RI rn = r + RG::SLOTS;
-            if (rn < f_end && (STEADY || per || rn >= 0)) {
+            if (rn < f_end && (STEADY || per || in_grid(rn))) {
                 if (per) {
                     if (lane == 0) {
                         fence_proxy_async();
@@ -892,7 +891,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
             if ((MODE == 2 || MODE == 5) && (lev & 1)) {
                 // second half of a Strang step: z sweep of rows q-2 and q into row q-1, then the x sweep of
                 // row q-1.  The input is 1/4 of the state (the phase carried 1/16), the z-swept row 1/2 of it.
-                const bool zrow_ok = STEADY || per || (q - 1 >= 0 && q - 1 < nr32);
+                const bool zrow_ok = STEADY || per || in_grid(q - 1);
                 Cx<T> zs[P][4];
 #pragma unroll
                 for (int j = 0; j < P; ++j) {
@@ -945,7 +944,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                 flux_row<T, P>(lu14, lu23, w14, w23, face_j, face_lane, lane, q - r_begin, q == r_end - 1,
                                gsm + lev * 8 * 32, 0.5 * a.flux_unit, facc[FT ? 0 : lev]);
             }
-            const bool out_row_ok = STEADY || per || (q - 1 >= 0 && q - 1 < nr32);
+            const bool out_row_ok = STEADY || per || in_grid(q - 1);
 #pragma unroll
             for (int j = 0; j < P; ++j) {
                 // x sweep (Eq. sol_dis_1), x2
@@ -969,7 +968,7 @@ __device__ __forceinline__ void sweep_warp(const SweepArgs &a, const int64_t wid
                         // phase (Eq. sol_dis_4) with the deferred 1/4
                         Cx<T> qu, qd;
                         if (a.full_table) {
-                            const int64_t rr = per ? (int64_t)grid_row(q - 1) : (int64_t)min(max(q - 1, (RI)0), nr32 - 1);
+                            const int64_t rr = per || in_grid(q - 1) ? grid_row(q - 1) : 0u;
                             load_tab(static_cast<const T *>(a.table) + (plane * nr * nx + rr * nx + xl[j]) * 4, qu, qd);
                         } else {
                             qu = pu[j];
@@ -1106,9 +1105,9 @@ __global__ void __launch_bounds__(128) zphase_kernel(const ZArgs a) {
     T *out = static_cast<T *>(a.out);
     const T *tab = static_cast<const T *>(a.table);
     Cx<T> pu, pd;
+    if (!FULL) load_tab(tab + x * 4, pu, pd);
     constexpr bool AHEAD = FULL && !IsF64<T>::value;
     Cx<T> tu, td;
-    if (!FULL) load_tab(tab + x * 4, pu, pd);
     Cx<T> UA[2] = {{T(0), T(0)}, {T(0), T(0)}}, UB[2] = {{T(0), T(0)}, {T(0), T(0)}};
     for (int64_t z = z_begin - 1; z <= z_end; ++z) {
         Cx<T> s[4];
