@@ -67,7 +67,7 @@ struct dirac_grid {
     size_t flux_used = 0;      // doubles of it that launches since the last fold write
     FluxFold flux{};           // and their places; empty between calls of dirac_step
     double *flux_dev = nullptr;
-    unsigned *ticket = nullptr;  // [1]: set by a step kernel whose bounded wait ran out
+    unsigned *wait_err = nullptr;  // set by a step kernel whose bounded wait ran out
     std::vector<double> absorb;      // per-x-column damping factors (empty: none)
     std::vector<double> v_host;      // last potential set (for rebuilding the table)
     int v_layout = DIRAC_V_NONE;
@@ -585,7 +585,7 @@ dirac_status enqueue_block(dirac_grid *g, int parity, int K, cudaStream_t s, int
     a.nsegs = p.nsegs;
     a.seg_h = p.seg_h;
     a.flux_face = flux ? g->cfg.flux_face : -1;
-    a.err = g->ticket + 1;
+    a.err = g->wait_err;
     a.periodic = g->cfg.boundary == DIRAC_BC_PERIODIC;
     a.full_table = g->table_full;
     a.ucoef = g->ucoef;
@@ -814,7 +814,7 @@ dirac_status enqueue_strang3d_run(dirac_grid *g, int parity, int64_t m, cudaStre
     a.nx = g->cfg.n[0];
     a.nplanes = 1;
     a.flux_face = flux ? g->cfg.flux_face : -1;
-    a.err = g->ticket + 1;
+    a.err = g->wait_err;
     a.periodic = g->cfg.boundary == DIRAC_BC_PERIODIC;
     const double *ucoef = field_on(g) ? g->ucoef : nullptr;
     const int64_t ucoef_n = (int64_t)(g->avec.size() / 3);
@@ -974,7 +974,7 @@ void release(dirac_grid *g) {
         if (p) cudaFree(p);
     if (g->flux_part) cudaFree(g->flux_part);
     if (g->flux_dev) cudaFree(g->flux_dev);
-    if (g->ticket) cudaFree(g->ticket);
+    if (g->wait_err) cudaFree(g->wait_err);
     if (g->obs_partial) cudaFree(g->obs_partial);
     if (g->obs_out) cudaFree(g->obs_out);
     if (g->density_tmp) cudaFree(g->density_tmp);
@@ -1340,7 +1340,7 @@ dirac_status dirac_create_grid(const dirac_config *cfg, dirac_grid **out) {
         void **p;
         size_t bytes;
     } allocs[] = {{&g->psi[0], state_bytes}, {&g->psi[1], state_bytes}, {(void **)&g->flux_dev, 8 * sizeof(double)},
-                  {(void **)&g->ticket, 16},
+                  {(void **)&g->wait_err, 16},
                   {(void **)&g->obs_partial, (size_t)kObsBlocksMax * 5 * sizeof(double)},
                   {(void **)&g->obs_out, 8 * sizeof(double)}};
     for (auto &al : allocs) {
@@ -1368,7 +1368,7 @@ dirac_status dirac_create_grid(const dirac_config *cfg, dirac_grid **out) {
     if (st == DIRAC_OK) {
         e = g->ext ? cudaSuccess : cudaMemsetAsync(g->psi[0], 0, state_bytes, g->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(g->flux_dev, 0, 8 * sizeof(double), g->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(g->ticket, 0, 16, g->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(g->wait_err, 0, 16, g->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
         if (e != cudaSuccess) st = cuda_fail(g, e, "initial clear");
     }
@@ -1524,7 +1524,7 @@ dirac_status dirac_set_state(dirac_grid *g, const void *psi, int on_device) {
                               g->stream));
     }
     CK(g, cudaMemsetAsync(g->flux_dev, 0, sizeof(double), g->stream));
-    CK(g, cudaMemsetAsync(g->ticket + 1, 0, sizeof(unsigned), g->stream));  // clear a reported timeout
+    CK(g, cudaMemsetAsync(g->wait_err, 0, sizeof(unsigned), g->stream));  // clear a reported timeout
     if (!on_device) CK(g, cudaStreamSynchronize(g->stream));
     g->step = 0;
     return DIRAC_OK;
@@ -1558,7 +1558,7 @@ dirac_status dirac_set_state_fx(dirac_grid *g, const int64_t *q, int shift, int 
         CK(g, cudaMemcpyAsync(g->psi[g->cur], q, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                               g->stream));
     CK(g, cudaMemsetAsync(g->flux_dev, 0, sizeof(double), g->stream));
-    CK(g, cudaMemsetAsync(g->ticket + 1, 0, sizeof(unsigned), g->stream));
+    CK(g, cudaMemsetAsync(g->wait_err, 0, sizeof(unsigned), g->stream));
     if (!on_device) CK(g, cudaStreamSynchronize(g->stream));
     set_fx_shift(g, shift);
     g->step = 0;
@@ -1637,7 +1637,7 @@ dirac_status dirac_observables(dirac_grid *g, dirac_obs *obs, double *density, i
     g->launches += 2;
     CK(g, cudaMemcpyAsync(g->host_obs, g->obs_out, 5 * sizeof(double), cudaMemcpyDeviceToHost, g->stream));
     CK(g, cudaMemcpyAsync(&g->host_obs[5], g->flux_dev, sizeof(double), cudaMemcpyDeviceToHost, g->stream));
-    CK(g, cudaMemcpyAsync(&g->host_obs[6], g->ticket + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, g->stream));
+    CK(g, cudaMemcpyAsync(&g->host_obs[6], g->wait_err, sizeof(unsigned), cudaMemcpyDeviceToHost, g->stream));
     if (density && !density_on_device)
         CK(g, cudaMemcpyAsync(density, dens, (size_t)g->ncells * sizeof(double), cudaMemcpyDeviceToHost, g->stream));
     CK(g, cudaStreamSynchronize(g->stream));

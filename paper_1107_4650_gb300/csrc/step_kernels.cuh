@@ -150,9 +150,6 @@ __device__ __forceinline__ void z_chars(const Cx<T> b[4], Cx<T> &U13, Cx<T> &W13
 template <bool HY, typename T> __device__ __forceinline__ void z_join(Cx<T> U13, Cx<T> W13, Cx<T> U24, Cx<T> W24, Cx<T> o[4]) {
     butterfly2<HY>(U13, W13, W24, U24, o[0], o[2], o[1], o[3]);
 }
-// i z and -i z (exact)
-template <typename T> __device__ __forceinline__ Cx<T> cmul_i(Cx<T> a) { return {-a.im, a.re}; }
-template <typename T> __device__ __forceinline__ Cx<T> cmul_mi(Cx<T> a) { return {a.im, -a.re}; }
 template <typename T> __device__ __forceinline__ Cx<T> cmulp(Cx<T> z, Cx<T> p) {
     return {Ar<T>::fma(z.re, p.re, -Ar<T>::mul(z.im, p.im)), Ar<T>::fma(z.re, p.im, Ar<T>::mul(z.im, p.re))};
 }
