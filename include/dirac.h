@@ -236,7 +236,8 @@ dirac_status dirac_set_counters(dirac_grid *g, int64_t step, double flux_cum);
 
 typedef struct {
     int steps_per_launch;   /* temporal block depth k in use */
-    int points_per_lane;    /* x cells per lane in the step kernel */
+    int points_per_lane;    /* x cells per lane in the step kernel (small 2-D grids, stepped in tiles of one cell a
+                               lane: of the configuration with the same steps per launch) */
     int64_t launch_warps;   /* warps in one step launch */
     int64_t strip_width;    /* x cells written by one warp */
     int64_t segment_rows;   /* rows written by one warp (small 2-D grids: by one block's tile) */

@@ -156,11 +156,11 @@ cudaError_t launch_axis(const void *in, void *out, const void *table, int64_t nx
                         double *flux_part, const double *ucoef,
                         int64_t ucoef_n, int64_t step0, int precision, int rshift, int blocks, cudaStream_t s);
 
-// Fused 3-D step (x, y, z sweeps and phase in one pass, `steps` = 1 or 2 steps per launch): blocks of
-// `warps` warps own a (32 - 2 steps)-cell x strip and warps - 2 steps rows along y and stream a z segment of
-// zseg_h planes (steps 1: 8 or 16 warps; steps 2: 16 warps in FP32, 8 in FP64; 64-bit fixed point: steps 1,
-// no vector potential).  precision: 0 FP64, 1 FP32, 2 int64 fixed point.  Flux parts:
-// [steps][nzsegs * nytiles * warps] (a.nsegs * a.nplanes must equal nzsegs * nytiles * warps).
+// Fused 3-D step (x, y, z sweeps and phase in one pass, `steps` = 1 or 2 steps per launch): blocks own a (32 - 2 steps)-cell
+// x strip and rows - 2 steps rows along y and stream a z segment of zseg_h planes.  One step: 8 or 16 warps of one row; two:
+// FP32 12 warps of two rows (no vector potential) or 16 of one, FP64 8 of one; 64-bit fixed point: one step, no vector
+// potential.  precision: 0 FP64, 1 FP32, 2 int64 fixed point.  Flux parts: [steps][nzsegs * nytiles * warps] (a.nsegs *
+// a.nplanes must equal nzsegs * nytiles * warps).
 cudaError_t launch_fused3d(const SweepArgs &a, int precision, int warps, int steps, int64_t ny, int64_t nz,
                            int64_t nstrips, int64_t nytiles, int64_t nzsegs, int64_t zseg_h, cudaStream_t s);
 

@@ -479,7 +479,7 @@ inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 // ---- Inference: the whole network for 128 queries per CTA in one launch.
 //
 // The weights of layers 2-4 are first packed into the canonical no-swizzle K-major layout the MMA reads
-// (the layout `stage` builds: B(k, n) = W[n][k], 256 rows n), so each layer's 128 KB operand reaches shared
+// (the layout `stage_async` builds: B(k, n) = W[n][k], 256 rows n), so each layer's 128 KB operand reaches shared
 // memory as bulk copies (cp.async.bulk, completion counted on an mbarrier), issued as soon as the previous
 // layer's MMAs have read the buffer and overlapping that layer's epilogue.  Layer 1 (K = 3) runs on the CUDA
 // cores and writes bf16(h1) straight into the A operand (128 queries x 256); each hidden layer is 16
@@ -487,8 +487,8 @@ inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 // (16 by default): the NW / 4 warps w, w + 4, ... read the same 32 TMEM lanes (queries 32 (w % 4)..), each a
 // block of 256 / (NW / 4) columns; they add the bias, take tanh and write bf16(h) over the A operand (16
 // warps ran 99 us against 116 for 8 on 65,536 queries).  The output layer then sums bf16(h4) bf16(w5)
-// per query in out_fwd_kernel's order (32 strided partial sums, then its shuffle tree), so every rounding
-// point is forward's.  Every wait is bounded; a timeout sets *err.
+// per query in out_layer_kernel's order (32 strided partial sums, then its shuffle tree), so every rounding
+// point is the training step's.  Every wait is bounded; a timeout sets *err.
 constexpr int IQ = 128;                          // queries per CTA (the MMA's M)
 constexpr int IW_SLAB = HID * 16 * 2;            // one 16-deep K slab of a 256-row weight operand (8 KB)
 constexpr int IH_SLAB = IQ * 16 * 2;             // one 16-deep K slab of the activations (4 KB)
@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(32 * NW, 1) mlp_infer_kernel(const float *x, c
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
     if (ok && warp < 4 && q < Bn) {
-        // output layer in out_fwd_kernel's order: partial sum l takes columns l, l + 32, ..., then the xor tree
+        // output layer in out_layer_kernel's order: partial sum l takes columns l, l + 32, ..., then the xor tree
         float s[32];
 #pragma unroll
         for (int l = 0; l < 32; ++l) s[l] = 0.f;

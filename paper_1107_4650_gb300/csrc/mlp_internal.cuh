@@ -51,7 +51,7 @@ inline void layout(Net &n) {
 // of mean((y - t)^2) into g, per-sample squared errors into a.sqerr; see mlp.cu.
 cudaError_t gradients(const Net &n, const Acts &a, const float *X, const float *T, const int *idx, float *g, int Bn,
                       cudaStream_t s);
-// Inference only: y = network(x) for Bn queries in one fused launch, with the same rounding points as forward.
+// Inference only: y = network(x) for Bn queries in one fused launch, with the same rounding points as gradients.
 // It reads W2-W4 from n.wpack, which pack_weights fills from n.wb (again after every change of the weights).
 constexpr int64_t WPACK_BYTES = 3 * (int64_t)HID * HID * 2;
 cudaError_t pack_weights(const Net &n, cudaStream_t s);

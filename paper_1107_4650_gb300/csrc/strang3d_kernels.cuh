@@ -18,7 +18,7 @@
 // plane); NH = 2 has two barriers per plane, which order every reuse of its two single buffers.
 // Face flux: every x sweep adds, on the face strip's owned rows, 1/2 (|u14|^2 + |u23|^2) of cell face - 1 and
 // subtracts 1/2 (|w14|^2 + |w23|^2) of cell face, of the state entering it, times 1 / s^2 for the state's
-// scale s (fscale); one part per (sweep, z segment, y tile, warp), folded by the last block.
+// scale s (fscale); one part per (sweep, z segment, y tile, warp).
 // 64-bit fixed-point state (q = psi 2^S): the sweeps are exact integer sums, the face terms are formed in FP64
 // (fscale carries 2^-2S), and the step's final division by 16 (rounded to nearest, halves up: the phase carries
 // only the first four halves) follows the step's last x sweep: at the end of a pass that ends a step and between
