@@ -22,7 +22,8 @@ def fake_lib(tmp_path_factory):
     if gxx is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
         pytest.skip("no g++ or no CUDA headers")
     lib = str(tmp_path_factory.mktemp("fake") / "libfake.so")
-    subprocess.run([gxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-fopenmp", "-I", cuda, "-I", B.CSRC, "-x", "c++",
+    # (bound to its own stand-ins whatever runtime the process has loaded)
+    subprocess.run([gxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-fopenmp", "-I", cuda, "-I", B.CSRC, "-x", "c++",
                     os.path.join(B.CSRC, "dirac_api.cu"), os.path.join(HERE, "fake_cuda.cpp"), "-o", lib], check=True)
     return lib
 
