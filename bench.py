@@ -54,11 +54,11 @@ FP64_ISSUE_PEAK_NOMINAL = FP64_INSTR_PER_SM_CLOCK * SM_COUNT * 2.07e9 / 1e12  # 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of the step kernel on the 2048^2 workload, keyed
 # by (steps per launch, points per lane) of the captured variant
 # (profiles/step_kernels_two_pipes_pairs_tiles.md).  A variant without a capture reports null.
-MEASURED_TRAFFIC_PER_LAUNCH = {"fp64": {(1, 1): 277.649248e6 + 222.500720e6},
-                               "fp32": {(4, 2): 167.320192e6 + 88.742166e6},
-                               "fx64": {(1, 1): 277.561088e6 + 219.967744e6}}
+MEASURED_TRAFFIC_PER_LAUNCH = {"fp64": {(1, 1): 277.660416e6 + 223.318528e6},
+                               "fp32": {(4, 2): 167.286528e6 + 88.852736e6},
+                               "fx64": {(1, 1): 277.541120e6 + 219.706368e6}}
 # ncu sm__pipe_fp64_cycles_active of the same captures (fraction of active cycles)
-MEASURED_FP64_PIPE = {(1, 1): 0.7937}
+MEASURED_FP64_PIPE = {(1, 1): 0.7974}
 
 
 def parse():

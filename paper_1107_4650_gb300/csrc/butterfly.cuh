@@ -10,7 +10,7 @@
 // nothing downstream can tell which pipe did it.
 // Measured, clocks an SM and warp at 1.92 GHz with four pairs a thread in flight: the pair alone 37.7, split 24.8 (the
 // integer side's); with one FP64 multiply-add beside each pair, the 2-D step's ratio, 56.2 and 38.2.  The 2-D step at
-// 2048^2: 9.6 -> 13.9 G point-steps/s, the FP64 pipe then 79 % busy.
+// 2048^2: 9.6 -> 13.9 G point-steps/s, the FP64 pipe then 80 % busy.
 #pragma once
 
 #include <stdint.h>

@@ -1049,8 +1049,8 @@ void default_plan(dirac_grid *g) {
     if (ndim_of(g) == 3) {
         // points_per_lane 0: the fused single-pass step; 1, 2 or 4: the x-y pass + z/phase pass with that P.  FP64, bound by
         // its pipe, recomputes no halo rows in the two passes, whose one point a lane splits its sums over both pipes: the
-        // library's choice from about 60^3 (64^3 66.9 us a step against 81.4 fused, 256^3 1855 against 2330, 384^3 6301
-        // against 7281; 48^3 46.5 against 38.1)
+        // library's choice from about 60^3 (64^3 60.5 us a step against 74.3 fused, 256^3 1798 against 2217, 384^3 5999
+        // against 6956)
         const bool two64 = !g->fp32 && !strang(g) && !field_on(g) && k == 0 && pp == 0 && g->ncells > 200000;
         g->plan.fused3d = pp > 0 || two64 ? 0 : 1;
         // FP64: 8-warp blocks, two on an SM (fused3d_kernels.cuh); FP32: 16, short y extents 8 (6-row tiles waste fewer
@@ -1098,9 +1098,9 @@ void default_plan(dirac_grid *g) {
         return;
     }
     // FP64: one point a lane, 16 warps an SM (four blocks of 128 registers): the sweeps' pairs split over the FP64 and
-    // the integer pipe need warps to overlap (2048^2: 13.1 against 10.0 G with two points and 8 warps; second order
-    // 6.35 against 5.1; in a laser field 7.6 against 6.4)
-    // FP32: four steps a launch (2048^2 21.2 us a step against 25.1 with two, 4096^2 70.6 against 87.2, where two move twice
+    // the integer pipe need warps to overlap (2048^2: 13.9 against 10.8 G with two points and 8 warps; second order
+    // 7.1 against 5.5; in a laser field 7.7 against 6.6)
+    // FP32: four steps a launch (2048^2 20.8 us a step against 25.1 with two, 4096^2 70.6 against 87.2, where two move twice
     // the bytes)
     int K = g->fp32 ? (pp == 0 || pp == 2 ? 4 : 2) : 1, P = g->fp32 ? 2 : 1;
     // with a field FP32 first order two (2048^2 43.9 us a step against 61.0 with one, 1000 x 777 12.0 and 17.0, 300^2 6.8 and

@@ -13,7 +13,7 @@
 // issue of about 60 instructions a cell and step (0.0135 us per row and step with R = 4, 0.018 with R = 1: the fewer rows go
 // through shared memory and the more chains a warp has, the better; two cells a lane gave nothing more), with three blocks of
 // 80 registers an SM (1024^2 6.3 -> 6.0 us a step against two, 1300^2 10.5 -> 9.2).
-// Measured, us a step with the face flux, row kernel -> this: FP64 128^2 9.1 -> 4.9, 256^2 12.2 -> 9.0 (second order 32.8 ->
+// Measured, us a step with the face flux, row kernel -> this: FP64 128^2 9.1 -> 4.9, 256^2 12.2 -> 8.8 (second order 32.8 ->
 // 14.9); FP32 128^2 4.2 -> 1.1, 512^2 5.9 -> 2.5, 1024^2 10.2 -> 6.0 (second order 256^2 7.8 -> 2.5); fixed point 256^2 7.2 ->
 // 3.6; in a uniform field, 300^2, FP64 25.0 -> 22.1 (second order 45.8 -> 33.6), FP32 6.6 -> 2.9 (10.9 -> 5.1).  A launch may
 // begin while the one before it drains (256^2 FP32 1.5 -> 1.3 us a step).
